@@ -15,10 +15,10 @@
 //      target;
 //   3. builds the boxes of every level at once: each leaf emits its level-k key where it
 //      heads its level-k row segment, one sort and one unique pass give every level's
-//      boxes; a second sort numbers each level's boxes in parity-class order (class,
-//      problem, (y >> 1, x >> 1) row by row: each class one contiguous range of compact
-//      ids), and one kernel finds parents, children and interaction lists by binary
-//      search;
+//      boxes; one stable partition by (level, class) numbers each level's boxes in
+//      parity-class order (class, problem, (y >> 1, x >> 1) row by row: each class one
+//      contiguous range of compact ids), and one kernel finds parents, children and
+//      interaction lists by binary search;
 //   4. lists the near-field strips (SW consecutive leaves of a row holding a target) and
 //      the occupied leaves of each strip's three neighbour-row segments.
 // The sorts are a stable least-significant-digit radix sort (8-bit digits, per-block
@@ -231,21 +231,28 @@ struct SortBufs {
 
 int64_t sort_hist_ints(int64_t n) { return (int64_t)kRadix * ((n + kTile - 1) / kTile) + 1; }
 
+// One stable pass over the digit at `shift`: (ki, vi) -> (ko, vo); values optional.
+cudaError_t radix_pass(const uint64_t* ki, const uint32_t* vi, uint64_t* ko, uint32_t* vo, int64_t n, int shift,
+                       SortBufs& b, cudaStream_t s) {
+    const int nblocks = (int)((n + kTile - 1) / kTile);
+    radix_hist_kernel<<<nblocks, kT, 0, s>>>(ki, n, shift, nblocks, b.hist);
+    cudaError_t e = exscan(b.hist, b.hist, (int64_t)kRadix * nblocks, b.sums, s);
+    if (e != cudaSuccess) return e;
+    radix_scatter_kernel<<<nblocks, kT, 0, s>>>(ki, vi, ko, vo, n, shift, nblocks, b.hist);
+    return cudaGetLastError();
+}
+
 // Sorts n keys (and values, when v is set) by their low `bits` bits (bits <= 64; the
 // keys hold no higher bits), stably, in place: the passes alternate between (k, v) and
 // the scratch, and after an odd number of them one copy brings the result back.
 cudaError_t radix_sort(uint64_t* k, uint32_t* v, int64_t n, int bits, SortBufs& b, cudaStream_t s) {
     if (n <= 1) return cudaSuccess;
-    const int nblocks = (int)((n + kTile - 1) / kTile);
     const int passes = std::max(1, (bits + 7) / 8);
     uint64_t *ki = k, *ko = b.k2;
     uint32_t *vi = v, *vo = v ? b.v2 : nullptr;
     for (int pass = 0; pass < passes; ++pass) {
-        const int shift = 8 * pass;
-        radix_hist_kernel<<<nblocks, kT, 0, s>>>(ki, n, shift, nblocks, b.hist);
-        cudaError_t e = exscan(b.hist, b.hist, (int64_t)kRadix * nblocks, b.sums, s);
+        cudaError_t e = radix_pass(ki, vi, ko, vo, n, 8 * pass, b, s);
         if (e != cudaSuccess) return e;
-        radix_scatter_kernel<<<nblocks, kT, 0, s>>>(ki, vi, ko, vo, n, shift, nblocks, b.hist);
         std::swap(ki, ko);
         std::swap(vi, vo);
     }
@@ -466,8 +473,11 @@ __global__ void head_key_kernel(const uint64_t* __restrict__ leaves, int64_t m, 
     }
 }
 
-// class-major key (k, class, problem, y >> 1, x >> 1) of every box of every level (value:
-// its position in the level-major row-major key array A)
+// Partition key 4 k + class of every box of every level (value: its position in the
+// level-major row-major key array A).  A is ordered by (level, problem, row, column), so a
+// stable partition by this one digit leaves every class in (problem, y >> 1, x >> 1) order:
+// one radix pass instead of a sort by the whole (class, box) key (five passes at 14 levels;
+// clustered_4m builds 1.3 M boxes).
 __global__ void class_key_kernel(const uint64_t* __restrict__ A, int64_t n, int kb, int kbits,
                                  uint64_t* __restrict__ ck, uint32_t* __restrict__ idx) {
     const uint64_t low = ((uint64_t)1 << kbits) - 1;
@@ -477,13 +487,13 @@ __global__ void class_key_kernel(const uint64_t* __restrict__ A, int64_t n, int 
         int p, y, x;
         unpack_key(key & low, kb, p, y, x);
         const uint64_t c = (uint64_t)((x & 1) | ((y & 1) << 1));
-        ck[g] = (k << (kbits + 2)) | (c << kbits) | pack_key(p, y >> 1, x >> 1, kb);
+        ck[g] = (k << 2) | c;
         idx[g] = (uint32_t)g;
     }
 }
 
 // first class-major position of class c of level k (entry 4 k + c; entry 4 nk: all boxes)
-__global__ void class_starts_kernel(const uint64_t* __restrict__ ck, int64_t n, int nk, int kbits,
+__global__ void class_starts_kernel(const uint64_t* __restrict__ ck, int64_t n, int nk,
                                     int64_t* __restrict__ cstart) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t > 4 * nk) return;
@@ -491,8 +501,7 @@ __global__ void class_starts_kernel(const uint64_t* __restrict__ ck, int64_t n, 
         cstart[t] = n;
         return;
     }
-    const uint64_t v = ((uint64_t)(t >> 2) << (kbits + 2)) | ((uint64_t)(t & 3) << kbits);
-    cstart[t] = lower_bound_key(ck, n, v);
+    cstart[t] = lower_bound_key(ck, n, (uint64_t)t);
 }
 
 // Box b of the class-major order (all levels, level-major) <- its row-major entry cm[b]
@@ -504,7 +513,7 @@ __global__ void box_records_kernel(const uint64_t* __restrict__ A, const uint64_
                                    int32_t* __restrict__ local_of, int32_t* __restrict__ leaf_rl) {
     const uint64_t low = ((uint64_t)1 << kbits) - 1;
     for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b < n; b += (int64_t)gridDim.x * blockDim.x) {
-        const int k = (int)(ck[b] >> (kbits + 2));
+        const int k = (int)(ck[b] >> 2);
         const uint32_t g = cm[b];
         int p, y, x;
         unpack_key(A[g] & low, kb, p, y, x);
@@ -537,7 +546,7 @@ __global__ void links_kernel(int64_t n, const uint64_t* __restrict__ ck, const u
     __syncthreads();
     const uint64_t cmask = ((uint64_t)1 << kb) - 1;
     for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b < n; b += (int64_t)gridDim.x * blockDim.x) {
-        const int k = (int)(ck[b] >> (kbits + 2));
+        const int k = (int)(ck[b] >> 2);
         const int p = bp[b];
         const int x = bxy[b] & 0xffff, y = bxy[b] >> 16;
         const int l = L[p] - k;
@@ -670,24 +679,31 @@ __global__ void same_points_kernel(const int2* __restrict__ a, const int2* __res
     }
 }
 
-// strip key (problem, leaf row, column / SW) of each occupied leaf with a target, the
-// skip value for the others (non-decreasing over the target leaves: leaves are row-major)
-__global__ void strip_key_kernel(const uint64_t* __restrict__ leaves, const int32_t* __restrict__ rt, int64_t m,
-                                 int kb, int SW, uint64_t skip, uint64_t* __restrict__ out) {
+// Strip (problem, leaf row, column / SW) of each occupied leaf: 1 where the leaf is the
+// strip's first one with a target.  Leaves are row-major, so a strip's leaves are
+// consecutive and at most SW of them: the leaves before this one in its strip are looked
+// at directly, and no sort has to bring the strips together.
+__global__ void strip_flag_kernel(const uint64_t* __restrict__ leaves, const int32_t* __restrict__ rt, int64_t m,
+                                  int kb, int SW, int32_t* __restrict__ flag) {
     for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x) {
         int p, y, x;
         unpack_key(leaves[j], kb, p, y, x);
-        out[j] = rt[j + 1] > rt[j] ? pack_key(p, y, x / SW, kb) : skip;
+        const uint64_t first = pack_key(p, y, x / SW * SW, kb);
+        bool head = rt[j + 1] > rt[j];
+        for (int64_t i = j - 1; head && i >= 0 && leaves[i] >= first; --i) head = rt[i + 1] == rt[i];
+        flag[j] = head ? 1 : 0;
     }
 }
 
-// strip records (problem, leaf row, first column, 0)
-__global__ void strip_record_kernel(const uint64_t* __restrict__ sk, int64_t m, int kb, int SW,
+// strip records (problem, leaf row, first column, 0), in the order of their first leaves
+__global__ void strip_record_kernel(const uint64_t* __restrict__ leaves, const int32_t* __restrict__ flag,
+                                    const int32_t* __restrict__ pos, int64_t m, int kb, int SW,
                                     int4* __restrict__ strips) {
     for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x) {
+        if (!flag[j]) continue;
         int p, y, x;
-        unpack_key(sk[j], kb, p, y, x);
-        strips[j] = make_int4(p, y, x * SW, 0);
+        unpack_key(leaves[j], kb, p, y, x);
+        strips[pos[j]] = make_int4(p, y, x / SW * SW, 0);
     }
 }
 
@@ -1116,10 +1132,12 @@ int forest_build(Forest& F, const int32_t* src, const int64_t* soff_h, int64_t n
         timer->add_launches(4 + 5 * ((kbits + lbits + 7) / 8));
     }
     const int64_t NB = (int64_t)M + U;
-    // class-major order of every level
+    // class-major order of every level (4 nk <= 84 partition keys: one digit)
     class_key_kernel<<<grid_of(NB), kT, 0, s>>>(A, NB, kb, kbits, ck, cidx);
     LFMM_CUDA_TRY(cudaGetLastError());
-    LFMM_CUDA_TRY(radix_sort(ck, cidx, NB, kbits + 2 + lbits, lsb, s));
+    LFMM_CUDA_TRY(radix_pass(ck, cidx, lsb.k2, lsb.v2, NB, 0, lsb, s));
+    std::swap(ck, lsb.k2);
+    std::swap(cidx, lsb.v2);
     // per-box records of all levels in one allocation (level k at box_off[k])
     if ((st = alloc(F, &vp, (size_t)NB * (3 + 27 + 4) * sizeof(int32_t) + (size_t)M * sizeof(int32_t) +
                                 (size_t)(4 * nk + 1 + 5 * nk) * sizeof(int64_t) + 16, s)))
@@ -1132,7 +1150,7 @@ int forest_build(Forest& F, const int32_t* src, const int64_t* soff_h, int64_t n
     int32_t* il_all = par_all + NB;
     int32_t* ch_all = il_all + 27 * NB;
     int32_t* leaf_rl = ch_all + 4 * NB;
-    class_starts_kernel<<<(4 * nk + 1 + kT - 1) / kT, kT, 0, s>>>(ck, NB, nk, kbits, cstart);
+    class_starts_kernel<<<(4 * nk + 1 + kT - 1) / kT, kT, 0, s>>>(ck, NB, nk, cstart);
     box_records_kernel<<<grid_of(NB), kT, 0, s>>>(A, ck, cidx, NB, cstart, kb, kbits, bp_all, bxy_all, local_of, leaf_rl);
     // the [first, end) of every box row of A, so that the links' searches (parent, two child
     // rows, six neighbour rows per box) cover one row instead of all of A; without it (a
@@ -1165,7 +1183,7 @@ int forest_build(Forest& F, const int32_t* src, const int64_t* soff_h, int64_t n
                                             row_off, np, par_all, ch_all, il_all);
     LFMM_CUDA_TRY(cudaGetLastError());
     LFMM_CUDA_TRY(cudaMemcpyAsync(F.rl_id, local_of, (size_t)M * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
-    timer->add_launches(4 + 5 * ((kbits + 2 + lbits + 7) / 8));
+    timer->add_launches(4 + 5);
     // class ranges of every level
     {
         std::vector<int64_t> hc((size_t)4 * nk + 1);
@@ -1199,24 +1217,21 @@ int forest_build(Forest& F, const int32_t* src, const int64_t* soff_h, int64_t n
                                                    " sources / " + std::to_string(mtg) + " targets)");
     F.SW = SW;
     {
-        // strip keys of the target leaves (the others: the skip value, sorted to the end)
-        const uint64_t skip = 1ull << kbits;  // above every key
-        strip_key_kernel<<<grid_of(M), kT, 0, s>>>(F.rl_key, F.rl_t, M, kb, SW, skip, kspare);
-        LFMM_CUDA_TRY(cudaGetLastError());
-        LFMM_CUDA_TRY(radix_sort(kspare, nullptr, M, kbits + 1, sbuf, s));
-        int nstr = 0;
-        if ((st = unique_runs(kspare, M, skip, ukeys, nullptr, flag, pos, ssum, &nstr, s))) return st;
+        strip_flag_kernel<<<grid_of(M), kT, 0, s>>>(F.rl_key, F.rl_t, M, kb, SW, flag);
+        LFMM_CUDA_TRY(exscan(flag, pos, M, ssum, s));
+        int32_t nstr = 0;
+        LFMM_CUDA_TRY(cudaMemcpyAsync(&nstr, pos + M, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+        LFMM_CUDA_TRY(cudaStreamSynchronize(s));
         const size_t n4 = (size_t)std::max(nstr, 1);
         if ((st = alloc(F, &vp, 3 * n4 * sizeof(int4) + 16, s))) return st;
         F.strips = (int4*)vp;
         F.strip_rows = F.strips + n4;
         F.n_strips_d = (int32_t*)(F.strip_rows + 2 * n4);
-        const int32_t ns32 = nstr;
-        LFMM_CUDA_TRY(cudaMemcpyAsync(F.n_strips_d, &ns32, sizeof(int32_t), cudaMemcpyHostToDevice, s));
-        strip_record_kernel<<<grid_of(nstr), kT, 0, s>>>(ukeys, nstr, kb, SW, F.strips);
+        LFMM_CUDA_TRY(cudaMemcpyAsync(F.n_strips_d, pos + M, sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
+        strip_record_kernel<<<grid_of(M), kT, 0, s>>>(F.rl_key, flag, pos, M, kb, SW, F.strips);
         strip_rows_kernel<<<grid_of(nstr), kT, 0, s>>>(F.strips, nstr, F.rl_key, M, dL, kb, SW, F.strip_rows);
         LFMM_CUDA_TRY(cudaGetLastError());
-        timer->add_launches(7 + 5 * ((kbits + 8) / 8));
+        timer->add_launches(6);
     }
     return LFMM_OK;  // temporaries are freed in stream order
 }
