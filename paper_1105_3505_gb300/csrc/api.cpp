@@ -381,8 +381,8 @@ int plan_build(lfmm_plan* p, const int32_t* src_xy, const int32_t* tgt_xy, cudaS
     while (((int64_t)nleaf << (2 * L_pig)) < nmax) ++L_pig;
     const int Lf_guess = L_pig + 1;
     Temp t4;
-    if ((st = talloc(t4, 10 * sizeof(int), s))) return st;
-    int* d4 = (int*)t4.ptr;
+    if ((st = talloc(t4, 11 * sizeof(int), s))) return st;
+    int* d4 = (int*)t4.ptr;  // bounding box, then the six words of the counts, then targets-differ
     Temp ranks;  // each point's arrival rank in its box of level Lf_last
     if ((st = talloc(ranks, (size_t)(p->ns + p->nt) * sizeof(int32_t), s))) return st;
     Temp guess;  // counts at level Lf_guess: [fine src][fine tgt][coarse src][coarse tgt]
@@ -395,7 +395,8 @@ int plan_build(lfmm_plan* p, const int32_t* src_xy, const int32_t* tgt_xy, cudaS
     tree_timer->add_launches(2);
     if (have_guess) {
         int32_t* fs = (int32_t*)guess.ptr;
-        LFMM_CUDA_TRY(launch_histogram_bbox(src, p->ns, tgt, p->nt, d4, Lf_guess, fs, fs + nf_g,
+        LFMM_CUDA_TRY(launch_histogram_bbox(src, p->ns, tgt, p->nt, d4, Lf_guess,
+                                            ilog2_ceil(p->opts.max_leaf_side), fs, fs + nf_g,
                                             (int32_t*)ranks.ptr, s));
         LFMM_CUDA_TRY(launch_coarsen(fs, fs + nf_g, nc_g, fs + 2 * nf_g, fs + 2 * nf_g + nc_g, d4 + 4, s));
         tree_timer->add_launches(2);
@@ -428,6 +429,11 @@ int plan_build(lfmm_plan* p, const int32_t* src_xy, const int32_t* tgt_xy, cudaS
     int chosen = -1;
     int early_side = 0;    // > 0: pruned storage decided on the way, the builder's first leaf side
     int64_t nonempty = 1;  // leaves holding a source or a target at the chosen level
+    // counting again: targets that are the sources are counted once (a device word tells the
+    // kernels, so no round trip).  clustered_4m counts 4^13 boxes: zeroing, counting and
+    // coarsening both arrays took 365 us, one array 190 us
+    int* differ = d4 + 10;
+    bool differ_known = false, same = false;
     for (;;) {
         if (Lf > kMaxLevel)
             return fail(LFMM_EUNSUPPORTED, "tree would need more than 4^14 leaves");
@@ -435,7 +441,7 @@ int plan_build(lfmm_plan* p, const int32_t* src_xy, const int32_t* tgt_xy, cudaS
         const int64_t nc = Lf >= 1 ? nf / 4 : 0;
         Temp c2;
         // [max fine src, max fine tgt, max coarse src, max coarse tgt, non-empty fine, non-empty coarse]
-        int m4[6] = {(int)std::min<int64_t>(p->ns, INT_MAX), (int)std::min<int64_t>(p->nt, INT_MAX), 0, 0, 1, 1};
+        int m4[7] = {(int)std::min<int64_t>(p->ns, INT_MAX), (int)std::min<int64_t>(p->nt, INT_MAX), 0, 0, 1, 1, 1};
         if (have_guess && Lf == Lf_guess) {  // counted with the bounding box
             c2.ptr = guess.ptr;
             c2.s = s;
@@ -444,23 +450,35 @@ int plan_build(lfmm_plan* p, const int32_t* src_xy, const int32_t* tgt_xy, cudaS
         } else {
             if ((st = talloc(c2, (size_t)(2 * nf + 2 * nc) * sizeof(int32_t), s))) return st;
             int32_t* f0 = (int32_t*)c2.ptr;
-            LFMM_CUDA_TRY(cudaMemsetAsync(f0, 0, (size_t)2 * nf * sizeof(int32_t), s));
+            const bool may_be_same = p->ns == p->nt && Lf >= 1;
+            LFMM_CUDA_TRY(cudaMemsetAsync(d4 + 4, 0, (differ_known ? 6 : 7) * sizeof(int), s));
+            if (may_be_same) {
+                if (!differ_known && src != tgt) {
+                    LFMM_CUDA_TRY(launch_differ(src, tgt, p->ns, differ, s));
+                    tree_timer->add_launches(1);
+                }
+                differ_known = true;
+                LFMM_CUDA_TRY(launch_zero_counts(f0, f0 + nf, nf, differ, s));
+            } else {
+                LFMM_CUDA_TRY(cudaMemsetAsync(f0, 0, (size_t)2 * nf * sizeof(int32_t), s));
+            }
             LFMM_CUDA_TRY(launch_histogram(src, p->ns, tgt, p->nt, p->x0, p->y0, p->K - Lf, f0, f0 + nf, s,
-                                           (int32_t*)ranks.ptr));
+                                           (int32_t*)ranks.ptr, may_be_same ? differ : nullptr));
             tree_timer->add_launches(1);
             if (Lf >= 1) {
-                LFMM_CUDA_TRY(cudaMemsetAsync(d4 + 4, 0, 6 * sizeof(int), s));
-                LFMM_CUDA_TRY(launch_coarsen(f0, f0 + nf, nc, f0 + 2 * nf, f0 + 2 * nf + nc, d4 + 4, s));
+                LFMM_CUDA_TRY(launch_coarsen(f0, f0 + nf, nc, f0 + 2 * nf, f0 + 2 * nf + nc, d4 + 4, s,
+                                             may_be_same ? differ : nullptr));
                 tree_timer->add_launches(1);
                 LFMM_CUDA_TRY(cudaMemcpyAsync(m4, d4 + 4, sizeof(m4), cudaMemcpyDeviceToHost, s));
                 LFMM_CUDA_TRY(cudaStreamSynchronize(s));
+                same = may_be_same && m4[6] == 0;
             }
         }
         have_guess = false;  // a later pass counts again (and overwrites the ranks)
         int32_t* fs = (int32_t*)c2.ptr;
-        int32_t* ft = fs + nf;
-        int32_t* ccs = ft + nf;
-        int32_t* cct = ccs + nc;
+        int32_t* ft = same ? fs : fs + nf;
+        int32_t* ccs = fs + 2 * nf;
+        int32_t* cct = same ? ccs : ccs + nc;
         // Clustered input: more than half of the boxes of the coarse level counted here are
         // empty, hence of every finer level too (a non-empty box has a non-empty parent), so
         // automatic storage is pruned whatever the leaf level turns out to be.  The forest
@@ -551,7 +569,7 @@ int plan_build(lfmm_plan* p, const int32_t* src_xy, const int32_t* tgt_xy, cudaS
         }
     }
     LFMM_CUDA_TRY(launch_scatter_ranked(tgt, p->nt, p->x0, p->y0, p->K, p->L, Lf_last, p->tgt_begin, ft_last,
-                                        (const int32_t*)ranks.ptr + p->ns, p->tgt_loc, p->tgt_perm, ts, p->tgt_leaf));
+                                        (const int32_t*)ranks.ptr + (same ? 0 : p->ns), p->tgt_loc, p->tgt_perm, ts, p->tgt_leaf));
     if (ts != s) {
         LFMM_CUDA_TRY(cudaEventRecord(p->tgt_ready, ts));
         ranks.s = ts;  // freed behind the target scatter

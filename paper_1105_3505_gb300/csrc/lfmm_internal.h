@@ -338,7 +338,13 @@ cudaError_t launch_bbox(const int32_t* a, int64_t na, const int32_t* b, int64_t 
 // ns + nt entries, sources first) receives each point's arrival rank in its box.
 cudaError_t launch_histogram(const int32_t* src, int64_t ns, const int32_t* tgt, int64_t nt,
                              int64_t x0, int64_t y0, int shift, int32_t* cnt_src,
-                             int32_t* cnt_tgt, cudaStream_t s, int32_t* rank = nullptr);
+                             int32_t* cnt_tgt, cudaStream_t s, int32_t* rank = nullptr,
+                             const int* differ = nullptr);
+// *differ (preset to 0 by the caller) = 1 if the two point lists differ.  With a device word
+// `differ` that stays 0, launch_histogram and launch_coarsen count the sources alone, and
+// launch_zero_counts (n a multiple of 4) zeroes the first array alone.
+cudaError_t launch_differ(const int32_t* a, const int32_t* b, int64_t n, int* differ, cudaStream_t s);
+cudaError_t launch_zero_counts(int32_t* a, int32_t* b, int64_t n, const int* differ, cudaStream_t s);
 // Leaf buckets from histogram ranks taken at level Lf (L or L + 1; fine = that level's
 // Morton counts): no atomics.
 cudaError_t launch_scatter_ranked(const int32_t* xy, int64_t n, int64_t x0, int64_t y0, int K, int L, int Lf,
@@ -348,11 +354,12 @@ cudaError_t launch_scatter_ranked(const int32_t* xy, int64_t n, int64_t x0, int6
 // largest fine source / target count and the largest coarse ones, max4[4..5] (atomic
 // add) the number of non-empty fine and coarse boxes.  max4 must be zeroed first.
 // Counts at level Lf with the root box taken from the device bbox words {min x, min y,
-// max x, max y} (no host round trip); ranks always recorded; nothing counted if K < Lf.
+// max x, max y} (no host round trip); ranks always recorded; nothing counted unless Lf is
+// the level that plan_build counts first (leaf sides up to 2^ls).
 cudaError_t launch_histogram_bbox(const int32_t* src, int64_t ns, const int32_t* tgt, int64_t nt, const int* bbox4,
-                                  int Lf, int32_t* cs, int32_t* ct, int32_t* rank, cudaStream_t s);
+                                  int Lf, int ls, int32_t* cs, int32_t* ct, int32_t* rank, cudaStream_t s);
 cudaError_t launch_coarsen(const int32_t* fs, const int32_t* ft, int64_t n_coarse, int32_t* cs,
-                           int32_t* ct, int* max4, cudaStream_t s);
+                           int32_t* ct, int* max4, cudaStream_t s, const int* differ = nullptr);
 // Exclusive scan over the 4^L leaves in row-major order of two Morton-indexed count
 // arrays; out has 4^L + 1 entries.
 cudaError_t launch_scan2(const int32_t* in_a, int32_t* out_a, const int32_t* in_b,

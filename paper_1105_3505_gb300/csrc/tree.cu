@@ -88,12 +88,14 @@ __device__ __forceinline__ uint32_t box_of(int2 p, int64_t x0, int64_t y0, int s
 // Counts points per box; with `rank` set, also records each point's arrival rank in
 // its box (the value its atomic increment returned), which places it in its bucket
 // later without a second atomic pass.
+// differ (optional): 0 when the targets are the sources; only the sources are then counted.
 __global__ void histogram_kernel(const int2* __restrict__ src, int64_t ns,
                                  const int2* __restrict__ tgt, int64_t nt, int64_t x0,
                                  int64_t y0, int shift, int32_t* __restrict__ cs,
-                                 int32_t* __restrict__ ct, int32_t* __restrict__ rank) {
+                                 int32_t* __restrict__ ct, int32_t* __restrict__ rank,
+                                 const int* __restrict__ differ) {
     griddep_wait();
-    const int64_t n = ns + nt;
+    const int64_t n = ns + (differ && *differ == 0 ? 0 : nt);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
         const int r = i < ns ? atomicAdd(cs + box_of(src[i], x0, y0, shift), 1)
@@ -104,17 +106,20 @@ __global__ void histogram_kernel(const int2* __restrict__ src, int64_t ns,
 
 // The same counts at level Lf before the host has read the bounding box: the root box
 // (corner and side 2^K, K the smallest with 2^K >= the larger extent) comes from the
-// bbox words the previous kernel wrote.  Nothing is counted when K < Lf (the host then
-// finds that level Lf was the wrong guess and counts again).
+// bbox words the previous kernel wrote.  Nothing is counted when the leaf-side bound 2^ls
+// or the root puts the first level to count elsewhere (the host finds the same from the
+// same words and counts that level): on clustered_4m (17-bit root, 4^9 cells guessed, 4^13
+// needed) the wasted count had cost 140 us.
 __global__ void histogram_bbox_kernel(const int2* __restrict__ src, int64_t ns, const int2* __restrict__ tgt,
-                                      int64_t nt, const int* __restrict__ bbox4, int Lf, int32_t* __restrict__ cs,
+                                      int64_t nt, const int* __restrict__ bbox4, int Lf, int ls,
+                                      int32_t* __restrict__ cs,
                                       int32_t* __restrict__ ct, int32_t* __restrict__ rank) {
     griddep_wait();
     const int64_t x0 = bbox4[0], y0 = bbox4[1];
     const int64_t ext = max((int64_t)bbox4[2] - x0, (int64_t)bbox4[3] - y0) + 1;
     if (ext < 1) return;
     const int K = ext <= 1 ? 0 : 64 - __clzll((unsigned long long)(ext - 1));
-    if (K < Lf) return;
+    if (min(K, max(K - ls, Lf - 1) + 1) != Lf) return;
     const int shift = K - Lf;
     const int64_t n = ns + nt;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
@@ -152,18 +157,20 @@ __global__ void scatter_ranked_kernel(const int2* __restrict__ xy, int64_t n, in
 }
 
 // coarse[b] = sum of fine[4b..4b+3]; max4 = {max fine src, max fine tgt, max coarse src,
-// max coarse tgt}.
+// max coarse tgt}.  differ (optional): 0 when the targets are the sources, whose counts
+// then stand for both (ft is not read, ct not written).
 __global__ void coarsen_kernel(const int4* __restrict__ fs, const int4* __restrict__ ft,
                                int64_t n_coarse, int32_t* __restrict__ cs,
-                               int32_t* __restrict__ ct, int* __restrict__ max4) {
+                               int32_t* __restrict__ ct, int* __restrict__ max4, const int* __restrict__ differ) {
     griddep_wait();
+    const bool same = differ && *differ == 0;
     int m0 = 0, m1 = 0, m2 = 0, m3 = 0, nf = 0, nc = 0;
     for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b < n_coarse;
          b += (int64_t)gridDim.x * blockDim.x) {
-        const int4 s = fs[b], t = ft[b];
+        const int4 s = fs[b], t = same ? s : ft[b];
         const int ss = s.x + s.y + s.z + s.w, tt = t.x + t.y + t.z + t.w;
         cs[b] = ss;
-        ct[b] = tt;
+        if (!same) ct[b] = tt;
         m0 = max(m0, max(max(s.x, s.y), max(s.z, s.w)));
         m1 = max(m1, max(max(t.x, t.y), max(t.z, t.w)));
         m2 = max(m2, ss);
@@ -299,6 +306,29 @@ __global__ void scatter_kernel(const int2* __restrict__ xy, int64_t n, int64_t x
     }
 }
 
+// *differ = 1 if the two point lists differ anywhere (else left as it is)
+__global__ void differ_kernel(const int2* __restrict__ a, const int2* __restrict__ b, int64_t n,
+                              int* __restrict__ differ) {
+    griddep_wait();
+    bool d = false;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const int2 u = a[i], v = b[i];
+        d |= u.x != v.x || u.y != v.y;
+    }
+    if (d) *differ = 1;
+}
+
+// n16 16-byte words of zeros at a, and as many at b unless *differ is 0
+__global__ void zero_counts_kernel(int4* __restrict__ a, int4* __restrict__ b, int64_t n16,
+                                   const int* __restrict__ differ) {
+    griddep_wait();
+    const bool both = *differ != 0;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n16; i += (int64_t)gridDim.x * blockDim.x) {
+        a[i] = make_int4(0, 0, 0, 0);
+        if (both) b[i] = make_int4(0, 0, 0, 0);
+    }
+}
+
 __global__ void set4_kernel(int* p, int a, int b, int c, int d) {
     p[0] = a;
     p[1] = b;
@@ -344,16 +374,16 @@ cudaError_t launch_bbox(const int32_t* a, int64_t na, const int32_t* b, int64_t 
 
 cudaError_t launch_histogram(const int32_t* src, int64_t ns, const int32_t* tgt, int64_t nt,
                              int64_t x0, int64_t y0, int shift, int32_t* cs, int32_t* ct,
-                             cudaStream_t s, int32_t* rank) {
+                             cudaStream_t s, int32_t* rank, const int* differ) {
     (void)launch_dependent(histogram_kernel, dim3(grid_for(ns + nt, kThreads)), dim3(kThreads), 0, s,
-        (const int2*)src, ns, (const int2*)tgt, nt, x0, y0, shift, cs, ct, rank);
+        (const int2*)src, ns, (const int2*)tgt, nt, x0, y0, shift, cs, ct, rank, differ);
     return cudaGetLastError();
 }
 
 cudaError_t launch_histogram_bbox(const int32_t* src, int64_t ns, const int32_t* tgt, int64_t nt, const int* bbox4,
-                                  int Lf, int32_t* cs, int32_t* ct, int32_t* rank, cudaStream_t s) {
+                                  int Lf, int ls, int32_t* cs, int32_t* ct, int32_t* rank, cudaStream_t s) {
     return launch_dependent(histogram_bbox_kernel, dim3(grid_for(ns + nt, kThreads)), dim3(kThreads), 0, s,
-                            (const int2*)src, ns, (const int2*)tgt, nt, bbox4, Lf, cs, ct, rank);
+                            (const int2*)src, ns, (const int2*)tgt, nt, bbox4, Lf, ls, cs, ct, rank);
 }
 
 cudaError_t launch_scatter_ranked(const int32_t* xy, int64_t n, int64_t x0, int64_t y0, int K, int L, int Lf,
@@ -364,9 +394,19 @@ cudaError_t launch_scatter_ranked(const int32_t* xy, int64_t n, int64_t x0, int6
 }
 
 cudaError_t launch_coarsen(const int32_t* fs, const int32_t* ft, int64_t n_coarse, int32_t* cs,
-                           int32_t* ct, int* max4, cudaStream_t s) {
+                           int32_t* ct, int* max4, cudaStream_t s, const int* differ) {
     return launch_dependent(coarsen_kernel, dim3(grid_for(n_coarse, kThreads)), dim3(kThreads), 0, s,
-                            (const int4*)fs, (const int4*)ft, n_coarse, cs, ct, max4);
+                            (const int4*)fs, (const int4*)ft, n_coarse, cs, ct, max4, differ);
+}
+
+cudaError_t launch_differ(const int32_t* a, const int32_t* b, int64_t n, int* differ, cudaStream_t s) {
+    return launch_dependent(differ_kernel, dim3(grid_for(n, kThreads)), dim3(kThreads), 0, s, (const int2*)a,
+                            (const int2*)b, n, differ);
+}
+
+cudaError_t launch_zero_counts(int32_t* a, int32_t* b, int64_t n, const int* differ, cudaStream_t s) {
+    return launch_dependent(zero_counts_kernel, dim3(grid_for(n / 4, kThreads)), dim3(kThreads), 0, s, (int4*)a,
+                            (int4*)b, n / 4, differ);
 }
 
 size_t scan_partials_size(int64_t n) {
