@@ -54,11 +54,13 @@ extern "C" {
 /* LFMM_FP64: every step in binary64 (the plain path, relative error <= 1e-10 at p >= 16).
  * LFMM_MIXED: near field, expansions and translations in binary32, charges rounded
  *   to binary32, the per-target sum of near and far parts in binary64 (<= 1e-6). */
-#define LFMM_FP64 0   /* every step in binary64                                         */
+#define LFMM_FP64 0   /* every step in binary64 (translations at p > 9: products of       */
+                      /* 53-bit operands split exactly over fp16 tensor-core products)    */
 #define LFMM_MIXED 1  /* binary32 near and far field, compensated charge channel, TF32    */
                       /* tensor-core M2L; binary64 final sum (relative error ~1e-7)       */
 #define LFMM_DF 2     /* binary64 inputs and outputs, every step in float-float pairs     */
-                      /* (~48 bits) on the FP32 pipes: binary64-level accuracy at a       */
+                      /* (~48 bits) on the FP32 pipes, translations at p > 9 in 53-bit    */
+                      /* split operands on the tensor cores: binary64-level accuracy at a */
                       /* fraction of the binary64 pipe's cost                             */
 
 typedef struct lfmm_plan lfmm_plan;
@@ -75,7 +77,10 @@ typedef struct lfmm_opts {
     int32_t tc_min_level;     /* mixed path: tree levels >= this run M2L on the tensor cores  */
                               /* (0 = default 6; a value > 30 disables them); pruned storage  */
                               /* and forests: every list level of >= 1024 boxes runs there    */
-                              /* unless this is > 30                                          */
+                              /* unless this is > 30.  Binary64 and float-float at p > 9: the */
+                              /* whole far field of pruned trees and forests, and of uniform  */
+                              /* trees whose leaf level is >= this, runs there in exactly     */
+                              /* split operands unless this is > 30                           */
     int32_t tree;             /* LFMM_TREE_AUTO, LFMM_TREE_UNIFORM or LFMM_TREE_PRUNED         */
     int32_t flags;            /* bitwise OR of LFMM_FLAG_* (0: none)                           */
     /* M2L tiling (0 everywhere: the library's rules; lfmm_autotune picks these).  They    */
@@ -115,7 +120,8 @@ typedef struct lfmm_opts {
  * levels of at least 1,024 boxes, as in the default form).  The results are
  * bit-identical either way; on the 4,096-problem forest the two forms measured within
  * 1 % of each other (per-level launches slightly ahead), and per-level launches are the
- * default. */
+ * default.  No effect on binary64 and float-float plans whose far field runs on the
+ * tensor cores (tc_min_level above). */
 #define LFMM_FLAG_PERSISTENT 4
 
 /* Tree storage.  UNIFORM: every box of every level is stored (Sec. 6), the layout for

@@ -7,6 +7,7 @@
 #include <new>
 
 #include "lfmm_internal.h"
+#include "split_tc.h"
 
 namespace lfmm {
 
@@ -75,6 +76,7 @@ struct lfmm_plan {
     int64_t m2l_part_bytes = 0;
     int m2l_part_nvec = 0;         // vectors the buffer has been sized for
     std::unique_ptr<Forest> forest;  // pruned tree or forest (null: uniform tree)
+    void* sg_work = nullptr;         // work space of the sliced far field (split_tc.h)
     void* tc_split = nullptr;        // TF32 hi/lo copies of q_hat and the parent u_hat for the tensor cores
     double* un_tmp = nullptr;        // near field per target (caller order) from the concurrent near-field pass
     double* uf_tmp = nullptr;        // far field per target (caller order), before the final sum
@@ -344,6 +346,12 @@ int forest_workspaces(lfmm_plan* p, cudaStream_t s) {
         if (need > 0 && (st = palloc(p, &b, (size_t)need * sizeof(float), s))) return st;
         F.tc_split = (float*)b;
     }
+    // sliced far field of the binary64-accurate paths (split_tc.cu)
+    if (F.kmax >= 0 && (int)F.levels.size() <= kSgMaxLevels &&
+        sg_applies(p->opts.precision, p->NP, p->opts.tc_min_level)) {
+        const int64_t need = sg_work_bytes(forest_sg_tree(F), p->opts.precision, p->num_sms);
+        if ((st = palloc(p, &F.sg_work, (size_t)need, s))) return st;
+    }
     if ((st = palloc(p, &p->Qbox, (size_t)boxes * 8, s))) return st;
     if ((st = palloc(p, &p->Cbox, (size_t)boxes * 8, s))) return st;
     void* stbuf;
@@ -608,6 +616,10 @@ int plan_build(lfmm_plan* p, const int32_t* src_xy, const int32_t* tgt_xy, cudaS
     if ((st = palloc(p, &p->uhat, (size_t)boxes * p->NP * esz, s))) return st;
     if ((st = palloc(p, &p->Qbox, (size_t)boxes * 8, s))) return st;
     if ((st = palloc(p, &p->Cbox, (size_t)boxes * 8, s))) return st;
+    if (sg_applies_uniform(p->opts.precision, p->NP, p->L, p->opts.tc_min_level) &&
+        (st = palloc(p, &p->sg_work,
+                     (size_t)sg_work_bytes(sg_uniform_tree(p->L, p->opts.m2l_split), p->opts.precision, p->num_sms), s)))
+        return st;
     if (p->L >= 2) {  // a far field: near and far parts go to these buffers, then one sum
         void* b;
         if ((st = palloc(p, &b, (size_t)2 * p->nt * sizeof(double), s))) return st;
@@ -697,6 +709,21 @@ int far_sweeps(lfmm_plan* p, const FarBufs& b, cudaStream_t s, Hook before_fine)
                     LFMM_CUDA_TRY(launch_m2m<T>(ops, L - l, l, Qx(l + 1, v), Qm(l + 1, v), Qx(l, v), Qm(l, v), s));
                     pt.add_launches(1);
                 }
+        }
+    }
+    if constexpr (sizeof(T) == 8) {
+        if (p->sg_work) {  // the binary64-accurate paths on the tensor cores, vector by vector
+            const int st = before_fine();
+            if (st) return st;
+            PhaseTimer pt(LFMM_PHASE_M2L_TC, s);
+            for (int v = 0; v < b.nvec; ++v) {
+                int n = 0;
+                LFMM_CUDA_TRY(sg_far_field<T>(sg_uniform_tree(L, p->opts.m2l_split), ops, (const T*)b.q + v * b.vq,
+                                              (T*)b.u + v * b.vq, (V8*)b.Q + v * b.vQ, (V8*)b.C + v * b.vQ, p->sg_work,
+                                              true, p->status, p->num_sms, s, &n));
+                pt.add_launches(n);
+            }
+            return LFMM_OK;
         }
     }
     int l_first = 2;  // first level left for the per-level M2L launches

@@ -25,6 +25,7 @@
 
 #include "device_common.h"
 #include "lfmm_internal.h"
+#include "split_tc.h"
 
 namespace lfmm {
 
@@ -963,11 +964,32 @@ static cudaError_t launch_coop(const void* fn, int grid, int threads, size_t sme
     return e;
 }
 
+SgTree forest_sg_tree(const Forest& F) {
+    SgTree t;
+    t.nk = (int)F.levels.size();
+    t.rows = F.total_boxes;
+    t.split = F.m2l_split;
+    for (int k = 0; k < t.nk && k < kSgMaxLevels; ++k) {
+        const ForestLevel& lv = F.levels[k];
+        SgTree::Level& o = t.lv[k];
+        o.nb = lv.nb;
+        o.off = lv.box_off;
+        std::copy(lv.cls, lv.cls + 5, o.cls);
+        o.il = lv.il;
+        o.par = lv.par;
+        o.ch = lv.ch;
+    }
+    return t;
+}
+
 template <typename T>
 int forest_eval(const Forest& F, const DeviceOps& ops, const double* f, T* f_sorted, T* qhat, T* uhat, void* Qbox,
                 void* Cbox, double* u, double* un, double* uf, int num_sms, cudaStream_t s, int* status_word,
                 bool persistent) {
-    int* status = persistent ? status_word : nullptr;
+    // the sliced far field (split_tc.cu) has one form; the persistent sweeps are those of the
+    // other kernels
+    const bool sliced = sizeof(T) == 8 && F.sg_work != nullptr && status_word != nullptr;
+    int* status = persistent && !sliced ? status_word : nullptr;
     using V = typename Mono<T>::V;
     const int NP = ops.NP;
     const int nk = (int)F.levels.size();
@@ -1025,7 +1047,17 @@ int forest_eval(const Forest& F, const DeviceOps& ops, const double* f, T* f_sor
             pt.add_launches(1);
         }
     }
-    if (far && !up_done) {
+    if constexpr (sizeof(T) == 8) {
+        if (far && sliced) {
+            PhaseTimer pt(LFMM_PHASE_M2L_TC, s);
+            int n = 0;
+            const cudaError_t e = sg_far_field<T>(forest_sg_tree(F), ops, qhat, uhat, Qbox, Cbox, F.sg_work, false,
+                                                  status_word, num_sms, s, &n);
+            if (e != cudaSuccess) return fail(LFMM_ECUDA, std::string("split_gemm_kernel: ") + cudaGetErrorString(e));
+            pt.add_launches(n);
+        }
+    }
+    if (far && !up_done && !sliced) {
         PhaseTimer pt(LFMM_PHASE_M2M, s);
         for (int k = 1; k < nk; ++k) {
             const ForestLevel& lv = F.levels[k];
@@ -1134,7 +1166,7 @@ int forest_eval(const Forest& F, const DeviceOps& ops, const double* f, T* f_sor
             down_done = true;  // every level with boxes runs on the tensor cores
         }
     }
-    if (far) {
+    if (far && !sliced) {
         for (int k = (down_done ? k_pers : nk) - 1; k >= 0; --k) {
             const ForestLevel& lv = F.levels[k];
             if (lv.nb == 0) continue;

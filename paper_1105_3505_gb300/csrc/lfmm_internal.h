@@ -178,6 +178,9 @@ struct DeviceOps {
     std::vector<void*> mono;              // per level k: deflation constants (hi[40], lo[40])
     std::vector<void*> tc;                // per level k (mixed, NP = 32): tensor-core B tiles,
                                           // [40 offsets + 4 L2L classes][hi, lo][32 x 32 fp32]
+    void* sg_base = nullptr;              // binary64-accurate paths, NP = 64: sliced operators
+    std::vector<uint8_t*> sg_tiles;       // per level k (split_tc.h: kSgOps tiles), and
+    std::vector<int32_t*> sg_e;           // their exponents
     std::vector<void*> retired;           // earlier, smaller uploads (kept alive)
 };
 
@@ -291,6 +294,7 @@ struct Forest {
     unsigned long long* sweep_ctr = nullptr;  // work-queue counters of the persistent sweeps (2 x 16)
     bool tc_list = false;                   // list M2L of large levels on the tensor cores (mixed path)
     float* tc_split = nullptr;              // TF32 hi / lo rows of those levels (plan-owned)
+    void* sg_work = nullptr;                // work space of the sliced far field (split_tc.h; plan-owned)
     void release(cudaStream_t s);
 };
 

@@ -21,6 +21,7 @@
 #include <mutex>
 
 #include "lfmm_internal.h"
+#include "split_tc.h"
 
 namespace lfmm {
 
@@ -169,7 +170,10 @@ extern "C" int lfmm_plan_shape_noalloc(const int32_t* src_xy, int64_t n_src, con
                          : o.precision == LFMM_MIXED ? m2l_fused_split_bytes_shape<float>(NP, has_tc, L, tc_min, num_sms, 1, o.m2l_split)
                          : o.precision == LFMM_DF    ? m2l_fused_split_bytes_shape<DF>(NP, has_tc, L, tc_min, num_sms, 1, o.m2l_split)
                                                      : m2l_fused_split_bytes_shape<double>(NP, has_tc, L, tc_min, num_sms, 1, o.m2l_split);
-    const int64_t bytes = a(2 * (n_leaves + 1) * 4) + a((2 * (n_src + n_tgt) + n_tgt) * 4) + a(n_src * esz) + split +
+    const int64_t sg = sg_applies_uniform(o.precision, NP, L, o.tc_min_level)
+                           ? sg_work_bytes(sg_uniform_tree(L, o.m2l_split), o.precision, num_sms)
+                           : 0;  // sliced far field of the binary64-accurate paths
+    const int64_t bytes = sg + a(2 * (n_leaves + 1) * 4) + a((2 * (n_src + n_tgt) + n_tgt) * 4) + a(n_src * esz) + split +
                           un_tmp + part +
                           2 * a(boxes * NP * esz) + 2 * a(boxes * 8) + 16 /* status word */;
 

@@ -32,6 +32,7 @@
 #include <tuple>
 
 #include "lfmm_internal.h"
+#include "split_tc.h"
 
 namespace lfmm {
 
@@ -475,6 +476,16 @@ const DeviceOps* get_device_ops(ModelOps* mo, int precision, int NP, int n_level
         d->l2l[k] = k >= 1 ? b + ol[k] * elem : nullptr;
         d->tifo[k] = b + ot[k] * elem;
         d->mono[k] = b + omono[k] * elem;
+    }
+    if (precision != LFMM_MIXED && NP == 64) {
+        e = sg_build_operators(*d, stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+        if (e != cudaSuccess) {
+            cudaFree(d->sg_base);
+            cudaFree(d->base);
+            if (err) *err = std::string("sliced operators: ") + cudaGetErrorString(e);
+            return nullptr;
+        }
     }
     if (slot) d->retired.push_back(slot.release());  // plans built earlier may still use it
     slot = std::move(d);
