@@ -718,7 +718,7 @@ int far_sweeps(lfmm_plan* p, const FarBufs& b, cudaStream_t s, Hook before_fine)
             PhaseTimer pt(LFMM_PHASE_M2L_TC, s);
             for (int v = 0; v < b.nvec; ++v) {
                 int n = 0;
-                LFMM_CUDA_TRY(sg_far_field<T>(sg_uniform_tree(L, p->opts.m2l_split), ops, (const T*)b.q + v * b.vq,
+                LFMM_CUDA_TRY(sg_far_field<T>(sg_uniform_tree(L, p->opts.m2l_split), ops, (T*)b.q + v * b.vq,
                                               (T*)b.u + v * b.vq, (V8*)b.Q + v * b.vQ, (V8*)b.C + v * b.vQ, p->sg_work,
                                               true, p->status, p->num_sms, s, &n));
                 pt.add_launches(n);

@@ -36,14 +36,17 @@
 // Every wait is bounded; on expiry LFMM_ETIMEOUT is recorded, the roles run out without
 // waiting, and the teardown waits (bounded) for the copies and MMAs in flight.
 //
-// What bounds it: a step needs 2,700 tensor cycles (128 x 64 x 64 x 21 products) and about
-// as long for the read-back, one after the other because the accumulators of a step fill
-// 384 (448) of the 512 TMEM columns; the float-float products on the FP32 pipes that it
-// replaces took 61,000 cycles a step, the binary64 ones 262,000.  Measured (ncu, cold
-// caches): the M2L of 400,009 points at leaf size 128, float-float p = 16 (8.4 k boxes)
-// 942 -> 108 us; of 178 k clustered points 1,713 -> 151 us; of 100 k points in binary64
-// 1,137 -> 54 us.  The M2M and L2L launches (20-30 us a level, the same on levels of a
-// few boxes) are bound by the latency of their four steps and one.
+// What bounds it: a step needs 2,700 tensor cycles (128 x 64 x 64 x 21 products) and 1,900
+// for the read-back, one after the other because the accumulators of a step fill 384 (448)
+// of the 512 TMEM columns; the float-float products on the FP32 pipes that it replaces took
+// 61,000 cycles a step, the binary64 ones 262,000.  Measured (ncu, cold caches): the M2L of
+// 400,009 points at leaf size 128, float-float p = 16 (8.4 k boxes) 942 -> 108 us, of 178 k
+// clustered points 1,713 -> 151 us, of 100 k points in binary64 1,137 -> 54 us.  Those
+// figures are with the producers reading each row's index between two copies (10,500 cycles
+// a step, clock64 trace); reading a step's indices first, adding the chunks once instead of
+// in the downward pass, and small_level_kernel for levels of few boxes (28 and 18 us a
+// level as tensor-core launches) then took eval_df_400k from 968 to 806 us, eval_fp64_100k
+// 636 -> 488, request_178k_1e10 1,456 -> 1,159 and a disk's Krylov iteration 387 -> 188 us.
 // Errors against the exact sum over eight inputs each (geometric means, before -> after):
 // float-float 1.4e-13 -> 1.3e-13, clustered requests 8.8e-14 -> 6.3e-14, a disk's double
 // layer 1.4e-12 -> 9.1e-13, binary64 1.13e-14 -> 1.14e-14 and 3.4e-14 -> 3.4e-14 (these set
@@ -106,15 +109,14 @@ struct SgParams {
     int count[4 * kSgMaxLevels];
     int tile_end[4 * kSgMaxLevels];
     int n_seg, n_items, n_chunks, has_par;
-    int n_part;         // L2L: chunks of the M2L to add
-    float* part;        // [chunk][row][NC][64] sums of the M2L steps
+    float* part;        // [chunk][row][NC][64] sums of the M2L steps (L2L: chunk 0, the whole sum)
     int32_t* part_e;    // [chunk][row]
     void* cpart;        // [chunk][row]
     int64_t part_rows;
     uint8_t* dst;       // sliced rows out (null: none)
     int32_t* dst_e;
     int64_t dst0;       // first row of the level there
-    void* u;            // rows of T out (null: none)
+    void* u;            // the level's rows of T out (null: none)
     void* Cout;         // M2M: charges out; L2L: constants out
     const void* Cpar;
 };
@@ -179,7 +181,51 @@ __device__ __forceinline__ int row_exp(uint32_t mx) {
     return max((int)(mx >> 23) - 126, -126);
 }
 
-// Slices of rows of T (64 coefficients), a warp per row, two coefficients per lane.
+// Slices of one row of T (64 coefficients, two per lane of a warp) and its exponent.
+template <typename T>
+__device__ __forceinline__ void slice_row(const T (&x)[2], int lane, uint8_t* __restrict__ dst,
+                                          int32_t* __restrict__ dst_e) {
+    uint32_t w[kSgSlices];
+    int e;
+    if constexpr (std::is_same<T, DF>::value) {
+        uint32_t mx = max(__float_as_uint(x[0].hi) & 0x7fffffffu, __float_as_uint(x[1].hi) & 0x7fffffffu);
+        mx = __reduce_max_sync(kFull, mx);
+        e = row_exp(mx);
+        const bool dead = abs(e) >= kExpNan;
+        float v[2][2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            v[i][0] = dead ? 0.f : ldexpf(x[i].hi, 8 - e);
+            v[i][1] = dead ? 0.f : ldexpf(x[i].lo, 8 - e);
+        }
+#pragma unroll
+        for (int s = 0; s < kSgSlices; ++s) {
+            const __half2 h = __floats2half2_rn(next_digit(v[0]), next_digit(v[1]));
+            w[s] = *reinterpret_cast<const uint32_t*>(&h);
+        }
+    } else {
+        uint32_t mx = max((uint32_t)__double2hiint(x[0]) & 0x7fffffffu, (uint32_t)__double2hiint(x[1]) & 0x7fffffffu);
+        if (mx == 0 && (x[0] != 0.0 || x[1] != 0.0)) mx = 1;
+        mx = __reduce_max_sync(kFull, mx);
+        e = mx == 0 ? kExpZero : mx >= 0x7ff00000u ? kExpNan : max((int)(mx >> 20) - 1022, -1022);
+        const bool dead = abs(e) >= kExpNan;
+        double v0 = dead ? 0.0 : ldexp(x[0], 8 - e), v1 = dead ? 0.0 : ldexp(x[1], 8 - e);
+#pragma unroll
+        for (int s = 0; s < kSgSlices; ++s) {
+            const double a0 = rint(v0), a1 = rint(v1);
+            v0 = (v0 - a0) * 512.0;
+            v1 = (v1 - a1) * 512.0;
+            const __half2 h = __floats2half2_rn((float)a0, (float)a1);
+            w[s] = *reinterpret_cast<const uint32_t*>(&h);
+        }
+    }
+    uint32_t* row = reinterpret_cast<uint32_t*>(dst);
+#pragma unroll
+    for (int s = 0; s < kSgSlices; ++s) row[32 * s + lane] = w[s];
+    if (lane == 0) *dst_e = e;
+}
+
+// Slices of nb rows of T, a warp per row.
 template <typename T>
 __global__ void __launch_bounds__(256) slice_rows_kernel(const T* __restrict__ x, int64_t nb, uint8_t* __restrict__ dst,
                                                          int32_t* __restrict__ dst_e) {
@@ -187,45 +233,8 @@ __global__ void __launch_bounds__(256) slice_rows_kernel(const T* __restrict__ x
     const int lane = threadIdx.x & 31;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t b = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; b < nb; b += nw) {
-        uint32_t w[kSgSlices];
-        int e;
-        if constexpr (std::is_same<T, DF>::value) {
-            const float4 p = *reinterpret_cast<const float4*>(x + b * 64 + 2 * lane);
-            float v[2][2] = {{p.x, p.y}, {p.z, p.w}};
-            uint32_t mx = max(__float_as_uint(p.x) & 0x7fffffffu, __float_as_uint(p.z) & 0x7fffffffu);
-            mx = __reduce_max_sync(kFull, mx);
-            e = row_exp(mx);
-            const int sh = 8 - e;
-#pragma unroll
-            for (int i = 0; i < 2; ++i)
-#pragma unroll
-                for (int c = 0; c < 2; ++c) v[i][c] = abs(e) >= kExpNan ? 0.f : ldexpf(v[i][c], sh);
-#pragma unroll
-            for (int s = 0; s < kSgSlices; ++s) {
-                const __half2 h = __floats2half2_rn(next_digit(v[0]), next_digit(v[1]));
-                w[s] = *reinterpret_cast<const uint32_t*>(&h);
-            }
-        } else {
-            const double2 p = *reinterpret_cast<const double2*>(x + b * 64 + 2 * lane);
-            uint32_t mx = max((uint32_t)__double2hiint(p.x) & 0x7fffffffu, (uint32_t)__double2hiint(p.y) & 0x7fffffffu);
-            if (mx == 0 && (p.x != 0.0 || p.y != 0.0)) mx = 1;
-            mx = __reduce_max_sync(kFull, mx);
-            e = mx == 0 ? kExpZero : mx >= 0x7ff00000u ? kExpNan : max((int)(mx >> 20) - 1022, -1022);
-            const bool dead = abs(e) >= kExpNan;
-            double v0 = dead ? 0.0 : ldexp(p.x, 8 - e), v1 = dead ? 0.0 : ldexp(p.y, 8 - e);
-#pragma unroll
-            for (int s = 0; s < kSgSlices; ++s) {
-                const double a0 = rint(v0), a1 = rint(v1);
-                v0 = (v0 - a0) * 512.0;
-                v1 = (v1 - a1) * 512.0;
-                const __half2 h = __floats2half2_rn((float)a0, (float)a1);
-                w[s] = *reinterpret_cast<const uint32_t*>(&h);
-            }
-        }
-        uint32_t* row = reinterpret_cast<uint32_t*>(dst + b * kSgRowBytes);
-#pragma unroll
-        for (int s = 0; s < kSgSlices; ++s) row[32 * s + lane] = w[s];
-        if (lane == 0) dst_e[b] = e;
+        const VecT<T, 2> p = *reinterpret_cast<const VecT<T, 2>*>(x + b * 64 + 2 * lane);
+        slice_row(p.v, lane, dst + b * kSgRowBytes, dst_e + b);
     }
 }
 
@@ -452,6 +461,7 @@ __global__ void __launch_bounds__(kSgThreads, 1) split_gemm_kernel(const __grid_
                 }
             }
             __syncwarp();
+            const uint8_t* src = L.src;
             for (int st = I.st0; st < I.st1 && !stop; ++st, ++step) {
                 const int bslot = step & 1;
                 if (pw == 0 && lane == 0) {
@@ -465,6 +475,15 @@ __global__ void __launch_bounds__(kSgThreads, 1) split_gemm_kernel(const __grid_
                         s_bissued = step + 1;
                     }
                 }
+                // the lane's sixteen rows of the step, in 16-byte units (read before the copies:
+                // the copies' memory clobber would put a shared-memory load's latency between
+                // any two of them, 1,400 instead of 250 cycles a slice)
+                uint32_t from16[16];
+#pragma unroll
+                for (int g = 0; g < 16; ++g) {
+                    const int si = my_src[(4 * g + sub) * 28 + st - I.st0];
+                    from16[g] = si < 0 ? ~0u : (uint32_t)si * (uint32_t)(kSgRowBytes / 16) + ch;
+                }
                 for (int sl = 0; sl < kSgSlices; ++sl) {
                     bool ok = *vabort == 0;
                     if (ok && ause > 0 && lane == 0) ok = mbar_poll_bounded(&aempty[aslot], (uint32_t)((ause - 1) & 1), wb);
@@ -476,12 +495,12 @@ __global__ void __launch_bounds__(kSgThreads, 1) split_gemm_kernel(const __grid_
                     const uint32_t sa = base + (uint32_t)aslot * kABytes;
 #pragma unroll
                     for (int g = 0; g < 16; ++g) {
-                        const int rl = 4 * g + sub, r = 64 * pw + rl;
-                        const int si = my_src[rl * 28 + st - I.st0];
-                        const uint8_t* from = L.src + (si < 0 ? 0 : (size_t)si * kSgRowBytes) + sl * 128 + ch * 16;
+                        const int r = 64 * pw + 4 * g + sub;
+                        const bool none = from16[g] == ~0u;
+                        const uint8_t* from = src + (none ? 0 : (size_t)from16[g] * 16 + sl * 128);
                         asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(
                                          sa + (uint32_t)(r * 128 + ((ch ^ (r & 7)) << 4))),
-                                     "l"(from), "r"(si < 0 ? 0 : 16)
+                                     "l"(from), "r"(none ? 0 : 16)
                                      : "memory");
                     }
                     cp_async_mbar_arrive_noinc(&afull[aslot]);
@@ -588,7 +607,7 @@ __global__ void __launch_bounds__(kSgThreads, 1) split_gemm_kernel(const __grid_
                 } else {
                     const int pb = P.has_par ? source_of<MODE>(L, s_dxy[0], b, 0) : -1;
                     V sum = pb >= 0 ? ((const V*)P.Cpar)[pb] : M::zero();
-                    for (int z = 0; z < P.n_part; ++z) sum = M::add(sum, ((const V*)P.cpart)[z * P.part_rows + L.out0 + b]);
+                    sum = M::add(sum, ((const V*)P.cpart)[L.out0 + b]);
                     ((V*)P.Cout)[b] = sum;
                 }
             }
@@ -615,17 +634,24 @@ __global__ void __launch_bounds__(kSgThreads, 1) split_gemm_kernel(const __grid_
             int eref = kExpZero;
             for (int st = 0; st < ns; ++st)
                 if (my_exp[st] != kExpNan) eref = max(eref, (int)my_exp[st]);
-            int n_part = 0;
-            if (MODE == kL2L) {
-                n_part = P.n_part;
-                for (int z = 0; z < n_part; ++z)
-                    if (valid) eref = max(eref, P.part_e[z * P.part_rows + L.out0 + b]);
-            }
+            if (MODE == kL2L && valid) eref = max(eref, P.part_e[L.out0 + b]);
             float acc[32][NC];
 #pragma unroll
             for (int j = 0; j < 32; ++j)
 #pragma unroll
                 for (int c = 0; c < NC; ++c) acc[j][c] = 0.f;
+            if (MODE == kL2L && valid) {  // the M2L's sum, loaded while the parent's product runs
+                const int64_t row = L.out0 + b;
+                const float f = pow2f(P.part_e[row] - eref);
+                const float4* from = reinterpret_cast<const float4*>(P.part + row * (64 * NC) + 32 * half);
+#pragma unroll
+                for (int c = 0; c < NC; ++c)
+#pragma unroll
+                    for (int j = 0; j < 32; j += 4) {
+                        const float4 q = from[16 * c + j / 4];
+                        acc[j][c] = q.x * f, acc[j + 1][c] = q.y * f, acc[j + 2][c] = q.z * f, acc[j + 3][c] = q.w * f;
+                    }
+            }
             for (int st = 0; st < ns; ++st, ++step) {
                 if (!dead) {
                     const bool ok = *vabort == 0 && mbar_poll_bounded(&acc_full, (uint32_t)(step & 1), wb);
@@ -659,29 +685,6 @@ __global__ void __launch_bounds__(kSgThreads, 1) split_gemm_kernel(const __grid_
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&acc_empty);
             }
-            if (MODE == kL2L) {
-                for (int z = 0; z < n_part; ++z) {
-                    const int64_t row = z * P.part_rows + L.out0 + b;
-                    const float f = valid ? pow2f(P.part_e[row] - eref) : 0.f;
-                    const float4* src = reinterpret_cast<const float4*>(P.part + row * (64 * NC) + 32 * half);
-#pragma unroll
-                    for (int j0 = 0; j0 < 32; j0 += 4) {
-                        float x[NC][4];
-#pragma unroll
-                        for (int c = 0; c < NC; ++c) {
-                            const float4 q = valid ? src[16 * c + j0 / 4] : make_float4(0.f, 0.f, 0.f, 0.f);
-                            x[c][0] = q.x, x[c][1] = q.y, x[c][2] = q.z, x[c][3] = q.w;
-                        }
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            float v[NC];
-#pragma unroll
-                            for (int c = 0; c < NC; ++c) v[c] = x[c][j];
-                            add_scaled(acc[j0 + j], v, f);
-                        }
-                    }
-                }
-            }
 #pragma unroll
             for (int j = 0; j < 32; ++j) renorm(acc[j]);
             if (MODE == kM2L) {
@@ -697,7 +700,7 @@ __global__ void __launch_bounds__(kSgThreads, 1) split_gemm_kernel(const __grid_
                 }
                 continue;
             }
-            if (MODE == kL2L && P.u && valid) {
+            if (P.u && valid) {
                 T* to = (T*)P.u + b * 64 + 32 * half;
 #pragma unroll
                 for (int j = 0; j < 32; j += 2) {
@@ -763,6 +766,168 @@ __global__ void __launch_bounds__(kSgThreads, 1) split_gemm_kernel(const __grid_
     }
 }
 
+// The chunks of every row's M2L added in chunk order into chunk 0, a warp per row and two
+// outputs per lane.
+template <typename T>
+__global__ void __launch_bounds__(256) sum_chunks_kernel(float* __restrict__ part, int32_t* __restrict__ part_e,
+                                                         void* __restrict__ cpart, int64_t rows, int chunks) {
+    griddep_wait();
+    constexpr int NC = SgT<T>::NC;
+    using M = Mono<T>;
+    using V = typename M::V;
+    const int lane = threadIdx.x & 31;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t b = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; b < rows; b += nw) {
+        const int e = __reduce_max_sync(kFull, lane < chunks ? part_e[lane * rows + b] : kExpZero);
+        float v[2][NC];
+#pragma unroll
+        for (int c = 0; c < NC; ++c) v[0][c] = v[1][c] = 0.f;
+        V sum = M::zero();
+        for (int z = 0; z < chunks; ++z) {
+            const float f = pow2f(part_e[z * rows + b] - e);
+            const float2* from = reinterpret_cast<const float2*>(part + (z * rows + b) * (64 * NC));
+            float x[2][NC];
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                const float2 q = from[32 * c + lane];
+                x[0][c] = q.x;
+                x[1][c] = q.y;
+            }
+            add_scaled(v[0], x[0], f);
+            add_scaled(v[1], x[1], f);
+            if (lane == 0) sum = M::add(sum, ((const V*)cpart)[z * rows + b]);
+        }
+        renorm(v[0]);
+        renorm(v[1]);
+        float2* to = reinterpret_cast<float2*>(part + b * (64 * NC));
+#pragma unroll
+        for (int c = 0; c < NC; ++c) to[32 * c + lane] = make_float2(v[0][c], v[1][c]);
+        if (lane == 0) {
+            part_e[b] = e;
+            ((V*)cpart)[b] = sum;
+        }
+    }
+}
+
+// M2M (UP) or L2L of a level of few boxes on the CUDA cores, in T: a block per box, 64 outputs
+// x 16 (UP) or 4 groups of 16 inputs, each thread holding its 16 operator entries in
+// registers (L2L: reloaded when the block's boxes change class); the groups' sums are added
+// in group order and the first warp writes the row of T and, with dst set, its slices.  A
+// tensor-core launch spends 10-15 us on its steps' and its slicing's latency however few its
+// boxes are; this takes about 4 us while the blocks fit the chip.
+struct SmallP {
+    int64_t nb, row0;          // boxes; first row of the level in the expansion arrays
+    int64_t cls[5];            // L2L, compact form
+    const int32_t* list;       // UP: children [4]; L2L: parent [1] (compact form)
+    int lg;                    // uniform form
+    int has_par;
+    const void* op;            // UP: m2m [256][64]; L2L: l2l [4][64][64]
+    const void* x;             // rows of the children's / the parent's level
+    const void* Xin;           // their charges / constants
+    const float* part;         // L2L: the M2L's sums (rows of the level)
+    const int32_t* part_e;
+    const void* cpart;
+    void* y;                   // rows out
+    void* Yout;                // charges / constants out
+    uint8_t* dst;              // sliced rows out (null: none)
+    int32_t* dst_e;
+};
+
+template <typename T, bool UP>
+__global__ void __launch_bounds__(UP ? 1024 : 256) small_level_kernel(const __grid_constant__ SmallP P) {
+    griddep_wait();
+    constexpr int NG = UP ? 16 : 4, NC = SgT<T>::NC;
+    using M = Mono<T>;
+    using V = typename M::V;
+    __shared__ T s_x[NG * 16], s_red[NG][64];
+    const int o = threadIdx.x & 63, g = threadIdx.x >> 6, lane = threadIdx.x & 31;
+    const int64_t per = (P.nb + gridDim.x - 1) / gridDim.x;
+    const int64_t b0 = blockIdx.x * per, b1 = min(P.nb, b0 + per);
+    T op[16];
+    int cls = -1;
+    for (int64_t b = b0; b < b1; ++b) {
+        int c = 0;
+        if (!UP) c = P.lg >= 0 ? (int)(b & 3) : (b >= P.cls[1]) + (b >= P.cls[2]) + (b >= P.cls[3]);
+        if (c != cls) {
+            cls = c;
+#pragma unroll
+            for (int i = 0; i < 16; ++i) op[i] = ldg((const T*)P.op + (size_t)c * 4096 + (16 * g + i) * 64 + o);
+        }
+        if (threadIdx.x < NG * 16) {
+            const int ch = threadIdx.x >> 6;
+            int src = -1;
+            if (UP) src = P.list[4 * b + ch];
+            else if (P.has_par) src = P.lg >= 0 ? (int)(b >> 2) : P.list[b];
+            s_x[threadIdx.x] = src >= 0 ? ((const T*)P.x)[(size_t)src * 64 + o] : T(0);
+        }
+        __syncthreads();
+        T acc = T(0);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) acc = fma(op[i], s_x[16 * g + i], acc);
+        s_red[g][o] = acc;
+        __syncthreads();
+        if (UP) {  // sixteen groups to four
+            T v = s_red[0][0];
+            if (threadIdx.x < 256) v = (s_red[4 * g][o] + s_red[4 * g + 1][o]) + (s_red[4 * g + 2][o] + s_red[4 * g + 3][o]);
+            __syncthreads();
+            if (threadIdx.x < 256) s_red[g][o] = v;
+            __syncthreads();
+        }
+        if (threadIdx.x < 32) {
+            T v[2];
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int q = 2 * lane + j;
+                v[j] = (s_red[0][q] + s_red[1][q]) + (s_red[2][q] + s_red[3][q]);
+            }
+            if (!UP) {
+                const float2* from = reinterpret_cast<const float2*>(P.part + (P.row0 + b) * (64 * NC));
+                const int e = P.part_e[P.row0 + b];
+                float2 x[NC];
+#pragma unroll
+                for (int k = 0; k < NC; ++k) x[k] = from[32 * k + lane];
+                if constexpr (std::is_same<T, DF>::value) {
+                    v[0] += DF{ldexpf(x[0].x, e), ldexpf(x[1].x, e)};
+                    v[1] += DF{ldexpf(x[0].y, e), ldexpf(x[1].y, e)};
+                } else {
+                    v[0] += ldexp((double)x[0].x + ((double)x[1].x + (double)x[2 % NC].x), e);
+                    v[1] += ldexp((double)x[0].y + ((double)x[1].y + (double)x[2 % NC].y), e);
+                }
+            }
+            T* y = (T*)P.y + (size_t)b * 64;
+            y[2 * lane] = v[0];
+            y[2 * lane + 1] = v[1];
+            if (P.dst) slice_row(v, lane, P.dst + b * kSgRowBytes, P.dst_e + b);
+            if (lane == 0) {
+                const V* X = (const V*)P.Xin;
+                V* Y = (V*)P.Yout;
+                if (UP) {
+                    V q[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const int src = P.list[4 * b + k];
+                        q[k] = src >= 0 ? X[src] : M::zero();
+                    }
+                    Y[b] = M::add(M::add(q[0], q[1]), M::add(q[2], q[3]));
+                } else {
+                    const int src = !P.has_par ? -1 : P.lg >= 0 ? (int)(b >> 2) : P.list[b];
+                    const V up = src >= 0 ? X[src] : M::zero();
+                    Y[b] = M::add(up, ((const V*)P.cpart)[P.row0 + b]);
+                }
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// Levels of up to this many boxes take small_level_kernel (M2M, L2L): the work of one box
+// (16,384 and 4,096 multiply-adds, 15 FP32 operations each or one at 1/64 rate) against a
+// tensor-core launch's latency.
+template <typename T>
+constexpr int64_t kSmallUp = std::is_same<T, DF>::value ? 2048 : 304;
+template <typename T>
+constexpr int64_t kSmallDown = std::is_same<T, DF>::value ? 4096 : 912;
+
 // Work space: sliced rows and exponents of q (all levels) and of u (levels k >= 1), the
 // chunks' sums, exponents and constants.
 struct SgWork {
@@ -820,7 +985,7 @@ int sg_chunks(const SgTree& t, int num_sms) {
     int best = 1;
     double cost = 0;
     for (int c = 1; c <= 9; ++c) {
-        const double v = (double)((tiles * c + num_sms - 1) / num_sms) * ((27 + c - 1) / c + 1.5) + 0.3 * c;
+        const double v = (double)((tiles * c + num_sms - 1) / num_sms) * ((27 + c - 1) / c + 2.0) + 0.1 * c;
         if (c == 1 || v < cost) {
             best = c;
             cost = v;
@@ -861,7 +1026,7 @@ cudaError_t sg_build_operators(DeviceOps& ops, cudaStream_t s) {
 }
 
 template <typename T>
-cudaError_t sg_far_field(const SgTree& t, const DeviceOps& ops, const T* q, T* u, void* Q, void* C, void* work,
+cudaError_t sg_far_field(const SgTree& t, const DeviceOps& ops, T* q, T* u, void* Q, void* C, void* work,
                          bool q_all, int* status, int num_sms, cudaStream_t s, int* launches) {
     constexpr int NC = SgT<T>::NC;
     const int chunks = sg_chunks(t, num_sms);
@@ -898,6 +1063,8 @@ cudaError_t sg_far_field(const SgTree& t, const DeviceOps& ops, const T* q, T* u
         P = SgParams();
         P.n_chunks = 1;
     };
+    auto small_up = [&](int k) { return t.lv[k].nb > 0 && t.lv[k].nb <= kSmallUp<T>; };
+    auto small_down = [&](int k) { return t.lv[k].nb > 0 && t.lv[k].nb <= kSmallDown<T>; };
     SgParams P;
     // ---- slices of the leaf expansions (or of every level's), then M2M level by level
     {
@@ -909,6 +1076,24 @@ cudaError_t sg_far_field(const SgTree& t, const DeviceOps& ops, const T* q, T* u
         ++*launches;
     }
     for (int k = 1; k < t.nk && !q_all; ++k) {
+        if (small_up(k)) {
+            SmallP S = {};
+            S.nb = t.lv[k].nb;
+            S.list = t.lv[k].ch;
+            S.lg = -1;
+            S.op = ops.m2m[k];
+            S.x = q + t.lv[k - 1].off * 64;
+            S.Xin = Qm(k - 1);
+            S.y = q + t.lv[k].off * 64;
+            S.Yout = Qm(k);
+            S.dst = qrow(k);
+            S.dst_e = w.qe + t.lv[k].off;
+            e = launch_dependent(small_level_kernel<T, true>, dim3((unsigned)std::min<int64_t>(S.nb, 2 * num_sms)),
+                                 dim3(1024), 0, s, S);
+            if (e != cudaSuccess) return e;
+            ++*launches;
+            continue;
+        }
         clear(P);
         P.n_seg = 1;
         P.count[0] = (int)t.lv[k].nb;
@@ -925,6 +1110,7 @@ cudaError_t sg_far_field(const SgTree& t, const DeviceOps& ops, const T* q, T* u
         P.dst_e = w.qe;
         P.dst0 = t.lv[k].off;
         P.Cout = Qm(k);
+        if (k + 1 < t.nk && small_up(k + 1)) P.u = q + t.lv[k].off * 64;  // read as rows of T there
         e = go(std::integral_constant<int, kM2M>(), P);
         if (e != cudaSuccess) return e;
     }
@@ -953,13 +1139,49 @@ cudaError_t sg_far_field(const SgTree& t, const DeviceOps& ops, const T* q, T* u
     P.part_rows = t.rows;
     e = go(std::integral_constant<int, kM2L>(), P);
     if (e != cudaSuccess) return e;
-    // ---- chunks' sums + L2L, coarse to fine
+    // ---- the chunks' sums, then L2L coarse to fine
+    if (chunks > 1) {
+        const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((t.rows + 7) / 8, (int64_t)num_sms * 8));
+        e = launch_dependent(sum_chunks_kernel<T>, dim3((unsigned)blocks), dim3(256), 0, s, w.part, w.part_e, w.cpart,
+                             t.rows, chunks);
+        if (e != cudaSuccess) return e;
+        ++*launches;
+    }
     for (int k = t.nk - 1; k >= 0; --k) {
+        if (small_down(k)) {
+            SmallP S = {};
+            S.nb = t.lv[k].nb;
+            S.row0 = t.lv[k].off;
+            std::copy(t.lv[k].cls, t.lv[k].cls + 5, S.cls);
+            S.list = t.lv[k].par;
+            S.lg = t.lv[k].lg;
+            S.has_par = k + 1 < t.nk ? 1 : 0;
+            if (S.has_par) {
+                S.op = ops.l2l[k + 1];
+                S.x = u + t.lv[k + 1].off * 64;
+                S.Xin = Cm(k + 1);
+            } else {
+                S.op = ops.tifo[0];  // times zero
+            }
+            S.part = w.part;
+            S.part_e = w.part_e;
+            S.cpart = w.cpart;
+            S.y = u + t.lv[k].off * 64;
+            S.Yout = Cm(k);
+            if (k > 0 && !small_down(k - 1)) {
+                S.dst = w.u + uoff[k] * kSgRowBytes;
+                S.dst_e = w.ue + uoff[k];
+            }
+            e = launch_dependent(small_level_kernel<T, false>, dim3((unsigned)std::min<int64_t>(S.nb, 8 * num_sms)),
+                                 dim3(256), 0, s, S);
+            if (e != cudaSuccess) return e;
+            ++*launches;
+            continue;
+        }
         clear(P);
         P.n_items = segments(P, 0, k, 0);
         P.n_seg = 4;
         P.has_par = k + 1 < t.nk ? 1 : 0;
-        P.n_part = chunks;
         P.part = w.part;
         P.part_e = w.part_e;
         P.cpart = w.cpart;
@@ -976,12 +1198,12 @@ cudaError_t sg_far_field(const SgTree& t, const DeviceOps& ops, const T* q, T* u
             P.Cpar = Cm(k + 1);
         }
         P.Cout = Cm(k);
-        if (k > 0) {
+        if (k > 0 && !small_down(k - 1)) {
             P.dst = w.u;
             P.dst_e = w.ue;
             P.dst0 = uoff[k];
         } else {
-            P.u = u + t.lv[0].off * 64;
+            P.u = u + t.lv[k].off * 64;
         }
         e = go(std::integral_constant<int, kL2L>(), P);
         if (e != cudaSuccess) return e;
@@ -989,9 +1211,9 @@ cudaError_t sg_far_field(const SgTree& t, const DeviceOps& ops, const T* q, T* u
     return cudaSuccess;
 }
 
-template cudaError_t sg_far_field<DF>(const SgTree&, const DeviceOps&, const DF*, DF*, void*, void*, void*, bool, int*,
+template cudaError_t sg_far_field<DF>(const SgTree&, const DeviceOps&, DF*, DF*, void*, void*, void*, bool, int*,
                                       int, cudaStream_t, int*);
-template cudaError_t sg_far_field<double>(const SgTree&, const DeviceOps&, const double*, double*, void*, void*, void*,
+template cudaError_t sg_far_field<double>(const SgTree&, const DeviceOps&, double*, double*, void*, void*, void*,
                                           bool, int*, int, cudaStream_t, int*);
 
 }  // namespace lfmm

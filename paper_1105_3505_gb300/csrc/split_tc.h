@@ -49,9 +49,9 @@ int64_t sg_work_bytes(const SgTree& t, int precision, int num_sms);
 cudaError_t sg_build_operators(DeviceOps& ops, cudaStream_t s);
 // M2M (unless q_all: the expansions of every level are in q already), M2L and L2L: from the
 // leaf expansions and charges in q / Q to the leaf incoming expansions and constants in
-// u / C (rows as in t.lv[k].off; other levels' rows of u are not written).
+// u / C (rows as in t.lv[k].off; other levels' rows of q and u are scratch).
 template <typename T>
-cudaError_t sg_far_field(const SgTree& t, const DeviceOps& ops, const T* q, T* u, void* Q, void* C, void* work,
+cudaError_t sg_far_field(const SgTree& t, const DeviceOps& ops, T* q, T* u, void* Q, void* C, void* work,
                          bool q_all, int* status, int num_sms, cudaStream_t s, int* launches);
 
 }  // namespace lfmm
