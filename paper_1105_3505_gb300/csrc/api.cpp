@@ -81,6 +81,7 @@ struct lfmm_plan {
     double* un_tmp = nullptr;        // near field per target (caller order) from the concurrent near-field pass
     double* uf_tmp = nullptr;        // far field per target (caller order), before the final sum
     struct AuxStream* aux = nullptr;  // near-field pass runs here, beside the far-field sweeps
+    struct AuxStream* far_aux = nullptr;  // pruned / forest, 8-byte types: the far field, beside the near field
     // uniform storage: the targets are bucketed on `aux` while the plan's creation and the
     // evaluation's upward sweep go on; whatever reads them waits for this event
     cudaEvent_t tgt_ready = nullptr;
@@ -113,6 +114,7 @@ struct AuxStream {
     cudaStream_t s = nullptr;
     cudaEvent_t fork = nullptr, join = nullptr;
     int device = -1;
+    bool high = false;  // one step above the default priority
 };
 
 namespace {
@@ -120,11 +122,11 @@ namespace {
 std::mutex g_aux_mu;
 std::vector<AuxStream*> g_aux_free;
 
-AuxStream* acquire_aux(int device) {
+AuxStream* acquire_aux(int device, bool high = false) {
     {
         std::lock_guard<std::mutex> g(g_aux_mu);
         for (size_t i = 0; i < g_aux_free.size(); ++i)
-            if (g_aux_free[i]->device == device) {
+            if (g_aux_free[i]->device == device && g_aux_free[i]->high == high) {
                 AuxStream* a = g_aux_free[i];
                 g_aux_free.erase(g_aux_free.begin() + i);
                 return a;
@@ -133,7 +135,8 @@ AuxStream* acquire_aux(int device) {
     AuxStream* a = new (std::nothrow) AuxStream();
     if (!a) return nullptr;
     a->device = device;
-    if (cudaStreamCreateWithFlags(&a->s, cudaStreamNonBlocking) != cudaSuccess ||
+    a->high = high;
+    if (cudaStreamCreateWithPriority(&a->s, cudaStreamNonBlocking, high ? -1 : 0) != cudaSuccess ||
         cudaEventCreateWithFlags(&a->fork, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&a->join, cudaEventDisableTiming) != cudaSuccess) {
         cudaGetLastError();
@@ -346,6 +349,11 @@ int forest_workspaces(lfmm_plan* p, cudaStream_t s) {
         if (need > 0 && (st = palloc(p, &b, (size_t)need * sizeof(float), s))) return st;
         F.tc_split = (float*)b;
     }
+    if (p->opts.precision != LFMM_MIXED && F.kmax >= 0) {  // near field, before the far part is added
+        void* b;
+        if ((st = palloc(p, &b, (size_t)p->nt * sizeof(double), s))) return st;
+        F.near_tmp = (double*)b;
+    }
     // sliced far field of the binary64-accurate paths (split_tc.cu)
     if (F.kmax >= 0 && (int)F.levels.size() <= kSgMaxLevels &&
         sg_applies(p->opts.precision, p->NP, p->opts.tc_min_level)) {
@@ -539,7 +547,8 @@ int plan_build(lfmm_plan* p, const int32_t* src_xy, const int32_t* tgt_xy, cudaS
         p->forest.reset(new (std::nothrow) Forest());
         if (!p->forest) return fail(LFMM_ENOMEM, "host allocation failed");
         const int64_t so[2] = {0, p->ns}, to[2] = {0, p->nt};
-        if ((st = forest_build(*p->forest, src, so, p->ns, tgt, to, p->nt, 1, p->opts.leaf_size, p->side, s, &pt)))
+        if ((st = forest_build(*p->forest, src, so, p->ns, tgt, to, p->nt, 1, p->opts.leaf_size, p->side,
+                               p->opts.precision != LFMM_MIXED, s, &pt)))
             return st;
         return forest_workspaces(p, s);
     }
@@ -765,9 +774,19 @@ int far_sweeps(lfmm_plan* p, const FarBufs& b, cudaStream_t s, Hook before_fine)
 
 template <typename T>
 int eval_impl(lfmm_plan* p, const double* f, double* u, double* un, double* uf, cudaStream_t s) {
-    if (p->forest)
-        return forest_eval<T>(*p->forest, *p->ops, f, (T*)p->f_sorted, (T*)p->qhat, (T*)p->uhat, p->Qbox, p->Cbox,
-                              u, un, uf, p->num_sms, s, p->status, (p->opts.flags & LFMM_FLAG_PERSISTENT) != 0);
+    if (p->forest) {
+        // 8-byte types: the far field on a second stream beside the near field (launches of
+        // few blocks, so of a higher priority), joined before L2P
+        SideStream side{};
+        const bool beside = sizeof(T) == 8 && p->forest->kmax >= 0 && !(p->opts.flags & LFMM_FLAG_SERIAL);
+        if (beside && !p->far_aux) p->far_aux = acquire_aux(p->device, true);
+        if (beside && p->far_aux) side = SideStream{p->far_aux->s, p->far_aux->fork, p->far_aux->join};
+        const int st = forest_eval<T>(*p->forest, *p->ops, f, (T*)p->f_sorted, (T*)p->qhat, (T*)p->uhat, p->Qbox,
+                                      p->Cbox, u, un, uf, p->num_sms, s, p->status,
+                                      (p->opts.flags & LFMM_FLAG_PERSISTENT) != 0, side.s ? &side : nullptr);
+        if (st && side.s) cudaStreamSynchronize(side.s);  // nothing forked is left behind a failure
+        return st;
+    }
     const TreeView t = tree_view(p);
     const DeviceOps& ops = *p->ops;
     const int NP = p->NP;
@@ -1069,6 +1088,7 @@ int lfmm_plan_create(lfmm_plan** plan, const int32_t* src_xy, int64_t n_src, con
         free_plan_buffers(p);
         if (p->tgt_ready) cudaEventDestroy(p->tgt_ready);
         release_aux(p->aux);
+        release_aux(p->far_aux);
         delete p;
         return st;
     }
@@ -1096,6 +1116,7 @@ int lfmm_plan_destroy(lfmm_plan* plan) {
     if (plan->graph) cudaGraphExecDestroy(plan->graph);
     if (plan->cap_stream) cudaStreamDestroy(plan->cap_stream);
     release_aux(plan->aux);
+    release_aux(plan->far_aux);
     delete plan;
     if (e != cudaSuccess) return fail(LFMM_ECUDA, std::string("plan destroy: ") + cudaGetErrorString(e));
     return LFMM_OK;
@@ -1389,7 +1410,7 @@ int lfmm_forest_create(lfmm_plan** plan, const int32_t* src_xy, const int64_t* s
         p->forest.reset(new (std::nothrow) Forest());
         if (!p->forest) return fail(LFMM_ENOMEM, "host allocation failed");
         if ((r = forest_build(*p->forest, src, src_offsets, ns, tgt, tgt_offsets, nt, (int)n_problems, o.leaf_size,
-                              o.max_leaf_side, s, &pt)))
+                              o.max_leaf_side, o.precision != LFMM_MIXED, s, &pt)))
             return r;
         return forest_workspaces(p, s);
     };

@@ -675,12 +675,37 @@ struct LStripCfg {
     static constexpr int CAPS = 2048;
     static constexpr int CAPT = 1536;
     static constexpr int MAXSW = 32;
-    // the builder sizes strips with the smallest of these (kStripCapSrc: the binary64 case)
+    // (the builder sizes strips with these, those of the 8-byte types with near8_caps)
     static_assert(MAXSW == kStripMaxSW && CAPT == kStripCapTgt && CAPS >= kStripCapSrc, "strip staging caps");
 };
 
-template <typename T, int NP>
-__global__ void __launch_bounds__(LStripCfg<T>::WARPS * 32) p2p_list_kernel(
+// The near field of the 8-byte types is its own launch (kNear; kFar then adds L2P), so that
+// it runs beside the far field and in blocks of its own shape: one block of 24 warps per
+// SM, because the float-float / binary64 table (146 KB at side 32) leaves no room for a
+// second block, and as many staged sources as fit (near8_caps).  Its warps share a strip's
+// work evenly whatever the number of targets: G = 1 .. 32 lanes take one target and every
+// G-th source of its three rows, and the lanes' sums are added by shuffles; strips of few
+// targets among many sources (clustered points, scattered targets) had kept one warp of
+// six busy.  Float-float pairs are added without renormalising each term (12 instead of
+// 15 operations).
+constexpr int kBoth = 0, kNear = 1, kFar = 2;
+constexpr int kNearThreads = 768;
+
+// acc += a b with the two-sum's and the product's errors collected in acc.lo
+__device__ __forceinline__ void near_add(DF& acc, DF a, DF b) {
+    const float p = a.hi * b.hi;
+    float e = fmaf(a.hi, b.hi, -p);
+    e = fmaf(a.hi, b.lo, e);
+    e = fmaf(a.lo, b.hi, e);
+    const float s = acc.hi + p, bb = s - acc.hi;
+    e += (acc.hi - (s - bb)) + (p - bb);
+    acc.hi = s;
+    acc.lo += e;
+}
+__device__ __forceinline__ void near_add(double& acc, double a, double b) { acc = fma(a, b, acc); }
+
+template <typename T, int NP, int PART>
+__global__ void __launch_bounds__(PART == kNear ? kNearThreads : LStripCfg<T>::WARPS * 32) p2p_list_kernel(
     const int4* __restrict__ strips, const int4* __restrict__ strip_rows, const int32_t* __restrict__ n_strips_d,
     const int32_t* __restrict__ Lp, const uint64_t* __restrict__ rl_key, const int32_t* __restrict__ rl_s,
     const int32_t* __restrict__ rl_t, const int32_t* __restrict__ rl_id, int kb, int side, int SW,
@@ -688,17 +713,19 @@ __global__ void __launch_bounds__(LStripCfg<T>::WARPS * 32) p2p_list_kernel(
     const T* __restrict__ f_sorted,
     const T* __restrict__ table, int tab_H, int tab_W, const T* __restrict__ uhat,
     const typename Mono<T>::V* __restrict__ Cleaf, const typename Mono<T>::V* __restrict__ Qleaf,
-    const T* __restrict__ tofsT, double* __restrict__ u, double* __restrict__ u_near, double* __restrict__ u_far) {
+    const T* __restrict__ tofsT, double* __restrict__ u, double* __restrict__ u_near, double* __restrict__ u_far,
+    int caps, double* __restrict__ near_tmp) {
     griddep_wait();
     using M = Mono<T>;
     using V = typename M::V;
     using Cfg = LStripCfg<T>;
+    constexpr bool kHasNear = PART != kFar, kHasFar = PART != kNear;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int tab_n = (2 * tab_H + 1) * tab_W;
+    const int tab_n = kHasNear ? (2 * tab_H + 1) * tab_W : 0;
     T* tab = reinterpret_cast<T*>(smem_raw);
     SrcEntry<T>* s_src = reinterpret_cast<SrcEntry<T>*>(tab + tab_n);
-    T* s_uhat = reinterpret_cast<T*>(s_src + Cfg::CAPS);      // [MAXSW][NP]
-    V* s_q = reinterpret_cast<V*>(s_uhat + Cfg::MAXSW * NP);  // [3][MAXSW+2]
+    T* s_uhat = reinterpret_cast<T*>(s_src + (kHasNear ? caps : 0));      // [MAXSW][NP]
+    V* s_q = reinterpret_cast<V*>(s_uhat + (kHasFar ? Cfg::MAXSW * NP : 0));  // [3][MAXSW+2]
     V* s_c = s_q + 3 * (Cfg::MAXSW + 2);                      // [MAXSW]
     int* s_tloc = reinterpret_cast<int*>(s_c + Cfg::MAXSW);   // [CAPT]
     int* s_tperm = s_tloc + Cfg::CAPT;                        // [CAPT]
@@ -711,8 +738,8 @@ __global__ void __launch_bounds__(LStripCfg<T>::WARPS * 32) p2p_list_kernel(
     __shared__ int s_rj[3][2];                 // leaf-list range [j0, j1) of each row (-1: outside)
     __shared__ int s_lc[3][Cfg::MAXSW + 2];    // column - c_lo of each listed leaf (ascending)
 
-    block_stage(tab, table, tab_n);
-    const V phi0 = M::make(table[tab_n], table[tab_n + 1]);
+    if (kHasNear) block_stage(tab, table, tab_n);
+    const V phi0 = kHasNear ? M::make(table[tab_n], table[tab_n + 1]) : M::zero();
     const T* tab_c = tab + (tab_H + tab_H * tab_W);
     const int n_strips = *n_strips_d;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -798,7 +825,7 @@ __global__ void __launch_bounds__(LStripCfg<T>::WARPS * 32) p2p_list_kernel(
         }
         __syncthreads();
         // the strip's leaf expansions (four loads in flight per thread)
-        for (int i0 = threadIdx.x; i0 < (bx1 - bx0) * NP; i0 += 4 * blockDim.x) {
+        for (int i0 = threadIdx.x; kHasFar && i0 < (bx1 - bx0) * NP; i0 += 4 * blockDim.x) {
             T vals[4];
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
@@ -812,7 +839,7 @@ __global__ void __launch_bounds__(LStripCfg<T>::WARPS * 32) p2p_list_kernel(
                 if (i < (bx1 - bx0) * NP) s_uhat[i] = vals[k];
             }
         }
-        for (int li = threadIdx.x; li < bx1 - bx0; li += blockDim.x) {
+        for (int li = threadIdx.x; kHasNear && li < bx1 - bx0; li += blockDim.x) {
             const int bx = bx0 + li;
             const int ca = max(bx - 1, 0) - c_lo, cb = min(bx + 1, n - 1) - c_lo + 1;
             int rs = 0;
@@ -837,12 +864,58 @@ __global__ void __launch_bounds__(LStripCfg<T>::WARPS * 32) p2p_list_kernel(
         }
         __syncthreads();
         const int ns_strip = s_rs[3];
-        stage_strip_sources<T>(s_src, ns_strip, s_rs, s_sb, Cfg::MAXSW + 3, ncol, c_lo, bx0, side, tab_W, sloc,
+        if (kHasNear) stage_strip_sources<T>(s_src, ns_strip, s_rs, s_sb, Cfg::MAXSW + 3, ncol, c_lo, bx0, side, tab_W, sloc,
                                f_sorted);
         const int tb0 = s_tb[0], nt_strip = s_tb[bx1 - bx0] - tb0;
         stage_strip_targets(s_tloc, s_tperm, nt_strip, s_tb, bx1 - bx0, tb0, tloc, tperm);
         __syncthreads();
 
+        if constexpr (PART == kNear) {
+            const int warps = blockDim.x >> 5;
+            int lg = 0;  // G = 2^lg lanes per target: at least two units of 32 / G targets per warp
+            while (lg < 5 && (nt_strip << lg) < 64 * warps) ++lg;
+            const int G = 1 << lg, sub = lane & (G - 1), per = 32 >> lg;
+            const int units = (nt_strip + per - 1) / per;
+            for (int unit = warp; unit < units; unit += warps) {
+                const int v = unit * per + (lane >> lg);
+                const bool active = v < nt_strip;
+                const int tl = s_tloc[active ? v : 0];
+                const int li = (tl >> 8) & 0xff, tx = tl & 0xff, ty = tl >> 16;
+                const T* tp = tab_c + (tx + tab_W * ty + li * side);
+                T acc = T(0);
+#pragma unroll
+                for (int r = 0; r < 3; ++r) {
+                    const SrcEntry<T>* src = s_src + s_ra[li][r];
+                    const int len = active ? s_rl[li][r] : 0;
+                    int j = sub;
+                    for (; j + 3 * G < len; j += 4 * G) {
+                        const SrcEntry<T> e0 = src[j], e1 = src[j + G], e2 = src[j + 2 * G], e3 = src[j + 3 * G];
+                        const T t0 = tp[-e0.off], t1 = tp[-e1.off], t2 = tp[-e2.off], t3 = tp[-e3.off];
+                        near_add(acc, t0, e0.f);
+                        near_add(acc, t1, e1.f);
+                        near_add(acc, t2, e2.f);
+                        near_add(acc, t3, e3.f);
+                    }
+                    for (; j < len; j += G) {
+                        const SrcEntry<T> e = src[j];
+                        near_add(acc, tp[-e.off], e.f);
+                    }
+                }
+                for (int o = 1; o < G; o <<= 1) acc += shfl_xor_v(acc, o);
+                if (active && sub == 0) {
+                    const double dn = (double)acc + s_nc[li];
+                    if (near_tmp) {
+                        near_tmp[tb0 + v] = dn;
+                    } else {  // no far field
+                        const int dst = s_tperm[v];
+                        if (u) u[dst] = dn;
+                        if (u_near) u_near[dst] = dn;
+                        if (u_far) u_far[dst] = 0.0;
+                    }
+                }
+            }
+            continue;
+        }
         const int n_chunks = (nt_strip + 31) >> 5;
         for (int chunk = warp; chunk < n_chunks; chunk += Cfg::WARPS) {
             const int v = chunk * 32 + lane;
@@ -852,7 +925,7 @@ __global__ void __launch_bounds__(LStripCfg<T>::WARPS * 32) p2p_list_kernel(
             const int li = (tl >> 8) & 0xff, tx = tl & 0xff, ty = tl >> 16;
             const T* tp = tab_c + (tx + tab_W * ty + li * side);
             T acc = T(0), cmp = T(0);
-            auto add = [&](T term) {
+            [[maybe_unused]] auto add = [&](T term) {
                 if constexpr (sizeof(T) == 4) {
                     const T y = term - cmp;
                     const T s2 = acc + y;
@@ -862,6 +935,7 @@ __global__ void __launch_bounds__(LStripCfg<T>::WARPS * 32) p2p_list_kernel(
                     acc += term;
                 }
             };
+            if constexpr (PART == kBoth) {
 #pragma unroll
             for (int r = 0; r < 3; ++r) {
                 const SrcEntry<T>* src = s_src + s_ra[li][r];
@@ -886,6 +960,7 @@ __global__ void __launch_bounds__(LStripCfg<T>::WARPS * 32) p2p_list_kernel(
                 }
             }
             acc -= cmp;
+            }
             T far = T(0);
             if (uhat) {
                 constexpr int PL = NP / 32;
@@ -907,7 +982,7 @@ __global__ void __launch_bounds__(LStripCfg<T>::WARPS * 32) p2p_list_kernel(
             }
             if (active) {
                 const int dst = s_tperm[v];
-                const double dn = (double)acc + s_nc[li];
+                const double dn = PART == kFar ? near_tmp[tb0 + v] : (double)acc + s_nc[li];
                 const double df = (double)far + M::to_double(s_c[li]);
                 if (u) u[dst] = dn + df;
                 if (u_near) u_near[dst] = dn;
@@ -982,10 +1057,47 @@ SgTree forest_sg_tree(const Forest& F) {
     return t;
 }
 
+template <typename T, int PART>
+static int launch_list_p2p(const Forest& F, const DeviceOps& ops, const T* f_sorted, const T* uhat, const void* Cleaf,
+                           const void* Qleaf, double* u, double* un, double* uf, int num_sms, cudaStream_t s,
+                           bool use_tmp) {
+    using Cfg = LStripCfg<T>;
+    using V = typename Mono<T>::V;
+    PhaseTimer pt(PART == kFar ? LFMM_PHASE_L2P : LFMM_PHASE_P2P, s);
+    const int NP = ops.NP;
+    const int caps = PART == kNear ? near8_caps(F.side) : Cfg::CAPS;
+    size_t smem = (size_t)(3 * (Cfg::MAXSW + 2) + Cfg::MAXSW) * sizeof(V) + (size_t)2 * Cfg::CAPT * sizeof(int) +
+                  (size_t)(3 * (Cfg::MAXSW + 3) + Cfg::MAXSW + 1) * sizeof(int);
+    if (PART != kFar)
+        smem += (size_t)(2 * ops.tab_H + 1) * ops.tab_W * sizeof(T) + (size_t)caps * sizeof(SrcEntry<T>);
+    if (PART != kNear) smem += (size_t)Cfg::MAXSW * NP * sizeof(T);
+    const int threads = PART == kNear ? kNearThreads : Cfg::WARPS * 32;
+    auto go = [&](auto np_tag) -> cudaError_t {
+        constexpr int NPc = decltype(np_tag)::value;
+        const void* fn = (const void*)p2p_list_kernel<T, NPc, PART>;
+        const cudaError_t e = ensure_dynamic_smem(fn, smem);
+        if (e != cudaSuccess) return e;
+        const int per_sm = blocks_per_sm(fn, threads, smem);
+        // the near field beside the far field: blocks of a few strips, so that the far
+        // field's launches (of a higher priority) find free SMs as blocks end
+        const int64_t waves = PART == kNear && use_tmp ? 6 : 1;
+        const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(F.n_strips, waves * num_sms * per_sm));
+        return launch_dependent(p2p_list_kernel<T, NPc, PART>, dim3((unsigned)grid), dim3(threads), smem, s, F.strips,
+                                F.strip_rows, F.n_strips_d, F.d_L, F.rl_key, F.rl_s, F.rl_t, F.rl_id, F.kb, F.side,
+                                F.SW, F.sloc, F.tloc, F.tperm, f_sorted, (const T*)ops.p2p_table, ops.tab_H, ops.tab_W,
+                                uhat, (const V*)Cleaf, (const V*)Qleaf, (const T*)ops.tofsT, u, un, uf, caps,
+                                use_tmp ? F.near_tmp : nullptr);
+    };
+    const cudaError_t e = NP == 32 ? go(std::integral_constant<int, 32>()) : go(std::integral_constant<int, 64>());
+    if (e != cudaSuccess) return fail(LFMM_ECUDA, std::string("p2p_list_kernel: ") + cudaGetErrorString(e));
+    pt.add_launches(1);
+    return LFMM_OK;
+}
+
 template <typename T>
 int forest_eval(const Forest& F, const DeviceOps& ops, const double* f, T* f_sorted, T* qhat, T* uhat, void* Qbox,
                 void* Cbox, double* u, double* un, double* uf, int num_sms, cudaStream_t s, int* status_word,
-                bool persistent) {
+                bool persistent, const SideStream* side) {
     // the sliced far field (split_tc.cu) has one form; the persistent sweeps are those of the
     // other kernels
     const bool sliced = sizeof(T) == 8 && F.sg_work != nullptr && status_word != nullptr;
@@ -1047,7 +1159,21 @@ int forest_eval(const Forest& F, const DeviceOps& ops, const double* f, T* f_sor
             pt.add_launches(1);
         }
     }
+    // the near field of the 8-byte types needs the sorted charges and the leaf charges only:
+    // it runs on the caller's stream, the rest of the far field on the side stream
+    const cudaStream_t s_main = s;
+    const bool fork = sizeof(T) == 8 && far && side != nullptr;
     if constexpr (sizeof(T) == 8) {
+        if (fork) {
+            LFMM_CUDA_TRY(cudaEventRecord(side->fork, s));
+            LFMM_CUDA_TRY(cudaStreamWaitEvent(side->s, side->fork, 0));
+            s = side->s;
+        }
+        if (far) {
+            const int st = launch_list_p2p<T, kNear>(F, ops, f_sorted, (const T*)nullptr, nullptr, Qm(0), nullptr, nullptr,
+                                                     nullptr, num_sms, s_main, true);
+            if (st) return st;
+        }
         if (far && sliced) {
             PhaseTimer pt(LFMM_PHASE_M2L_TC, s);
             int n = 0;
@@ -1216,40 +1342,26 @@ int forest_eval(const Forest& F, const DeviceOps& ops, const double* f, T* f_sor
             pt.add_launches(nc > 1 ? 2 : 1);
         }
     }
-    {
-        PhaseTimer pt(LFMM_PHASE_P2P, s);
-        using Cfg = LStripCfg<T>;
-        const size_t tab_bytes = (size_t)(2 * ops.tab_H + 1) * ops.tab_W * sizeof(T);
-        const size_t smem = tab_bytes + (size_t)Cfg::CAPS * sizeof(SrcEntry<T>) +
-                            (size_t)Cfg::MAXSW * NP * sizeof(T) +
-                            (size_t)(3 * (Cfg::MAXSW + 2) + Cfg::MAXSW) * sizeof(V) + (size_t)2 * Cfg::CAPT * sizeof(int) +
-                            (size_t)(3 * (Cfg::MAXSW + 3) + Cfg::MAXSW + 1) * sizeof(int);
-        auto go = [&](auto np_tag) -> cudaError_t {
-            constexpr int NPc = decltype(np_tag)::value;
-            {
-                cudaError_t e = ensure_dynamic_smem((const void*)p2p_list_kernel<T, NPc>, smem);
-                if (e != cudaSuccess) return e;
-            }
-            const int per_sm = blocks_per_sm((const void*)p2p_list_kernel<T, NPc>, Cfg::WARPS * 32, smem);
-            (void)launch_dependent(p2p_list_kernel<T, NPc>, dim3(num_sms * per_sm), dim3(Cfg::WARPS * 32), smem, s,
-                F.strips, F.strip_rows, F.n_strips_d, F.d_L, F.rl_key, F.rl_s, F.rl_t, F.rl_id, F.kb, F.side, F.SW,
-                F.sloc, F.tloc, F.tperm, f_sorted,
-                (const T*)ops.p2p_table, ops.tab_H, ops.tab_W, far ? Ux(0) : nullptr, far ? Cm(0) : nullptr, Qm(0),
-                (const T*)ops.tofsT, u, un, uf);
-            return cudaGetLastError();
-        };
-        cudaError_t e = NP == 32 ? go(std::integral_constant<int, 32>()) : go(std::integral_constant<int, 64>());
-        if (e != cudaSuccess) return fail(LFMM_ECUDA, std::string("p2p_list_kernel: ") + cudaGetErrorString(e));
-        pt.add_launches(1);
+    // near field (+ L2P): one launch for binary32; for the 8-byte types the near field was
+    // launched beside the far field and L2P follows it here
+    if constexpr (sizeof(T) == 8) {
+        if (!far) return launch_list_p2p<T, kNear>(F, ops, f_sorted, (const T*)nullptr, nullptr, Qm(0), u, un, uf, num_sms, s, false);
+        if (fork) {
+            LFMM_CUDA_TRY(cudaEventRecord(side->join, s));
+            LFMM_CUDA_TRY(cudaStreamWaitEvent(s_main, side->join, 0));
+        }
+        return launch_list_p2p<T, kFar>(F, ops, f_sorted, (const T*)Ux(0), Cm(0), Qm(0), u, un, uf, num_sms, s_main, true);
+    } else {
+        return launch_list_p2p<T, kBoth>(F, ops, f_sorted, (const T*)(far ? Ux(0) : nullptr), far ? Cm(0) : nullptr, Qm(0), u, un, uf, num_sms, s,
+                                         false);
     }
-    return LFMM_OK;
 }
 
 template int forest_eval<float>(const Forest&, const DeviceOps&, const double*, float*, float*, float*, void*, void*,
-                                double*, double*, double*, int, cudaStream_t, int*, bool);
+                                double*, double*, double*, int, cudaStream_t, int*, bool, const SideStream*);
 template int forest_eval<double>(const Forest&, const DeviceOps&, const double*, double*, double*, double*, void*,
-                                 void*, double*, double*, double*, int, cudaStream_t, int*, bool);
+                                 void*, double*, double*, double*, int, cudaStream_t, int*, bool, const SideStream*);
 template int forest_eval<DF>(const Forest&, const DeviceOps&, const double*, DF*, DF*, DF*, void*, void*, double*,
-                             double*, double*, int, cudaStream_t, int*, bool);
+                             double*, double*, int, cudaStream_t, int*, bool, const SideStream*);
 
 }  // namespace lfmm

@@ -797,8 +797,8 @@ int unique_runs(const uint64_t* key, int64_t n, uint64_t skip, uint64_t* out, in
 }  // namespace
 
 int forest_build(Forest& F, const int32_t* src, const int64_t* soff_h, int64_t ns, const int32_t* tgt,
-                 const int64_t* toff_h, int64_t nt, int np, int leaf_size, int max_leaf_side, cudaStream_t s,
-                 PhaseTimer* timer) {
+                 const int64_t* toff_h, int64_t nt, int np, int leaf_size, int max_leaf_side, bool wide,
+                 cudaStream_t s, PhaseTimer* timer) {
     int st;
     F.np = np;
     F.ns = ns;
@@ -1215,9 +1215,10 @@ int forest_build(Forest& F, const int32_t* src, const int64_t* soff_h, int64_t n
     const int SW = std::min({kStripMaxSW, kStripCapSrc / (3 * msr) - 2, kStripCapTgt / mtg});
     if (SW < 1) return fail(LFMM_EUNSUPPORTED, "leaves too full for the near-field staging (" + std::to_string(msr) +
                                                    " sources / " + std::to_string(mtg) + " targets)");
-    F.SW = SW;
+    // (the same leaves are refused whatever the element type)
+    F.SW = wide ? std::min({kStripMaxSW, near8_caps(F.side) / (3 * msr) - 2, kStripCapTgt / mtg}) : SW;
     {
-        strip_flag_kernel<<<grid_of(M), kT, 0, s>>>(F.rl_key, F.rl_t, M, kb, SW, flag);
+        strip_flag_kernel<<<grid_of(M), kT, 0, s>>>(F.rl_key, F.rl_t, M, kb, F.SW, flag);
         LFMM_CUDA_TRY(exscan(flag, pos, M, ssum, s));
         int32_t nstr = 0;
         LFMM_CUDA_TRY(cudaMemcpyAsync(&nstr, pos + M, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
@@ -1228,8 +1229,9 @@ int forest_build(Forest& F, const int32_t* src, const int64_t* soff_h, int64_t n
         F.strip_rows = F.strips + n4;
         F.n_strips_d = (int32_t*)(F.strip_rows + 2 * n4);
         LFMM_CUDA_TRY(cudaMemcpyAsync(F.n_strips_d, pos + M, sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
-        strip_record_kernel<<<grid_of(M), kT, 0, s>>>(F.rl_key, flag, pos, M, kb, SW, F.strips);
-        strip_rows_kernel<<<grid_of(nstr), kT, 0, s>>>(F.strips, nstr, F.rl_key, M, dL, kb, SW, F.strip_rows);
+        strip_record_kernel<<<grid_of(M), kT, 0, s>>>(F.rl_key, flag, pos, M, kb, F.SW, F.strips);
+        F.n_strips = nstr;
+        strip_rows_kernel<<<grid_of(nstr), kT, 0, s>>>(F.strips, nstr, F.rl_key, M, dL, kb, F.SW, F.strip_rows);
         LFMM_CUDA_TRY(cudaGetLastError());
         timer->add_launches(6);
     }

@@ -261,6 +261,20 @@ struct ForestLevel {
 constexpr int kStripMaxSW = 32;
 constexpr int kStripCapSrc = 2048;
 constexpr int kStripCapTgt = 1536;
+// Row width of the P2P table of a leaf side: at least 2H + 1 = 4 side - 1, and 16 mod 32 so
+// that targets in the same column but in rows of different parity fall in different
+// shared-memory banks.
+inline int p2p_table_width(int side) {
+    int w = 16;
+    while (w < 4 * side - 1) w += 32;
+    return w;
+}
+// Staged sources of the 8-byte types' near field (one block per SM): what 220,000 bytes of
+// shared memory leave beside the table, the targets and the strip's bookkeeping.
+inline int near8_caps(int side) {
+    const int tab = (4 * side - 1) * p2p_table_width(side) * 8;
+    return std::min(8192, (220000 - tab - 2 * kStripCapTgt * 4 - 3072) / 16);
+}
 
 struct Forest {
     int np = 0;
@@ -287,6 +301,8 @@ struct Forest {
     // 2 int4 per strip {j0 r0, j1 r0, j0 r1, j1 r1}, {j0 r2, j1 r2, 0, 0}
     int4* strip_rows = nullptr;
     int32_t* n_strips_d = nullptr;
+    int64_t n_strips = 0;
+    double* near_tmp = nullptr;                 // near field per sorted target, before the far part is added
     std::vector<void*> owned;
     int64_t bytes = 0;
     void* m2l_part = nullptr;               // partial sums of K-split list M2L levels (plan-owned)
@@ -306,18 +322,25 @@ int64_t forest_m2l_split_bytes(const Forest& F, int NP, size_t esz, int num_sms,
 
 // Builds the tree of every problem (offsets: n_problems + 1 entries, host memory).
 // Leaf side: the largest power of two <= max_leaf_side at which no leaf holds more than
-// leaf_size sources or targets.  Synchronises the stream.
+// leaf_size sources or targets.  wide: strips for the near field of the 8-byte types.
+// Synchronises the stream.
 int forest_build(Forest& F, const int32_t* src, const int64_t* soff_h, int64_t ns, const int32_t* tgt,
-                 const int64_t* toff_h, int64_t nt, int np, int leaf_size, int max_leaf_side, cudaStream_t s,
-                 PhaseTimer* timer);
+                 const int64_t* toff_h, int64_t nt, int np, int leaf_size, int max_leaf_side, bool wide,
+                 cudaStream_t s, PhaseTimer* timer);
 // status: the plan's status word (grid-barrier words beside it; timed-out waits are
 // recorded there); persistent: run each sweep as one persistent cooperative launch
 // (LFMM_FLAG_PERSISTENT), else one launch per level, the list M2L of levels with at
 // least kTcListMinBoxes boxes on the tensor cores when F.tc_list is set.
+// side: a second stream (of higher priority) with its fork and join events, for the far
+// field beside the near field; null: one after the other on s.
+struct SideStream {
+    cudaStream_t s;
+    cudaEvent_t fork, join;
+};
 template <typename T>
 int forest_eval(const Forest& F, const DeviceOps& ops, const double* f, T* f_sorted, T* qhat, T* uhat, void* Qbox,
                 void* Cbox, double* u, double* un, double* uf, int num_sms, cudaStream_t s, int* status,
-                bool persistent);
+                bool persistent, const SideStream* side);
 // Tensor-core M2L + L2L over the compact box lists of one pruned / forest level (mixed
 // path, P_pad 32 or 64): splits the level's expansions (nb rows) and the parent level's
 // incoming expansions (nb_parent rows, none without L2L) into TF32 hi / lo rows in
