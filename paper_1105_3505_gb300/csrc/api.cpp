@@ -27,6 +27,20 @@ const char* last_error_cstr() { return t_last_error.c_str(); }
 // lfmm_fault_inject_alloc: allocations left until the failing one (0: disarmed)
 std::atomic<int64_t> g_alloc_fail_in{0};
 
+// Page-locked host words for the tree build's readbacks (one set per host thread): a
+// copy into pageable memory would be staged by the driver and complete later.
+int* readback_words() {
+    static thread_local int* words = [] {
+        void* h = nullptr;
+        if (cudaMallocHost(&h, kReadbackWords * sizeof(int)) != cudaSuccess) {
+            cudaGetLastError();
+            h = nullptr;
+        }
+        return (int*)h;
+    }();
+    return words;
+}
+
 cudaError_t dev_malloc(void** ptr, size_t bytes, cudaStream_t s) {
     int64_t n = g_alloc_fail_in.load(std::memory_order_relaxed);
     while (n > 0) {
@@ -256,20 +270,6 @@ int validate_opts(const lfmm_opts& o) {
     if (o.m2l_split < 0 || o.m2l_split > 9) return fail(LFMM_EINVAL, "opts.m2l_split must be in [0, 9]");
     if (o.reserved != 0) return fail(LFMM_EINVAL, "opts.reserved must be 0");
     return LFMM_OK;
-}
-
-// Page-locked host words for the tree build's readbacks (one set per host thread): a
-// copy into pageable memory would be staged by the driver and complete later.
-int* readback_words() {
-    static thread_local int* words = [] {
-        void* h = nullptr;
-        if (cudaMallocHost(&h, 16 * sizeof(int)) != cudaSuccess) {
-            cudaGetLastError();
-            h = nullptr;
-        }
-        return (int*)h;
-    }();
-    return words;
 }
 
 int ilog2_ceil(int64_t v) {
@@ -547,8 +547,9 @@ int plan_build(lfmm_plan* p, const int32_t* src_xy, const int32_t* tgt_xy, cudaS
         p->forest.reset(new (std::nothrow) Forest());
         if (!p->forest) return fail(LFMM_ENOMEM, "host allocation failed");
         const int64_t so[2] = {0, p->ns}, to[2] = {0, p->nt};
+        const ForestHint hint{h10[0], h10[1], h10[2], h10[3], p->ns != p->nt ? 0 : differ_known ? (int)same : -1};
         if ((st = forest_build(*p->forest, src, so, p->ns, tgt, to, p->nt, 1, p->opts.leaf_size, p->side,
-                               p->opts.precision != LFMM_MIXED, s, &pt)))
+                               p->opts.precision != LFMM_MIXED, &hint, s, &pt)))
             return st;
         return forest_workspaces(p, s);
     }
@@ -1410,7 +1411,7 @@ int lfmm_forest_create(lfmm_plan** plan, const int32_t* src_xy, const int64_t* s
         p->forest.reset(new (std::nothrow) Forest());
         if (!p->forest) return fail(LFMM_ENOMEM, "host allocation failed");
         if ((r = forest_build(*p->forest, src, src_offsets, ns, tgt, tgt_offsets, nt, (int)n_problems, o.leaf_size,
-                              o.max_leaf_side, o.precision != LFMM_MIXED, s, &pt)))
+                              o.max_leaf_side, o.precision != LFMM_MIXED, nullptr, s, &pt)))
             return r;
         return forest_workspaces(p, s);
     };

@@ -13,12 +13,15 @@
 //      grids, else the sorted keys), so the sources of a leaf row segment are one
 //      contiguous range, and lists the occupied leaves with their first source and
 //      target;
-//   3. builds the boxes of every level at once: each leaf emits its level-k key where it
-//      heads its level-k row segment, one sort and one unique pass give every level's
-//      boxes; one stable partition by (level, class) numbers each level's boxes in
-//      parity-class order (class, problem, (y >> 1, x >> 1) row by row: each class one
-//      contiguous range of compact ids), and one kernel finds parents, children and
-//      interaction lists by binary search;
+//   3. builds the boxes of every level at once, numbered level by level in parity-class
+//      order (class, problem, (y >> 1, x >> 1) row by row: each class one contiguous range
+//      of compact ids).  While a bit per cell of every level is affordable (grid_words_max),
+//      the boxes are the set bits of grids laid out in that very order: a leaf sets its
+//      ancestors' bits, one scan of the words' populations numbers the boxes, and parents,
+//      children and interaction lists are bit tests and ranks.  Deeper trees of few points
+//      keep sorted keys: each leaf emits its level-k key where it heads its level-k row
+//      segment, one sort and one unique pass give every level's boxes, one stable partition
+//      by (level, class) their numbers, and the links are binary searches;
 //   4. lists the near-field strips (SW consecutive leaves of a row holding a target) and
 //      the occupied leaves of each strip's three neighbour-row segments.
 // The sorts are a stable least-significant-digit radix sort (8-bit digits, per-block
@@ -43,12 +46,19 @@ int grid_of(int64_t n, int threads = kT, int cap = 152 * 16) {
 // ------------------------------------------------------------------------- exclusive scan
 constexpr int kScanBlock = 1024;
 
+// POP: the items are the populations of the words in[i]
+template <bool POP>
+__device__ __forceinline__ int32_t scan_item(int32_t v) {
+    return POP ? __popc((unsigned)v) : v;
+}
+
+template <bool POP>
 __global__ void scan_reduce_kernel(const int32_t* __restrict__ in, int64_t n, int32_t* __restrict__ sums) {
     __shared__ int32_t w[kT / 32];
     const int64_t base = (int64_t)blockIdx.x * kScanBlock;
     int32_t v = 0;
     for (int i = threadIdx.x; i < kScanBlock; i += blockDim.x)
-        if (base + i < n) v += in[base + i];
+        if (base + i < n) v += scan_item<POP>(in[base + i]);
     for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
     if ((threadIdx.x & 31) == 0) w[threadIdx.x >> 5] = v;
     __syncthreads();
@@ -94,6 +104,7 @@ __global__ void scan_sums_kernel(int32_t* __restrict__ sums, int nb) {
     if (threadIdx.x == 0) sums[nb] = carry_s;
 }
 
+template <bool POP>
 __global__ void scan_apply_kernel(const int32_t* __restrict__ in, int64_t n, const int32_t* __restrict__ sums,
                                   int32_t* __restrict__ out) {
     __shared__ int32_t w[kT / 32];
@@ -102,7 +113,7 @@ __global__ void scan_apply_kernel(const int32_t* __restrict__ in, int64_t n, con
     int32_t v[PER], t = 0;
 #pragma unroll
     for (int j = 0; j < PER; ++j) {
-        v[j] = base + j < n ? in[base + j] : 0;
+        v[j] = base + j < n ? scan_item<POP>(in[base + j]) : 0;
         t += v[j];
     }
     int32_t x = t;
@@ -134,13 +145,62 @@ __global__ void scan_apply_kernel(const int32_t* __restrict__ in, int64_t n, con
 
 int64_t scan_tmp_ints(int64_t n) { return (n + kScanBlock - 1) / kScanBlock + 1; }
 
+// The whole scan in one block, for arrays of up to kScanSmall items: 32 items per thread and
+// turn, one launch instead of three (5 instead of 8 us of device time on 16,384 items, and
+// two launches fewer on the host, which is what the building of small trees waits for).
+constexpr int64_t kScanSmall = 65536;
+template <bool POP>
+__global__ void __launch_bounds__(1024) scan_small_kernel(const int32_t* __restrict__ in, int n,
+                                                          int32_t* __restrict__ out) {
+    __shared__ int32_t w[32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    int32_t carry = 0;
+    for (int base = 0; base < n; base += 16384) {
+        const int i0 = base + 16 * threadIdx.x;
+        int32_t v[16], t = 0;
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+            v[j] = i0 + j < n ? scan_item<POP>(in[i0 + j]) : 0;
+            t += v[j];
+        }
+        int32_t x = t;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t y = __shfl_up_sync(kFull, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) w[wid] = x;
+        __syncthreads();
+        int32_t s = w[lane];
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t y = __shfl_up_sync(kFull, s, o);
+            if (lane >= o) s += y;
+        }
+        const int32_t before = wid > 0 ? __shfl_sync(kFull, s, wid - 1) : 0;
+        const int32_t total = __shfl_sync(kFull, s, 31);
+        int32_t run = carry + before + x - t;
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+            if (i0 + j < n) out[i0 + j] = run;
+            run += v[j];
+        }
+        carry += total;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) out[n] = carry;
+}
+
 // out[0..n] = exclusive prefix sums of in[0..n) (out[n] = total); sums: scan_tmp_ints(n)
+template <bool POP = false>
 cudaError_t exscan(const int32_t* in, int32_t* out, int64_t n, int32_t* sums, cudaStream_t s) {
     const int64_t nb = (n + kScanBlock - 1) / kScanBlock;
     if (nb == 0) return cudaMemsetAsync(out, 0, sizeof(int32_t), s);
-    scan_reduce_kernel<<<(unsigned)nb, kT, 0, s>>>(in, n, sums);
+    if (n <= kScanSmall) {
+        scan_small_kernel<POP><<<1, 1024, 0, s>>>(in, (int)n, out);
+        return cudaGetLastError();
+    }
+    scan_reduce_kernel<POP><<<(unsigned)nb, kT, 0, s>>>(in, n, sums);
     scan_sums_kernel<<<1, 1024, 0, s>>>(sums, (int)nb);
-    scan_apply_kernel<<<(unsigned)nb, kT, 0, s>>>(in, n, sums, out);
+    scan_apply_kernel<POP><<<(unsigned)nb, kT, 0, s>>>(in, n, sums, out);
     return cudaGetLastError();
 }
 
@@ -366,7 +426,7 @@ __global__ void leaf_key_kernel(const int2* __restrict__ xy, int64_t n, const in
                                 const int32_t* __restrict__ x0, const int32_t* __restrict__ y0, int ls, int kb,
                                 uint64_t* __restrict__ key, uint32_t* __restrict__ idx) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int p = pid[i];
+        const int p = pid ? pid[i] : 0;
         const int2 v = xy[i];
         const int bx = (int)(((int64_t)v.x - x0[p]) >> ls), by = (int)(((int64_t)v.y - y0[p]) >> ls);
         key[i] = pack_key(p, by, bx, kb);
@@ -411,7 +471,7 @@ __global__ void point_order_kernel(const int2* __restrict__ xy, int64_t n, const
     const int mask = (1 << ls) - 1;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t j = idx[i];
-        const int p = pid[j];
+        const int p = pid ? pid[j] : 0;
         const int2 v = xy[j];
         const int lx = (int)(((int64_t)v.x - x0[p]) & mask), ly = (int)(((int64_t)v.y - y0[p]) & mask);
         loc[i] = lx | (ly << 16);
@@ -598,6 +658,197 @@ __global__ void links_kernel(int64_t n, const uint64_t* __restrict__ ck, const u
     }
 }
 
+// ------------------------------------------------------------------------- bit grids
+// One bit per cell of every level: level k, class c, problem p is a grid of h x h bits, row
+// by row from a word boundary, h = max(1, 2^(L_p - k) / 2), at word
+// base[k] + c stride[k] + off[k np + p].  The words' order is the order of the compact ids,
+// so a box's id is the number of set bits before its own (rank).
+constexpr int kGridLevels = 21;
+struct BitGrid {
+    uint32_t base[kGridLevels], stride[kGridLevels];
+    int nk, np, kmax;
+    const uint32_t* off;  // null with one problem
+    const int32_t* L;
+    uint32_t* bits;
+    const int32_t* before;  // set bits before each word
+};
+__device__ __forceinline__ uint32_t grid_word(const BitGrid& G, int k, int c, int p) {
+    return G.base[k] + (uint32_t)c * G.stride[k] + (G.off ? G.off[k * G.np + p] : 0u);
+}
+
+// Every leaf's bit and those of its ancestors (levels >= 2 of its problem's tree).  A leaf
+// that follows another of the same box in its row leaves that box's and all higher bits to
+// the first one.
+__global__ void grid_set_kernel(const BitGrid G, const uint64_t* __restrict__ leaves, const int32_t* __restrict__ m_d,
+                                int kb) {
+    const int64_t m = *m_d;
+    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x) {
+        int p, y, x, pp = -1, yy = 0, xx = 0;
+        unpack_key(leaves[j], kb, p, y, x);
+        if (j > 0) unpack_key(leaves[j - 1], kb, pp, yy, xx);
+        const bool row = pp == p && yy == y;
+        const int l = G.L[p];
+        for (int k = 0; k < G.nk; ++k) {
+            if (k > 0 && (l - k < 2 || (row && (xx >> k) == (x >> k)))) break;
+            const int X = x >> k, Y = y >> k, h = max(1, (1 << (l - k)) >> 1);
+            const uint32_t i = (uint32_t)(Y >> 1) * (uint32_t)h + (uint32_t)(X >> 1);
+            atomicOr(G.bits + grid_word(G, k, (X & 1) | ((Y & 1) << 1), p) + (i >> 5), 1u << (i & 31));
+        }
+    }
+}
+
+// first id of every class of every level (entry 4 nk: all boxes), the level-local class
+// starts, and what the host waits for: {M, class starts}
+__global__ void grid_starts_kernel(const BitGrid G, int64_t words, const int32_t* __restrict__ m_d,
+                                   int64_t* __restrict__ cstart, int64_t* __restrict__ dcls, int* __restrict__ out) {
+    for (int t = threadIdx.x; t <= 4 * G.nk; t += blockDim.x) {
+        auto start = [&](int i) -> int32_t {
+            return G.before[i >= 4 * G.nk ? words : (int64_t)G.base[i >> 2] + (i & 3) * (int64_t)G.stride[i >> 2]];
+        };
+        const int32_t v = start(t);
+        cstart[t] = v;
+        out[1 + t] = v;
+        if (t < 4 * G.nk) {
+            dcls[5 * (t >> 2) + (t & 3)] = v - start(t & ~3);
+            if ((t & 3) == 3) dcls[5 * (t >> 2) + 4] = start(t + 1) - start(t & ~3);
+        }
+    }
+    if (threadIdx.x == 0) out[0] = *m_d;
+}
+
+// problem and coordinates of every box, word by word
+__global__ void grid_records_kernel(const BitGrid G, int64_t words, int32_t* __restrict__ bp,
+                                    int32_t* __restrict__ bxy) {
+    for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < words; w += (int64_t)gridDim.x * blockDim.x) {
+        uint32_t v = G.bits[w];
+        if (!v) continue;
+        int k = 0;
+        while (k + 1 < G.nk && (uint32_t)w >= G.base[k + 1]) ++k;
+        const uint32_t r = (uint32_t)w - G.base[k];
+        const int c = (int)(r / G.stride[k]);
+        const uint32_t in = r - (uint32_t)c * G.stride[k];
+        int p = 0;
+        if (G.off) {
+            int lo = 0, hi = G.np;  // off[p] <= in < off[p + 1]
+            while (hi - lo > 1) {
+                const int mid = (lo + hi) >> 1;
+                if (G.off[k * G.np + mid] <= in) lo = mid;
+                else hi = mid;
+            }
+            p = lo;
+        }
+        const int lh = max(0, G.L[p] - k - 1);
+        int id = G.before[w];
+        const uint32_t i0 = (in - (G.off ? G.off[k * G.np + p] : 0u)) * 32;
+        for (; v; v &= v - 1, ++id) {
+            const uint32_t i = i0 + (uint32_t)__ffs(v) - 1;
+            const int x = 2 * (int)(i & ((1u << lh) - 1)) + (c & 1), y = 2 * (int)(i >> lh) + (c >> 1);
+            bp[id] = p;
+            bxy[id] = x | (y << 16);
+        }
+    }
+}
+
+// the level-0 id of every leaf, and the leaf of every level-0 id
+__global__ void grid_leaves_kernel(const BitGrid G, const uint64_t* __restrict__ leaves, int64_t m, int kb,
+                                   int32_t* __restrict__ rl_id, int32_t* __restrict__ leaf_rl) {
+    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x) {
+        int p, y, x;
+        unpack_key(leaves[j], kb, p, y, x);
+        const int h = max(1, (1 << G.L[p]) >> 1);
+        const uint32_t i = (uint32_t)(y >> 1) * (uint32_t)h + (uint32_t)(x >> 1);
+        const uint32_t w = grid_word(G, 0, (x & 1) | ((y & 1) << 1), p) + (i >> 5);
+        const int id = G.before[w] + __popc(G.bits[w] & ((1u << (i & 31)) - 1));
+        rl_id[j] = id;
+        leaf_rl[id] = (int32_t)j;
+    }
+}
+
+// Parent, children and interaction list of every box (as links_kernel): bit tests in the
+// grids, ranks from the words' running counts.  The 27 candidates are, in each class, the
+// 3 x 3 cells around the parent's: three bits in a row, in one word or two.  The lists are
+// gathered in shared memory (27 words a box, an odd stride) and written in one piece.
+__global__ void __launch_bounds__(kT) grid_links_kernel(const BitGrid G, int64_t n, const int64_t* __restrict__ cstart,
+                                                        const int32_t* __restrict__ bp,
+                                                        const int32_t* __restrict__ bxy, int32_t* __restrict__ par,
+                                                        int32_t* __restrict__ ch, int32_t* __restrict__ il) {
+    __shared__ signed char s_slot[4][36];
+    __shared__ int s_start[kGridLevels + 1];
+    __shared__ int32_t s_il[kT * 27];
+    for (int t = threadIdx.x; t < 4 * 36; t += blockDim.x) (&s_slot[0][0])[t] = -1;
+    for (int t = threadIdx.x; t <= G.nk; t += blockDim.x) s_start[t] = (int)cstart[4 * t];
+    __syncthreads();
+    for (int t = threadIdx.x; t < 4 * 27; t += blockDim.x) {
+        const int c = t / 27, st = t % 27, px = c & 1, py = c >> 1;
+        int dx, dy;
+        interaction_slot(px, py, st, dx, dy);
+        s_slot[c][(dy + 2 + py) * 6 + dx + 2 + px] = (signed char)st;
+    }
+    const int64_t tiles = (n + kT - 1) / kT;
+    for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        const int64_t b = tile * kT + threadIdx.x;
+        int32_t* my = s_il + threadIdx.x * 27;
+        __syncthreads();  // slots are set; the previous tile's lists are written
+        for (int st = 0; st < 27; ++st) my[st] = -1;
+        if (b < n) {
+            int k = 0;
+            while (b >= s_start[k + 1]) ++k;
+            const int p = bp[b], x = bxy[b] & 0xffff, y = bxy[b] >> 16;
+            const int l = G.L[p] - k, hn = 1 << l, h = max(1, hn >> 1);
+            const int c = (x & 1) | ((y & 1) << 1), X = x >> 1, Y = y >> 1;
+            int pr = -1;
+            if (k + 1 <= G.kmax && l - 1 >= 2) {  // its parent is a box of level k + 1
+                const uint32_t i = (uint32_t)(Y >> 1) * (uint32_t)(h >> 1) + (uint32_t)(X >> 1);
+                const uint32_t w = grid_word(G, k + 1, (X & 1) | ((Y & 1) << 1), p) + (i >> 5);
+                pr = G.before[w] + __popc(G.bits[w] & ((1u << (i & 31)) - 1)) - s_start[k + 1];
+            }
+            par[b] = pr;
+            if (k >= 1) {
+                const uint32_t i = (uint32_t)y * (uint32_t)hn + (uint32_t)x;  // the same cell of all four classes
+                int cc[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const uint32_t w = grid_word(G, k - 1, q, p) + (i >> 5), v = G.bits[w];
+                    cc[q] = (v >> (i & 31)) & 1 ? G.before[w] + __popc(v & ((1u << (i & 31)) - 1)) - s_start[k - 1] : -1;
+                }
+                reinterpret_cast<int4*>(ch)[b] = make_int4(cc[0], cc[1], cc[2], cc[3]);
+            }
+            const int x0 = max(X - 1, 0), x1 = min(X + 1, h - 1);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const uint32_t wq = grid_word(G, k, q, p);
+#pragma unroll
+                for (int dy = -1; dy <= 1; ++dy) {
+                    const int yy = Y + dy;
+                    if (yy < 0 || yy >= h) continue;
+                    const uint32_t i0 = (uint32_t)yy * (uint32_t)h + (uint32_t)x0, i1 = i0 + (uint32_t)(x1 - x0);
+                    const uint32_t w0 = wq + (i0 >> 5), w1 = wq + (i1 >> 5);
+                    const uint32_t v0 = G.bits[w0], v1 = w1 == w0 ? v0 : G.bits[w1];
+                    const uint64_t v = (uint64_t)v0 | (w1 == w0 ? 0ull : (uint64_t)v1 << 32);
+                    const int sh = (int)(i0 & 31);
+                    if (!((v >> sh) & ((1u << (x1 - x0 + 1)) - 1))) continue;
+                    int id = G.before[w0] + __popcll(v & (((uint64_t)1 << sh) - 1)) - s_start[k];
+                    for (int xx = x0; xx <= x1; ++xx)
+                        if ((v >> (sh + xx - x0)) & 1) {
+                            const int sl = s_slot[c][(2 * dy + (q >> 1) + 2) * 6 + 2 * (xx - X) + (q & 1) + 2];
+                            if (sl >= 0) my[sl] = id;
+                            ++id;
+                        }
+                }
+            }
+        }
+        __syncthreads();
+        const int64_t first = tile * kT * 27, count = min((int64_t)kT, n - tile * kT) * 27;
+        for (int t = threadIdx.x; t < count; t += kT) il[first + t] = s_il[t];
+    }
+}
+
+// Words of bit grids that are affordable: a few bytes per point, and at least what a leaf
+// grid of 4,096 x 4,096 cells takes (clustered_4m: 11.2 M words for 8.4 M points).
+int64_t grid_words_max(int64_t points) {
+    return std::min<int64_t>(std::max<int64_t>((int64_t)1 << 20, 2 * points), (int64_t)1 << 30);
+}
+
 // leaf occupancy of every problem's dense leaf grid at side 2^ls (L: leaf levels at that
 // side, cell_off: first cell of each problem)
 __global__ void dense_count_kernel(const int2* __restrict__ xy, int64_t n, const int32_t* __restrict__ pid,
@@ -605,7 +856,7 @@ __global__ void dense_count_kernel(const int2* __restrict__ xy, int64_t n, const
                                    const int32_t* __restrict__ L, const int64_t* __restrict__ cell_off, int ls,
                                    int32_t* __restrict__ cnt) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int p = pid[i];
+        const int p = pid ? pid[i] : 0;
         const int2 v = xy[i];
         const int64_t bx = ((int64_t)v.x - x0[p]) >> ls, by = ((int64_t)v.y - y0[p]) >> ls;
         atomicAdd(cnt + cell_off[p] + (by << L[p]) + bx, 1);
@@ -623,7 +874,7 @@ __global__ void dense_scatter_kernel(const int2* __restrict__ xy, int64_t n, con
                                      int32_t* __restrict__ perm) {
     const int mask = (1 << ls) - 1;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int p = pid[i];
+        const int p = pid ? pid[i] : 0;
         const int2 v = xy[i];
         const int64_t dx = (int64_t)v.x - x0[p], dy = (int64_t)v.y - y0[p];
         const int pos = atomicAdd(cursor + cell_off[p] + ((dy >> ls) << L[p]) + (dx >> ls), 1);
@@ -646,6 +897,11 @@ __global__ void occupied_compact_kernel(const int32_t* __restrict__ flag, const 
                                         const int32_t* __restrict__ ts, uint64_t* __restrict__ key,
                                         int32_t* __restrict__ rs, int32_t* __restrict__ rt) {
     for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < cells; c += (int64_t)gridDim.x * blockDim.x) {
+        if (c == cells - 1) {  // the totals behind the last leaf
+            const int m = pos[cells];
+            rs[m] = ss[cells];
+            rt[m] = ts[cells];
+        }
         if (!flag[c]) continue;
         int lo = 0, hi = np;  // problem p: cell_off[p] <= c < cell_off[p + 1]
         while (hi - lo > 1) {
@@ -711,9 +967,10 @@ __global__ void strip_record_kernel(const uint64_t* __restrict__ leaves, const i
 // columns max(bx0 - 1, 0) .. min(bx0 + SW, n - 1)): index ranges [j0, j1) in the sorted
 // occupied-leaf keys, found by binary search.  The end key is column c_hi + 1 taken as a
 // sum, so that one past the row's last column carries into the next row.
-__global__ void strip_rows_kernel(const int4* __restrict__ strips, int64_t nstr, const uint64_t* __restrict__ leaves,
-                                  int64_t m, const int32_t* __restrict__ L, int kb, int SW,
-                                  int4* __restrict__ rows) {
+__global__ void strip_rows_kernel(const int4* __restrict__ strips, const int32_t* __restrict__ nstr_d,
+                                  const uint64_t* __restrict__ leaves, int64_t m, const int32_t* __restrict__ L,
+                                  int kb, int SW, int4* __restrict__ rows) {
+    const int64_t nstr = *nstr_d;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nstr; i += (int64_t)gridDim.x * blockDim.x) {
         const int4 q = strips[i];
         const int p = q.x, by = q.y, bx0 = q.z;
@@ -798,7 +1055,7 @@ int unique_runs(const uint64_t* key, int64_t n, uint64_t skip, uint64_t* out, in
 
 int forest_build(Forest& F, const int32_t* src, const int64_t* soff_h, int64_t ns, const int32_t* tgt,
                  const int64_t* toff_h, int64_t nt, int np, int leaf_size, int max_leaf_side, bool wide,
-                 cudaStream_t s, PhaseTimer* timer) {
+                 const ForestHint* hint, cudaStream_t s, PhaseTimer* timer) {
     int st;
     F.np = np;
     F.ns = ns;
@@ -807,39 +1064,54 @@ int forest_build(Forest& F, const int32_t* src, const int64_t* soff_h, int64_t n
     void* v;
     // targets = sources (same counts, offsets and coordinates): one sort serves both sides
     bool same = ns == nt && std::equal(soff_h, soff_h + np + 1, toff_h);
-    // problem offsets and per-point problem ids (temporaries)
+    // problem offsets and per-point problem ids (temporaries; none with one problem)
     DevBuf offs, pids;
     if ((st = offs.get((size_t)2 * (np + 1) * sizeof(int64_t) + 16, s))) return st;
     int64_t* soff = (int64_t*)offs.ptr;
     int64_t* toff = soff + (np + 1);
     int* word = (int*)(toff + (np + 1));  // the coordinate comparison's flag
-    LFMM_CUDA_TRY(cudaMemcpyAsync(soff, soff_h, (np + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s));
-    LFMM_CUDA_TRY(cudaMemcpyAsync(toff, toff_h, (np + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s));
-    LFMM_CUDA_TRY(cudaMemsetAsync(word, 0, sizeof(int), s));
-    if (same && src != tgt) same_points_kernel<<<grid_of(ns), kT, 0, s>>>((const int2*)src, (const int2*)tgt, ns, word);
-    // bounding boxes first (int4: 16-byte aligned at the allocation's start), then the ids
-    if ((st = pids.get((size_t)np * sizeof(int4) + (size_t)(ns + nt) * sizeof(int32_t), s))) return st;
-    int4* bb = (int4*)pids.ptr;
-    int32_t* spid = (int32_t*)(bb + np);
-    int32_t* tpid = spid + ns;
-    if (np == 1) {
-        LFMM_CUDA_TRY(cudaMemsetAsync(spid, 0, (size_t)(ns + nt) * sizeof(int32_t), s));
-        LFMM_CUDA_TRY(launch_set4((int*)bb, INT_MAX, INT_MAX, INT_MIN, INT_MIN, s));
-        LFMM_CUDA_TRY(launch_bbox(src, ns, tgt, nt, (int*)bb, s));
-    } else {
-        pid_kernel<<<std::min(np, 152 * 8), kT, 0, s>>>(soff, np, spid);
-        pid_kernel<<<std::min(np, 152 * 8), kT, 0, s>>>(toff, np, tpid);
-        bbox_forest_kernel<<<std::min(np, 152 * 8), kT, 0, s>>>((const int2*)src, soff, (const int2*)tgt, toff, np,
-                                                               bb);
-    }
-    LFMM_CUDA_TRY(cudaGetLastError());
-    timer->add_launches(5);
+    int32_t *spid = nullptr, *tpid = nullptr;
     std::vector<int4> hbb(np);
-    int hdiff = 0;
-    LFMM_CUDA_TRY(cudaMemcpyAsync(hbb.data(), bb, np * sizeof(int4), cudaMemcpyDeviceToHost, s));
-    LFMM_CUDA_TRY(cudaMemcpyAsync(&hdiff, word, sizeof(int), cudaMemcpyDeviceToHost, s));
-    LFMM_CUDA_TRY(cudaStreamSynchronize(s));
-    same = same && hdiff == 0;
+    const bool compare = same && src != tgt && !(hint && hint->same >= 0);
+    if (hint && hint->same >= 0) same = same && hint->same == 1;
+    if (compare) {
+        LFMM_CUDA_TRY(cudaMemsetAsync(word, 0, sizeof(int), s));
+        same_points_kernel<<<grid_of(ns), kT, 0, s>>>((const int2*)src, (const int2*)tgt, ns, word);
+        timer->add_launches(1);
+    }
+    int* hw = readback_words();  // page-locked words for the readbacks
+    if (!hw) return fail(LFMM_ENOMEM, "page-locked readback words");
+    if (hint) {  // one problem, its box known
+        hbb[0] = make_int4(hint->x0, hint->y0, hint->x1, hint->y1);
+        if (compare) {
+            LFMM_CUDA_TRY(cudaMemcpyAsync(hw, word, sizeof(int), cudaMemcpyDeviceToHost, s));
+            LFMM_CUDA_TRY(cudaStreamSynchronize(s));
+            same = hw[0] == 0;
+        }
+    } else {
+        // bounding boxes first (int4: 16-byte aligned at the allocation's start), then the ids
+        if ((st = pids.get((size_t)np * sizeof(int4) + (size_t)(np > 1 ? ns + nt : 0) * sizeof(int32_t), s))) return st;
+        int4* bb = (int4*)pids.ptr;
+        if (np == 1) {
+            LFMM_CUDA_TRY(launch_set4((int*)bb, INT_MAX, INT_MAX, INT_MIN, INT_MIN, s));
+            LFMM_CUDA_TRY(launch_bbox(src, ns, tgt, nt, (int*)bb, s));
+        } else {
+            LFMM_CUDA_TRY(cudaMemcpyAsync(soff, soff_h, (np + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s));
+            LFMM_CUDA_TRY(cudaMemcpyAsync(toff, toff_h, (np + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s));
+            spid = (int32_t*)(bb + np);
+            tpid = spid + ns;
+            pid_kernel<<<std::min(np, 152 * 8), kT, 0, s>>>(soff, np, spid);
+            pid_kernel<<<std::min(np, 152 * 8), kT, 0, s>>>(toff, np, tpid);
+            bbox_forest_kernel<<<std::min(np, 152 * 8), kT, 0, s>>>((const int2*)src, soff, (const int2*)tgt, toff, np,
+                                                                   bb);
+        }
+        LFMM_CUDA_TRY(cudaGetLastError());
+        timer->add_launches(np == 1 ? 2 : 3);
+        LFMM_CUDA_TRY(cudaMemcpyAsync(hbb.data(), bb, np * sizeof(int4), cudaMemcpyDeviceToHost, s));
+        if (compare) LFMM_CUDA_TRY(cudaMemcpyAsync(hw, word, sizeof(int), cudaMemcpyDeviceToHost, s));
+        LFMM_CUDA_TRY(cudaStreamSynchronize(s));
+        if (compare) same = hw[0] == 0;
+    }
     F.x0.resize(np);
     F.y0.resize(np);
     F.K.resize(np);
@@ -860,8 +1132,9 @@ int forest_build(Forest& F, const int32_t* src, const int64_t* soff_h, int64_t n
     int32_t* dy0 = dx0 + np;
     int32_t* dL = dy0 + np;
     F.d_L = dL;
-    LFMM_CUDA_TRY(cudaMemcpyAsync(dx0, F.x0.data(), np * sizeof(int32_t), cudaMemcpyHostToDevice, s));
-    LFMM_CUDA_TRY(cudaMemcpyAsync(dy0, F.y0.data(), np * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+    std::vector<int32_t> xyl((size_t)3 * np);  // x0, y0, L of every problem: one upload
+    std::copy(F.x0.begin(), F.x0.end(), xyl.begin());
+    std::copy(F.y0.begin(), F.y0.end(), xyl.begin() + np);
 
     // sorting scratch, sized for the largest sort of this phase (the union of source and
     // target leaves)
@@ -942,7 +1215,8 @@ int forest_build(Forest& F, const int32_t* src, const int64_t* soff_h, int64_t n
         kb = std::max(1, Lmax);
         if (Lmax > 20 || pbits + 2 * kb + 7 > 63)
             return fail(LFMM_EUNSUPPORTED, "forest problem needs more than 2^20 leaves per side");
-        LFMM_CUDA_TRY(cudaMemcpyAsync(dL, F.L.data(), np * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+        std::copy(F.L.begin(), F.L.end(), xyl.begin() + 2 * np);
+        LFMM_CUDA_TRY(cudaMemcpyAsync(dx0, xyl.data(), xyl.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s));
         const int bits = pbits + 2 * kb;
         dense = cells <= std::max<int64_t>(2 * (ns + nt), (int64_t)1 << 22);
         DevBuf cb;
@@ -961,12 +1235,11 @@ int forest_build(Forest& F, const int32_t* src, const int64_t* soff_h, int64_t n
                 max_count_kernel<<<grid_of(cells), kT, 0, s>>>(cnt + cells, cells, mx + 1);
             }
             LFMM_CUDA_TRY(cudaGetLastError());
-            int h[2] = {0, 0};
-            LFMM_CUDA_TRY(cudaMemcpyAsync(h, mx, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
+            LFMM_CUDA_TRY(cudaMemcpyAsync(hw, mx, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
             LFMM_CUDA_TRY(cudaStreamSynchronize(s));
-            timer->add_launches(4);
-            maxs = h[0];
-            maxt = same ? h[0] : h[1];
+            timer->add_launches(same ? 2 : 4);
+            maxs = hw[0];
+            maxt = same ? hw[0] : hw[1];
         } else {
             if ((st = sort_side(true, bits, &maxs))) return st;
             if (same) maxt = maxs;
@@ -998,6 +1271,10 @@ int forest_build(Forest& F, const int32_t* src, const int64_t* soff_h, int64_t n
     F.tloc = same ? F.sloc : F.sperm + ns;
     F.tperm = same ? F.sperm : F.tloc + nt;
     int M = 0;
+    // the number of leaves on the device; on the host it is known with the boxes below
+    // (dense grids), or already (sorted keys)
+    DevBuf gb, mbuf;
+    const int32_t* M_d = nullptr;
     if (dense) {
         // counting sort on the grids: first slot of every leaf by one exclusive scan of the
         // counts, points placed by atomic cursors; occupied leaves by one compaction
@@ -1006,7 +1283,6 @@ int forest_build(Forest& F, const int32_t* src, const int64_t* soff_h, int64_t n
         int64_t* doff = (int64_t*)cbk.ptr;
         int32_t* cs = (int32_t*)(doff + np + 1);
         int32_t* ct = same ? nullptr : cs + cells;
-        DevBuf gb;
         const int64_t sc = scan_tmp_ints(cells);
         if ((st = gb.get((size_t)(4 * (cells + 1) + 2 * sc) * sizeof(int32_t), s))) return st;
         int32_t* ss = (int32_t*)gb.ptr;      // [cells + 1] first source of each leaf
@@ -1019,18 +1295,16 @@ int forest_build(Forest& F, const int32_t* src, const int64_t* soff_h, int64_t n
         LFMM_CUDA_TRY(exscan(gflag, gpos, cells, gsum, s));
         LFMM_CUDA_TRY(exscan(cs, ss, cells, gsum + sc, s));
         if (!same) LFMM_CUDA_TRY(exscan(ct, ts, cells, gsum + sc, s));
-        LFMM_CUDA_TRY(cudaMemcpyAsync(&M, gpos + cells, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-        LFMM_CUDA_TRY(cudaStreamSynchronize(s));
-        if ((st = alloc(F, &vp, (size_t)(M + 1) * sizeof(uint64_t), s))) return st;
+        M_d = gpos + cells;
+        const int64_t cap = std::min<int64_t>(cells, same ? ns : ns + nt);  // leaves at most
+        if ((st = alloc(F, &vp, (size_t)(cap + 1) * sizeof(uint64_t), s))) return st;
         F.rl_key = (uint64_t*)vp;
-        if ((st = alloc(F, &vp, (size_t)(same ? 2 : 3) * (M + 1) * sizeof(int32_t), s))) return st;
+        if ((st = alloc(F, &vp, (size_t)(same ? 2 : 3) * (cap + 1) * sizeof(int32_t), s))) return st;
         F.rl_s = (int32_t*)vp;
-        F.rl_id = F.rl_s + (M + 1);
-        F.rl_t = same ? F.rl_s : F.rl_id + (M + 1);
+        F.rl_id = F.rl_s + (cap + 1);
+        F.rl_t = same ? F.rl_s : F.rl_id + (cap + 1);
         occupied_compact_kernel<<<grid_of(cells), kT, 0, s>>>(gflag, gpos, cells, doff, np, dL, kb, ss, same ? ss : ts,
                                                               F.rl_key, F.rl_s, F.rl_t);
-        LFMM_CUDA_TRY(cudaMemcpyAsync(F.rl_s + M, ss + cells, sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
-        if (!same) LFMM_CUDA_TRY(cudaMemcpyAsync(F.rl_t + M, ts + cells, sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
         // the counts become cursors (each leaf's first slot), then the points are placed
         LFMM_CUDA_TRY(cudaMemcpyAsync(cs, ss, (size_t)cells * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
         dense_scatter_kernel<<<grid_of(ns), kT, 0, s>>>((const int2*)src, ns, spid, dx0, dy0, dL, doff, ls, cs, F.sloc,
@@ -1070,15 +1344,108 @@ int forest_build(Forest& F, const int32_t* src, const int64_t* soff_h, int64_t n
         LFMM_CUDA_TRY(cudaGetLastError());
         timer->add_launches(12);
     }
-    F.n_leaves = M;
 
-    // ---- 3. boxes of every level: A = the leaves (k = 0), then the boxes of levels
-    // k = 1 .. kmax, sorted by (k, problem, row, column); compact ids number each level's
-    // boxes in class-major order; links by search in A
+    // ---- 3. boxes of every level
     F.kmax = Lmax - 2;  // may be negative: no far field anywhere
     const int nk = std::max(F.kmax, 0) + 1;
-    const int lbits = ceil_log2(nk);
     const int kmx = std::max(F.kmax, 0);
+    int64_t NB = 0;
+    std::vector<int64_t> hc((size_t)4 * nk + 1);
+    int64_t* dcls = nullptr;
+    int32_t *bp_all = nullptr, *bxy_all = nullptr, *par_all = nullptr, *il_all = nullptr, *ch_all = nullptr,
+            *leaf_rl = nullptr;
+    // per-box records of all levels in one allocation (level k at box_off[k])
+    int64_t* cstart = nullptr;
+    auto alloc_records = [&]() -> int {
+        int r;
+        if ((r = alloc(F, &vp, (size_t)NB * (4 + 3 + 27) * sizeof(int32_t) + (size_t)M * sizeof(int32_t) +
+                                   (size_t)(5 * nk) * sizeof(int64_t) + 16, s)))
+            return r;
+        ch_all = (int32_t*)vp;  // (16-byte records first)
+        dcls = (int64_t*)(ch_all + 4 * NB);  // 5 nk, level-local class starts
+        bp_all = (int32_t*)(dcls + 5 * nk);
+        bxy_all = bp_all + NB;
+        par_all = bxy_all + NB;
+        il_all = par_all + NB;
+        leaf_rl = il_all + 27 * NB;
+        return LFMM_OK;
+    };
+    BitGrid G = {};
+    int64_t words = 0;
+    std::vector<uint32_t> goff;
+    if (nk <= kGridLevels) {
+        if (np > 1) goff.resize((size_t)nk * np);
+        for (int k = 0; k < nk && words >= 0; ++k) {
+            int64_t stride = 0;
+            for (int p = 0; p < np; ++p) {
+                if (np > 1) goff[(size_t)k * np + p] = (uint32_t)stride;
+                if (k > 0 && F.L[p] - k < 2) continue;
+                const int64_t h = std::max<int64_t>(1, ((int64_t)1 << (F.L[p] - k)) >> 1);
+                stride += (h * h + 31) / 32;
+            }
+            G.base[k] = (uint32_t)words;
+            G.stride[k] = (uint32_t)stride;
+            words += 4 * stride;
+            if (words > grid_words_max(ns + nt)) words = -1;
+        }
+    } else {
+        words = -1;
+    }
+    DevBuf gbits, starts;
+    if ((st = starts.get((size_t)(4 * nk + 1) * sizeof(int64_t) + (size_t)(4 * nk + 2) * sizeof(int), s))) return st;
+    cstart = (int64_t*)starts.ptr;  // 4 nk + 1
+    int* starts_out = (int*)(cstart + 4 * nk + 1);
+    if (!dense) {
+        if ((st = mbuf.get(sizeof(int32_t), s))) return st;
+        LFMM_CUDA_TRY(cudaMemcpyAsync(mbuf.ptr, &M, sizeof(int32_t), cudaMemcpyHostToDevice, s));
+        M_d = (const int32_t*)mbuf.ptr;
+    }
+    if (words > 0 && 4 * nk + 2 <= kReadbackWords) {
+        // bits, running counts, scan sums, offsets
+        const int64_t sc = scan_tmp_ints(words);
+        if ((st = gbits.get((size_t)(2 * words + 1 + sc) * sizeof(int32_t) + goff.size() * sizeof(uint32_t), s))) return st;
+        G.nk = nk;
+        G.np = np;
+        G.kmax = F.kmax;
+        G.L = dL;
+        G.bits = (uint32_t*)gbits.ptr;
+        int32_t* before = (int32_t*)(G.bits + words);
+        int32_t* wsum = before + words + 1;
+        G.before = before;
+        if (np > 1) {
+            G.off = (const uint32_t*)(wsum + sc);
+            LFMM_CUDA_TRY(cudaMemcpyAsync((void*)G.off, goff.data(), goff.size() * sizeof(uint32_t), cudaMemcpyHostToDevice, s));
+        }
+        LFMM_CUDA_TRY(cudaMemsetAsync(G.bits, 0, (size_t)words * sizeof(uint32_t), s));
+        const int64_t cap = dense ? std::min<int64_t>(cells_k, ns + nt) : M;
+        grid_set_kernel<<<grid_of(cap), kT, 0, s>>>(G, F.rl_key, M_d, kb);
+        LFMM_CUDA_TRY(exscan<true>((const int32_t*)G.bits, before, words, wsum, s));
+        DevBuf dc;  // (the level-local class starts, copied into the records once these exist)
+        if ((st = dc.get((size_t)5 * nk * sizeof(int64_t), s))) return st;
+        grid_starts_kernel<<<1, 128, 0, s>>>(G, words, M_d, cstart, (int64_t*)dc.ptr, starts_out);
+        LFMM_CUDA_TRY(cudaGetLastError());
+        LFMM_CUDA_TRY(cudaMemcpyAsync(hw, starts_out, (size_t)(4 * nk + 2) * sizeof(int), cudaMemcpyDeviceToHost, s));
+        LFMM_CUDA_TRY(cudaStreamSynchronize(s));
+        M = hw[0];
+        for (int t = 0; t <= 4 * nk; ++t) hc[t] = hw[1 + t];
+        NB = hc[4 * nk];
+        if ((st = alloc_records())) return st;
+        LFMM_CUDA_TRY(cudaMemcpyAsync(dcls, dc.ptr, (size_t)5 * nk * sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
+        grid_records_kernel<<<grid_of(words), kT, 0, s>>>(G, words, bp_all, bxy_all);
+        grid_leaves_kernel<<<grid_of(M), kT, 0, s>>>(G, F.rl_key, M, kb, F.rl_id, leaf_rl);
+        grid_links_kernel<<<grid_of(NB), kT, 0, s>>>(G, NB, cstart, bp_all, bxy_all, par_all, ch_all, il_all);
+        LFMM_CUDA_TRY(cudaGetLastError());
+        timer->add_launches(words <= kScanSmall ? 6 : 8);
+    } else {
+    if (dense) {  // the number of leaves
+        LFMM_CUDA_TRY(cudaMemcpyAsync(hw, M_d, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+        LFMM_CUDA_TRY(cudaStreamSynchronize(s));
+        M = hw[0];
+    }
+    // without the grids: A = the leaves (k = 0), then the boxes of levels
+    // k = 1 .. kmax, sorted by (k, problem, row, column); compact ids number each level's
+    // boxes in class-major order; links by search in A
+    const int lbits = ceil_log2(nk);
     int E = 0, U = 0;
     DevBuf ebuf, abuf;
     // level >= 1 keys of the row-segment heads
@@ -1131,25 +1498,14 @@ int forest_build(Forest& F, const int32_t* src, const int64_t* soff_h, int64_t n
         if ((st = unique_runs(ek, E, ~0ull, A + M, nullptr, lflag, lpos, lsum, &U, s))) return st;
         timer->add_launches(4 + 5 * ((kbits + lbits + 7) / 8));
     }
-    const int64_t NB = (int64_t)M + U;
+    NB = (int64_t)M + U;
     // class-major order of every level (4 nk <= 84 partition keys: one digit)
     class_key_kernel<<<grid_of(NB), kT, 0, s>>>(A, NB, kb, kbits, ck, cidx);
     LFMM_CUDA_TRY(cudaGetLastError());
     LFMM_CUDA_TRY(radix_pass(ck, cidx, lsb.k2, lsb.v2, NB, 0, lsb, s));
     std::swap(ck, lsb.k2);
     std::swap(cidx, lsb.v2);
-    // per-box records of all levels in one allocation (level k at box_off[k])
-    if ((st = alloc(F, &vp, (size_t)NB * (3 + 27 + 4) * sizeof(int32_t) + (size_t)M * sizeof(int32_t) +
-                                (size_t)(4 * nk + 1 + 5 * nk) * sizeof(int64_t) + 16, s)))
-        return st;
-    int64_t* cstart = (int64_t*)vp;                 // 4 nk + 1
-    int64_t* dcls = cstart + (4 * nk + 1);          // 5 nk, level-local class starts
-    int32_t* bp_all = (int32_t*)(dcls + 5 * nk);
-    int32_t* bxy_all = bp_all + NB;
-    int32_t* par_all = bxy_all + NB;
-    int32_t* il_all = par_all + NB;
-    int32_t* ch_all = il_all + 27 * NB;
-    int32_t* leaf_rl = ch_all + 4 * NB;
+    if ((st = alloc_records())) return st;
     class_starts_kernel<<<(4 * nk + 1 + kT - 1) / kT, kT, 0, s>>>(ck, NB, nk, cstart);
     box_records_kernel<<<grid_of(NB), kT, 0, s>>>(A, ck, cidx, NB, cstart, kb, kbits, bp_all, bxy_all, local_of, leaf_rl);
     // the [first, end) of every box row of A, so that the links' searches (parent, two child
@@ -1184,19 +1540,23 @@ int forest_build(Forest& F, const int32_t* src, const int64_t* soff_h, int64_t n
     LFMM_CUDA_TRY(cudaGetLastError());
     LFMM_CUDA_TRY(cudaMemcpyAsync(F.rl_id, local_of, (size_t)M * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
     timer->add_launches(4 + 5);
+    LFMM_CUDA_TRY(cudaMemcpyAsync(hc.data(), cstart, hc.size() * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+    LFMM_CUDA_TRY(cudaStreamSynchronize(s));
+    std::vector<int64_t> hl((size_t)5 * nk);
+    for (int k = 0; k < nk; ++k)
+        for (int c = 0; c <= 4; ++c) hl[5 * k + c] = hc[4 * k + c] - hc[4 * k];
+    LFMM_CUDA_TRY(cudaMemcpyAsync(dcls, hl.data(), hl.size() * sizeof(int64_t), cudaMemcpyHostToDevice, s));
+    LFMM_CUDA_TRY(cudaStreamSynchronize(s));  // hl is a local
+    }
+    F.n_leaves = M;
     // class ranges of every level
     {
-        std::vector<int64_t> hc((size_t)4 * nk + 1);
-        LFMM_CUDA_TRY(cudaMemcpyAsync(hc.data(), cstart, hc.size() * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-        LFMM_CUDA_TRY(cudaStreamSynchronize(s));
         F.levels.assign(nk, ForestLevel());
-        std::vector<int64_t> hl((size_t)5 * nk);
         for (int k = 0; k < nk; ++k) {
             ForestLevel& lv = F.levels[k];
             lv.box_off = hc[4 * k];
             lv.nb = hc[4 * k + 4] - hc[4 * k];
             for (int c = 0; c <= 4; ++c) lv.cls[c] = hc[4 * k + c] - lv.box_off;
-            for (int c = 0; c <= 4; ++c) hl[5 * k + c] = lv.cls[c];
             lv.d_cls = dcls + 5 * k;
             lv.bp = bp_all + lv.box_off;
             lv.bxy = bxy_all + lv.box_off;
@@ -1206,8 +1566,6 @@ int forest_build(Forest& F, const int32_t* src, const int64_t* soff_h, int64_t n
             lv.rl = k == 0 ? leaf_rl : nullptr;
         }
         F.total_boxes = NB;
-        LFMM_CUDA_TRY(cudaMemcpyAsync(dcls, hl.data(), hl.size() * sizeof(int64_t), cudaMemcpyHostToDevice, s));
-        LFMM_CUDA_TRY(cudaStreamSynchronize(s));  // hl is a local
     }
 
     // ---- 4. strips of the near-field sweep
@@ -1220,20 +1578,17 @@ int forest_build(Forest& F, const int32_t* src, const int64_t* soff_h, int64_t n
     {
         strip_flag_kernel<<<grid_of(M), kT, 0, s>>>(F.rl_key, F.rl_t, M, kb, F.SW, flag);
         LFMM_CUDA_TRY(exscan(flag, pos, M, ssum, s));
-        int32_t nstr = 0;
-        LFMM_CUDA_TRY(cudaMemcpyAsync(&nstr, pos + M, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-        LFMM_CUDA_TRY(cudaStreamSynchronize(s));
-        const size_t n4 = (size_t)std::max(nstr, 1);
+        const size_t n4 = (size_t)std::max(M, 1);  // strips at most; their number stays on the device
         if ((st = alloc(F, &vp, 3 * n4 * sizeof(int4) + 16, s))) return st;
         F.strips = (int4*)vp;
         F.strip_rows = F.strips + n4;
         F.n_strips_d = (int32_t*)(F.strip_rows + 2 * n4);
+        F.n_strips = M;
         LFMM_CUDA_TRY(cudaMemcpyAsync(F.n_strips_d, pos + M, sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
         strip_record_kernel<<<grid_of(M), kT, 0, s>>>(F.rl_key, flag, pos, M, kb, F.SW, F.strips);
-        F.n_strips = nstr;
-        strip_rows_kernel<<<grid_of(nstr), kT, 0, s>>>(F.strips, nstr, F.rl_key, M, dL, kb, F.SW, F.strip_rows);
+        strip_rows_kernel<<<grid_of(M), kT, 0, s>>>(F.strips, F.n_strips_d, F.rl_key, M, dL, kb, F.SW, F.strip_rows);
         LFMM_CUDA_TRY(cudaGetLastError());
-        timer->add_launches(6);
+        timer->add_launches(M <= kScanSmall ? 4 : 6);
     }
     return LFMM_OK;  // temporaries are freed in stream order
 }

@@ -66,6 +66,10 @@ int fail(int status, const std::string& msg);
                                 std::string(#expr) + ": " + cudaGetErrorString(_e));   \
     } while (0)
 
+// Page-locked host words for readbacks (one set per host thread; null: none to be had).
+constexpr int kReadbackWords = 256;
+int* readback_words();
+
 // Every device allocation of plans, temporaries and staging buffers goes through here
 // (the stream-ordered pool); lfmm_fault_inject_alloc can make the n-th call fail with
 // cudaErrorMemoryAllocation, as a full device would.
@@ -301,7 +305,7 @@ struct Forest {
     // 2 int4 per strip {j0 r0, j1 r0, j0 r1, j1 r1}, {j0 r2, j1 r2, 0, 0}
     int4* strip_rows = nullptr;
     int32_t* n_strips_d = nullptr;
-    int64_t n_strips = 0;
+    int64_t n_strips = 0;                       // at most this many strips (the count is on the device)
     double* near_tmp = nullptr;                 // near field per sorted target, before the far part is added
     std::vector<void*> owned;
     int64_t bytes = 0;
@@ -320,13 +324,19 @@ int m2l_list_chunks(int64_t maxc, int num_sms, int split = 0);
 // Bytes of partial sums the K-split list M2L levels of F need (0: none split).
 int64_t forest_m2l_split_bytes(const Forest& F, int NP, size_t esz, int num_sms, int split = 0);
 
+// What the caller knows of a single problem: its bounding box, and whether the targets are
+// the sources (1, 0; -1: not known).
+struct ForestHint {
+    int x0, y0, x1, y1;
+    int same;
+};
 // Builds the tree of every problem (offsets: n_problems + 1 entries, host memory).
 // Leaf side: the largest power of two <= max_leaf_side at which no leaf holds more than
 // leaf_size sources or targets.  wide: strips for the near field of the 8-byte types.
 // Synchronises the stream.
 int forest_build(Forest& F, const int32_t* src, const int64_t* soff_h, int64_t ns, const int32_t* tgt,
                  const int64_t* toff_h, int64_t nt, int np, int leaf_size, int max_leaf_side, bool wide,
-                 cudaStream_t s, PhaseTimer* timer);
+                 const ForestHint* hint, cudaStream_t s, PhaseTimer* timer);
 // status: the plan's status word (grid-barrier words beside it; timed-out waits are
 // recorded there); persistent: run each sweep as one persistent cooperative launch
 // (LFMM_FLAG_PERSISTENT), else one launch per level, the list M2L of levels with at
