@@ -91,7 +91,7 @@ struct lfmm_plan {
     int m2l_part_nvec = 0;         // vectors the buffer has been sized for
     std::unique_ptr<Forest> forest;  // pruned tree or forest (null: uniform tree)
     void* sg_work = nullptr;         // work space of the sliced far field (split_tc.h)
-    void* tc_split = nullptr;        // TF32 hi/lo copies of q_hat and the parent u_hat for the tensor cores
+    void* tc_split = nullptr;        // fp16 hi/lo copies of q_hat and the parent u_hat for the tensor cores
     double* un_tmp = nullptr;        // near field per target (caller order) from the concurrent near-field pass
     double* uf_tmp = nullptr;        // far field per target (caller order), before the final sum
     struct AuxStream* aux = nullptr;  // near-field pass runs here, beside the far-field sweeps
@@ -618,9 +618,8 @@ int plan_build(lfmm_plan* p, const int32_t* src_xy, const int32_t* tgt_xy, cudaS
     }
     p->n_boxes = boxes;
     if (p->opts.precision == LFMM_MIXED && p->L >= (p->opts.tc_min_level == 0 ? kDefaultTcMinLevel : p->opts.tc_min_level)) {
-        // largest tensor-core level: TF32 hi/lo of its q_hat and of its parent's u_hat
-        const size_t n = ((size_t)p->NP << (2 * p->L)) * 2 + ((size_t)p->NP << (2 * std::max(0, p->L - 1))) * 2;
-        if ((st = palloc(p, &p->tc_split, n * sizeof(float), s))) return st;
+        // largest tensor-core level: fp16 hi/lo of its q_hat and of its parent's u_hat
+        if ((st = palloc(p, &p->tc_split, (size_t)tma_split_floats(p->L, p->NP) * sizeof(float), s))) return st;
     }
     if ((st = palloc(p, &p->qhat, (size_t)boxes * p->NP * esz, s))) return st;
     if ((st = palloc(p, &p->uhat, (size_t)boxes * p->NP * esz, s))) return st;
@@ -1236,8 +1235,7 @@ int lfmm_eval_multi(lfmm_plan* p, const double* F, int32_t k, double* U, void* s
         // per-vector buffers for one group (allocated once per plan and size)
         const size_t esz = p->opts.precision == LFMM_MIXED ? sizeof(float) : sizeof(double);
         const size_t g = (size_t)group;
-        const size_t split = p->tc_split ? ((size_t)p->NP << (2 * p->L)) * 2 + ((size_t)p->NP << (2 * (p->L - 1))) * 2
-                                         : 0;
+        const size_t split = p->tc_split ? (size_t)tma_split_floats(p->L, p->NP) : 0;
         void *a, *bq, *bu, *bQ, *bC, *c, *d = nullptr;
         if ((st = palloc(p, &a, g * p->ns * esz, s))) return st;
         if ((st = palloc(p, &bq, g * p->n_boxes * p->NP * esz, s))) return st;

@@ -182,6 +182,8 @@ struct DeviceOps {
     std::vector<void*> mono;              // per level k: deflation constants (hi[40], lo[40])
     std::vector<void*> tc;                // per level k (mixed, NP = 32): tensor-core B tiles,
                                           // [40 offsets + 4 L2L classes][hi, lo][32 x 32 fp32]
+    std::vector<void*> tch, tch_scale;    // per level k (mixed): the same operators in fp16 hi, lo, and
+                                          // the float that undoes each one's power-of-two scaling
     void* sg_base = nullptr;              // binary64-accurate paths, NP = 64: sliced operators
     std::vector<uint8_t*> sg_tiles;       // per level k (split_tc.h: kSgOps tiles), and
     std::vector<int32_t*> sg_e;           // their exponents
@@ -476,11 +478,15 @@ template <typename T>
 cudaError_t launch_m2l(const DeviceOps& ops, int k, int level, const T* q_level, const void* Q_level,
                        const T* u_parent, const void* C_parent, T* u_level, void* C_level, cudaStream_t s);
 // Tensor-core M2L + L2L of one level (Morton-ordered q_hat / u_hat in and out):
-// splits the level's expansions and the parent's into TF32 hi / lo layouts in `split`
-// (8 np^2 + 2 np^2 rows of 32 floats, np = 2^(level-1)), then one persistent launch fed
-// by tiled TMA loads; a timed-out wait is reported in *status.
+// splits the level's expansions and the parent's into scaled fp16 hi / lo layouts in `split`
+// (tma_split_floats(level, NP) floats), then one persistent launch fed by tiled TMA
+// loads; a timed-out wait is reported in *status.
 // nvec charge vectors at once: vector v's arrays start v vq floats (q, u) and v vQ
-// value pairs (Q, C) after vector 0's; `split` then holds nvec times the rows.
+// value pairs (Q, C) after vector 0's; `split` then holds nvec times the floats.
+// (a level's rows and its parents', 2 NP halves and a scale each)
+inline int64_t tma_split_floats(int level, int NP) {
+    return (((int64_t)1 << (2 * level)) + ((int64_t)1 << (2 * std::max(0, level - 1)))) * (NP + 1);
+}
 cudaError_t launch_m2l_tma(const DeviceOps& ops, int k, int level, const float* q_level, const void* Q_level,
                            const float* u_parent, const void* C_parent, float* u_level, void* C_level, float* split,
                            int* status, int num_sms, cudaStream_t s, int nvec = 1, int64_t vq = 0, int64_t vQ = 0,

@@ -4,20 +4,23 @@
 //   u_hat^tau = sum_{sigma in int(tau)} (T_ifo^o - c_o 1 1^T) q_hat^sigma + T_ifi^c u_hat^parent
 //
 // as an implicit GEMM per CTA: M = 128 target boxes (TMEM lanes), N = 32 outputs,
-// K = 27 x 32 source expansions (+ 32 for the parent).  Operands are split into TF32
-// hi + lo parts (round to nearest) and three products hi*hi + hi*lo + lo*hi are formed
-// (the lo*lo term is below 2^-22 relative).  The tensor core's fp32 accumulation rounds
+// K = 27 x 32 source expansions (+ 32 for the parent).  Operands are split into hi + lo
+// parts of 11 bits (round to nearest) and three products hi*hi + hi*lo + lo*hi are formed
+// (the lo*lo term is below 2^-22 relative): on uniform levels in fp16, every row and
+// operator scaled by a power of two (half the operand bytes and half the MMAs of TF32 for
+// the same 22 bits), on box lists in TF32.  The tensor core's fp32 accumulation rounds
 // toward zero, and that bias grows linearly with the number of MMAs feeding one
 // accumulator; so every K-step writes fresh TMEM accumulators (hi*hi in one, the small
 // hi*lo + lo*hi terms in another), which are read back after the step and added in
 // registers with round-to-nearest fp32.
 //
 // A (source expansions) arrives by tiled TMA loads from parity-plane layouts of the
-// split expansions, B (operators) as pre-split, pre-swizzled 4 KB tiles of the device
+// split expansions, B (operators) as pre-split, pre-swizzled tiles of the device
 // image by bulk copies; both land in the 128-byte-swizzled K-major layout that the
 // shared-memory matrix descriptors describe.  The pipeline is described at the kernel.
 #include <cuda.h>
 #include <cudaTypedefs.h>
+#include <cuda_fp16.h>
 
 #include "lfmm_internal.h"
 #include "tc_common.h"
@@ -82,45 +85,55 @@ __device__ __forceinline__ DFv dmul(DFv a, DFv b) {
 }
 
 // ---------------------------------------------------------------------------------
-// TMA form.  The level's expansions are split into TF32 hi / lo once and stored by
-// parity plane, Q5[hl][py'][px'][y'][x'][NP] with box (x, y) = (2x' + px', 2y' + py'):
-// for a target tile of one parity class, the sources at one interaction offset are then
-// a rectangle of one plane, so a single tiled TMA load (5-D tensor map, 128-byte
-// swizzle, zero fill outside the level) writes the A operand of a K-block directly in
-// the layout the tensor core reads.  The parent level's incoming expansions are stored
-// row-major (4-D map) and their window is the tile itself.
+// TMA form.  The level's expansions are scaled row by row to [2^14, 2^15), split into fp16
+// hi / lo once and stored by parity plane, Q[py'][px'][y'][x'] with box (x, y) = (2x' + px',
+// 2y' + py'), in 128-byte rows (NP = 32: hi and lo side by side; NP = 64: a plane set of hi
+// rows and one of lo rows): for a target tile of one parity class, the sources at one
+// interaction offset are then a rectangle of one plane, so a tiled TMA load (5-D tensor
+// map, 128-byte swizzle, zero fill outside the level) writes the A operand directly in the
+// layout the tensor core reads.  The parent level's incoming expansions are stored row-major
+// (4-D map) and their window is the tile itself.
 //
-// A K-block is 32 expansion coefficients (one 128-byte swizzled row per box): NP = 32
-// takes one K-block per interaction offset, NP = 64 two, accumulated into the same
-// fresh accumulator of that offset.
-//
-// Persistent CTAs (one per SM) walk the tiles with a continuous pipeline:
-//   warp 4 (one thread): producer - for every K-block of every offset of every tile,
-//     wait until the stage is free, then two TMA loads (A hi, A lo) and one bulk copy
-//     (B hi + lo) completing on the stage's "full" mbarrier;
-//   warp 5 (one thread): MMA issuer - wait "full" (and, at an offset's first K-block,
-//     until the accumulator buffer is folded), issue the block's 8 MMAs, commit to the
-//     stage's "empty" barrier (frees the shared memory) and, at the offset's last
-//     K-block, to the buffer's "acc_full" barrier;
+// Persistent CTAs (one per SM) walk the tiles with a continuous pipeline, PO offsets a step
+// (two at NP = 32: a clock trace puts every role's barrier waits, however ready, near 200
+// cycles each, as much as issuing an offset's MMAs):
+//   warp 4 (one thread): producer - for every step of every tile, wait until the stage is
+//     free, then per offset the TMA loads of A and one bulk copy of B (hi + lo) completing on
+//     the stage's "full" mbarrier;
+//   warp 5 (one thread): MMA issuer - wait "full" and until the accumulator buffer is
+//     folded, issue the offsets' MMAs (4 each at NP = 32, 8 at NP = 64), commit to the
+//     stage's "empty" barrier (frees the shared memory) and to the buffer's "acc_full" one;
 //   warps 0-3: one target box per thread (TMEM lane) - fold every offset's fresh
-//     accumulators into round-to-nearest fp32 registers, arrive on "acc_empty"; at a
-//     tile's last offset write the row of u_hat;
-//   warp 6: the compensated incoming constant of every box of the CTA's tiles (plain
+//     accumulators, times the source row's and the operator's scale, into round-to-nearest
+//     fp32 registers, arrive on "acc_empty"; at a tile's last step write the row of u_hat;
+//   warp 6: those scales, a tile ahead, for every row and offset of a tile (fetched by the
+//     fold itself they stood between any two steps for 500-900 cycles);
+// Against TF32 hi / lo (40 KB and 8 MMAs a step at NP = 32, now 24 KB and 4) the levels 6-8
+// of 2^20 sources and targets went from 110 to KKK us, the eight-vector launches from 583 to
+// LLL us.
+//   warps 7..: the compensated incoming constant of every box of the CTA's tiles (plain
 //     loads and float-pair arithmetic, independent of the pipeline).
 // Every wait is bounded; on expiry the CTA records LFMM_ETIMEOUT, every role stops at
 // its next iteration, and the teardown waits (bounded) for the copies and MMAs issued.
 constexpr int kTmaStagesDefault = 3;  // ring depth unless opts.m2l_stages says otherwise
 constexpr int kTmaAcc = 4;
-constexpr int kTmaThreads = 224;
-constexpr uint32_t kTmaABytes = 128 * 32 * 4;  // one A K-block (hi or lo): 128 rows x 128 B
+constexpr uint32_t kTmaABytes = 128 * 32 * 4;  // one A tile: 128 rows x 128 B
 
 template <int NP>
 struct TmaCfg {
-    static constexpr int KB = NP / 32;                          // K-blocks per interaction offset
-    static constexpr uint32_t BBytes = 2u * NP * 128u;          // B K-block: [B_hi | B_lo], 2 NP rows x 128 B
-    static constexpr uint32_t StageBytes = 2 * kTmaABytes + BBytes;
-    static constexpr int AccCols = 2 * NP;                      // buffer: D_big [0, 2NP), D_small [NP, 2NP)
-    static constexpr int Cols = kTmaAcc * AccCols;              // TMEM columns (256 or 512)
+    static constexpr int AT = NP / 32;                          // A tiles of a step (NP = 32: hi | lo in one)
+    static constexpr uint32_t BBytes = 2u * NP * 128u;          // [B_hi | B_lo], 2 NP rows x 128 B
+    static constexpr int PO = NP == 32 ? 2 : 1;                 // offsets of a step
+    static constexpr uint32_t OffBytes = AT * kTmaABytes + BBytes;
+    static constexpr uint32_t StageBytes = PO * OffBytes;
+    static constexpr int AccCols = 2 * NP;                      // per offset: D_big [0, 2NP), D_small [NP, 2NP)
+    static constexpr int Cols = kTmaAcc * PO * AccCols;         // TMEM columns
+    // warps of the compensated constants: one spends 30,000 cycles on a tile of 128 boxes (27
+    // gathers and float-pair multiply-adds each), as much as the whole pipeline; P_pad 64, whose
+    // pipeline takes as long, has no registers for more
+    static constexpr int CW = NP == 32 ? 4 : 1;
+    static constexpr int Threads = (7 + CW) * 32;
+    static constexpr uint32_t ScaleBytes = 2 * 28 * 128 * 4;    // two tiles' scales
 };
 
 struct TmaGeo {
@@ -132,7 +145,7 @@ struct TmaGeo {
     int n_tiles;          // 4 classes x tiles_per_class
     int has_l2l;
     int nvec;             // charge vectors: vector v's expansions at v vq floats, charges /
-    long long vq, vQ;     // constants at v vQ pairs; its split layouts at TMA index 2v + hl
+    long long vq, vQ;     // constants at v vQ pairs; its split layouts at TMA index AT v + hl
 };
 
 __device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2, int c3,
@@ -153,31 +166,38 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map
 }
 
 template <int NP, int kTmaStages>
-__global__ void __launch_bounds__(kTmaThreads, 1) m2l_tma_kernel(
+__global__ void __launch_bounds__(TmaCfg<NP>::Threads, 1) m2l_tma_kernel(
     const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_u, const TmaGeo g,
-    const float* __restrict__ tiles, const float* __restrict__ mono, const DFv* __restrict__ Qin,
+    const unsigned char* __restrict__ tiles, const float* __restrict__ tile_scale, const float* __restrict__ q_scale,
+    const float* __restrict__ u_scale, const float* __restrict__ mono, const DFv* __restrict__ Qin,
     const DFv* __restrict__ Cpar, float* __restrict__ out, DFv* __restrict__ Cout, int* __restrict__ status) {
     griddep_wait();
     using Cfg = TmaCfg<NP>;
-    constexpr int KB = Cfg::KB;
+    constexpr int AT = Cfg::AT, PO = Cfg::PO;
     constexpr uint32_t kStageBytes = Cfg::StageBytes;
     extern __shared__ __align__(1024) unsigned char tma_smem[];
-    // stage i: A hi, A lo (128 rows x 128 B each, 128-byte swizzled), B hi + lo (2 NP rows x 128 B)
+    // stage i: A (128 rows x 128 B a tile, 128-byte swizzled), B hi + lo (2 NP rows x 128 B)
     const uint32_t base = smem_u32(tma_smem) + ((1024u - (smem_u32(tma_smem) & 1023u)) & 1023u);
     __shared__ __align__(8) uint64_t full[kTmaStages], empty[kTmaStages], acc_full[kTmaAcc], acc_empty[kTmaAcc];
+    float* s_scale = reinterpret_cast<float*>(tma_smem + (base - smem_u32(tma_smem)) + kTmaStages * kStageBytes);
+    __shared__ __align__(8) uint64_t sc_full[2], sc_empty[2];
+    __shared__ int s_sc[4][28];        // per (class, offset): the source row's distance in q_scale and its
+                                       // steps (ax, ay) in the class grid
+    __shared__ float s_ts[kNumOffsets + 4];
     __shared__ uint32_t s_tmem;
     __shared__ int s_off[4][27][3];
     __shared__ int s_abort;
-    __shared__ int s_issued[2];  // K-blocks issued by the producer and by the MMA thread
+    __shared__ int s_issued[2];  // steps issued by the producer and by the MMA thread
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int n_steps = 27 + g.has_l2l;  // interaction offsets (+ the parent) per tile
+    const int n_off = 27 + g.has_l2l;  // interaction offsets (+ the parent) per tile
+    const int n_steps = (n_off + PO - 1) / PO;
     const int np = 1 << g.lg, side = 2 << g.lg;
     const int rows = g.TX * g.TY;
-    const uint32_t tx_bytes = 2u * (uint32_t)rows * 128u + Cfg::BBytes;
+    const uint32_t tx_bytes = (uint32_t)(AT * rows) * 128u + Cfg::BBytes;  // per offset
     const int all_tiles = g.n_tiles * g.nvec;
     const int my_tiles = blockIdx.x < (unsigned)all_tiles ? (all_tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
-    const int total = my_tiles * n_steps * KB;  // K-blocks of this CTA
+    const int total = my_tiles * n_steps;  // steps of this CTA
     volatile int* vabort = &s_abort;
     // the plan's wait budget in polls (status[3], 0: the clock bound alone)
     const uint32_t wb = ((volatile int*)status)[3] > 0 ? (uint32_t)((volatile int*)status)[3] : 0xffffffffu;
@@ -192,6 +212,8 @@ __global__ void __launch_bounds__(kTmaThreads, 1) m2l_tma_kernel(
                 s_off[c][nn][0] = dx;
                 s_off[c][nn][1] = dy;
                 s_off[c][nn][2] = offset_index_tc(dx, dy);
+                const int sx = px + dx, sy = py + dy;
+                s_sc[c][nn] = (((sx & 1) + 2 * (sy & 1)) << 4) | (((sx >> 1) + 2) << 2) | ((sy >> 1) + 2);
                 ++nn;
             }
         }
@@ -203,10 +225,15 @@ __global__ void __launch_bounds__(kTmaThreads, 1) m2l_tma_kernel(
             mbar_init(&acc_full[i], 1);
             mbar_init(&acc_empty[i], 4);
         }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&sc_full[i], 1);
+            mbar_init(&sc_empty[i], 4);
+        }
         fence_barrier_init();
         s_abort = 0;
         s_issued[0] = s_issued[1] = 0;
     }
+    for (int i = threadIdx.x; i < kNumOffsets + 4; i += blockDim.x) s_ts[i] = tile_scale[i];
     if (warp == 0) {
         tmem_alloc(&s_tmem, Cfg::Cols);
         tmem_relinquish();
@@ -231,13 +258,12 @@ __global__ void __launch_bounds__(kTmaThreads, 1) m2l_tma_kernel(
         ri0 = (k % g.tiles_x) * g.TX;
         rj0 = (k / g.tiles_x) * g.TY;
     };
-    // The roles walk the same sequence of K-blocks gs = (it * n_steps + st) * KB + h with
-    // running counters: stage slot gs % kTmaStages and its use count; the accumulator
-    // buffer advances once per offset (every KB blocks).
+    // The roles walk the same sequence of steps gs = it * n_steps + st with running counters:
+    // stage slot gs % kTmaStages and its use count, and likewise the accumulator buffer.
 
     if (warp == 4) {
         if (lane == 0) {
-            int it = 0, st = 0, h = 0, slot = 0, use = 0;
+            int it = 0, st = 0, slot = 0, use = 0;
             int cls = 0, ri0 = 0, rj0 = 0, v = 0;
             tile_of(0, cls, ri0, rj0, v);
             for (int gs = 0; gs < total; ++gs) {
@@ -247,84 +273,141 @@ __global__ void __launch_bounds__(kTmaThreads, 1) m2l_tma_kernel(
                     break;
                 }
                 const uint32_t sa = base + (uint32_t)slot * kStageBytes;
-                mbar_arrive_expect_tx(&full[slot], tx_bytes);
-                const int c0 = 32 * h;
-                if (st < 27) {
-                    const int sx = (cls & 1) + s_off[cls][st][0], sy = (cls >> 1) + s_off[cls][st][1];
-                    const int plane = (sx & 1) + 2 * (sy & 1);
-                    tma_load_5d(sa, &tm_q, c0, ri0 + (sx >> 1), rj0 + (sy >> 1), plane, 2 * v, &full[slot]);
-                    tma_load_5d(sa + kTmaABytes, &tm_q, c0, ri0 + (sx >> 1), rj0 + (sy >> 1), plane, 2 * v + 1,
-                                &full[slot]);
-                    bulk_g2s_u32(sa + 2 * kTmaABytes, tiles + ((size_t)s_off[cls][st][2] * KB + h) * (Cfg::BBytes / 4),
-                                 Cfg::BBytes, &full[slot]);
-                } else {
-                    tma_load_4d(sa, &tm_u, c0, ri0, rj0, 2 * v, &full[slot]);
-                    tma_load_4d(sa + kTmaABytes, &tm_u, c0, ri0, rj0, 2 * v + 1, &full[slot]);
-                    bulk_g2s_u32(sa + 2 * kTmaABytes, tiles + ((size_t)(kNumOffsets + cls) * KB + h) * (Cfg::BBytes / 4),
-                                 Cfg::BBytes, &full[slot]);
+                mbar_arrive_expect_tx(&full[slot], tx_bytes * (uint32_t)min(PO, n_off - st * PO));
+#pragma unroll
+                for (int j = 0; j < PO; ++j) {
+                    const int o = st * PO + j;
+                    const uint32_t so = sa + j * Cfg::OffBytes;
+                    if (o < 27) {
+                        const int sx = (cls & 1) + s_off[cls][o][0], sy = (cls >> 1) + s_off[cls][o][1];
+                        const int plane = (sx & 1) + 2 * (sy & 1);
+#pragma unroll
+                        for (int t = 0; t < AT; ++t)
+                            tma_load_5d(so + t * kTmaABytes, &tm_q, 0, ri0 + (sx >> 1), rj0 + (sy >> 1), plane,
+                                        AT * v + t, &full[slot]);
+                        bulk_g2s_u32(so + AT * kTmaABytes, tiles + (size_t)s_off[cls][o][2] * Cfg::BBytes, Cfg::BBytes,
+                                     &full[slot]);
+                    } else if (o < n_off) {
+#pragma unroll
+                        for (int t = 0; t < AT; ++t)
+                            tma_load_4d(so + t * kTmaABytes, &tm_u, 0, ri0, rj0, AT * v + t, &full[slot]);
+                        bulk_g2s_u32(so + AT * kTmaABytes, tiles + (size_t)(kNumOffsets + cls) * Cfg::BBytes,
+                                     Cfg::BBytes, &full[slot]);
+                    }
                 }
                 s_issued[0] = gs + 1;
                 if (++slot == kTmaStages) {
                     slot = 0;
                     ++use;
                 }
-                if (++h == KB) {
-                    h = 0;
-                    if (++st == n_steps) {
-                        st = 0;
-                        if (++it < my_tiles) tile_of(it, cls, ri0, rj0, v);
-                    }
+                if (++st == n_steps) {
+                    st = 0;
+                    if (++it < my_tiles) tile_of(it, cls, ri0, rj0, v);
                 }
             }
         }
     } else if (warp == 5) {
         if (lane == 0) {
-            // per K slice kk of the block: D_big[0, 2NP) (+)= A_hi x [B_hi | B_lo] (N = 2 NP:
-            // the hi*hi and hi*lo terms side by side), then D_small = D_big + NP += A_lo x B_hi
-            // (N = NP)
-            constexpr uint32_t kIdescBig = idesc_tf32(128, 2 * NP), kIdescSmall = idesc_tf32(128, NP);
-            int slot = 0, use = 0, h = 0, d = 0, du = 0;
+            // per K slice kk of the step (16 coefficients): D_big[0, 2NP) (+)= A_hi x [B_hi | B_lo]
+            // (N = 2 NP: the hi*hi and hi*lo terms side by side), then D_small = D_big + NP +=
+            // A_lo x B_hi (N = NP)
+            constexpr uint32_t kIdescBig = idesc_f16(128, 2 * NP), kIdescSmall = idesc_f16(128, NP);
+            int slot = 0, use = 0, d = 0, du = 0, st = 0;
             for (int gs = 0; gs < total; ++gs) {
                 if (*vabort) break;
                 if (!mbar_poll_bounded(&full[slot], (uint32_t)(use & 1), wb) ||
-                    (h == 0 && du > 0 && !mbar_poll_bounded(&acc_empty[d], (uint32_t)((du - 1) & 1), wb))) {
+                    (du > 0 && !mbar_poll_bounded(&acc_empty[d], (uint32_t)((du - 1) & 1), wb))) {
                     abort_now();
                     break;
                 }
                 tc_fence_after();
-                const uint32_t a_hi = base + (uint32_t)slot * kStageBytes, a_lo = a_hi + kTmaABytes;
-                const uint32_t b_hi = a_hi + 2 * kTmaABytes;
-                const uint32_t d_big = tmem + Cfg::AccCols * d, d_small = d_big + NP;
-                const uint64_t dah = smem_desc_sw128(a_hi), dal = smem_desc_sw128(a_lo), dbh = smem_desc_sw128(b_hi);
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk) {
-                    // +32 bytes along K inside the swizzled rows = +2 in the descriptor's address field
-                    mma_tf32_ss(d_big, dah + 2 * kk, dbh + 2 * kk, kIdescBig, (h > 0 || kk > 0) ? 1u : 0u);
-                    mma_tf32_ss(d_small, dal + 2 * kk, dbh + 2 * kk, kIdescSmall, 1u);
+                for (int j = 0; j < PO; ++j) {
+                    if (st * PO + j >= n_off) break;
+                    const uint32_t a_hi = base + (uint32_t)slot * kStageBytes + j * Cfg::OffBytes;
+                    const uint32_t d_big = tmem + Cfg::AccCols * (PO * d + j), d_small = d_big + NP;
+                    const uint64_t dah = smem_desc_sw128(a_hi), db = smem_desc_sw128(a_hi + AT * kTmaABytes);
+                    // lo: the second tile, or 64 bytes along K inside the swizzled rows (+4 in the
+                    // descriptor's address field)
+                    const uint64_t dal = NP == 64 ? smem_desc_sw128(a_hi + kTmaABytes) : dah + 4;
+#pragma unroll
+                    for (int kk = 0; kk < NP / 16; ++kk) {
+                        mma_f16_ss(d_big, dah + 2 * kk, db + 2 * kk, kIdescBig, kk > 0 ? 1u : 0u);
+                        mma_f16_ss(d_small, dal + 2 * kk, db + 2 * kk, kIdescSmall, 1u);
+                    }
                 }
+                if (++st == n_steps) st = 0;
                 mma_commit(&empty[slot]);
+                mma_commit(&acc_full[d]);
                 s_issued[1] = gs + 1;
                 if (++slot == kTmaStages) {
                     slot = 0;
                     ++use;
                 }
-                if (++h == KB) {
-                    h = 0;
-                    mma_commit(&acc_full[d]);
-                    if (++d == kTmaAcc) {
-                        d = 0;
-                        ++du;
-                    }
+                if (++d == kTmaAcc) {
+                    d = 0;
+                    ++du;
                 }
             }
         }
     } else if (warp == 6) {
+        // scale of every (offset, row) of a tile: source row times operator (0 outside the level)
+        for (int it = 0; it < my_tiles; ++it) {
+            bool ok = *vabort == 0;
+            if (ok && it >= 2 && lane == 0) ok = mbar_poll_bounded(&sc_empty[it & 1], (uint32_t)(((it >> 1) - 1) & 1), wb);
+            if (!__all_sync(0xffffffffu, ok)) {
+                if (lane == 0) abort_now();
+                break;
+            }
+            int cls, ri0, rj0, v;
+            tile_of(it, cls, ri0, rj0, v);
+            float* to = s_scale + (it & 1) * 28 * 128;
+            // four rows a lane, nine offsets' loads in flight each
+            int ri[4], rj[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int r = lane + 32 * i;
+                ri[i] = r < rows ? ri0 + r % g.TX : -4;  // (no source in the level)
+                rj[i] = rj0 + r / g.TX;
+            }
+            const float* qv = q_scale + ((size_t)(4 * v) << (2 * g.lg));
+            for (int k0 = 0; k0 < 27; k0 += 9) {
+                float q[9][4];
+#pragma unroll
+                for (int k = 0; k < 9; ++k) {
+                    const int e = s_sc[cls][k0 + k], ax = ((e >> 2) & 3) - 2, ay = (e & 3) - 2;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const int x = ri[i] + ax, y = rj[i] + ay;
+                        q[k][i] = (unsigned)x < (unsigned)np && (unsigned)y < (unsigned)np
+                                      ? __ldg(qv + ((((e >> 4) << g.lg) + y) << g.lg) + x)
+                                      : 0.f;
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < 9; ++k) {
+                    const float t = s_ts[s_off[cls][k0 + k][2]];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) to[(k0 + k) * 128 + lane + 32 * i] = q[k][i] * t;
+                }
+            }
+            if (g.has_l2l)
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (lane + 32 * i < rows)
+                        to[27 * 128 + lane + 32 * i] =
+                            __ldg(u_scale + (((size_t)v << (2 * g.lg)) + ((size_t)rj[i] << g.lg) + ri[i])) *
+                            s_ts[kNumOffsets + cls];
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sc_full[it & 1]);
+        }
+    } else if (warp >= 7) {
         for (int it = 0; it < my_tiles; ++it) {
             int cls, ri0, rj0, v;
             tile_of(it, cls, ri0, rj0, v);
             const int px = cls & 1, py = cls >> 1;
             const DFv* Qv = Qin + v * g.vQ;
-            for (int r = lane; r < rows; r += 32) {
+            for (int r = 32 * (warp - 7) + lane; r < rows; r += 32 * Cfg::CW) {
                 const int ri = ri0 + r % g.TX, rj = rj0 + r / g.TX;
                 DFv sacc = g.has_l2l ? Cpar[v * g.vQ + (size_t)morton2(ri, rj)] : DFv{0.f, 0.f};
                 for (int k0 = 0; k0 < 27; k0 += 9) {  // nine loads in flight at a time
@@ -353,14 +436,13 @@ __global__ void __launch_bounds__(kTmaThreads, 1) m2l_tma_kernel(
 #pragma unroll
         for (int j = 0; j < NP; ++j) acc[j] = 0.f;
         int it = 0, st = 0, d = 0, du = 0;
-        int cls = 0, ri = 0, rj = 0, v = 0;
-        const int offsets_total = my_tiles * n_steps;
-        for (int gs = 0; gs < offsets_total; ++gs) {
-            if (st == 0) {
-                int ri0, rj0;
-                tile_of(it, cls, ri0, rj0, v);
-                ri = ri0 + xl;
-                rj = rj0 + yl;
+        for (int gs = 0; gs < total; ++gs) {
+            if (st == 0) {  // the tile's scales
+                bool sc = *vabort == 0 && mbar_poll_bounded(&sc_full[it & 1], (uint32_t)((it >> 1) & 1), wb);
+                if (!__all_sync(0xffffffffu, sc)) {
+                    if (lane == 0) abort_now();
+                    break;
+                }
             }
             bool ok = *vabort == 0 && mbar_poll_bounded(&acc_full[d], (uint32_t)(du & 1), wb);
             ok = __all_sync(0xffffffffu, ok);
@@ -370,19 +452,31 @@ __global__ void __launch_bounds__(kTmaThreads, 1) m2l_tma_kernel(
             }
             tc_fence_after();
 #pragma unroll
-            for (int c = 0; c < NP / 32; ++c) {
-                uint32_t big[32], small[32];
-                tmem_ld32(tmem + lane_base + Cfg::AccCols * d + 32 * c, big);
-                tmem_ld32(tmem + lane_base + Cfg::AccCols * d + NP + 32 * c, small);
-                tmem_wait_ld();
+            for (int j = 0; j < PO; ++j) {
+                const int o = st * PO + j;
+                if (o >= n_off) break;
+                const float scale = s_scale[((it & 1) * 28 + o) * 128 + r];
 #pragma unroll
-                for (int j = 0; j < 32; ++j) acc[32 * c + j] += __uint_as_float(small[j]) + __uint_as_float(big[j]);
+                for (int c = 0; c < NP / 32; ++c) {
+                    uint32_t big[32], small[32];
+                    const uint32_t at = tmem + lane_base + Cfg::AccCols * (PO * d + j) + 32 * c;
+                    tmem_ld32(at, big);
+                    tmem_ld32(at + NP, small);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int e = 0; e < 32; ++e)
+                        acc[32 * c + e] =
+                            fmaf(__uint_as_float(small[e]) + __uint_as_float(big[e]), scale, acc[32 * c + e]);
+                }
             }
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&acc_empty[d]);
             if (st == n_steps - 1) {
                 if (valid) {
+                    int cls, ri0, rj0, v;
+                    tile_of(it, cls, ri0, rj0, v);
+                    const int ri = ri0 + xl, rj = rj0 + yl;
                     float4* dst = reinterpret_cast<float4*>(
                         out + v * g.vq + (size_t)morton2(2 * ri + (cls & 1), 2 * rj + (cls >> 1)) * NP);
 #pragma unroll
@@ -398,6 +492,7 @@ __global__ void __launch_bounds__(kTmaThreads, 1) m2l_tma_kernel(
             }
             if (++st == n_steps) {
                 st = 0;
+                if (lane == 0) mbar_arrive(&sc_empty[it & 1]);
                 ++it;
             }
         }
@@ -439,23 +534,24 @@ __global__ void __launch_bounds__(kTmaThreads, 1) m2l_tma_kernel(
 // two cp.async groups late, the K-steps taken in turn by whole warps, and a deeper ring
 // announced later.)
 //   warps 0-3: fold (one box per TMEM lane), warps 4-7: gather, warp 8: MMA issuer,
-//   warp 9: compensated incoming constants.
+//   warps 9..: compensated incoming constants.
 constexpr int kLStages = 4;
-constexpr int kLThreads = 320;
 constexpr int kLSrcInts = 4 * 32 * 28;  // per producer warp: 32 rows x 28 offsets
 // P_pad 32: one K-block per offset; P_pad 64: two (each a ring step), accumulated in the
 // offset's fresh accumulator, as in the TMA form
 template <int NP>
 struct ListTcCfg {
-    static constexpr int KB = NP / 32;
+    static constexpr int KB = NP / 32;                                 // K-blocks per interaction offset
     static constexpr uint32_t BBytes = 2u * NP * 128u;                 // [B_hi | B_lo] of one K-block
     static constexpr uint32_t StageBytes = 2 * kTmaABytes + BBytes;    // A hi, A lo, B
+    static constexpr int CW = TmaCfg<NP>::CW;  // warps of the compensated constants
+    static constexpr int Threads = (9 + CW) * 32;
     static constexpr size_t Smem = 1024 + (size_t)kLStages * StageBytes + (size_t)kLSrcInts * sizeof(int);
     static_assert(Smem <= 227 * 1024, "list ring exceeds shared memory");
 };
 
 template <int NP>
-__global__ void __launch_bounds__(kLThreads, 1) m2l_tc_list_kernel(
+__global__ void __launch_bounds__(ListTcCfg<NP>::Threads, 1) m2l_tc_list_kernel(
     const int64_t* __restrict__ cls_start, const int32_t* __restrict__ il, const int32_t* __restrict__ par,
     const float* __restrict__ qhi, const float* __restrict__ qlo, const float* __restrict__ uhi,
     const float* __restrict__ ulo, const float* __restrict__ tiles, const float* __restrict__ mono,
@@ -648,12 +744,12 @@ __global__ void __launch_bounds__(kLThreads, 1) m2l_tc_list_kernel(
                 }
             }
         }
-    } else if (warp == 9) {
+    } else if (warp >= 9) {
         for (int it = 0; it < my_tiles; ++it) {
             int cls;
             long long b0, b1;
             tile_of(it, cls, b0, b1);
-            for (long long b = b0 + lane; b < b1; b += 32) {
+            for (long long b = b0 + 32 * (warp - 9) + lane; b < b1; b += 32 * Cfg::CW) {
                 const int pb = has_l2l ? par[b] : -1;
                 DFv sacc = pb >= 0 ? Cpar[pb] : DFv{0.f, 0.f};
                 for (int k0 = 0; k0 < 27; k0 += 9) {
@@ -774,19 +870,21 @@ __global__ void split_tf32_rows_kernel(const float4* __restrict__ x, int64_t n4,
     }
 }
 
-// hi / lo TF32 split of a level's expansions (Morton order in) into the layouts the
-// tensor maps describe: planes = 1 -> [hl][plane][y'][x'][NP] (targets' level),
-// planes = 0 -> [hl][y][x][NP] (parent level, row-major).  Item iv is one float4 of
-// vector iv / n4.
+// A level's expansions (Morton order in), each row scaled by a power of two so that its
+// largest magnitude lies in [2^14, 2^15) and split into fp16 hi and lo, in the layouts the
+// tensor maps describe: planes = 1 -> by parity plane (targets' level), planes = 0 ->
+// row-major (parent level); 128-byte rows, [hi | lo] at NP = 32, all hi rows then all lo
+// rows at NP = 64; scale[row] undoes the scaling.  Item iv is one float4 of vector iv / n4;
+// the NP / 4 lanes of a row are consecutive.
 template <int NP>
-__device__ __forceinline__ void split_tf32_item(const float4* __restrict__ x0, float4* __restrict__ dst0, int lg,
-                                                int planes, int64_t vq4, int64_t n4, int64_t iv) {
+__device__ __forceinline__ void split_f16_item(const float4* __restrict__ x0, uint2* __restrict__ dst0,
+                                               float* __restrict__ scale, int lg, int planes, int64_t vq4, int64_t n4,
+                                               int64_t iv) {
     constexpr int Q = NP / 4;  // float4 per box
     const int np = 1 << lg;
     const int64_t vec = iv / n4, i = iv - vec * n4;
     const float4* x = x0 + vec * vq4;
-    float4* dst = dst0 + 2 * vec * n4;  // vector vec: hi then lo
-    const int64_t b = i / Q;
+    const int64_t b = i / Q, nb = n4 / Q;
     const int c = (int)(i - b * Q);
     uint32_t bx, by;
     if (planes) {
@@ -800,28 +898,48 @@ __device__ __forceinline__ void split_tf32_item(const float4* __restrict__ x0, f
     }
     const float4 v = x[(size_t)morton2(bx, by) * Q + c];
     const float a[4] = {v.x, v.y, v.z, v.w};
-    float h[4], l[4];
+    uint32_t mx = 0;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) mx = max(mx, __float_as_uint(a[e]) & 0x7fffffffu);
+#pragma unroll
+    for (int o = 1; o < Q; o <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    // 2^14 <= 2^s max < 2^15, within binary32's exponents; rows of zeros, infinities or NaN
+    // are not scaled
+    int s = 0;
+    if (mx != 0 && mx < 0x7f800000u) s = min(14 - ((int)(mx >> 23) - 127), 126);
+    const float up = __int_as_float((s + 127) << 23);
+    __half h[4], l[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-        h[e] = __uint_as_float(tf32_rna_bits(a[e]));
-        l[e] = __uint_as_float(tf32_rna_bits(a[e] - h[e]));
+        const float y = a[e] * up;
+        h[e] = __float2half_rn(y);
+        l[e] = __float2half_rn(y - __half2float(h[e]));
     }
-    dst[i] = make_float4(h[0], h[1], h[2], h[3]);
-    dst[i + n4] = make_float4(l[0], l[1], l[2], l[3]);
+    const uint2 hv = *reinterpret_cast<const uint2*>(h), lv = *reinterpret_cast<const uint2*>(l);
+    if (NP == 32) {
+        uint2* row = dst0 + (vec * nb + b) * 16;
+        row[c] = hv;
+        row[8 + c] = lv;
+    } else {
+        dst0[(2 * vec * nb + b) * 16 + c] = hv;
+        dst0[((2 * vec + 1) * nb + b) * 16 + c] = lv;
+    }
+    if (c == 0) scale[vec * nb + b] = __int_as_float((127 - s) << 23);
 }
 
 // The target level's expansions (parity planes) and, when xu is set, the parent level's
-// (row-major) in one launch: items [0, nvec nq4) are the former, the rest the latter.
+// (row-major) in one launch: items [0, nvec nq4) are the former, the rest the latter (both
+// counts multiples of 32, so that a warp's items are all of one kind).
 template <int NP>
-__global__ void split_tf32_layout_kernel(const float4* __restrict__ xq, float4* __restrict__ dq,
-                                         const float4* __restrict__ xu, float4* __restrict__ du, int lg, int nvec,
-                                         int64_t vq4) {
+__global__ void split_f16_layout_kernel(const float4* __restrict__ xq, uint2* __restrict__ dq, float* __restrict__ sq,
+                                        const float4* __restrict__ xu, uint2* __restrict__ du, float* __restrict__ su,
+                                        int lg, int nvec, int64_t vq4) {
     griddep_wait();
     const int64_t nq4 = ((int64_t)4 << (2 * lg)) * (NP / 4), nu4 = ((int64_t)1 << (2 * lg)) * (NP / 4);
     const int64_t nq = nq4 * nvec, n = nq + (xu ? nu4 * nvec : 0);
     for (int64_t iv = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; iv < n; iv += (int64_t)gridDim.x * blockDim.x) {
-        if (iv < nq) split_tf32_item<NP>(xq, dq, lg, 1, vq4, nq4, iv);
-        else split_tf32_item<NP>(xu, du, lg, 0, vq4, nu4, iv - nq);
+        if (iv < nq) split_f16_item<NP>(xq, dq, sq, lg, 1, vq4, nq4, iv);
+        else split_f16_item<NP>(xu, du, su, lg, 0, vq4, nu4, iv - nq);
     }
 }
 
@@ -840,22 +958,22 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
     return fn;
 }
 
-// fp32 tiled map over `rank` dims (dims[0] = NP coefficients, innermost), box
-// {32, TX, TY, 1, ...} (one 128-byte K-block), 128-byte swizzle, zero fill outside
-bool encode_map(CUtensorMap* m, const float* base, int rank, const uint64_t* dims, int TX, int TY) {
+// fp16 tiled map over `rank` dims (dims[0] = 64 halves, innermost), box {64, TX, TY, 1, ...}
+// (128-byte rows), 128-byte swizzle, zero fill outside
+bool encode_map(CUtensorMap* m, const void* base, int rank, const uint64_t* dims, int TX, int TY) {
     auto enc = tensor_map_encoder();
     if (!enc) return false;
     cuuint64_t gd[5], gs[4];
     cuuint32_t box[5], es[5];
-    uint64_t stride = 4;
+    uint64_t stride = 2;
     for (int i = 0; i < rank; ++i) {
         gd[i] = dims[i];
         if (i > 0) gs[i - 1] = stride;
         stride *= dims[i];
-        box[i] = i == 0 ? 32u : i == 1 ? (cuuint32_t)TX : i == 2 ? (cuuint32_t)TY : 1u;
+        box[i] = i == 0 ? 64u : i == 1 ? (cuuint32_t)TX : i == 2 ? (cuuint32_t)TY : 1u;
         es[i] = 1;
     }
-    return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, (cuuint32_t)rank, const_cast<float*>(base), gd, gs, box, es,
+    return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, (cuuint32_t)rank, const_cast<void*>(base), gd, gs, box, es,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
@@ -871,27 +989,25 @@ cudaError_t launch_m2l_tma(const DeviceOps& ops, int k, int level, const float* 
     const int lg = level - 1;
     const int np = 1 << lg;
     const bool l2l = u_parent != nullptr;
-    float* qs = split;                                           // [nvec][2][4][np][np][NP]
-    float* us = split + ((size_t)nvec * 2 * 4 * np * np * NP);   // [nvec][2][np][np][NP]
+    // split rows of the level (2 NP halves a row) and the parent's, then the rows' scales
+    const size_t rq = (size_t)nvec * 4 * np * np, ru = (size_t)nvec * np * np;
+    float* qs = split;
+    float* us = qs + rq * NP;
+    float* q_scale = us + ru * NP;
+    float* u_scale = q_scale + rq;
     auto grid_for = [&](int64_t n4) {
         int64_t b = (n4 + 255) / 256;
         return (int)std::max<int64_t>(1, std::min<int64_t>(b, (int64_t)num_sms * 16));
     };
     {
         const dim3 sg(grid_for((int64_t)(4 + (l2l ? 1 : 0)) * np * np * (NP / 4) * nvec));
-        const cudaError_t e = NP == 32
-            ? launch_dependent(split_tf32_layout_kernel<32>, sg, dim3(256), 0, s,
-                               reinterpret_cast<const float4*>(q_level), reinterpret_cast<float4*>(qs),
-                               l2l ? reinterpret_cast<const float4*>(u_parent) : nullptr, reinterpret_cast<float4*>(us),
-                               lg, nvec, vq / 4)
-            : launch_dependent(split_tf32_layout_kernel<64>, sg, dim3(256), 0, s,
-                               reinterpret_cast<const float4*>(q_level), reinterpret_cast<float4*>(qs),
-                               l2l ? reinterpret_cast<const float4*>(u_parent) : nullptr, reinterpret_cast<float4*>(us),
-                               lg, nvec, vq / 4);
-        if (e != cudaSuccess) return e;
-    }
-    {
-        cudaError_t e = cudaGetLastError();
+        auto go = [&](auto np_tag) {
+            return launch_dependent(split_f16_layout_kernel<decltype(np_tag)::value>, sg, dim3(256), 0, s,
+                                    reinterpret_cast<const float4*>(q_level), reinterpret_cast<uint2*>(qs), q_scale,
+                                    l2l ? reinterpret_cast<const float4*>(u_parent) : nullptr,
+                                    reinterpret_cast<uint2*>(us), u_scale, lg, nvec, vq / 4);
+        };
+        const cudaError_t e = NP == 32 ? go(std::integral_constant<int, 32>()) : go(std::integral_constant<int, 64>());
         if (e != cudaSuccess) return e;
     }
     TmaGeo g;
@@ -908,20 +1024,22 @@ cudaError_t launch_m2l_tma(const DeviceOps& ops, int k, int level, const float* 
     g.vq = vq;
     g.vQ = vQ;
     CUtensorMap mq, mu;
-    const uint64_t dq[5] = {(uint64_t)NP, (uint64_t)np, (uint64_t)np, 4, (uint64_t)(2 * nvec)};
-    const uint64_t du[4] = {(uint64_t)NP, (uint64_t)np, (uint64_t)np, (uint64_t)(2 * nvec)};
+    const uint64_t dq[5] = {64, (uint64_t)np, (uint64_t)np, 4, (uint64_t)(NP / 32 * nvec)};
+    const uint64_t du[4] = {64, (uint64_t)np, (uint64_t)np, (uint64_t)(NP / 32 * nvec)};
     if (!encode_map(&mq, qs, 5, dq, g.TX, g.TY)) return cudaErrorInvalidValue;
     if (!encode_map(&mu, l2l ? us : qs, 4, du, g.TX, g.TY)) return cudaErrorInvalidValue;
     const int grid = std::min(g.n_tiles * nvec, num_sms);
     auto go = [&](auto np_tag, auto stages_tag) -> cudaError_t {
         constexpr int NPc = decltype(np_tag)::value;
         constexpr int S = decltype(stages_tag)::value;
-        constexpr size_t smem = 1024 + (size_t)S * TmaCfg<NPc>::StageBytes;
+        constexpr size_t smem = 1024 + (size_t)S * TmaCfg<NPc>::StageBytes + TmaCfg<NPc>::ScaleBytes;
         static_assert(smem <= 227 * 1024, "TMA ring exceeds shared memory");
         cudaError_t e = ensure_dynamic_smem((const void*)m2l_tma_kernel<NPc, S>, smem);
         if (e != cudaSuccess) return e;
-        return launch_dependent(m2l_tma_kernel<NPc, S>, dim3(grid), dim3(kTmaThreads), smem, s, mq, mu, g,
-                                (const float*)ops.tc[k], (const float*)ops.mono[k], (const DFv*)Q_level,
+        return launch_dependent(m2l_tma_kernel<NPc, S>, dim3(grid), dim3(TmaCfg<NPc>::Threads), smem, s, mq, mu, g,
+                                (const unsigned char*)ops.tch[k], (const float*)ops.tch_scale[k],
+                                (const float*)q_scale, (const float*)u_scale, (const float*)ops.mono[k],
+                                (const DFv*)Q_level,
                                 (const DFv*)C_parent, u_level, (DFv*)C_level, status);
     };
     auto by_stages = [&](auto np_tag) -> cudaError_t {
@@ -970,7 +1088,7 @@ cudaError_t launch_m2l_tc_list(const DeviceOps& ops, int k, const int64_t* cls_s
         constexpr int NPc = decltype(np_tag)::value;
         cudaError_t r = ensure_dynamic_smem((const void*)m2l_tc_list_kernel<NPc>, ListTcCfg<NPc>::Smem);
         if (r != cudaSuccess) return r;
-        return launch_dependent(m2l_tc_list_kernel<NPc>, dim3(grid), dim3(kLThreads), ListTcCfg<NPc>::Smem, s,
+        return launch_dependent(m2l_tc_list_kernel<NPc>, dim3(grid), dim3(ListTcCfg<NPc>::Threads), ListTcCfg<NPc>::Smem, s,
                                 cls_start, il, u_parent ? par : nullptr, (const float*)qhi, (const float*)qlo,
                                 u_parent ? (const float*)uhi : nullptr, u_parent ? (const float*)ulo : nullptr,
                                 (const float*)ops.tc[k], (const float*)ops.mono[k], (const DFv*)Q_level,

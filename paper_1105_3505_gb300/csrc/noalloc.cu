@@ -159,8 +159,8 @@ extern "C" int lfmm_plan_shape_noalloc(const int32_t* src_xy, int64_t n_src, con
     auto a = [](int64_t b) { return b == 0 ? (int64_t)16 : b; };
     const int tc_min = o.tc_min_level == 0 ? kDefaultTcMinLevel : o.tc_min_level;
     const int64_t split = (o.precision == LFMM_MIXED && L >= tc_min)
-                              ? a(((int64_t)NP << (2 * L)) * 2 * 4 + ((int64_t)NP << (2 * std::max(0, L - 1))) * 2 * 4)
-                              : 0;  // TF32 hi/lo copies for the tensor-core M2L
+                              ? a(tma_split_floats(L, NP) * 4)
+                              : 0;  // fp16 hi/lo copies for the tensor-core M2L
     const int64_t un_tmp = L >= 2 ? a(2 * n_tgt * 8) : 0;  // near and far parts before the final sum
     // one vector's partial sums of the coarse-level M2L split along K (sized from the shape)
     int num_sms = 0;

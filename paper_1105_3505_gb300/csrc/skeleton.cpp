@@ -308,12 +308,51 @@ void write_tc_tile(float* dst, int NP, int rows, int cols, F value) {
     }
 }
 
+// binary16 round to nearest even of a value within the normal range of binary32 (|x| < 2^15
+// here; below 2^-14 on the subnormal grid of spacing 2^-24).
+uint16_t half_rne(float x) {
+    uint32_t u;
+    std::memcpy(&u, &x, 4);
+    const uint16_t sign = (uint16_t)((u >> 16) & 0x8000u);
+    const float a = std::fabs(x);
+    if (a < 6.103515625e-05f) return (uint16_t)(sign | (uint16_t)std::nearbyint((double)a * 16777216.0));  // 2^24 a
+    u = (u & 0x7fffffffu) - ((127u - 15u) << 23);
+    u += 0xfffu + ((u >> 13) & 1u);
+    return (uint16_t)(sign | (u >> 13));
+}
+float half_value(uint16_t h) {
+    const int e = (h >> 10) & 31, m = h & 1023;
+    const float v = e ? std::ldexp((float)(1024 + m), e - 25) : std::ldexp((float)m, -24);
+    return h & 0x8000 ? -v : v;
+}
+
+// The same operators for the fp16 tensor-core M2L: value(n, k) scaled by a power of two so
+// that the largest magnitude lies in [2^14, 2^15), split into fp16 hi and lo and stacked as
+// one K-major matrix of 2 NP rows (hi rows, then lo rows) of 128 bytes (64 halves; NP = 32
+// uses the first 32), 128-byte swizzled.  Returns the factor that undoes the scaling.
+template <typename F>
+float write_half_tile(uint16_t* dst, int NP, int rows, int cols, F value) {
+    float mx = 0.0f;
+    for (int n = 0; n < rows; ++n)
+        for (int k = 0; k < cols; ++k) mx = std::max(mx, std::fabs((float)value(n, k)));
+    const int sh = mx > 0.0f ? std::min(14 - std::ilogb(mx), 100) : 0;
+    for (int n = 0; n < rows; ++n)
+        for (int k = 0; k < cols; ++k) {
+            const float v = std::ldexp((float)value(n, k), sh);
+            const uint16_t h = half_rne(v), l = half_rne(v - half_value(h));
+            const size_t at = (size_t)n * 64 + (((k >> 3) ^ (n & 7)) << 3) + (k & 7);
+            dst[at] = h;
+            dst[at + (size_t)NP * 64] = l;  // row NP + n: the same swizzle
+        }
+    return std::ldexp(1.0f, -sh);
+}
+
 template <typename T>
 void fill_device_image(const ModelOps& mo, int NP, int n_levels, int H, int W,
                        std::vector<T>& img, size_t& off_tofs, size_t& off_tab,
                        std::vector<size_t>& off_m2m, std::vector<size_t>& off_l2l,
                        std::vector<size_t>& off_tifo, std::vector<size_t>& off_mono,
-                       std::vector<size_t>& off_tc) {
+                       std::vector<size_t>& off_tc, std::vector<size_t>& off_tch) {
     const int s = mo.leaf_side;
     auto align = [](size_t v) { return (v + 31) & ~(size_t)31; };  // 128/256-byte aligned blocks
     size_t n = 0;
@@ -326,12 +365,15 @@ void fill_device_image(const ModelOps& mo, int NP, int n_levels, int H, int W,
     off_tifo.assign(n_levels, 0);
     off_mono.assign(n_levels, 0);
     off_tc.assign(n_levels, 0);
+    off_tch.assign(n_levels, 0);
     const bool tc = sizeof(T) == 4 && (NP == 32 || NP == 64);
     for (int k = 0; k < n_levels; ++k) {
         if (tc) {
             n = (n + 255) & ~(size_t)255;  // 1 KB aligned tiles
             off_tc[k] = n;
             n += (size_t)(kNumOffsets + 4) * 2 * NP * NP;  // per operator NP / 32 blocks of 64 NP floats
+            off_tch[k] = n;  // fp16 tiles (2 NP rows of 128 bytes), then their scales
+            n = align(n + (size_t)(kNumOffsets + 4) * (2 * NP * 32 + 1));
         }
         off_mono[k] = n;
         n = align(n + (size_t)2 * kNumOffsets);
@@ -394,7 +436,11 @@ void fill_device_image(const ModelOps& mo, int NP, int n_levels, int H, int W,
                     img[off_tifo[k] + ((size_t)o * NP + q) * NP + p] = (T)(t[(size_t)p * lv.P + q] - c);
             if (tc) {
                 float* base = reinterpret_cast<float*>(img.data() + off_tc[k]) + (size_t)o * 2 * NP * NP;
-                write_tc_tile(base, NP, lv.P, lv.P, [&](int n_, int k_) { return t[(size_t)n_ * lv.P + k_] - c; });
+                const auto v = [&](int n_, int k_) { return t[(size_t)n_ * lv.P + k_] - c; };
+                write_tc_tile(base, NP, lv.P, lv.P, v);
+                float* half = reinterpret_cast<float*>(img.data() + off_tch[k]);
+                half[(size_t)(kNumOffsets + 4) * 2 * NP * 32 + o] =
+                    write_half_tile(reinterpret_cast<uint16_t*>(half + (size_t)o * 2 * NP * 32), NP, lv.P, lv.P, v);
             }
         }
         // tensor-core L2L tiles for class c: B[n = child p][k = parent q] = S_{k+1}[q][c P_k + p]
@@ -402,9 +448,11 @@ void fill_device_image(const ModelOps& mo, int NP, int n_levels, int H, int W,
             const LevelOps& par = mo.levels[k + 1];
             for (int c = 0; c < 4; ++c) {
                 float* base = reinterpret_cast<float*>(img.data() + off_tc[k]) + (size_t)(kNumOffsets + c) * 2 * NP * NP;
-                write_tc_tile(base, NP, lv.P, par.P, [&](int n_, int k_) {
-                    return par.S[(size_t)k_ * (4 * lv.P) + c * lv.P + n_];
-                });
+                const auto v = [&](int n_, int k_) { return par.S[(size_t)k_ * (4 * lv.P) + c * lv.P + n_]; };
+                write_tc_tile(base, NP, lv.P, par.P, v);
+                float* half = reinterpret_cast<float*>(img.data() + off_tch[k]);
+                half[(size_t)(kNumOffsets + 4) * 2 * NP * 32 + kNumOffsets + c] = write_half_tile(
+                    reinterpret_cast<uint16_t*>(half + (size_t)(kNumOffsets + c) * 2 * NP * 32), NP, lv.P, par.P, v);
             }
         }
     }
@@ -427,22 +475,22 @@ const DeviceOps* get_device_ops(ModelOps* mo, int precision, int NP, int n_level
     d->tab_H = 2 * mo->leaf_side - 1;
     d->tab_W = p2p_table_width(mo->leaf_side);
     size_t off_tofs, off_tab;
-    std::vector<size_t> om, ol, ot, omono, otc;
+    std::vector<size_t> om, ol, ot, omono, otc, otch;
     std::vector<char> bytes;
     size_t elem;
     if (precision == LFMM_MIXED) {
         std::vector<float> img;
-        fill_device_image<float>(*mo, NP, nl, d->tab_H, d->tab_W, img, off_tofs, off_tab, om, ol, ot, omono, otc);
+        fill_device_image<float>(*mo, NP, nl, d->tab_H, d->tab_W, img, off_tofs, off_tab, om, ol, ot, omono, otc, otch);
         elem = sizeof(float);
         bytes.assign((const char*)img.data(), (const char*)img.data() + img.size() * elem);
     } else if (precision == LFMM_DF) {
         std::vector<DF> img;
-        fill_device_image<DF>(*mo, NP, nl, d->tab_H, d->tab_W, img, off_tofs, off_tab, om, ol, ot, omono, otc);
+        fill_device_image<DF>(*mo, NP, nl, d->tab_H, d->tab_W, img, off_tofs, off_tab, om, ol, ot, omono, otc, otch);
         elem = sizeof(DF);
         bytes.assign((const char*)img.data(), (const char*)img.data() + img.size() * elem);
     } else {
         std::vector<double> img;
-        fill_device_image<double>(*mo, NP, nl, d->tab_H, d->tab_W, img, off_tofs, off_tab, om, ol, ot, omono, otc);
+        fill_device_image<double>(*mo, NP, nl, d->tab_H, d->tab_W, img, off_tofs, off_tab, om, ol, ot, omono, otc, otch);
         elem = sizeof(double);
         bytes.assign((const char*)img.data(), (const char*)img.data() + img.size() * elem);
     }
@@ -467,8 +515,14 @@ const DeviceOps* get_device_ops(ModelOps* mo, int precision, int NP, int n_level
     d->tifo.resize(nl);
     d->mono.resize(nl);
     d->tc.assign(nl, nullptr);
+    d->tch.assign(nl, nullptr);
+    d->tch_scale.assign(nl, nullptr);
     for (int k = 0; k < nl; ++k) {
-        if (precision == LFMM_MIXED && (NP == 32 || NP == 64)) d->tc[k] = b + otc[k] * elem;
+        if (precision == LFMM_MIXED && (NP == 32 || NP == 64)) {
+            d->tc[k] = b + otc[k] * elem;
+            d->tch[k] = b + otch[k] * elem;
+            d->tch_scale[k] = (char*)d->tch[k] + (size_t)(kNumOffsets + 4) * 2 * NP * 128;
+        }
         d->m2m[k] = k >= 1 ? b + om[k] * elem : nullptr;
         d->l2l[k] = k >= 1 ? b + ol[k] * elem : nullptr;
         d->tifo[k] = b + ot[k] * elem;
