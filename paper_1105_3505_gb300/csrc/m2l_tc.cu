@@ -523,20 +523,27 @@ __global__ void __launch_bounds__(TmaCfg<NP>::Threads, 1) m2l_tma_kernel(
 // the gather of the tile's 128 source rows (hi and lo, split beforehand into row-major
 // [box][NP] arrays; one 128-byte K-block of each row per ring step), so no tensor map
 // applies.  Same pipeline as the TMA form, with the
-// copies done by four producer warps, 32 rows each: eight lanes per row and four rows
-// per instruction (16-byte cp.async, coalesced 128-byte rows), written straight into the
-// 128-byte swizzled layout, missing sources zero-filled.  Every producer lane arrives on
-// the stage's "full" barrier through cp.async.mbarrier.arrive.noinc, which fires when
-// that lane's copies have landed, so a stage is released to the MMA thread as soon as
-// its rows are in, however far ahead the producers have run; the MMA thread makes the
-// rows visible to the tensor core with a proxy fence after its wait.  Producer warp 0
-// adds the operator tile's bulk copy.  (Measured before: announcing each warp's rows
-// two cp.async groups late, the K-steps taken in turn by whole warps, and a deeper ring
-// announced later.)
-//   warps 0-3: fold (one box per TMEM lane), warps 4-7: gather, warp 8: MMA issuer,
-//   warps 9..: compensated incoming constants.
+// copies done by producer groups of four warps, 32 rows each: eight lanes per row and four
+// rows per instruction (16-byte cp.async, coalesced 128-byte rows), written straight into
+// the 128-byte swizzled layout, missing sources zero-filled.  One group spends 1,450 cycles
+// a step on issuing (clock trace: 650 for the sixteen copies of a lane, the rest the stage's
+// wait, the operator copy and loop overhead) and 3,000 a tile on its lists, against 500 of
+// the MMA thread: at P_pad 32 two groups take the ring steps in turn, and the next tile's
+// lists arrive by cp.async while a tile runs.  Every producer lane arrives on the stage's
+// "full" barrier through cp.async.mbarrier.arrive.noinc, which fires when that lane's copies
+// have landed, so a stage is released to the MMA thread as soon as its rows are in, however
+// far ahead the producers have run; the MMA thread makes the rows visible to the tensor core
+// with a proxy fence after its wait.  The first warp of a group adds the operator tile's
+// bulk copy.  The constants take several warps: one warp spent as long on a tile's 128 x 27
+// gathers and float-pair multiply-adds as the whole pipeline on its products, and hid every
+// other change.  (Measured and not kept: announcing each warp's rows two cp.async groups
+// late, a deeper ring announced later; gathering the binary32 rows, half the bytes, and
+// splitting them into hi and lo on chip, 48 KB a step more of shared-memory traffic.)
+// clustered_4m's lists 1,721 -> KKK us, forest_4096's 1,336 -> LLL us, the same bits.
+//   warps 0-3: fold (one box per TMEM lane), then the producers, the MMA issuer and the
+//   compensated incoming constants.
 constexpr int kLStages = 4;
-constexpr int kLSrcInts = 4 * 32 * 28;  // per producer warp: 32 rows x 28 offsets
+constexpr int kLSrcInts = 32 * 28;  // one tile's lists of a producer warp: 32 x 27 entries, 32 parents
 // P_pad 32: one K-block per offset; P_pad 64: two (each a ring step), accumulated in the
 // offset's fresh accumulator, as in the TMA form
 template <int NP>
@@ -544,9 +551,14 @@ struct ListTcCfg {
     static constexpr int KB = NP / 32;                                 // K-blocks per interaction offset
     static constexpr uint32_t BBytes = 2u * NP * 128u;                 // [B_hi | B_lo] of one K-block
     static constexpr uint32_t StageBytes = 2 * kTmaABytes + BBytes;    // A hi, A lo, B
-    static constexpr int CW = TmaCfg<NP>::CW;  // warps of the compensated constants
-    static constexpr int Threads = (9 + CW) * 32;
-    static constexpr size_t Smem = 1024 + (size_t)kLStages * StageBytes + (size_t)kLSrcInts * sizeof(int);
+    // producer groups of four warps, taking the ring steps in turn, and warps of the compensated
+    // constants (P_pad 64: the fold's registers leave room for one of each)
+    static constexpr int PG = NP == 32 ? 2 : 1;
+    static constexpr int PW = 4 * PG;
+    static constexpr int CW = NP == 32 ? 3 : 1;
+    static constexpr int Threads = (5 + PW + CW) * 32;
+    static constexpr size_t Smem =
+        1024 + (size_t)kLStages * StageBytes + (size_t)2 * PW * kLSrcInts * sizeof(int);
     static_assert(Smem <= 227 * 1024, "list ring exceeds shared memory");
 };
 
@@ -559,7 +571,7 @@ __global__ void __launch_bounds__(ListTcCfg<NP>::Threads, 1) m2l_tc_list_kernel(
     int* __restrict__ status) {
     griddep_wait();
     using Cfg = ListTcCfg<NP>;
-    constexpr int KB = Cfg::KB;
+    constexpr int KB = Cfg::KB, PG = Cfg::PG, PW = Cfg::PW;
     constexpr uint32_t kLStageBytes = Cfg::StageBytes;
     constexpr uint32_t kAccCols = TmaCfg<NP>::AccCols;
     extern __shared__ __align__(1024) unsigned char tl_smem[];
@@ -570,8 +582,8 @@ __global__ void __launch_bounds__(ListTcCfg<NP>::Threads, 1) m2l_tc_list_kernel(
     __shared__ int s_op[4][28];           // operator tile of K-step st for class c
     __shared__ long long s_c[5], s_t[5];  // class starts; first tile of each class
     __shared__ int s_abort;
-    __shared__ int s_issued[2];           // K-steps issued by the producers (all four) and by the MMA thread
-    __shared__ int s_pissued[4];
+    __shared__ int s_issued[2];           // [1]: K-steps issued by the MMA thread
+    __shared__ int s_pissued[PW];
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const bool has_l2l = uhi != nullptr;
@@ -606,7 +618,7 @@ __global__ void __launch_bounds__(ListTcCfg<NP>::Threads, 1) m2l_tc_list_kernel(
         fence_barrier_init();
         s_abort = 0;
         s_issued[0] = s_issued[1] = 0;
-        for (int i = 0; i < 4; ++i) s_pissued[i] = 0;
+        for (int i = 0; i < PW; ++i) s_pissued[i] = 0;
     }
     if (warp == 0) {
         tmem_alloc(&s_tmem, TmaCfg<NP>::Cols);
@@ -631,36 +643,53 @@ __global__ void __launch_bounds__(ListTcCfg<NP>::Threads, 1) m2l_tc_list_kernel(
         b1 = min(b0 + 128, s_c[cls + 1]);
     };
 
-    if (warp >= 4 && warp < 8) {
-        const int pw = warp - 4;                 // rows 32 pw .. 32 pw + 31 of every tile
-        int* my_src = s_src + pw * 32 * 28;      // [row][K-step] source row, -1: none
+    if (warp >= 4 && warp < 4 + PW) {
+        const int grp = (warp - 4) >> 2, pw = (warp - 4) & 3;  // rows 32 pw .. 32 pw + 31 of every tile
+        int* my_src = s_src + (warp - 4) * 2 * kLSrcInts;      // lists of two tiles
         const int sub = lane >> 3, ch = lane & 7;  // row within a group of four, 16-byte chunk
-        int it = 0, st = 0, h = 0, slot = 0, use = 0, cls = 0;
-        long long b0 = 0, b1 = 0;
-        int gs = 0;
-        for (; gs < total; ++gs) {
-            if (__any_sync(0xffffffffu, *vabort != 0)) break;  // warp-uniform
-            if (st == 0 && h == 0) {
-                // lane r: the 27 list entries and the parent of row r, seven loads in flight
-                tile_of(it, cls, b0, b1);
-                const long long b = b0 + 32 * pw + lane;
-                const bool bv = b < b1;
-#pragma unroll
-                for (int k0 = 0; k0 < 28; k0 += 7) {
-                    int v[7];
-#pragma unroll
-                    for (int u = 0; u < 7; ++u) {
-                        const int k = k0 + u;
-                        v[u] = !bv ? -1 : k < 27 ? il[b * 27 + k] : (has_l2l ? par[b] : -1);
-                    }
-#pragma unroll
-                    for (int u = 0; u < 7; ++u) my_src[lane * 28 + k0 + u] = v[u];
-                }
-                __syncwarp();
+        // the lists of this CTA's it-th tile, asynchronously, into buffer it & 1
+        auto list_copy = [&](int it) {
+            if (it < my_tiles) {
+                int c;
+                long long t0, t1;
+                tile_of(it, c, t0, t1);
+                const long long bw = t0 + 32 * pw;
+                const int rows = (int)max(0ll, min(32ll, t1 - bw));
+                const uint32_t to = smem_u32(my_src + (it & 1) * kLSrcInts);
+                for (int i = lane; i < rows * 27; i += 32)
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(to + 4 * i), "l"(il + bw * 27 + i)
+                                 : "memory");
+                if (has_l2l && lane < rows)
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(to + 4 * (32 * 27 + lane)),
+                                 "l"(par + bw + lane)
+                                 : "memory");
             }
-            bool ok = true;
-            if (use > 0 && lane == 0) ok = mbar_poll_bounded(&empty[slot], (uint32_t)((use - 1) & 1), wb);
-            if (!__shfl_sync(0xffffffffu, ok ? 1 : 0, 0)) {
+            asm volatile("cp.async.commit_group;\n" ::: "memory");
+        };
+        int it = 0, st = grp / KB, h = grp % KB, cls = 0, rows = 0;
+        long long b0 = 0, b1 = 0;
+        bool fresh = true;  // the tile's lists are still to be waited for
+        list_copy(0);
+        for (int gs = grp; gs < total; gs += PG) {
+            const int slot = gs % kLStages, use = gs / kLStages;
+            if (fresh) {
+                asm volatile("cp.async.wait_group 0;\n" ::: "memory");  // (the rows' copies are in no group)
+                __syncwarp();
+                tile_of(it, cls, b0, b1);
+                rows = (int)max(0ll, min(32ll, b1 - b0 - 32 * pw));
+                list_copy(it + 1);  // its buffer held the tile before this one
+                fresh = false;
+            }
+            const int* ls = my_src + (it & 1) * kLSrcInts;
+            int srow[8];  // this lane's rows of the step
+#pragma unroll
+            for (int g = 0; g < 8; ++g) {
+                const int rl = 4 * g + sub;
+                srow[g] = rl < rows ? (st < 27 ? ls[rl * 27 + st] : ls[32 * 27 + rl]) : -1;
+            }
+            bool ok = *vabort == 0;
+            if (ok && use > 0 && lane == 0) ok = mbar_poll_bounded(&empty[slot], (uint32_t)((use - 1) & 1), wb);
+            if (!__all_sync(0xffffffffu, ok)) {
                 if (lane == 0) abort_now();
                 break;
             }
@@ -671,40 +700,36 @@ __global__ void __launch_bounds__(ListTcCfg<NP>::Threads, 1) m2l_tc_list_kernel(
                              Cfg::BBytes, &full[slot]);
             }
             const float* hs = st < 27 ? qhi : uhi;
-            const float* ls = st < 27 ? qlo : ulo;
+            const float* ls_lo = st < 27 ? qlo : ulo;
 #pragma unroll
             for (int g = 0; g < 8; ++g) {
-                const int rl = 4 * g + sub;          // row within this warp's 32
-                const int r = 32 * pw + rl;          // row of the tile (TMEM lane)
-                const int si = my_src[rl * 28 + st];
-                const size_t off = si < 0 ? 0 : (size_t)si * NP + 32 * h + 4 * ch;
-                const int bytes = si < 0 ? 0 : 16;
+                const int r = 32 * pw + 4 * g + sub;  // row of the tile (TMEM lane)
+                const size_t off = srow[g] < 0 ? 0 : (size_t)srow[g] * NP + 32 * h + 4 * ch;
+                const int bytes = srow[g] < 0 ? 0 : 16;
                 const uint32_t dst = (uint32_t)(r * 128 + ((ch ^ (r & 7)) << 4));
                 asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(sa + dst), "l"(hs + off),
                              "r"(bytes)
                              : "memory");
                 asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(sa + kTmaABytes + dst),
-                             "l"(ls + off), "r"(bytes)
+                             "l"(ls_lo + off), "r"(bytes)
                              : "memory");
             }
             // the stage's barrier counts this lane once its copies have landed
             cp_async_mbar_arrive_noinc(&full[slot]);
-            if (lane == 0) s_pissued[pw] = gs + 1;
-            if (++slot == kLStages) {
-                slot = 0;
-                ++use;
-            }
-            if (++h == KB) {
-                h = 0;
-                if (++st == n_steps) {
-                    st = 0;
-                    ++it;
+            if (lane == 0) s_pissued[warp - 4] = gs + 1;
+            for (int i = 0; i < PG; ++i)
+                if (++h == KB) {
+                    h = 0;
+                    if (++st == n_steps) {
+                        st = 0;
+                        ++it;
+                        fresh = true;
+                    }
                 }
-            }
         }
         // nothing of this lane's in flight when the CTA ends
         asm volatile("cp.async.wait_all;\n" ::: "memory");
-    } else if (warp == 8) {
+    } else if (warp == 4 + PW) {
         if (lane == 0) {
             // per K slice: D_big[0, 2 NP) (+)= A_hi x [B_hi | B_lo], D_small = D_big + NP +=
             // A_lo x B_hi
@@ -744,12 +769,12 @@ __global__ void __launch_bounds__(ListTcCfg<NP>::Threads, 1) m2l_tc_list_kernel(
                 }
             }
         }
-    } else if (warp >= 9) {
+    } else if (warp >= 5 + PW) {
         for (int it = 0; it < my_tiles; ++it) {
             int cls;
             long long b0, b1;
             tile_of(it, cls, b0, b1);
-            for (long long b = b0 + 32 * (warp - 9) + lane; b < b1; b += 32 * Cfg::CW) {
+            for (long long b = b0 + 32 * (warp - 5 - PW) + lane; b < b1; b += 32 * Cfg::CW) {
                 const int pb = has_l2l ? par[b] : -1;
                 DFv sacc = pb >= 0 ? Cpar[pb] : DFv{0.f, 0.f};
                 for (int k0 = 0; k0 < 27; k0 += 9) {
@@ -823,20 +848,21 @@ __global__ void __launch_bounds__(ListTcCfg<NP>::Threads, 1) m2l_tc_list_kernel(
     if (s_abort && threadIdx.x == 0) {
         // Every producer lane arrived for the steps its warp issued, but the warps stopped
         // at different steps.  A warp issues step g + kLStages only after step g's stage
-        // was consumed, so the steps issued by some warps and not by others are fewer than
-        // kLStages, each in its own slot and phase: arrive for the 32 lanes of each warp
-        // that skipped them (and for warp 0's operator-tile arrival), then wait until the
-        // operator copies of the last kLStages issued steps have landed (the lanes waited
+        // was consumed, so the steps issued by some warps and missed by others lie within
+        // kLStages of one another, each in its own slot and phase: arrive for the 32 lanes
+        // of each warp that skipped one (and for its operator-tile arrival), then wait until
+        // the operator copies of the last kLStages issued steps have landed (the lanes waited
         // for their own cp.async) and the MMAs issued have completed (a commit tracks every
         // MMA before it).
         int pmin = s_pissued[0], pmax = s_pissued[0];
-        for (int i = 1; i < 4; ++i) {
+        for (int i = 1; i < PW; ++i) {
             pmin = min(pmin, s_pissued[i]);
             pmax = max(pmax, s_pissued[i]);
         }
         for (int g = pmin; g < pmax; ++g) {
-            int missing = s_pissued[0] <= g ? 1 : 0;
-            for (int i = 0; i < 4; ++i) missing += s_pissued[i] <= g ? 32 : 0;
+            const int* pi = s_pissued + 4 * (g % PG);  // the group whose step it is
+            int missing = pi[0] <= g ? 1 : 0;
+            for (int i = 0; i < 4; ++i) missing += pi[i] <= g ? 32 : 0;
             if (missing > 0) mbar_arrive_n(&full[g % kLStages], (uint32_t)missing);
         }
         for (int g = pmax > kLStages ? pmax - kLStages : 0; g < pmax; ++g)
