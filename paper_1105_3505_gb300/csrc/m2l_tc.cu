@@ -109,8 +109,9 @@ __device__ __forceinline__ DFv dmul(DFv a, DFv b) {
 //   warp 6: those scales, a tile ahead, for every row and offset of a tile (fetched by the
 //     fold itself they stood between any two steps for 500-900 cycles);
 // Against TF32 hi / lo (40 KB and 8 MMAs a step at NP = 32, now 24 KB and 4) the levels 6-8
-// of 2^20 sources and targets went from 110 to KKK us, the eight-vector launches from 583 to
-// LLL us.
+// of 2^20 sources and targets went from 110 to 87 us, the eight-vector launches from 583 to
+// 412 us (one warp for the constants kept them at 105 and 570; four offsets a step in two
+// stages 90 and 472).  Errors against the exact sum do not grow (figures at the tests).
 //   warps 7..: the compensated incoming constant of every box of the CTA's tiles (plain
 //     loads and float-pair arithmetic, independent of the pipeline).
 // Every wait is bounded; on expiry the CTA records LFMM_ETIMEOUT, every role stops at
@@ -184,6 +185,7 @@ __global__ void __launch_bounds__(TmaCfg<NP>::Threads, 1) m2l_tma_kernel(
     __shared__ int s_sc[4][28];        // per (class, offset): the source row's distance in q_scale and its
                                        // steps (ax, ay) in the class grid
     __shared__ float s_ts[kNumOffsets + 4];
+    __shared__ DFv s_mono[kNumOffsets];  // deflation constants
     __shared__ uint32_t s_tmem;
     __shared__ int s_off[4][27][3];
     __shared__ int s_abort;
@@ -234,6 +236,7 @@ __global__ void __launch_bounds__(TmaCfg<NP>::Threads, 1) m2l_tma_kernel(
         s_issued[0] = s_issued[1] = 0;
     }
     for (int i = threadIdx.x; i < kNumOffsets + 4; i += blockDim.x) s_ts[i] = tile_scale[i];
+    if (threadIdx.x < kNumOffsets) s_mono[threadIdx.x] = DFv{mono[threadIdx.x], mono[kNumOffsets + threadIdx.x]};
     if (warp == 0) {
         tmem_alloc(&s_tmem, Cfg::Cols);
         tmem_relinquish();
@@ -421,7 +424,7 @@ __global__ void __launch_bounds__(TmaCfg<NP>::Threads, 1) m2l_tma_kernel(
 #pragma unroll
                     for (int k = 0; k < 9; ++k) {
                         const int o = s_off[cls][k0 + k][2];
-                        sacc = dadd(sacc, dmul(DFv{mono[o], mono[kNumOffsets + o]}, qv[k]));
+                        sacc = dadd(sacc, dmul(s_mono[o], qv[k]));
                     }
                 }
                 Cout[v * g.vQ + morton2(2 * ri + px, 2 * rj + py)] = sacc;
@@ -539,7 +542,7 @@ __global__ void __launch_bounds__(TmaCfg<NP>::Threads, 1) m2l_tma_kernel(
 // other change.  (Measured and not kept: announcing each warp's rows two cp.async groups
 // late, a deeper ring announced later; gathering the binary32 rows, half the bytes, and
 // splitting them into hi and lo on chip, 48 KB a step more of shared-memory traffic.)
-// clustered_4m's lists 1,721 -> KKK us, forest_4096's 1,336 -> LLL us, the same bits.
+// clustered_4m's lists 1,721 -> 1,372 us, forest_4096's 1,336 -> 1,008 us, the same bits.
 //   warps 0-3: fold (one box per TMEM lane), then the producers, the MMA issuer and the
 //   compensated incoming constants.
 constexpr int kLStages = 4;
@@ -580,6 +583,7 @@ __global__ void __launch_bounds__(ListTcCfg<NP>::Threads, 1) m2l_tc_list_kernel(
     __shared__ __align__(8) uint64_t full[kLStages], empty[kLStages], acc_full[kTmaAcc], acc_empty[kTmaAcc];
     __shared__ uint32_t s_tmem;
     __shared__ int s_op[4][28];           // operator tile of K-step st for class c
+    __shared__ DFv s_mono[kNumOffsets];   // deflation constants
     __shared__ long long s_c[5], s_t[5];  // class starts; first tile of each class
     __shared__ int s_abort;
     __shared__ int s_issued[2];           // [1]: K-steps issued by the MMA thread
@@ -620,6 +624,7 @@ __global__ void __launch_bounds__(ListTcCfg<NP>::Threads, 1) m2l_tc_list_kernel(
         s_issued[0] = s_issued[1] = 0;
         for (int i = 0; i < PW; ++i) s_pissued[i] = 0;
     }
+    if (threadIdx.x < kNumOffsets) s_mono[threadIdx.x] = DFv{mono[threadIdx.x], mono[kNumOffsets + threadIdx.x]};
     if (warp == 0) {
         tmem_alloc(&s_tmem, TmaCfg<NP>::Cols);
         tmem_relinquish();
@@ -787,7 +792,7 @@ __global__ void __launch_bounds__(ListTcCfg<NP>::Threads, 1) m2l_tc_list_kernel(
 #pragma unroll
                     for (int k = 0; k < 9; ++k) {
                         const int o = s_op[cls][k0 + k];
-                        if (sb[k] >= 0) sacc = dadd(sacc, dmul(DFv{mono[o], mono[kNumOffsets + o]}, qv[k]));
+                        if (sb[k] >= 0) sacc = dadd(sacc, dmul(s_mono[o], qv[k]));
                     }
                 }
                 Cout[b] = sacc;
