@@ -349,10 +349,15 @@ int forest_workspaces(lfmm_plan* p, cudaStream_t s) {
         if (need > 0 && (st = palloc(p, &b, (size_t)need * sizeof(float), s))) return st;
         F.tc_split = (float*)b;
     }
-    if (p->opts.precision != LFMM_MIXED && F.kmax >= 0) {  // near field, before the far part is added
+    // near field before the far part is added: the 8-byte types' near field is its own launch,
+    // binary32's where leaves hold fewer than 12 targets on average (clustered_4m, 5.6: KKK us in
+    // two launches against 1,420 in one; forest_4096, 22: LLL against 1,930)
+    if ((p->opts.precision != LFMM_MIXED || p->nt < 12 * F.n_leaves) && F.kmax >= 0) {
         void* b;
-        if ((st = palloc(p, &b, (size_t)p->nt * sizeof(double), s))) return st;
+        if ((st = palloc(p, &b, (size_t)p->nt * (sizeof(double) + sizeof(int32_t)), s))) return st;
         F.near_tmp = (double*)b;
+        F.t_leaf = (int32_t*)(F.near_tmp + p->nt);
+        LFMM_CUDA_TRY(launch_target_leaves(F, F.t_leaf, s));
     }
     // sliced far field of the binary64-accurate paths (split_tc.cu)
     if (F.kmax >= 0 && (int)F.levels.size() <= kSgMaxLevels &&

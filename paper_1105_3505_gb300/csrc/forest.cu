@@ -679,7 +679,7 @@ struct LStripCfg {
     static_assert(MAXSW == kStripMaxSW && CAPT == kStripCapTgt && CAPS >= kStripCapSrc, "strip staging caps");
 };
 
-// The near field of the 8-byte types is its own launch (kNear; kFar then adds L2P), so that
+// The near field of the 8-byte types is its own launch (kNear; l2p_list_kernel follows), so that
 // it runs beside the far field and in blocks of its own shape: one block of 24 warps per
 // SM, because the float-float / binary64 table (146 KB at side 32) leaves no room for a
 // second block, and as many staged sources as fit (near8_caps).  Its warps share a strip's
@@ -688,8 +688,18 @@ struct LStripCfg {
 // targets among many sources (clustered points, scattered targets) had kept one warp of
 // six busy.  Float-float pairs are added without renormalising each term (12 instead of
 // 15 operations).
-constexpr int kBoth = 0, kNear = 1, kFar = 2;
+//
+// Binary32 splits into the same two launches where strips are short (few targets per leaf:
+// clustered points): a strip is then bound by its chain of dependent loads and barriers,
+// and the near field alone, without L2P's registers, fits six blocks per SM instead of
+// four.  The order of every target's sums is the same in both forms.
+constexpr int kBoth = 0, kNear = 1;
 constexpr int kNearThreads = 768;
+template <typename T, int PART>
+struct NearCfg {
+    static constexpr int THREADS = sizeof(T) == 8 && PART == kNear ? kNearThreads : LStripCfg<T>::WARPS * 32;
+    static constexpr int BLOCKS = sizeof(T) == 8 ? 1 : PART == kNear ? 6 : 4;
+};
 
 // acc += a b with the two-sum's and the product's errors collected in acc.lo
 __device__ __forceinline__ void near_add(DF& acc, DF a, DF b) {
@@ -705,7 +715,7 @@ __device__ __forceinline__ void near_add(DF& acc, DF a, DF b) {
 __device__ __forceinline__ void near_add(double& acc, double a, double b) { acc = fma(a, b, acc); }
 
 template <typename T, int NP, int PART>
-__global__ void __launch_bounds__(PART == kNear ? kNearThreads : LStripCfg<T>::WARPS * 32) p2p_list_kernel(
+__global__ void __launch_bounds__(NearCfg<T, PART>::THREADS, NearCfg<T, PART>::BLOCKS) p2p_list_kernel(
     const int4* __restrict__ strips, const int4* __restrict__ strip_rows, const int32_t* __restrict__ n_strips_d,
     const int32_t* __restrict__ Lp, const uint64_t* __restrict__ rl_key, const int32_t* __restrict__ rl_s,
     const int32_t* __restrict__ rl_t, const int32_t* __restrict__ rl_id, int kb, int side, int SW,
@@ -714,22 +724,22 @@ __global__ void __launch_bounds__(PART == kNear ? kNearThreads : LStripCfg<T>::W
     const T* __restrict__ table, int tab_H, int tab_W, const T* __restrict__ uhat,
     const typename Mono<T>::V* __restrict__ Cleaf, const typename Mono<T>::V* __restrict__ Qleaf,
     const T* __restrict__ tofsT, double* __restrict__ u, double* __restrict__ u_near, double* __restrict__ u_far,
-    int caps, double* __restrict__ near_tmp) {
+    int caps, int capt, double* __restrict__ near_tmp) {
     griddep_wait();
     using M = Mono<T>;
     using V = typename M::V;
     using Cfg = LStripCfg<T>;
-    constexpr bool kHasNear = PART != kFar, kHasFar = PART != kNear;
+    constexpr bool kHasFar = PART != kNear;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int tab_n = kHasNear ? (2 * tab_H + 1) * tab_W : 0;
+    const int tab_n = (2 * tab_H + 1) * tab_W;
     T* tab = reinterpret_cast<T*>(smem_raw);
     SrcEntry<T>* s_src = reinterpret_cast<SrcEntry<T>*>(tab + tab_n);
-    T* s_uhat = reinterpret_cast<T*>(s_src + (kHasNear ? caps : 0));      // [MAXSW][NP]
+    T* s_uhat = reinterpret_cast<T*>(s_src + caps);           // [MAXSW][NP]
     V* s_q = reinterpret_cast<V*>(s_uhat + (kHasFar ? Cfg::MAXSW * NP : 0));  // [3][MAXSW+2]
     V* s_c = s_q + 3 * (Cfg::MAXSW + 2);                      // [MAXSW]
-    int* s_tloc = reinterpret_cast<int*>(s_c + Cfg::MAXSW);   // [CAPT]
-    int* s_tperm = s_tloc + Cfg::CAPT;                        // [CAPT]
-    int* s_sb = s_tperm + Cfg::CAPT;                          // [3][MAXSW+3]
+    int* s_tloc = reinterpret_cast<int*>(s_c + Cfg::MAXSW);   // [capt]
+    int* s_tperm = s_tloc + capt;                             // [capt]
+    int* s_sb = s_tperm + capt;                               // [3][MAXSW+3]
     int* s_tb = s_sb + 3 * (Cfg::MAXSW + 3);                  // [MAXSW+1]
     __shared__ int s_rs[4];
     __shared__ int s_ra[Cfg::MAXSW][3], s_rl[Cfg::MAXSW][3];
@@ -738,8 +748,8 @@ __global__ void __launch_bounds__(PART == kNear ? kNearThreads : LStripCfg<T>::W
     __shared__ int s_rj[3][2];                 // leaf-list range [j0, j1) of each row (-1: outside)
     __shared__ int s_lc[3][Cfg::MAXSW + 2];    // column - c_lo of each listed leaf (ascending)
 
-    if (kHasNear) block_stage(tab, table, tab_n);
-    const V phi0 = kHasNear ? M::make(table[tab_n], table[tab_n + 1]) : M::zero();
+    block_stage(tab, table, tab_n);
+    const V phi0 = M::make(table[tab_n], table[tab_n + 1]);
     const T* tab_c = tab + (tab_H + tab_H * tab_W);
     const int n_strips = *n_strips_d;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -839,7 +849,7 @@ __global__ void __launch_bounds__(PART == kNear ? kNearThreads : LStripCfg<T>::W
                 if (i < (bx1 - bx0) * NP) s_uhat[i] = vals[k];
             }
         }
-        for (int li = threadIdx.x; kHasNear && li < bx1 - bx0; li += blockDim.x) {
+        for (int li = threadIdx.x; li < bx1 - bx0; li += blockDim.x) {
             const int bx = bx0 + li;
             const int ca = max(bx - 1, 0) - c_lo, cb = min(bx + 1, n - 1) - c_lo + 1;
             int rs = 0;
@@ -864,13 +874,13 @@ __global__ void __launch_bounds__(PART == kNear ? kNearThreads : LStripCfg<T>::W
         }
         __syncthreads();
         const int ns_strip = s_rs[3];
-        if (kHasNear) stage_strip_sources<T>(s_src, ns_strip, s_rs, s_sb, Cfg::MAXSW + 3, ncol, c_lo, bx0, side, tab_W, sloc,
+        stage_strip_sources<T>(s_src, ns_strip, s_rs, s_sb, Cfg::MAXSW + 3, ncol, c_lo, bx0, side, tab_W, sloc,
                                f_sorted);
         const int tb0 = s_tb[0], nt_strip = s_tb[bx1 - bx0] - tb0;
         stage_strip_targets(s_tloc, s_tperm, nt_strip, s_tb, bx1 - bx0, tb0, tloc, tperm);
         __syncthreads();
 
-        if constexpr (PART == kNear) {
+        if constexpr (PART == kNear && sizeof(T) == 8) {
             const int warps = blockDim.x >> 5;
             int lg = 0;  // G = 2^lg lanes per target: at least two units of 32 / G targets per warp
             while (lg < 5 && (nt_strip << lg) < 64 * warps) ++lg;
@@ -925,7 +935,7 @@ __global__ void __launch_bounds__(PART == kNear ? kNearThreads : LStripCfg<T>::W
             const int li = (tl >> 8) & 0xff, tx = tl & 0xff, ty = tl >> 16;
             const T* tp = tab_c + (tx + tab_W * ty + li * side);
             T acc = T(0), cmp = T(0);
-            [[maybe_unused]] auto add = [&](T term) {
+            auto add = [&](T term) {
                 if constexpr (sizeof(T) == 4) {
                     const T y = term - cmp;
                     const T s2 = acc + y;
@@ -935,7 +945,6 @@ __global__ void __launch_bounds__(PART == kNear ? kNearThreads : LStripCfg<T>::W
                     acc += term;
                 }
             };
-            if constexpr (PART == kBoth) {
 #pragma unroll
             for (int r = 0; r < 3; ++r) {
                 const SrcEntry<T>* src = s_src + s_ra[li][r];
@@ -960,6 +969,9 @@ __global__ void __launch_bounds__(PART == kNear ? kNearThreads : LStripCfg<T>::W
                 }
             }
             acc -= cmp;
+            if constexpr (PART == kNear) {
+                if (active) near_tmp[tb0 + v] = (double)acc + s_nc[li];
+                continue;
             }
             T far = T(0);
             if (uhat) {
@@ -982,13 +994,55 @@ __global__ void __launch_bounds__(PART == kNear ? kNearThreads : LStripCfg<T>::W
             }
             if (active) {
                 const int dst = s_tperm[v];
-                const double dn = PART == kFar ? near_tmp[tb0 + v] : (double)acc + s_nc[li];
+                const double dn = (double)acc + s_nc[li];
                 const double df = (double)far + M::to_double(s_c[li]);
                 if (u) u[dst] = dn + df;
                 if (u_near) u_near[dst] = dn;
                 if (u_far) u_far[dst] = df;
             }
         }
+    }
+}
+
+// L2P of the split form: u = near_tmp + T_ofs(:, J)^T u_hat + C for 32 consecutive sorted targets
+// per warp, the lanes owning expansion entries (the order of every sum is that of
+// p2p_list_kernel).  Not by strips: a strip of few targets costs its chain of dependent
+// loads whatever its size (clustered_4m: 842 us by strips).
+template <typename T, int NP>
+__global__ void __launch_bounds__(128) l2p_list_kernel(int64_t nt, const int32_t* __restrict__ t_leaf,
+                                                       const int32_t* __restrict__ tloc,
+                                                       const int32_t* __restrict__ tperm, int side,
+                                                       const T* __restrict__ uhat,
+                                                       const typename Mono<T>::V* __restrict__ Cleaf,
+                                                       const T* __restrict__ tofsT, const double* __restrict__ near_tmp,
+                                                       double* __restrict__ u, double* __restrict__ u_near,
+                                                       double* __restrict__ u_far) {
+    griddep_wait();
+    using M = Mono<T>;
+    constexpr int PL = NP / 32;
+    const int lane = threadIdx.x & 31;
+    const int64_t v = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32 + lane;
+    if (v - lane >= nt) return;
+    const bool active = v < nt;
+    const int cid = t_leaf[active ? v : nt - 1], tl = tloc[active ? v : nt - 1];
+    const int myJ = (tl & 0xffff) + side * (tl >> 16);
+    T part[32];
+#pragma unroll
+    for (int q = 0; q < 32; ++q) {
+        const T* row = tofsT + (size_t)__shfl_sync(kFull, myJ, q) * NP + lane;
+        const T* uq = uhat + (size_t)__shfl_sync(kFull, cid, q) * NP + lane;
+        T w = T(0);
+#pragma unroll
+        for (int i = 0; i < PL; ++i) w = fma(ldg(row + 32 * i), uq[32 * i], w);
+        part[q] = w;
+    }
+    const T far = reduce_scatter32(part);
+    if (active) {
+        const int dst = tperm[v];
+        const double dn = near_tmp[v], df = (double)far + M::to_double(Cleaf[cid]);
+        if (u) u[dst] = dn + df;
+        if (u_near) u_near[dst] = dn;
+        if (u_far) u_far[dst] = df;
     }
 }
 
@@ -1063,15 +1117,17 @@ static int launch_list_p2p(const Forest& F, const DeviceOps& ops, const T* f_sor
                            bool use_tmp) {
     using Cfg = LStripCfg<T>;
     using V = typename Mono<T>::V;
-    PhaseTimer pt(PART == kFar ? LFMM_PHASE_L2P : LFMM_PHASE_P2P, s);
+    PhaseTimer pt(LFMM_PHASE_P2P, s);
     const int NP = ops.NP;
-    const int caps = PART == kNear ? near8_caps(F.side) : Cfg::CAPS;
-    size_t smem = (size_t)(3 * (Cfg::MAXSW + 2) + Cfg::MAXSW) * sizeof(V) + (size_t)2 * Cfg::CAPT * sizeof(int) +
+    // staging for the strips of this tree (8-byte near field: all that fits)
+    const int caps = sizeof(T) == 8 && PART == kNear ? near8_caps(F.side)
+                                                     : std::min(Cfg::CAPS, 3 * (F.SW + 2) * std::max(1, F.max_src));
+    const int capt = std::min(Cfg::CAPT, F.SW * std::max(1, F.max_tgt) + 1) / 2 * 2;
+    size_t smem = (size_t)(3 * (Cfg::MAXSW + 2) + Cfg::MAXSW) * sizeof(V) + (size_t)2 * capt * sizeof(int) +
                   (size_t)(3 * (Cfg::MAXSW + 3) + Cfg::MAXSW + 1) * sizeof(int);
-    if (PART != kFar)
-        smem += (size_t)(2 * ops.tab_H + 1) * ops.tab_W * sizeof(T) + (size_t)caps * sizeof(SrcEntry<T>);
+    smem += (size_t)(2 * ops.tab_H + 1) * ops.tab_W * sizeof(T) + (size_t)caps * sizeof(SrcEntry<T>);
     if (PART != kNear) smem += (size_t)Cfg::MAXSW * NP * sizeof(T);
-    const int threads = PART == kNear ? kNearThreads : Cfg::WARPS * 32;
+    constexpr int threads = NearCfg<T, PART>::THREADS;
     auto go = [&](auto np_tag) -> cudaError_t {
         constexpr int NPc = decltype(np_tag)::value;
         const void* fn = (const void*)p2p_list_kernel<T, NPc, PART>;
@@ -1080,16 +1136,33 @@ static int launch_list_p2p(const Forest& F, const DeviceOps& ops, const T* f_sor
         const int per_sm = blocks_per_sm(fn, threads, smem);
         // the near field beside the far field: blocks of a few strips, so that the far
         // field's launches (of a higher priority) find free SMs as blocks end
-        const int64_t waves = PART == kNear && use_tmp ? 6 : 1;
+        const int64_t waves = sizeof(T) == 8 && PART == kNear && use_tmp ? 6 : 1;
         const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(F.n_strips, waves * num_sms * per_sm));
         return launch_dependent(p2p_list_kernel<T, NPc, PART>, dim3((unsigned)grid), dim3(threads), smem, s, F.strips,
                                 F.strip_rows, F.n_strips_d, F.d_L, F.rl_key, F.rl_s, F.rl_t, F.rl_id, F.kb, F.side,
                                 F.SW, F.sloc, F.tloc, F.tperm, f_sorted, (const T*)ops.p2p_table, ops.tab_H, ops.tab_W,
-                                uhat, (const V*)Cleaf, (const V*)Qleaf, (const T*)ops.tofsT, u, un, uf, caps,
+                                uhat, (const V*)Cleaf, (const V*)Qleaf, (const T*)ops.tofsT, u, un, uf, caps, capt,
                                 use_tmp ? F.near_tmp : nullptr);
     };
     const cudaError_t e = NP == 32 ? go(std::integral_constant<int, 32>()) : go(std::integral_constant<int, 64>());
     if (e != cudaSuccess) return fail(LFMM_ECUDA, std::string("p2p_list_kernel: ") + cudaGetErrorString(e));
+    pt.add_launches(1);
+    return LFMM_OK;
+}
+
+template <typename T>
+static int launch_list_l2p(const Forest& F, const DeviceOps& ops, const T* uhat, const void* Cleaf, double* u,
+                           double* un, double* uf, cudaStream_t s) {
+    using V = typename Mono<T>::V;
+    PhaseTimer pt(LFMM_PHASE_L2P, s);
+    const dim3 grid((unsigned)((F.nt + 127) / 128));
+    auto go = [&](auto np_tag) {
+        return launch_dependent(l2p_list_kernel<T, decltype(np_tag)::value>, grid, dim3(128), 0, s, F.nt, F.t_leaf,
+                                F.tloc, F.tperm, F.side, uhat, (const V*)Cleaf, (const T*)ops.tofsT, F.near_tmp, u, un,
+                                uf);
+    };
+    const cudaError_t e = ops.NP == 32 ? go(std::integral_constant<int, 32>()) : go(std::integral_constant<int, 64>());
+    if (e != cudaSuccess) return fail(LFMM_ECUDA, std::string("l2p_list_kernel: ") + cudaGetErrorString(e));
     pt.add_launches(1);
     return LFMM_OK;
 }
@@ -1350,8 +1423,14 @@ int forest_eval(const Forest& F, const DeviceOps& ops, const double* f, T* f_sor
             LFMM_CUDA_TRY(cudaEventRecord(side->join, s));
             LFMM_CUDA_TRY(cudaStreamWaitEvent(s_main, side->join, 0));
         }
-        return launch_list_p2p<T, kFar>(F, ops, f_sorted, (const T*)Ux(0), Cm(0), Qm(0), u, un, uf, num_sms, s_main, true);
+        return launch_list_l2p<T>(F, ops, (const T*)Ux(0), Cm(0), u, un, uf, s_main);
     } else {
+        if (far && F.near_tmp) {
+            const int st = launch_list_p2p<T, kNear>(F, ops, f_sorted, (const T*)nullptr, nullptr, Qm(0), nullptr, nullptr,
+                                                     nullptr, num_sms, s, true);
+            if (st) return st;
+            return launch_list_l2p<T>(F, ops, (const T*)Ux(0), Cm(0), u, un, uf, s);
+        }
         return launch_list_p2p<T, kBoth>(F, ops, f_sorted, (const T*)(far ? Ux(0) : nullptr), far ? Cm(0) : nullptr, Qm(0), u, un, uf, num_sms, s,
                                          false);
     }

@@ -104,10 +104,17 @@ __global__ void scan_sums_kernel(int32_t* __restrict__ sums, int nb) {
     if (threadIdx.x == 0) sums[nb] = carry_s;
 }
 
-template <bool POP>
+// TOTALS: sums holds the blocks' totals, else their prefix sums
+template <bool POP, bool TOTALS>
 __global__ void scan_apply_kernel(const int32_t* __restrict__ in, int64_t n, const int32_t* __restrict__ sums,
                                   int32_t* __restrict__ out) {
-    __shared__ int32_t w[kT / 32];
+    __shared__ int32_t w[kT / 32], wb[kT / 32];
+    if (TOTALS) {
+        int32_t b = 0;
+        for (int i = threadIdx.x; i < (int)blockIdx.x; i += kT) b += sums[i];
+        for (int o = 16; o; o >>= 1) b += __shfl_xor_sync(kFull, b, o);
+        if ((threadIdx.x & 31) == 0) wb[threadIdx.x >> 5] = b;
+    }
     constexpr int PER = kScanBlock / kT;  // 4 consecutive items per thread
     const int64_t base = (int64_t)blockIdx.x * kScanBlock + (int64_t)threadIdx.x * PER;
     int32_t v[PER], t = 0;
@@ -130,63 +137,65 @@ __global__ void scan_apply_kernel(const int32_t* __restrict__ in, int64_t n, con
             const int32_t y = __shfl_up_sync(kFull, s, o);
             if (lane >= o) s += y;
         }
-        w[lane] = s;
+        if (lane < kT / 32) w[lane] = s;
     }
     __syncthreads();
-    int32_t run = sums[blockIdx.x] + x - t + (wid > 0 ? w[wid - 1] : 0);
+    int32_t before = 0;
+    if (TOTALS) {
+#pragma unroll
+        for (int i = 0; i < kT / 32; ++i) before += wb[i];
+    } else {
+        before = sums[blockIdx.x];
+    }
+    int32_t run = before + x - t + (wid > 0 ? w[wid - 1] : 0);
 #pragma unroll
     for (int j = 0; j < PER; ++j) {
         if (base + j < n) out[base + j] = run;
         run += v[j];
     }
     const int64_t nblk = (n + kScanBlock - 1) / kScanBlock;
-    if (blockIdx.x == nblk - 1 && threadIdx.x == blockDim.x - 1) out[n] = sums[nblk];
+    if (blockIdx.x == nblk - 1 && threadIdx.x == blockDim.x - 1) out[n] = run;
 }
 
 int64_t scan_tmp_ints(int64_t n) { return (n + kScanBlock - 1) / kScanBlock + 1; }
 
-// The whole scan in one block, for arrays of up to kScanSmall items: 32 items per thread and
-// turn, one launch instead of three (5 instead of 8 us of device time on 16,384 items, and
-// two launches fewer on the host, which is what the building of small trees waits for).
-constexpr int64_t kScanSmall = 65536;
+// The scan of up to kScanSmall items in one block (16,384 items that way took 12 us, 65,536
+// 41 us), and up to kScanTwo block totals without a launch of their own: every block adds the
+// totals before it itself.  Two launches fewer, or one, on the host, which is what the
+// building of small trees waits for.
+constexpr int64_t kScanSmall = 4096;
+constexpr int64_t kScanTwo = 2048;
 template <bool POP>
 __global__ void __launch_bounds__(1024) scan_small_kernel(const int32_t* __restrict__ in, int n,
                                                           int32_t* __restrict__ out) {
     __shared__ int32_t w[32];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    int32_t carry = 0;
-    for (int base = 0; base < n; base += 16384) {
-        const int i0 = base + 16 * threadIdx.x;
-        int32_t v[16], t = 0;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, i0 = 4 * threadIdx.x;
+    int32_t v[4], t = 0;
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-            v[j] = i0 + j < n ? scan_item<POP>(in[i0 + j]) : 0;
-            t += v[j];
-        }
-        int32_t x = t;
-        for (int o = 1; o < 32; o <<= 1) {
-            const int32_t y = __shfl_up_sync(kFull, x, o);
-            if (lane >= o) x += y;
-        }
-        if (lane == 31) w[wid] = x;
-        __syncthreads();
-        int32_t s = w[lane];
-        for (int o = 1; o < 32; o <<= 1) {
-            const int32_t y = __shfl_up_sync(kFull, s, o);
-            if (lane >= o) s += y;
-        }
-        const int32_t before = wid > 0 ? __shfl_sync(kFull, s, wid - 1) : 0;
-        const int32_t total = __shfl_sync(kFull, s, 31);
-        int32_t run = carry + before + x - t;
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-            if (i0 + j < n) out[i0 + j] = run;
-            run += v[j];
-        }
-        carry += total;
-        __syncthreads();
+    for (int j = 0; j < 4; ++j) {
+        v[j] = i0 + j < n ? scan_item<POP>(in[i0 + j]) : 0;
+        t += v[j];
     }
-    if (threadIdx.x == 0) out[n] = carry;
+    int32_t x = t;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int32_t y = __shfl_up_sync(kFull, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) w[wid] = x;
+    __syncthreads();
+    int32_t s = w[lane];
+    for (int o = 1; o < 32; o <<= 1) {
+        const int32_t y = __shfl_up_sync(kFull, s, o);
+        if (lane >= o) s += y;
+    }
+    const int32_t before = __shfl_sync(kFull, s, max(wid - 1, 0));
+    int32_t run = (wid > 0 ? before : 0) + x - t;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        if (i0 + j < n) out[i0 + j] = run;
+        run += v[j];
+    }
+    if (threadIdx.x == 1023) out[n] = run;
 }
 
 // out[0..n] = exclusive prefix sums of in[0..n) (out[n] = total); sums: scan_tmp_ints(n)
@@ -199,9 +208,16 @@ cudaError_t exscan(const int32_t* in, int32_t* out, int64_t n, int32_t* sums, cu
         return cudaGetLastError();
     }
     scan_reduce_kernel<POP><<<(unsigned)nb, kT, 0, s>>>(in, n, sums);
+    if (nb <= kScanTwo) {
+        scan_apply_kernel<POP, true><<<(unsigned)nb, kT, 0, s>>>(in, n, sums, out);
+        return cudaGetLastError();
+    }
     scan_sums_kernel<<<1, 1024, 0, s>>>(sums, (int)nb);
-    scan_apply_kernel<POP><<<(unsigned)nb, kT, 0, s>>>(in, n, sums, out);
+    scan_apply_kernel<POP, false><<<(unsigned)nb, kT, 0, s>>>(in, n, sums, out);
     return cudaGetLastError();
+}
+int exscan_launches(int64_t n) {
+    return n <= kScanSmall ? 1 : n <= kScanTwo * kScanBlock ? 2 : 3;
 }
 
 // ------------------------------------------------------------------------- radix sort
@@ -1051,7 +1067,22 @@ int unique_runs(const uint64_t* key, int64_t n, uint64_t skip, uint64_t* out, in
     return LFMM_OK;
 }
 
+// the compact id of every sorted target's leaf, eight lanes per leaf
+__global__ void target_leaf_kernel(const int32_t* __restrict__ rl_t, const int32_t* __restrict__ rl_id, int64_t m,
+                                   int32_t* __restrict__ t_leaf) {
+    const int64_t n8 = ((int64_t)gridDim.x * blockDim.x) >> 3;
+    for (int64_t j = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 3; j < m; j += n8) {
+        const int id = rl_id[j];
+        for (int v = rl_t[j] + (threadIdx.x & 7); v < rl_t[j + 1]; v += 8) t_leaf[v] = id;
+    }
+}
+
 }  // namespace
+
+cudaError_t launch_target_leaves(const Forest& F, int32_t* t_leaf, cudaStream_t s) {
+    target_leaf_kernel<<<grid_of(8 * F.n_leaves), kT, 0, s>>>(F.rl_t, F.rl_id, F.n_leaves, t_leaf);
+    return cudaGetLastError();
+}
 
 int forest_build(Forest& F, const int32_t* src, const int64_t* soff_h, int64_t ns, const int32_t* tgt,
                  const int64_t* toff_h, int64_t nt, int np, int leaf_size, int max_leaf_side, bool wide,
@@ -1435,7 +1466,7 @@ int forest_build(Forest& F, const int32_t* src, const int64_t* soff_h, int64_t n
         grid_leaves_kernel<<<grid_of(M), kT, 0, s>>>(G, F.rl_key, M, kb, F.rl_id, leaf_rl);
         grid_links_kernel<<<grid_of(NB), kT, 0, s>>>(G, NB, cstart, bp_all, bxy_all, par_all, ch_all, il_all);
         LFMM_CUDA_TRY(cudaGetLastError());
-        timer->add_launches(words <= kScanSmall ? 6 : 8);
+        timer->add_launches(5 + exscan_launches(words));
     } else {
     if (dense) {  // the number of leaves
         LFMM_CUDA_TRY(cudaMemcpyAsync(hw, M_d, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
@@ -1588,7 +1619,7 @@ int forest_build(Forest& F, const int32_t* src, const int64_t* soff_h, int64_t n
         strip_record_kernel<<<grid_of(M), kT, 0, s>>>(F.rl_key, flag, pos, M, kb, F.SW, F.strips);
         strip_rows_kernel<<<grid_of(M), kT, 0, s>>>(F.strips, F.n_strips_d, F.rl_key, M, dL, kb, F.SW, F.strip_rows);
         LFMM_CUDA_TRY(cudaGetLastError());
-        timer->add_launches(M <= kScanSmall ? 4 : 6);
+        timer->add_launches(3 + exscan_launches(M));
     }
     return LFMM_OK;  // temporaries are freed in stream order
 }

@@ -309,6 +309,7 @@ struct Forest {
     int32_t* n_strips_d = nullptr;
     int64_t n_strips = 0;                       // at most this many strips (the count is on the device)
     double* near_tmp = nullptr;                 // near field per sorted target, before the far part is added
+    int32_t* t_leaf = nullptr;                  // (with near_tmp) compact id of each sorted target's leaf
     std::vector<void*> owned;
     int64_t bytes = 0;
     void* m2l_part = nullptr;               // partial sums of K-split list M2L levels (plan-owned)
@@ -326,6 +327,8 @@ int m2l_list_chunks(int64_t maxc, int num_sms, int split = 0);
 // Bytes of partial sums the K-split list M2L levels of F need (0: none split).
 int64_t forest_m2l_split_bytes(const Forest& F, int NP, size_t esz, int num_sms, int split = 0);
 
+// t_leaf[v] = compact id of sorted target v's leaf.
+cudaError_t launch_target_leaves(const Forest& F, int32_t* t_leaf, cudaStream_t s);
 // What the caller knows of a single problem: its bounding box, and whether the targets are
 // the sources (1, 0; -1: not known).
 struct ForestHint {
