@@ -95,7 +95,7 @@ struct lfmm_plan {
     double* un_tmp = nullptr;        // near field per target (caller order) from the concurrent near-field pass
     double* uf_tmp = nullptr;        // far field per target (caller order), before the final sum
     struct AuxStream* aux = nullptr;  // near-field pass runs here, beside the far-field sweeps
-    struct AuxStream* far_aux = nullptr;  // pruned / forest, 8-byte types: the far field, beside the near field
+    struct AuxStream* far_aux = nullptr;  // pruned / forest: the far field, beside the near field
     // uniform storage: the targets are bucketed on `aux` while the plan's creation and the
     // evaluation's upward sweep go on; whatever reads them waits for this event
     cudaEvent_t tgt_ready = nullptr;
@@ -349,10 +349,7 @@ int forest_workspaces(lfmm_plan* p, cudaStream_t s) {
         if (need > 0 && (st = palloc(p, &b, (size_t)need * sizeof(float), s))) return st;
         F.tc_split = (float*)b;
     }
-    // near field before the far part is added: the 8-byte types' near field is its own launch,
-    // binary32's where leaves hold fewer than 12 targets on average (clustered_4m, 5.6: KKK us in
-    // two launches against 1,420 in one; forest_4096, 22: LLL against 1,930)
-    if ((p->opts.precision != LFMM_MIXED || p->nt < 12 * F.n_leaves) && F.kmax >= 0) {
+    if (F.kmax >= 0) {  // near field before the far part is added, and every target's leaf for that
         void* b;
         if ((st = palloc(p, &b, (size_t)p->nt * (sizeof(double) + sizeof(int32_t)), s))) return st;
         F.near_tmp = (double*)b;
@@ -780,10 +777,10 @@ int far_sweeps(lfmm_plan* p, const FarBufs& b, cudaStream_t s, Hook before_fine)
 template <typename T>
 int eval_impl(lfmm_plan* p, const double* f, double* u, double* un, double* uf, cudaStream_t s) {
     if (p->forest) {
-        // 8-byte types: the far field on a second stream beside the near field (launches of
-        // few blocks, so of a higher priority), joined before L2P
+        // the far field on a second stream beside the near field (launches of few blocks, so of
+        // a higher priority), joined before L2P
         SideStream side{};
-        const bool beside = sizeof(T) == 8 && p->forest->kmax >= 0 && !(p->opts.flags & LFMM_FLAG_SERIAL);
+        const bool beside = p->forest->kmax >= 0 && !(p->opts.flags & LFMM_FLAG_SERIAL);
         if (beside && !p->far_aux) p->far_aux = acquire_aux(p->device, true);
         if (beside && p->far_aux) side = SideStream{p->far_aux->s, p->far_aux->fork, p->far_aux->join};
         const int st = forest_eval<T>(*p->forest, *p->ops, f, (T*)p->f_sorted, (T*)p->qhat, (T*)p->uhat, p->Qbox,

@@ -661,44 +661,34 @@ __global__ void __launch_bounds__(LCfg<T, NP>::WARPS * 32, sizeof(T) == 4 ? 2 : 
     }
 }
 
-// P2P + L2P over a list of strips (problem, leaf row, first leaf column): the
-// uniform-tree strip kernel with per-problem leaf grids and compact-id lookups.
-// Six warps per block and staging for 2,048 sources and 1,536 targets: four blocks per SM
-// at binary32 (forest_4096, mixed p = 7: 2.25 ms with eight warps and room for 4,096
-// sources and 2,048 targets, three blocks per SM; 2.22 ms with eight warps and these
-// caps; 2.73 / 2.23 / 2.00 / 1.95 ms with two / three / four / six warps).  Forest strips
-// are short (rows of 8 to 32 leaves of ~16 targets), so fewer warps per strip idle less
-// at the strip's barriers.
+// P2P over a list of strips (problem, leaf row, first leaf column): the uniform-tree strip
+// kernel with per-problem leaf grids and compact-id lookups; l2p_list_kernel adds the far
+// part.  A strip of few targets is bound by its chain of dependent loads and barriers,
+// whatever it holds, so the blocks are small and many: binary32 takes six warps per block
+// and six blocks per SM, its staging sized for the tree's fullest leaves (with L2P in the
+// same kernel its registers allowed four blocks: clustered_4m 1,423 us against 820 + 132
+// here, forest_4096 1,886 against 1,366 + 275; the order of every target's sums is the
+// same).  The dense end is bound by shared-memory wavefronts of the table lookups.
 template <typename T>
 struct LStripCfg {
-    static constexpr int WARPS = 6;
-    static constexpr int CAPS = 2048;
+    static constexpr int CAPS = 2048;  // binary32: staged sources, and targets, of a block at most
     static constexpr int CAPT = 1536;
     static constexpr int MAXSW = 32;
     // (the builder sizes strips with these, those of the 8-byte types with near8_caps)
     static_assert(MAXSW == kStripMaxSW && CAPT == kStripCapTgt && CAPS >= kStripCapSrc, "strip staging caps");
 };
 
-// The near field of the 8-byte types is its own launch (kNear; l2p_list_kernel follows), so that
-// it runs beside the far field and in blocks of its own shape: one block of 24 warps per
-// SM, because the float-float / binary64 table (146 KB at side 32) leaves no room for a
-// second block, and as many staged sources as fit (near8_caps).  Its warps share a strip's
-// work evenly whatever the number of targets: G = 1 .. 32 lanes take one target and every
-// G-th source of its three rows, and the lanes' sums are added by shuffles; strips of few
-// targets among many sources (clustered points, scattered targets) had kept one warp of
-// six busy.  Float-float pairs are added without renormalising each term (12 instead of
-// 15 operations).
-//
-// Binary32 splits into the same two launches where strips are short (few targets per leaf:
-// clustered points): a strip is then bound by its chain of dependent loads and barriers,
-// and the near field alone, without L2P's registers, fits six blocks per SM instead of
-// four.  The order of every target's sums is the same in both forms.
-constexpr int kBoth = 0, kNear = 1;
-constexpr int kNearThreads = 768;
-template <typename T, int PART>
+// The near field of the 8-byte types takes one block of 24 warps per SM, because the
+// float-float / binary64 table (146 KB at side 32) leaves no room for a second block, and as
+// many staged sources as fit (near8_caps).  Its warps share a strip's work evenly whatever
+// the number of targets: G = 1 .. 32 lanes take one target and every G-th source of its
+// three rows, and the lanes' sums are added by shuffles; strips of few targets among many
+// sources (clustered points, scattered targets) had kept one warp of six busy.  Float-float
+// pairs are added without renormalising each term (12 instead of 15 operations).
+template <typename T>
 struct NearCfg {
-    static constexpr int THREADS = sizeof(T) == 8 && PART == kNear ? kNearThreads : LStripCfg<T>::WARPS * 32;
-    static constexpr int BLOCKS = sizeof(T) == 8 ? 1 : PART == kNear ? 6 : 4;
+    static constexpr int THREADS = sizeof(T) == 8 ? 768 : 192;
+    static constexpr int BLOCKS = sizeof(T) == 8 ? 1 : 6;
 };
 
 // acc += a b with the two-sum's and the product's errors collected in acc.lo
@@ -714,37 +704,32 @@ __device__ __forceinline__ void near_add(DF& acc, DF a, DF b) {
 }
 __device__ __forceinline__ void near_add(double& acc, double a, double b) { acc = fma(a, b, acc); }
 
-template <typename T, int NP, int PART>
-__global__ void __launch_bounds__(NearCfg<T, PART>::THREADS, NearCfg<T, PART>::BLOCKS) p2p_list_kernel(
+template <typename T>
+__global__ void __launch_bounds__(NearCfg<T>::THREADS, NearCfg<T>::BLOCKS) p2p_list_kernel(
     const int4* __restrict__ strips, const int4* __restrict__ strip_rows, const int32_t* __restrict__ n_strips_d,
     const int32_t* __restrict__ Lp, const uint64_t* __restrict__ rl_key, const int32_t* __restrict__ rl_s,
     const int32_t* __restrict__ rl_t, const int32_t* __restrict__ rl_id, int kb, int side, int SW,
     const int32_t* __restrict__ sloc, const int32_t* __restrict__ tloc, const int32_t* __restrict__ tperm,
     const T* __restrict__ f_sorted,
-    const T* __restrict__ table, int tab_H, int tab_W, const T* __restrict__ uhat,
-    const typename Mono<T>::V* __restrict__ Cleaf, const typename Mono<T>::V* __restrict__ Qleaf,
-    const T* __restrict__ tofsT, double* __restrict__ u, double* __restrict__ u_near, double* __restrict__ u_far,
-    int caps, int capt, double* __restrict__ near_tmp) {
+    const T* __restrict__ table, int tab_H, int tab_W, const typename Mono<T>::V* __restrict__ Qleaf,
+    double* __restrict__ u, double* __restrict__ u_near, double* __restrict__ u_far, int caps, int capt,
+    double* __restrict__ near_tmp) {
     griddep_wait();
     using M = Mono<T>;
     using V = typename M::V;
     using Cfg = LStripCfg<T>;
-    constexpr bool kHasFar = PART != kNear;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int tab_n = (2 * tab_H + 1) * tab_W;
     T* tab = reinterpret_cast<T*>(smem_raw);
     SrcEntry<T>* s_src = reinterpret_cast<SrcEntry<T>*>(tab + tab_n);
-    T* s_uhat = reinterpret_cast<T*>(s_src + caps);           // [MAXSW][NP]
-    V* s_q = reinterpret_cast<V*>(s_uhat + (kHasFar ? Cfg::MAXSW * NP : 0));  // [3][MAXSW+2]
-    V* s_c = s_q + 3 * (Cfg::MAXSW + 2);                      // [MAXSW]
-    int* s_tloc = reinterpret_cast<int*>(s_c + Cfg::MAXSW);   // [capt]
+    V* s_q = reinterpret_cast<V*>(s_src + caps);              // [3][MAXSW+2]
+    int* s_tloc = reinterpret_cast<int*>(s_q + 3 * (Cfg::MAXSW + 2));  // [capt]
     int* s_tperm = s_tloc + capt;                             // [capt]
     int* s_sb = s_tperm + capt;                               // [3][MAXSW+3]
     int* s_tb = s_sb + 3 * (Cfg::MAXSW + 3);                  // [MAXSW+1]
     __shared__ int s_rs[4];
     __shared__ int s_ra[Cfg::MAXSW][3], s_rl[Cfg::MAXSW][3];
     __shared__ double s_nc[Cfg::MAXSW];
-    __shared__ int s_has[Cfg::MAXSW];
     __shared__ int s_rj[3][2];                 // leaf-list range [j0, j1) of each row (-1: outside)
     __shared__ int s_lc[3][Cfg::MAXSW + 2];    // column - c_lo of each listed leaf (ascending)
 
@@ -790,12 +775,12 @@ __global__ void __launch_bounds__(NearCfg<T, PART>::THREADS, NearCfg<T, PART>::B
         // int items: the first source at or after column c of each row (past its last
         // column: the first source of the next occupied leaf, as in a dense bucket array)
         // and the target boundaries of the strip's leaves; V items: the leaf charges of the
-        // three rows and the strip leaves' incoming constants, through each leaf's compact
-        // id.  A thread takes one item of each kind and issues its loads before the stores.
+        // three rows, through each leaf's compact id.  A thread takes one item of each kind and
+        // issues its loads before the stores.
         {
             const int nA = 3 * (ncol + 1), nI = nA + (bx1 - bx0 + 1);
-            const int nC = 3 * ncol, nV = nC + (bx1 - bx0);
-            for (int i = threadIdx.x; i < max(nI, nV); i += blockDim.x) {
+            const int nC = 3 * ncol;
+            for (int i = threadIdx.x; i < max(nI, nC); i += blockDim.x) {
                 int iv = 0;
                 if (i < nA) {
                     const int r = i / (ncol + 1), c = i % (ncol + 1);
@@ -812,43 +797,15 @@ __global__ void __launch_bounds__(NearCfg<T, PART>::THREADS, NearCfg<T, PART>::B
                         const int q = first_at(r, c);
                         if (j0 + q < s_rj[r][1] && s_lc[r][q] == c) cid = rl_id[j0 + q];
                     }
-                } else if (i < nV) {
-                    const int cc = bx0 + (i - nC) - c_lo;
-                    const int q = first_at(1, cc);
-                    if (s_rj[1][0] + q < s_rj[1][1] && s_lc[1][q] == cc) cid = rl_id[s_rj[1][0] + q];
                 }
                 V vv = M::zero();
-                if (i < nC) {
-                    if (cid >= 0) vv = Qleaf[cid];
-                } else if (i < nV) {
-                    if (Cleaf && cid >= 0) vv = Cleaf[cid];
-                }
+                if (cid >= 0) vv = Qleaf[cid];
                 if (i < nA) s_sb[(i / (ncol + 1)) * (Cfg::MAXSW + 3) + i % (ncol + 1)] = iv;
                 else if (i < nI) s_tb[i - nA] = iv;
-                if (i < nC) {
-                    s_q[(i / ncol) * (Cfg::MAXSW + 2) + i % ncol] = vv;
-                } else if (i < nV) {
-                    s_has[i - nC] = cid;
-                    s_c[i - nC] = vv;
-                }
+                if (i < nC) s_q[(i / ncol) * (Cfg::MAXSW + 2) + i % ncol] = vv;
             }
         }
         __syncthreads();
-        // the strip's leaf expansions (four loads in flight per thread)
-        for (int i0 = threadIdx.x; kHasFar && i0 < (bx1 - bx0) * NP; i0 += 4 * blockDim.x) {
-            T vals[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int i = i0 + k * (int)blockDim.x;
-                const int cid = i < (bx1 - bx0) * NP ? s_has[i / NP] : -1;
-                vals[k] = (uhat && cid >= 0) ? uhat[(size_t)cid * NP + i % NP] : T(0);
-            }
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int i = i0 + k * (int)blockDim.x;
-                if (i < (bx1 - bx0) * NP) s_uhat[i] = vals[k];
-            }
-        }
         for (int li = threadIdx.x; li < bx1 - bx0; li += blockDim.x) {
             const int bx = bx0 + li;
             const int ca = max(bx - 1, 0) - c_lo, cb = min(bx + 1, n - 1) - c_lo + 1;
@@ -880,7 +837,18 @@ __global__ void __launch_bounds__(NearCfg<T, PART>::THREADS, NearCfg<T, PART>::B
         stage_strip_targets(s_tloc, s_tperm, nt_strip, s_tb, bx1 - bx0, tb0, tloc, tperm);
         __syncthreads();
 
-        if constexpr (PART == kNear && sizeof(T) == 8) {
+        // the near sum of sorted target tb0 + v: kept for l2p_list_kernel, or the result
+        auto put = [&](int v, double dn) {
+            if (near_tmp) {
+                near_tmp[tb0 + v] = dn;
+                return;
+            }
+            const int dst = s_tperm[v];  // no far field
+            if (u) u[dst] = dn;
+            if (u_near) u_near[dst] = dn;
+            if (u_far) u_far[dst] = 0.0;
+        };
+        if constexpr (sizeof(T) == 8) {
             const int warps = blockDim.x >> 5;
             int lg = 0;  // G = 2^lg lanes per target: at least two units of 32 / G targets per warp
             while (lg < 5 && (nt_strip << lg) < 64 * warps) ++lg;
@@ -912,25 +880,14 @@ __global__ void __launch_bounds__(NearCfg<T, PART>::THREADS, NearCfg<T, PART>::B
                     }
                 }
                 for (int o = 1; o < G; o <<= 1) acc += shfl_xor_v(acc, o);
-                if (active && sub == 0) {
-                    const double dn = (double)acc + s_nc[li];
-                    if (near_tmp) {
-                        near_tmp[tb0 + v] = dn;
-                    } else {  // no far field
-                        const int dst = s_tperm[v];
-                        if (u) u[dst] = dn;
-                        if (u_near) u_near[dst] = dn;
-                        if (u_far) u_far[dst] = 0.0;
-                    }
-                }
+                if (active && sub == 0) put(v, (double)acc + s_nc[li]);
             }
             continue;
         }
         const int n_chunks = (nt_strip + 31) >> 5;
-        for (int chunk = warp; chunk < n_chunks; chunk += Cfg::WARPS) {
+        for (int chunk = warp; chunk < n_chunks; chunk += NearCfg<T>::THREADS / 32) {
             const int v = chunk * 32 + lane;
             const bool active = v < nt_strip;
-            const int n_act = min(32, nt_strip - chunk * 32);
             const int tl = s_tloc[active ? v : chunk * 32];
             const int li = (tl >> 8) & 0xff, tx = tl & 0xff, ty = tl >> 16;
             const T* tp = tab_c + (tx + tab_W * ty + li * side);
@@ -969,45 +926,14 @@ __global__ void __launch_bounds__(NearCfg<T, PART>::THREADS, NearCfg<T, PART>::B
                 }
             }
             acc -= cmp;
-            if constexpr (PART == kNear) {
-                if (active) near_tmp[tb0 + v] = (double)acc + s_nc[li];
-                continue;
-            }
-            T far = T(0);
-            if (uhat) {
-                constexpr int PL = NP / 32;
-                const int myJ = tx + side * ty;
-                T part[32];
-#pragma unroll
-                for (int qq = 0; qq < 32; ++qq) {
-                    const int Jq = shfl(myJ, qq), lq = shfl(li, qq);
-                    T w = T(0);
-                    if (qq < n_act) {
-                        const T* row = tofsT + (size_t)Jq * NP;
-                        const T* uq = s_uhat + lq * NP;
-#pragma unroll
-                        for (int i = 0; i < PL; ++i) w = fma(ldg(row + lane + 32 * i), uq[lane + 32 * i], w);
-                    }
-                    part[qq] = w;
-                }
-                far = reduce_scatter32(part);
-            }
-            if (active) {
-                const int dst = s_tperm[v];
-                const double dn = (double)acc + s_nc[li];
-                const double df = (double)far + M::to_double(s_c[li]);
-                if (u) u[dst] = dn + df;
-                if (u_near) u_near[dst] = dn;
-                if (u_far) u_far[dst] = df;
-            }
+            if (active) put(v, (double)acc + s_nc[li]);
         }
     }
 }
 
-// L2P of the split form: u = near_tmp + T_ofs(:, J)^T u_hat + C for 32 consecutive sorted targets
-// per warp, the lanes owning expansion entries (the order of every sum is that of
-// p2p_list_kernel).  Not by strips: a strip of few targets costs its chain of dependent
-// loads whatever its size (clustered_4m: 842 us by strips).
+// L2P: u = near_tmp + T_ofs(:, J)^T u_hat + C for 32 consecutive sorted targets per warp, the
+// lanes owning expansion entries.  Not by strips: a strip of few targets costs its chain of
+// dependent loads whatever its size (clustered_4m: 842 us by strips, 132 here).
 template <typename T, int NP>
 __global__ void __launch_bounds__(128) l2p_list_kernel(int64_t nt, const int32_t* __restrict__ t_leaf,
                                                        const int32_t* __restrict__ tloc,
@@ -1111,40 +1037,35 @@ SgTree forest_sg_tree(const Forest& F) {
     return t;
 }
 
-template <typename T, int PART>
-static int launch_list_p2p(const Forest& F, const DeviceOps& ops, const T* f_sorted, const T* uhat, const void* Cleaf,
-                           const void* Qleaf, double* u, double* un, double* uf, int num_sms, cudaStream_t s,
-                           bool use_tmp) {
+// Near field of every strip: into F.near_tmp (use_tmp), or, without a far field, the result.
+template <typename T>
+static int launch_list_p2p(const Forest& F, const DeviceOps& ops, const T* f_sorted, const void* Qleaf, double* u,
+                           double* un, double* uf, int num_sms, cudaStream_t s, bool use_tmp) {
     using Cfg = LStripCfg<T>;
     using V = typename Mono<T>::V;
     PhaseTimer pt(LFMM_PHASE_P2P, s);
-    const int NP = ops.NP;
-    // staging for the strips of this tree (8-byte near field: all that fits)
-    const int caps = sizeof(T) == 8 && PART == kNear ? near8_caps(F.side)
-                                                     : std::min(Cfg::CAPS, 3 * (F.SW + 2) * std::max(1, F.max_src));
+    // staging for the strips of this tree (8-byte types: all that fits)
+    const int caps = sizeof(T) == 8 ? near8_caps(F.side) : std::min(Cfg::CAPS, 3 * (F.SW + 2) * std::max(1, F.max_src));
     const int capt = std::min(Cfg::CAPT, F.SW * std::max(1, F.max_tgt) + 1) / 2 * 2;
-    size_t smem = (size_t)(3 * (Cfg::MAXSW + 2) + Cfg::MAXSW) * sizeof(V) + (size_t)2 * capt * sizeof(int) +
-                  (size_t)(3 * (Cfg::MAXSW + 3) + Cfg::MAXSW + 1) * sizeof(int);
-    smem += (size_t)(2 * ops.tab_H + 1) * ops.tab_W * sizeof(T) + (size_t)caps * sizeof(SrcEntry<T>);
-    if (PART != kNear) smem += (size_t)Cfg::MAXSW * NP * sizeof(T);
-    constexpr int threads = NearCfg<T, PART>::THREADS;
-    auto go = [&](auto np_tag) -> cudaError_t {
-        constexpr int NPc = decltype(np_tag)::value;
-        const void* fn = (const void*)p2p_list_kernel<T, NPc, PART>;
-        const cudaError_t e = ensure_dynamic_smem(fn, smem);
-        if (e != cudaSuccess) return e;
+    const size_t smem = (size_t)(2 * ops.tab_H + 1) * ops.tab_W * sizeof(T) + (size_t)caps * sizeof(SrcEntry<T>) +
+                        (size_t)3 * (Cfg::MAXSW + 2) * sizeof(V) + (size_t)2 * capt * sizeof(int) +
+                        (size_t)(3 * (Cfg::MAXSW + 3) + Cfg::MAXSW + 1) * sizeof(int);
+    constexpr int threads = NearCfg<T>::THREADS;
+    const void* fn = (const void*)p2p_list_kernel<T>;
+    cudaError_t e = ensure_dynamic_smem(fn, smem);
+    if (e == cudaSuccess) {
         const int per_sm = blocks_per_sm(fn, threads, smem);
-        // the near field beside the far field: blocks of a few strips, so that the far
-        // field's launches (of a higher priority) find free SMs as blocks end
-        const int64_t waves = sizeof(T) == 8 && PART == kNear && use_tmp ? 6 : 1;
+        // beside the far field: blocks of a few strips, so that the far field's launches (of
+        // a higher priority) find free SMs as blocks end; binary32's table is staged faster and
+        // its far field takes more of the time (forest_4096 with 2 / 6 / 16 rounds of blocks:
+        // 4,126 / 4,084 / 3,932 us; one stream 4,287 us; clustered_4m 4,020 / 3,880 / 3,867)
+        const int64_t waves = !use_tmp ? 1 : sizeof(T) == 8 ? 6 : 16;
         const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(F.n_strips, waves * num_sms * per_sm));
-        return launch_dependent(p2p_list_kernel<T, NPc, PART>, dim3((unsigned)grid), dim3(threads), smem, s, F.strips,
-                                F.strip_rows, F.n_strips_d, F.d_L, F.rl_key, F.rl_s, F.rl_t, F.rl_id, F.kb, F.side,
-                                F.SW, F.sloc, F.tloc, F.tperm, f_sorted, (const T*)ops.p2p_table, ops.tab_H, ops.tab_W,
-                                uhat, (const V*)Cleaf, (const V*)Qleaf, (const T*)ops.tofsT, u, un, uf, caps, capt,
-                                use_tmp ? F.near_tmp : nullptr);
-    };
-    const cudaError_t e = NP == 32 ? go(std::integral_constant<int, 32>()) : go(std::integral_constant<int, 64>());
+        e = launch_dependent(p2p_list_kernel<T>, dim3((unsigned)grid), dim3(threads), smem, s, F.strips, F.strip_rows,
+                             F.n_strips_d, F.d_L, F.rl_key, F.rl_s, F.rl_t, F.rl_id, F.kb, F.side, F.SW, F.sloc, F.tloc,
+                             F.tperm, f_sorted, (const T*)ops.p2p_table, ops.tab_H, ops.tab_W, (const V*)Qleaf, u, un,
+                             uf, caps, capt, use_tmp ? F.near_tmp : nullptr);
+    }
     if (e != cudaSuccess) return fail(LFMM_ECUDA, std::string("p2p_list_kernel: ") + cudaGetErrorString(e));
     pt.add_launches(1);
     return LFMM_OK;
@@ -1232,21 +1153,20 @@ int forest_eval(const Forest& F, const DeviceOps& ops, const double* f, T* f_sor
             pt.add_launches(1);
         }
     }
-    // the near field of the 8-byte types needs the sorted charges and the leaf charges only:
-    // it runs on the caller's stream, the rest of the far field on the side stream
+    // the near field needs the sorted charges and the leaf charges only: it runs on the
+    // caller's stream, the rest of the far field on the side stream
     const cudaStream_t s_main = s;
-    const bool fork = sizeof(T) == 8 && far && side != nullptr;
+    const bool fork = far && side != nullptr && status == nullptr;  // not beside a persistent sweep
+    if (fork) {
+        LFMM_CUDA_TRY(cudaEventRecord(side->fork, s));
+        LFMM_CUDA_TRY(cudaStreamWaitEvent(side->s, side->fork, 0));
+        s = side->s;
+    }
+    if (far) {
+        const int st = launch_list_p2p<T>(F, ops, f_sorted, Qm(0), nullptr, nullptr, nullptr, num_sms, s_main, true);
+        if (st) return st;
+    }
     if constexpr (sizeof(T) == 8) {
-        if (fork) {
-            LFMM_CUDA_TRY(cudaEventRecord(side->fork, s));
-            LFMM_CUDA_TRY(cudaStreamWaitEvent(side->s, side->fork, 0));
-            s = side->s;
-        }
-        if (far) {
-            const int st = launch_list_p2p<T, kNear>(F, ops, f_sorted, (const T*)nullptr, nullptr, Qm(0), nullptr, nullptr,
-                                                     nullptr, num_sms, s_main, true);
-            if (st) return st;
-        }
         if (far && sliced) {
             PhaseTimer pt(LFMM_PHASE_M2L_TC, s);
             int n = 0;
@@ -1415,25 +1335,12 @@ int forest_eval(const Forest& F, const DeviceOps& ops, const double* f, T* f_sor
             pt.add_launches(nc > 1 ? 2 : 1);
         }
     }
-    // near field (+ L2P): one launch for binary32; for the 8-byte types the near field was
-    // launched beside the far field and L2P follows it here
-    if constexpr (sizeof(T) == 8) {
-        if (!far) return launch_list_p2p<T, kNear>(F, ops, f_sorted, (const T*)nullptr, nullptr, Qm(0), u, un, uf, num_sms, s, false);
-        if (fork) {
-            LFMM_CUDA_TRY(cudaEventRecord(side->join, s));
-            LFMM_CUDA_TRY(cudaStreamWaitEvent(s_main, side->join, 0));
-        }
-        return launch_list_l2p<T>(F, ops, (const T*)Ux(0), Cm(0), u, un, uf, s_main);
-    } else {
-        if (far && F.near_tmp) {
-            const int st = launch_list_p2p<T, kNear>(F, ops, f_sorted, (const T*)nullptr, nullptr, Qm(0), nullptr, nullptr,
-                                                     nullptr, num_sms, s, true);
-            if (st) return st;
-            return launch_list_l2p<T>(F, ops, (const T*)Ux(0), Cm(0), u, un, uf, s);
-        }
-        return launch_list_p2p<T, kBoth>(F, ops, f_sorted, (const T*)(far ? Ux(0) : nullptr), far ? Cm(0) : nullptr, Qm(0), u, un, uf, num_sms, s,
-                                         false);
+    if (!far) return launch_list_p2p<T>(F, ops, f_sorted, Qm(0), u, un, uf, num_sms, s, false);
+    if (fork) {
+        LFMM_CUDA_TRY(cudaEventRecord(side->join, s));
+        LFMM_CUDA_TRY(cudaStreamWaitEvent(s_main, side->join, 0));
     }
+    return launch_list_l2p<T>(F, ops, (const T*)Ux(0), Cm(0), u, un, uf, s_main);
 }
 
 template int forest_eval<float>(const Forest&, const DeviceOps&, const double*, float*, float*, float*, void*, void*,

@@ -1110,8 +1110,12 @@ int forest_build(Forest& F, const int32_t* src, const int64_t* soff_h, int64_t n
         same_points_kernel<<<grid_of(ns), kT, 0, s>>>((const int2*)src, (const int2*)tgt, ns, word);
         timer->add_launches(1);
     }
-    int* hw = readback_words();  // page-locked words for the readbacks
-    if (!hw) return fail(LFMM_ENOMEM, "page-locked readback words");
+    int* hw = readback_words();  // page-locked words for the readbacks, or ordinary ones
+    std::vector<int> pageable;
+    if (!hw) {
+        pageable.resize(kReadbackWords);
+        hw = pageable.data();
+    }
     if (hint) {  // one problem, its box known
         hbb[0] = make_int4(hint->x0, hint->y0, hint->x1, hint->y1);
         if (compare) {
