@@ -984,12 +984,13 @@ __global__ void __launch_bounds__(StripCfg<T>::WARPS * 32) p2p_strip_kernel(
                     b = fma(tp[-e3.off], e3.f, b);
                     add(b);
                 }
-                if (j < len) {
-                    T b = T(0);
-                    for (; j < len; ++j) {
-                        const SrcEntry<T> e = src[j];
-                        b = fma(tp[-e.off], e.f, b);
-                    }
+                if (j < len) {  // the last one to three: their loads side by side
+                    const int last = len - 1 - j;
+                    const SrcEntry<T> e0 = src[j], e1 = src[j + min(last, 1)], e2 = src[j + last];
+                    const T t0 = tp[-e0.off], t1 = tp[-e1.off], t2 = tp[-e2.off];
+                    T b = fma(t0, e0.f, T(0));
+                    if (last >= 1) b = fma(t1, e1.f, b);
+                    if (last == 2) b = fma(t2, e2.f, b);
                     add(b);
                 }
             }
@@ -1167,18 +1168,17 @@ __global__ void __launch_bounds__(StripMultiCfg<T, KR>::WARPS * 32) p2p_strip_mu
                         add(k, b);
                     }
                 }
-                if (j < len) {
-                    T b[KR];
+                if (j < len) {  // the last one to three: their loads side by side
+                    const int last = len - 1 - j, j1 = j + min(last, 1), j2 = j + last;
+                    const T p0 = tp[-so[j]], p1 = tp[-so[j1]], p2 = tp[-so[j2]];
+                    const FV f0 = sf[j], f1 = sf[j1], f2 = sf[j2];
 #pragma unroll
-                    for (int k = 0; k < KR; ++k) b[k] = T(0);
-                    for (; j < len; ++j) {
-                        const T pj = tp[-so[j]];
-                        const FV fj = sf[j];
-#pragma unroll
-                        for (int k = 0; k < KR; ++k) b[k] = fma(pj, fj.v[k], b[k]);
+                    for (int k = 0; k < KR; ++k) {
+                        T b = fma(p0, f0.v[k], T(0));
+                        if (last >= 1) b = fma(p1, f1.v[k], b);
+                        if (last == 2) b = fma(p2, f2.v[k], b);
+                        add(k, b);
                     }
-#pragma unroll
-                    for (int k = 0; k < KR; ++k) add(k, b[k]);
                 }
             }
             if (active) {

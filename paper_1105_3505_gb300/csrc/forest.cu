@@ -916,12 +916,13 @@ __global__ void __launch_bounds__(NearCfg<T>::THREADS, NearCfg<T>::BLOCKS) p2p_l
                     b = fma(tp[-e3.off], e3.f, b);
                     add(b);
                 }
-                if (j < len) {
-                    T b = T(0);
-                    for (; j < len; ++j) {
-                        const SrcEntry<T> e = src[j];
-                        b = fma(tp[-e.off], e.f, b);
-                    }
+                if (j < len) {  // the last one to three: their loads side by side
+                    const int last = len - 1 - j;
+                    const SrcEntry<T> e0 = src[j], e1 = src[j + min(last, 1)], e2 = src[j + last];
+                    const T t0 = tp[-e0.off], t1 = tp[-e1.off], t2 = tp[-e2.off];
+                    T b = fma(t0, e0.f, T(0));
+                    if (last >= 1) b = fma(t1, e1.f, b);
+                    if (last == 2) b = fma(t2, e2.f, b);
                     add(b);
                 }
             }
