@@ -69,26 +69,46 @@ __device__ __forceinline__ void p2m_list_quad(int64_t b0, int64_t nb, int lane, 
 #pragma unroll
     for (int i = 0; i < PL; ++i) acc[i] = T(0);
     typename M::V qsum = M::zero();
-    for (int j0 = 0; j0 < cmax; j0 += G) {
-        T fj = T(0);
-        int J = 0;
-        if (j0 + hl < cnt) {
-            const int j = s0 + j0 + hl;
-            const int l = loc[j];
-            J = (l & 0xffff) + side * (l >> 16);
-            const double fd = f[perm[j]];
-            fj = (T)fd;
-            f_sorted[j] = fj;
-            qsum = M::add(qsum, M::from_double(fd));
-        }
-        const int cc = min(G, cmax - j0);
-        for (int k = 0; k < cc; ++k) {
-            // lanes of a quarter with fewer sources multiply row 0 by zero
-            const T fk = shfl(fj, (grp << 3) + k);
-            const int Jk = __shfl_sync(kFull, J, (grp << 3) + k);
-            const Row r = *reinterpret_cast<const Row*>(tofsT + (size_t)Jk * NP + hl * PL);
+    // rounds of G sources per leaf whose loads (index, then charge) are in flight together; bound
+    // by those loads (clustered_4m 128 us with one round, 107 with two; forest_4096 204, 179)
+    constexpr int R = 2;
+    for (int j0 = 0; j0 < cmax; j0 += R * G) {
+        T fj[R];
+        int J[R], pj[R];
+        double fd[R];
 #pragma unroll
-            for (int i = 0; i < PL; ++i) acc[i] = fma(r.v[i], fk, acc[i]);
+        for (int u = 0; u < R; ++u) {
+            const int j = j0 + u * G + hl;
+            J[u] = pj[u] = 0;
+            if (j < cnt) {
+                const int l = loc[s0 + j];
+                J[u] = (l & 0xffff) + side * (l >> 16);
+                pj[u] = perm[s0 + j];
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < R; ++u) fd[u] = j0 + u * G + hl < cnt ? f[pj[u]] : 0.0;
+#pragma unroll
+        for (int u = 0; u < R; ++u) {
+            const int j = j0 + u * G + hl;
+            fj[u] = T(0);
+            if (j < cnt) {
+                fj[u] = (T)fd[u];
+                f_sorted[s0 + j] = fj[u];
+                qsum = M::add(qsum, M::from_double(fd[u]));
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < R; ++u) {
+            const int cc = min(G, cmax - j0 - u * G);
+            for (int k = 0; k < cc; ++k) {
+                // lanes of a quarter with fewer sources multiply row 0 by zero
+                const T fk = shfl(fj[u], (grp << 3) + k);
+                const int Jk = __shfl_sync(kFull, J[u], (grp << 3) + k);
+                const Row r = *reinterpret_cast<const Row*>(tofsT + (size_t)Jk * NP + hl * PL);
+#pragma unroll
+                for (int i = 0; i < PL; ++i) acc[i] = fma(r.v[i], fk, acc[i]);
+            }
         }
     }
     if (lv) {
@@ -951,22 +971,36 @@ __global__ void __launch_bounds__(128) l2p_list_kernel(int64_t nt, const int32_t
     const int64_t v = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32 + lane;
     if (v - lane >= nt) return;
     const bool active = v < nt;
-    const int cid = t_leaf[active ? v : nt - 1], tl = tloc[active ? v : nt - 1];
-    const int myJ = (tl & 0xffff) + side * (tl >> 16);
+    // {row, leaf} of two targets as one broadcast word instead of four shuffles, and the last
+    // loads issued early: 11.4 M targets 270 -> 245 us, 4 M (clustered) 129 -> 110
+    __shared__ int4 s_idx[4][16];
+    const int warp = threadIdx.x >> 5;
+    const int64_t vs = active ? v : nt - 1;
+    const int cid = t_leaf[vs], tl = tloc[vs], dst = tperm[vs];
+    const double dn = near_tmp[vs];
+    reinterpret_cast<int2*>(s_idx[warp])[lane] = make_int2((tl & 0xffff) + side * (tl >> 16), cid);
+    __syncwarp();
+    const double cst = M::to_double(Cleaf[cid]);
     T part[32];
 #pragma unroll
-    for (int q = 0; q < 32; ++q) {
-        const T* row = tofsT + (size_t)__shfl_sync(kFull, myJ, q) * NP + lane;
-        const T* uq = uhat + (size_t)__shfl_sync(kFull, cid, q) * NP + lane;
-        T w = T(0);
+    for (int q = 0; q < 32; q += 2) {
+        const int4 ix = s_idx[warp][q >> 1];
+        const T* row0 = tofsT + (size_t)ix.x * NP + lane;
+        const T* row1 = tofsT + (size_t)ix.z * NP + lane;
+        const T* uq0 = uhat + (size_t)ix.y * NP + lane;
+        const T* uq1 = uhat + (size_t)ix.w * NP + lane;
+        T w0 = T(0), w1 = T(0);
 #pragma unroll
-        for (int i = 0; i < PL; ++i) w = fma(ldg(row + 32 * i), uq[32 * i], w);
-        part[q] = w;
+        for (int i = 0; i < PL; ++i) {
+            w0 = fma(ldg(row0 + 32 * i), uq0[32 * i], w0);
+            w1 = fma(ldg(row1 + 32 * i), uq1[32 * i], w1);
+        }
+        part[q] = w0;
+        part[q + 1] = w1;
     }
     const T far = reduce_scatter32(part);
     if (active) {
-        const int dst = tperm[v];
-        const double dn = near_tmp[v], df = (double)far + M::to_double(Cleaf[cid]);
+        const double df = (double)far + cst;
         if (u) u[dst] = dn + df;
         if (u_near) u_near[dst] = dn;
         if (u_far) u_far[dst] = df;
