@@ -36,7 +36,6 @@ WORKLOAD = "uniform_1m: 2^20 distinct sources + 2^20 distinct targets uniform in
 L2_FLUSH_BYTES = 256 << 20
 SM_COUNT = 152
 TC_MIN_LEVEL = 6            # library default: levels >= 6 of the fp32 path on the tensor cores
-TF32_PER_BF16 = 1.1 / 2.25  # nominal dense tf32 : bf16 tensor throughput
 
 
 def parse_args():
@@ -156,19 +155,19 @@ def m2l_flops(info, P, levels=None) -> int:
 
 def m2l_tc_roofline(info, P, tc_levels, phases, n_prof, peaks, peak_src):
     """Tensor-core M2L (+ fused L2L) of the step's tensor-core levels: useful flops per
-    level over the phase's device time per level (which also holds each level's TF32
+    level over the phase's device time per level (which also holds each level's
     split launch, so the fraction is a lower bound for the kernel itself)."""
     ms_level = phases["m2l_tc"][0] / n_prof / max(1, len(tc_levels))
     flops = m2l_flops(info, P, tc_levels) // max(1, len(tc_levels))
     achieved = flops / (ms_level * 1e-3) / 1e12
-    peak = float(peaks["bf16_tflops"]) * TF32_PER_BF16
+    peak = float(peaks["bf16_tflops"])
     return {"kernel": "m2l_tma_kernel", "bound": "tensor", "achieved": achieved, "peak": peak,
             "unit": "TFLOP/s", "frac": achieved / peak, "traffic": traffic_for("m2l_tma_kernel"),
-            "peak_basis": f"tf32 dense = measured bf16 burst {peaks['bf16_tflops']} x {TF32_PER_BF16:.3f} "
-                          f"(nominal 1.1 / 2.25 PFLOP/s) ({peak_src}); useful flops only, the 3xTF32 split "
-                          f"issues 3 MMAs per useful product",
+            "peak_basis": f"fp16 dense = measured bf16 burst {peaks['bf16_tflops']} "
+                          f"({peak_src}); useful flops only, the split into fp16 halves "
+                          f"forms 3 products per useful one",
             "levels": tc_levels, "units_per_launch": flops, "ms_per_launch": ms_level,
-            "time_basis": "tensor-core phase per level, TF32 split launch included"}
+            "time_basis": "tensor-core phase per level, split launch included"}
 
 
 # ---------------------------------------------------------------- reference arm (oracle)

@@ -56,8 +56,10 @@ extern "C" {
  *   to binary32, the per-target sum of near and far parts in binary64 (<= 1e-6). */
 #define LFMM_FP64 0   /* every step in binary64 (translations at p > 9: products of       */
                       /* 53-bit operands split exactly over fp16 tensor-core products)    */
-#define LFMM_MIXED 1  /* binary32 near and far field, compensated charge channel, TF32    */
-                      /* tensor-core M2L; binary64 final sum (relative error ~1e-7)       */
+#define LFMM_MIXED 1  /* binary32 near and far field, compensated charge channel,         */
+                      /* tensor-core M2L in three products of 11-bit halves (fp16 on      */
+                      /* uniform levels, TF32 on box lists); binary64 final sum           */
+                      /* (relative error ~1e-7)                                           */
 #define LFMM_DF 2     /* binary64 inputs and outputs, every step in float-float pairs     */
                       /* (~48 bits) on the FP32 pipes, translations at p > 9 in 53-bit    */
                       /* split operands on the tensor cores: binary64-level accuracy at a */
