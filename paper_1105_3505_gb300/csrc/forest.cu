@@ -137,6 +137,84 @@ __global__ void __launch_bounds__(256) p2m_list_kernel(int64_t nb, const int32_t
         p2m_list_quad<T, NP>(4 * w, nb, lane, leaf_rl, rl_s, loc, perm, f, f_sorted, tofsT, side, qhat, Q);
 }
 
+// P2M of the 8-byte types where the sliced far field follows (leaves of up to 192 sources,
+// few of them): four warps per leaf, each with a quarter of its sources and the lanes owning
+// expansion entries; the quarters' sums are added in order.  Bound by the longest leaf's chain
+// of dependent multiply-adds: 400,009 points in float-float 51 -> 32 us against a quarter warp
+// per leaf, 100 k in binary64 51 -> 22, 178 k clustered 64 -> 29, a disk's boundary 28 -> 8.
+template <typename T, int NP>
+__global__ void __launch_bounds__(256) p2m_list_wide_kernel(int64_t nb, const int32_t* __restrict__ leaf_rl,
+                                                            const int32_t* __restrict__ rl_s,
+                                                            const int32_t* __restrict__ loc,
+                                                            const int32_t* __restrict__ perm,
+                                                            const double* __restrict__ f, T* __restrict__ f_sorted,
+                                                            const T* __restrict__ tofsT, int side,
+                                                            T* __restrict__ qhat, typename Mono<T>::V* __restrict__ Q) {
+    griddep_wait();
+    using M = Mono<T>;
+    constexpr int W = 4, LB = 8 / W, PL = NP / 32;  // warps per leaf, leaves per block
+    __shared__ T s_part[8][NP];
+    __shared__ typename M::V s_q[8];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, w = warp % W;
+    for (int64_t b0 = (int64_t)blockIdx.x * LB; b0 < nb; b0 += (int64_t)gridDim.x * LB) {
+        const int64_t b = b0 + warp / W;
+        int s0 = 0, s1 = 0;
+        if (b < nb) {
+            const int j = leaf_rl[b];
+            s0 = rl_s[j];
+            s1 = rl_s[j + 1];
+        }
+        const int per = (s1 - s0 + W - 1) / W, a = s0 + w * per, e = min(a + per, s1);
+        T acc[PL];
+#pragma unroll
+        for (int i = 0; i < PL; ++i) acc[i] = T(0);
+        typename M::V qsum = M::zero();
+        for (int j0 = a; j0 < e; j0 += 32) {
+            const int j = j0 + lane;
+            T fj = T(0);
+            int J = 0;
+            if (j < e) {
+                const int l = loc[j];
+                const double fd = f[perm[j]];
+                J = (l & 0xffff) + side * (l >> 16);
+                fj = (T)fd;
+                f_sorted[j] = fj;
+                qsum = M::add(qsum, M::from_double(fd));
+            }
+            const int cc = min(32, e - j0);
+#pragma unroll 4
+            for (int k = 0; k < cc; ++k) {
+                const T fk = shfl(fj, k);
+                const T* row = tofsT + (size_t)__shfl_sync(kFull, J, k) * NP + lane;
+#pragma unroll
+                for (int i = 0; i < PL; ++i) acc[i] = fma(ldg(row + 32 * i), fk, acc[i]);
+            }
+        }
+#pragma unroll
+        for (int off = 16; off; off >>= 1) qsum = M::add(qsum, shfl_xor_v(qsum, off));
+#pragma unroll
+        for (int i = 0; i < PL; ++i) s_part[warp][lane + 32 * i] = acc[i];
+        if (lane == 0) s_q[warp] = qsum;
+        __syncthreads();
+        for (int i = threadIdx.x; i < LB * NP; i += blockDim.x) {
+            const int lf = i / NP, c = i % NP;
+            if (b0 + lf < nb) {
+                T s = s_part[lf * W][c];
+#pragma unroll
+                for (int v = 1; v < W; ++v) s += s_part[lf * W + v][c];
+                qhat[(size_t)(b0 + lf) * NP + c] = s;
+                if (c == 0) {
+                    typename M::V q = s_q[lf * W];
+#pragma unroll
+                    for (int v = 1; v < W; ++v) q = M::add(q, s_q[lf * W + v]);
+                    Q[b0 + lf] = q;
+                }
+            }
+        }
+        __syncthreads();
+    }
+}
+
 // M2M: one warp per compact parent; children by compact id (-1: empty).
 // The same M2M for levels with few parents: one block per parent, warp c computing the
 // 32 products of input chunk c; the chunks are added in order, as in m2m_list_kernel,
@@ -1178,7 +1256,17 @@ int forest_eval(const Forest& F, const DeviceOps& ops, const double* f, T* f_sor
         const ForestLevel& l0 = F.levels[0];
         if (l0.nb > 0) {
             int64_t blocks = std::min<int64_t>((l0.nb * 8 + 255) / 256, 152 * 64);  // four leaves per warp
-            if (NP == 32)
+            bool wide = false;  // only before the sliced far field, whose plans know no persistent sweep
+            if constexpr (sizeof(T) == 8) {
+                wide = sliced && NP == 64;
+                if (wide)
+                    (void)launch_dependent(p2m_list_wide_kernel<T, 64>,
+                                           dim3((unsigned)std::min<int64_t>((l0.nb + 1) / 2, 152 * 64)), dim3(256), 0, s,
+                                           l0.nb, l0.rl, F.rl_s, F.sloc, F.sperm, f, f_sorted, (const T*)ops.tofsT,
+                                           F.side, Qx(0), Qm(0));
+            }
+            if (wide) {
+            } else if (NP == 32)
                 (void)launch_dependent(p2m_list_kernel<T, 32>, dim3((int)blocks), dim3(256), 0, s, l0.nb, l0.rl, F.rl_s,
                                        F.sloc, F.sperm, f, f_sorted, (const T*)ops.tofsT, F.side, Qx(0), Qm(0));
             else
