@@ -17,14 +17,10 @@ namespace {
 
 constexpr int kThreads = 256;
 
-__device__ __forceinline__ int warp_min(int v) {
-    for (int o = 16; o; o >>= 1) v = min(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
-}
-__device__ __forceinline__ int warp_max(int v) {
-    for (int o = 16; o; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
-}
+// one reduction instruction each (a five-step shuffle chain before)
+__device__ __forceinline__ int warp_min(int v) { return __reduce_min_sync(0xffffffffu, v); }
+__device__ __forceinline__ int warp_max(int v) { return __reduce_max_sync(0xffffffffu, v); }
+__device__ __forceinline__ int warp_sum(int v) { return __reduce_add_sync(0xffffffffu, v); }
 
 // out4 = {min x, min y, max x, max y} over both point sets; out4 preset by the host.
 // Warp and block reductions first: one set of atomics per block.
@@ -198,22 +194,23 @@ __global__ void coarsen_kernel(const int4* __restrict__ fs, const int4* __restri
     m1 = warp_max(m1);
     m2 = warp_max(m2);
     m3 = warp_max(m3);
-    for (int o = 16; o; o >>= 1) {
-        nf += __shfl_xor_sync(0xffffffffu, nf, o);
-        nc += __shfl_xor_sync(0xffffffffu, nc, o);
-    }
+    nf = warp_sum(nf);
+    nc = warp_sum(nc);
     const int w = threadIdx.x >> 5;
     if ((threadIdx.x & 31) == 0) {
         red[0][w] = m0, red[1][w] = m1, red[2][w] = m2, red[3][w] = m3;
         red[4][w] = nf, red[5][w] = nc;
     }
     __syncthreads();
-    if (threadIdx.x < 6) {
-        int a = 0;
-        for (int i = 0; i < (int)(blockDim.x >> 5); ++i)
-            a = threadIdx.x < 4 ? max(a, red[threadIdx.x][i]) : a + red[threadIdx.x][i];
-        if (threadIdx.x < 4) atomicMax(max4 + threadIdx.x, a);
-        else atomicAdd(max4 + threadIdx.x, a);
+    // warp q < 6: word q
+    if (w < 6) {
+        const int l = threadIdx.x & 31;
+        const int v = l < (int)(blockDim.x >> 5) ? red[w][l] : 0;
+        const int a = w < 4 ? warp_max(v) : warp_sum(v);
+        if (l == 0) {
+            if (w < 4) atomicMax(max4 + w, a);
+            else atomicAdd(max4 + w, a);
+        }
     }
 }
 
