@@ -154,7 +154,9 @@ __global__ void __launch_bounds__(256) p2m_list_wide_kernel(int64_t nb, const in
     using M = Mono<T>;
     constexpr int W = 4, LB = 8 / W, PL = NP / 32;  // warps per leaf, leaves per block
     __shared__ T s_part[8][NP];
-    __shared__ typename M::V s_q[8];
+    // charges are added in binary64 whatever T: their sums' rounding, times the constants of the
+    // far field, was what a double layer's error came from (1.2e-12 -> 5.1e-13)
+    __shared__ double s_q[8];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, w = warp % W;
     for (int64_t b0 = (int64_t)blockIdx.x * LB; b0 < nb; b0 += (int64_t)gridDim.x * LB) {
         const int64_t b = b0 + warp / W;
@@ -168,7 +170,7 @@ __global__ void __launch_bounds__(256) p2m_list_wide_kernel(int64_t nb, const in
         T acc[PL];
 #pragma unroll
         for (int i = 0; i < PL; ++i) acc[i] = T(0);
-        typename M::V qsum = M::zero();
+        double qsum = 0.0;
         for (int j0 = a; j0 < e; j0 += 32) {
             const int j = j0 + lane;
             T fj = T(0);
@@ -179,7 +181,7 @@ __global__ void __launch_bounds__(256) p2m_list_wide_kernel(int64_t nb, const in
                 J = (l & 0xffff) + side * (l >> 16);
                 fj = (T)fd;
                 f_sorted[j] = fj;
-                qsum = M::add(qsum, M::from_double(fd));
+                qsum += fd;
             }
             const int cc = min(32, e - j0);
 #pragma unroll 4
@@ -191,7 +193,7 @@ __global__ void __launch_bounds__(256) p2m_list_wide_kernel(int64_t nb, const in
             }
         }
 #pragma unroll
-        for (int off = 16; off; off >>= 1) qsum = M::add(qsum, shfl_xor_v(qsum, off));
+        for (int off = 16; off; off >>= 1) qsum += __shfl_xor_sync(kFull, qsum, off);
 #pragma unroll
         for (int i = 0; i < PL; ++i) s_part[warp][lane + 32 * i] = acc[i];
         if (lane == 0) s_q[warp] = qsum;
@@ -204,10 +206,10 @@ __global__ void __launch_bounds__(256) p2m_list_wide_kernel(int64_t nb, const in
                 for (int v = 1; v < W; ++v) s += s_part[lf * W + v][c];
                 qhat[(size_t)(b0 + lf) * NP + c] = s;
                 if (c == 0) {
-                    typename M::V q = s_q[lf * W];
+                    double q = s_q[lf * W];
 #pragma unroll
-                    for (int v = 1; v < W; ++v) q = M::add(q, s_q[lf * W + v]);
-                    Q[b0 + lf] = q;
+                    for (int v = 1; v < W; ++v) q += s_q[lf * W + v];
+                    Q[b0 + lf] = M::from_double(q);
                 }
             }
         }
