@@ -783,26 +783,66 @@ struct LStripCfg {
 // many staged sources as fit (near8_caps).  Its warps share a strip's work evenly whatever
 // the number of targets: G = 1 .. 32 lanes take one target and every G-th source of its
 // three rows, and the lanes' sums are added by shuffles; strips of few targets among many
-// sources (clustered points, scattered targets) had kept one warp of six busy.  Float-float
-// pairs are added without renormalising each term (12 instead of 15 operations).
+// sources (clustered points, scattered targets) had kept one warp of six busy.
 template <typename T>
 struct NearCfg {
     static constexpr int THREADS = sizeof(T) == 8 ? 768 : 192;
     static constexpr int BLOCKS = sizeof(T) == 8 ? 1 : 6;
 };
 
-// acc += a b with the two-sum's and the product's errors collected in acc.lo
-__device__ __forceinline__ void near_add(DF& acc, DF a, DF b) {
-    const float p = a.hi * b.hi;
-    float e = fmaf(a.hi, b.hi, -p);
-    e = fmaf(a.hi, b.lo, e);
-    e = fmaf(a.lo, b.hi, e);
-    const float s = acc.hi + p, bb = s - acc.hi;
-    e += (acc.hi - (s - bb)) + (p - bb);
-    acc.hi = s;
-    acc.lo += e;
-}
-__device__ __forceinline__ void near_add(double& acc, double a, double b) { acc = fma(a, b, acc); }
+// A lane's near sum of the 8-byte types.
+//
+// Float-float: four products at a time are summed from zero, their rounding errors gathered in
+// the block's low word, and the block is added to the sum by the normalising df_add: 15
+// operations a term (20 with normalised multiply-adds inside the block, the same errors).
+// Gathering the errors of a whole row in one low word takes 12 but outgrows that word's
+// fraction: near sums of 60,000 points were off by 3.6e-15 with normalised terms, 6.4e-15 with
+// one low word a row, 2.6e-15 here (rows that begin with large terms: 90 times further off).
+// 400,009 points at leaf size 128: the call 484 us with one low word a row, 497 here.
+// The terms left over by the three rows' blocks, at most nine, make one more block.
+//
+// Binary64: one chain, shared by at least four lanes (2^LG_MIN): n / 4 roundings of a quarter
+// of the sum each, which is what blocks of four in one chain give.  (Two chains a lane cost
+// 15 % at 100,003 points and leaf size 128, 305 -> 350 us; two lanes 1.35 times the error.)
+template <typename T>
+struct NearSum;
+template <>
+struct NearSum<DF> {
+    static constexpr int LG_MIN = 0;
+    DF acc = DF(0), rest = DF(0);
+    // s += a b, s.lo left as it comes
+    static __device__ __forceinline__ void add(DF& s, DF a, DF b) {
+        const float p = a.hi * b.hi;
+        float e = fmaf(a.hi, b.hi, -p);
+        e = fmaf(a.hi, b.lo, e);
+        e = fmaf(a.lo, b.hi, e);
+        const DF t = two_sum(s.hi, p);
+        s.hi = t.hi;
+        s.lo += e + t.lo;
+    }
+    __device__ __forceinline__ void add4(const DF (&t)[4], const DF (&f)[4]) {
+        const float p = t[0].hi * f[0].hi;
+        float e = fmaf(t[0].hi, f[0].hi, -p);
+        e = fmaf(t[0].hi, f[0].lo, e);
+        DF b{p, fmaf(t[0].lo, f[0].hi, e)};
+#pragma unroll
+        for (int i = 1; i < 4; ++i) add(b, t[i], f[i]);
+        acc += b;
+    }
+    __device__ __forceinline__ void add1(DF t, DF f) { add(rest, t, f); }
+    __device__ __forceinline__ DF total() const { return acc + rest; }
+};
+template <>
+struct NearSum<double> {
+    static constexpr int LG_MIN = 2;
+    double acc = 0.0;
+    __device__ __forceinline__ void add4(const double (&t)[4], const double (&f)[4]) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc = fma(t[i], f[i], acc);
+    }
+    __device__ __forceinline__ void add1(double t, double f) { acc = fma(t, f, acc); }
+    __device__ __forceinline__ double total() const { return acc; }
+};
 
 template <typename T>
 __global__ void __launch_bounds__(NearCfg<T>::THREADS, NearCfg<T>::BLOCKS) p2p_list_kernel(
@@ -950,7 +990,8 @@ __global__ void __launch_bounds__(NearCfg<T>::THREADS, NearCfg<T>::BLOCKS) p2p_l
         };
         if constexpr (sizeof(T) == 8) {
             const int warps = blockDim.x >> 5;
-            int lg = 0;  // G = 2^lg lanes per target: at least two units of 32 / G targets per warp
+            // G = 2^lg lanes per target: at least two units of 32 / G targets per warp
+            int lg = NearSum<T>::LG_MIN;
             while (lg < 5 && (nt_strip << lg) < 64 * warps) ++lg;
             const int G = 1 << lg, sub = lane & (G - 1), per = 32 >> lg;
             const int units = (nt_strip + per - 1) / per;
@@ -960,7 +1001,7 @@ __global__ void __launch_bounds__(NearCfg<T>::THREADS, NearCfg<T>::BLOCKS) p2p_l
                 const int tl = s_tloc[active ? v : 0];
                 const int li = (tl >> 8) & 0xff, tx = tl & 0xff, ty = tl >> 16;
                 const T* tp = tab_c + (tx + tab_W * ty + li * side);
-                T acc = T(0);
+                NearSum<T> sum;
 #pragma unroll
                 for (int r = 0; r < 3; ++r) {
                     const SrcEntry<T>* src = s_src + s_ra[li][r];
@@ -968,17 +1009,14 @@ __global__ void __launch_bounds__(NearCfg<T>::THREADS, NearCfg<T>::BLOCKS) p2p_l
                     int j = sub;
                     for (; j + 3 * G < len; j += 4 * G) {
                         const SrcEntry<T> e0 = src[j], e1 = src[j + G], e2 = src[j + 2 * G], e3 = src[j + 3 * G];
-                        const T t0 = tp[-e0.off], t1 = tp[-e1.off], t2 = tp[-e2.off], t3 = tp[-e3.off];
-                        near_add(acc, t0, e0.f);
-                        near_add(acc, t1, e1.f);
-                        near_add(acc, t2, e2.f);
-                        near_add(acc, t3, e3.f);
+                        sum.add4({tp[-e0.off], tp[-e1.off], tp[-e2.off], tp[-e3.off]}, {e0.f, e1.f, e2.f, e3.f});
                     }
                     for (; j < len; j += G) {
                         const SrcEntry<T> e = src[j];
-                        near_add(acc, tp[-e.off], e.f);
+                        sum.add1(tp[-e.off], e.f);
                     }
                 }
+                T acc = sum.total();
                 for (int o = 1; o < G; o <<= 1) acc += shfl_xor_v(acc, o);
                 if (active && sub == 0) put(v, (double)acc + s_nc[li]);
             }
