@@ -95,7 +95,7 @@ struct lfmm_plan {
     double* un_tmp = nullptr;        // near field per target (caller order) from the concurrent near-field pass
     double* uf_tmp = nullptr;        // far field per target (caller order), before the final sum
     struct AuxStream* aux = nullptr;  // near-field pass runs here, beside the far-field sweeps
-    struct AuxStream* far_aux = nullptr;  // pruned / forest: the far field, beside the near field
+    std::vector<struct AuxStream*> side_aux;  // pruned / forest: near and far field beside each other
     // uniform storage: the targets are bucketed on `aux` while the plan's creation and the
     // evaluation's upward sweep go on; whatever reads them waits for this event
     cudaEvent_t tgt_ready = nullptr;
@@ -128,7 +128,7 @@ struct AuxStream {
     cudaStream_t s = nullptr;
     cudaEvent_t fork = nullptr, join = nullptr;
     int device = -1;
-    bool high = false;  // one step above the default priority
+    int priority = 0;
 };
 
 namespace {
@@ -136,11 +136,11 @@ namespace {
 std::mutex g_aux_mu;
 std::vector<AuxStream*> g_aux_free;
 
-AuxStream* acquire_aux(int device, bool high = false) {
+AuxStream* acquire_aux(int device, int priority = 0) {
     {
         std::lock_guard<std::mutex> g(g_aux_mu);
         for (size_t i = 0; i < g_aux_free.size(); ++i)
-            if (g_aux_free[i]->device == device && g_aux_free[i]->high == high) {
+            if (g_aux_free[i]->device == device && g_aux_free[i]->priority == priority) {
                 AuxStream* a = g_aux_free[i];
                 g_aux_free.erase(g_aux_free.begin() + i);
                 return a;
@@ -149,8 +149,8 @@ AuxStream* acquire_aux(int device, bool high = false) {
     AuxStream* a = new (std::nothrow) AuxStream();
     if (!a) return nullptr;
     a->device = device;
-    a->high = high;
-    if (cudaStreamCreateWithPriority(&a->s, cudaStreamNonBlocking, high ? -1 : 0) != cudaSuccess ||
+    a->priority = priority;
+    if (cudaStreamCreateWithPriority(&a->s, cudaStreamNonBlocking, priority) != cudaSuccess ||
         cudaEventCreateWithFlags(&a->fork, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&a->join, cudaEventDisableTiming) != cudaSuccess) {
         cudaGetLastError();
@@ -167,6 +167,26 @@ void release_aux(AuxStream* a) {
     cudaStreamSynchronize(a->s);
     std::lock_guard<std::mutex> g(g_aux_mu);
     g_aux_free.push_back(a);
+}
+
+// Priorities of the two streams of a pruned evaluation called on `s`: the far field's launches
+// are one step more urgent than the near field's, and both stay within a step of the caller's
+// stream, so that the order of its requests among those of other streams is kept.  The side
+// stream carries the far field one step above the caller's priority, or, where the caller has
+// the most urgent one already, the near field one step below it.
+struct SidePriority {
+    int priority;
+    bool near;
+};
+SidePriority side_priority(cudaStream_t s) {
+    int least = 0, greatest = 0, own = 0;
+    if (cudaDeviceGetStreamPriorityRange(&least, &greatest) != cudaSuccess ||
+        cudaStreamGetPriority(s, &own) != cudaSuccess) {
+        cudaGetLastError();
+        return {0, false};
+    }
+    if (own > greatest) return {own - 1, false};
+    return {std::min(least, own + 1), true};
 }
 
 // Work on `s` that reads the bucketed targets waits for their bucketing (a no-op once it
@@ -777,12 +797,17 @@ int far_sweeps(lfmm_plan* p, const FarBufs& b, cudaStream_t s, Hook before_fine)
 template <typename T>
 int eval_impl(lfmm_plan* p, const double* f, double* u, double* un, double* uf, cudaStream_t s) {
     if (p->forest) {
-        // the far field on a second stream beside the near field (launches of few blocks, so of
-        // a higher priority), joined before L2P
+        // near field and far field beside each other, the far field (launches of few blocks) at
+        // the higher priority, joined before L2P
         SideStream side{};
-        const bool beside = p->forest->kmax >= 0 && !(p->opts.flags & LFMM_FLAG_SERIAL);
-        if (beside && !p->far_aux) p->far_aux = acquire_aux(p->device, true);
-        if (beside && p->far_aux) side = SideStream{p->far_aux->s, p->far_aux->fork, p->far_aux->join};
+        if (p->forest->kmax >= 0 && !(p->opts.flags & LFMM_FLAG_SERIAL)) {
+            const SidePriority sp = side_priority(s);
+            AuxStream* a = nullptr;
+            for (AuxStream* have : p->side_aux)
+                if (have->priority == sp.priority) a = have;
+            if (!a && (a = acquire_aux(p->device, sp.priority))) p->side_aux.push_back(a);
+            if (a) side = SideStream{a->s, a->fork, a->join, sp.near};
+        }
         const int st = forest_eval<T>(*p->forest, *p->ops, f, (T*)p->f_sorted, (T*)p->qhat, (T*)p->uhat, p->Qbox,
                                       p->Cbox, u, un, uf, p->num_sms, s, p->status,
                                       (p->opts.flags & LFMM_FLAG_PERSISTENT) != 0, side.s ? &side : nullptr);
@@ -1090,7 +1115,7 @@ int lfmm_plan_create(lfmm_plan** plan, const int32_t* src_xy, int64_t n_src, con
         free_plan_buffers(p);
         if (p->tgt_ready) cudaEventDestroy(p->tgt_ready);
         release_aux(p->aux);
-        release_aux(p->far_aux);
+        for (AuxStream* a : p->side_aux) release_aux(a);
         delete p;
         return st;
     }
@@ -1118,7 +1143,7 @@ int lfmm_plan_destroy(lfmm_plan* plan) {
     if (plan->graph) cudaGraphExecDestroy(plan->graph);
     if (plan->cap_stream) cudaStreamDestroy(plan->cap_stream);
     release_aux(plan->aux);
-    release_aux(plan->far_aux);
+    for (AuxStream* a : plan->side_aux) release_aux(a);
     delete plan;
     if (e != cudaSuccess) return fail(LFMM_ECUDA, std::string("plan destroy: ") + cudaGetErrorString(e));
     return LFMM_OK;

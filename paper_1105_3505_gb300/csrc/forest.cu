@@ -1316,17 +1316,18 @@ int forest_eval(const Forest& F, const DeviceOps& ops, const double* f, T* f_sor
             pt.add_launches(1);
         }
     }
-    // the near field needs the sorted charges and the leaf charges only: it runs on the
-    // caller's stream, the rest of the far field on the side stream
+    // the near field needs the sorted charges and the leaf charges only: it runs beside the
+    // rest of the far field, one of them on the side stream
     const cudaStream_t s_main = s;
+    cudaStream_t s_near = s;
     const bool fork = far && side != nullptr && status == nullptr;  // not beside a persistent sweep
     if (fork) {
         LFMM_CUDA_TRY(cudaEventRecord(side->fork, s));
         LFMM_CUDA_TRY(cudaStreamWaitEvent(side->s, side->fork, 0));
-        s = side->s;
+        (side->near ? s_near : s) = side->s;
     }
     if (far) {
-        const int st = launch_list_p2p<T>(F, ops, f_sorted, Qm(0), nullptr, nullptr, nullptr, num_sms, s_main, true);
+        const int st = launch_list_p2p<T>(F, ops, f_sorted, Qm(0), nullptr, nullptr, nullptr, num_sms, s_near, true);
         if (st) return st;
     }
     if constexpr (sizeof(T) == 8) {
@@ -1500,7 +1501,7 @@ int forest_eval(const Forest& F, const DeviceOps& ops, const double* f, T* f_sor
     }
     if (!far) return launch_list_p2p<T>(F, ops, f_sorted, Qm(0), u, un, uf, num_sms, s, false);
     if (fork) {
-        LFMM_CUDA_TRY(cudaEventRecord(side->join, s));
+        LFMM_CUDA_TRY(cudaEventRecord(side->join, side->s));
         LFMM_CUDA_TRY(cudaStreamWaitEvent(s_main, side->join, 0));
     }
     return launch_list_l2p<T>(F, ops, (const T*)Ux(0), Cm(0), u, un, uf, s_main);

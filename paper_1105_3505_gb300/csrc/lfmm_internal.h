@@ -346,11 +346,13 @@ int forest_build(Forest& F, const int32_t* src, const int64_t* soff_h, int64_t n
 // recorded there); persistent: run each sweep as one persistent cooperative launch
 // (LFMM_FLAG_PERSISTENT), else one launch per level, the list M2L of levels with at
 // least kTcListMinBoxes boxes on the tensor cores when F.tc_list is set.
-// side: a second stream (of higher priority) with its fork and join events, for the far
-// field beside the near field; null: one after the other on s.
+// side: a second stream with its fork and join events, for the far field beside the near
+// field (near: it carries the near field, else the far field; the far field's stream is the
+// more urgent of the two where there is a difference); null: one after the other on s.
 struct SideStream {
     cudaStream_t s;
     cudaEvent_t fork, join;
+    bool near;
 };
 template <typename T>
 int forest_eval(const Forest& F, const DeviceOps& ops, const double* f, T* f_sorted, T* qhat, T* uhat, void* Qbox,
