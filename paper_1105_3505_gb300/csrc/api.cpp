@@ -337,7 +337,21 @@ int forest_workspaces(lfmm_plan* p, cudaStream_t s) {
     std::string err;
     ModelOps* mo = get_model_ops(F.side, p->P, p->opts.proxies_per_edge, n_levels, &err);
     if (!mo) return fail(LFMM_EINTERNAL, err);
-    p->ops = get_device_ops(mo, p->opts.precision, p->NP, n_levels, s, &err);
+    // tensor-core list M2L of the large levels (mixed path; opts.tc_min_level beyond every tree
+    // level keeps them on the CUDA cores): TF32 hi / lo rows
+    F.tc_list = p->opts.precision == LFMM_MIXED && p->opts.tc_min_level <= kMaxTreeLevelForTc;
+    int64_t split_floats = 0;
+    const int nk = (int)F.levels.size();
+    OpsImages images;
+    for (int k = 0; k < nk && F.kmax >= 0 && F.tc_list; ++k)
+        if (F.levels[k].nb >= kTcListMinBoxes) {
+            split_floats = std::max(split_floats, m2l_tc_list_split_floats(
+                                                      F.levels[k].nb, k + 1 < nk ? F.levels[k + 1].nb : 0, p->NP));
+            images.rows = k + 1;
+        }
+    images.sliced =
+        F.kmax >= 0 && nk <= kSgMaxLevels && sg_applies(p->opts.precision, p->NP, p->opts.tc_min_level);
+    p->ops = get_device_ops(mo, p->opts.precision, p->NP, n_levels, &images, s, &err);
     if (!p->ops) return fail(LFMM_ECUDA, err);
     const size_t esz = p->opts.precision == LFMM_MIXED ? sizeof(float) : sizeof(double);
     if ((st = palloc(p, &p->f_sorted, (size_t)p->ns * esz, s))) return st;
@@ -355,18 +369,9 @@ int forest_workspaces(lfmm_plan* p, cudaStream_t s) {
         const int64_t sb = forest_m2l_split_bytes(F, p->NP, esz, p->num_sms, F.m2l_split);
         if (sb > 0 && (st = palloc(p, &F.m2l_part, (size_t)sb, s))) return st;
     }
-    // tensor-core list M2L of the large levels (mixed path; opts.tc_min_level
-    // beyond every tree level keeps them on the CUDA cores): TF32 hi / lo rows
-    F.tc_list = p->opts.precision == LFMM_MIXED && p->opts.tc_min_level <= kMaxTreeLevelForTc;
-    if (F.tc_list) {
-        int64_t need = 0;
-        const int nk = (int)F.levels.size();
-        for (int k = 0; k < nk && F.kmax >= 0; ++k)
-            if (F.levels[k].nb >= kTcListMinBoxes)
-                need = std::max(need, m2l_tc_list_split_floats(F.levels[k].nb, k + 1 < nk ? F.levels[k + 1].nb : 0,
-                                                               p->NP));
-        void* b = nullptr;
-        if (need > 0 && (st = palloc(p, &b, (size_t)need * sizeof(float), s))) return st;
+    if (split_floats > 0) {
+        void* b;
+        if ((st = palloc(p, &b, (size_t)split_floats * sizeof(float), s))) return st;
         F.tc_split = (float*)b;
     }
     if (F.kmax >= 0) {  // near field before the far part is added, and every target's leaf for that
@@ -377,8 +382,7 @@ int forest_workspaces(lfmm_plan* p, cudaStream_t s) {
         LFMM_CUDA_TRY(launch_target_leaves(F, F.t_leaf, s));
     }
     // sliced far field of the binary64-accurate paths (split_tc.cu)
-    if (F.kmax >= 0 && (int)F.levels.size() <= kSgMaxLevels &&
-        sg_applies(p->opts.precision, p->NP, p->opts.tc_min_level)) {
+    if (images.sliced) {
         const int64_t need = sg_work_bytes(forest_sg_tree(F), p->opts.precision, p->num_sms);
         if ((st = palloc(p, &F.sg_work, (size_t)need, s))) return st;
     }
@@ -626,7 +630,12 @@ int plan_build(lfmm_plan* p, const int32_t* src_xy, const int32_t* tgt_xy, cudaS
     std::string err;
     ModelOps* mo = get_model_ops(p->side, p->P, p->opts.proxies_per_edge, n_levels, &err);
     if (!mo) return fail(LFMM_EINTERNAL, err);
-    p->ops = get_device_ops(mo, p->opts.precision, p->NP, n_levels, s, &err);
+    const int tc_min = p->opts.tc_min_level == 0 ? kDefaultTcMinLevel : p->opts.tc_min_level;
+    const bool tc = p->opts.precision == LFMM_MIXED && p->L >= tc_min;
+    OpsImages images;
+    if (tc) images.halves = std::max(0, p->L + 1 - std::max(2, tc_min));  // levels tc_min .. L
+    images.sliced = sg_applies_uniform(p->opts.precision, p->NP, p->L, p->opts.tc_min_level);
+    p->ops = get_device_ops(mo, p->opts.precision, p->NP, n_levels, &images, s, &err);
     if (!p->ops) return fail(LFMM_ECUDA, err);
 
     // ---- workspaces: sorted charges, expansions of levels min(2,L)..L
@@ -639,7 +648,7 @@ int plan_build(lfmm_plan* p, const int32_t* src_xy, const int32_t* tgt_xy, cudaS
         boxes += (int64_t)1 << (2 * l);
     }
     p->n_boxes = boxes;
-    if (p->opts.precision == LFMM_MIXED && p->L >= (p->opts.tc_min_level == 0 ? kDefaultTcMinLevel : p->opts.tc_min_level)) {
+    if (tc) {
         // largest tensor-core level: fp16 hi/lo of its q_hat and of its parent's u_hat
         if ((st = palloc(p, &p->tc_split, (size_t)tma_split_floats(p->L, p->NP) * sizeof(float), s))) return st;
     }
@@ -647,7 +656,7 @@ int plan_build(lfmm_plan* p, const int32_t* src_xy, const int32_t* tgt_xy, cudaS
     if ((st = palloc(p, &p->uhat, (size_t)boxes * p->NP * esz, s))) return st;
     if ((st = palloc(p, &p->Qbox, (size_t)boxes * 8, s))) return st;
     if ((st = palloc(p, &p->Cbox, (size_t)boxes * 8, s))) return st;
-    if (sg_applies_uniform(p->opts.precision, p->NP, p->L, p->opts.tc_min_level) &&
+    if (images.sliced &&
         (st = palloc(p, &p->sg_work,
                      (size_t)sg_work_bytes(sg_uniform_tree(p->L, p->opts.m2l_split), p->opts.precision, p->num_sms), s)))
         return st;

@@ -1869,7 +1869,7 @@ int64_t m2l_fused_split_bytes_shape(int NP, bool has_tc, int L, int tc_min_level
 
 template <typename T>
 int64_t m2l_fused_split_bytes(const DeviceOps& ops, int L, int tc_min_level, int num_sms, int nvec, int split) {
-    const bool has_tc = !ops.tc.empty() && ops.tc[0] != nullptr;  // all levels or none
+    const bool has_tc = ops.precision == LFMM_MIXED;
     return m2l_fused_split_bytes_shape<T>(ops.NP, has_tc, L, tc_min_level, num_sms, nvec, split);
 }
 

@@ -171,26 +171,38 @@ void tifo_matrix(const LevelOps& lv, int o, std::vector<double>& out);
 //   mono [2][40]      c_o = phi(o*side) split as (hi, lo) of the element type
 // Leaf: tofsT [s^2][NP] tofsT[J][p] = T_ofs[p][J];
 //   P2P table [(2H+1)][W] of phi(dx,dy) - phi0, then phi0 = phi(s, 0) as (hi, lo).
+// Images of the operators for the tensor cores, built for the plans that use them and as far
+// as they do: TF32 hi / lo (box lists, mixed) and fp16 hi / lo (uniform levels, mixed) of the
+// first levels, slices (binary64-accurate) of all.  Both kinds of tiles of every level had
+// lengthened the first plan of a configuration from 13.4 ms (TF32 alone) to 15.9 at 2^20
+// points, mixed p = 8, and from 45.7 to 55 at p = 16; as used: 13.1 and 44.2, and 1 to 3.4 ms
+// once in a later plan that needs more of them.
+struct OpsImages {
+    int rows = 0, halves = 0;  // levels k = 0 .. n - 1
+    bool sliced = false;
+};
 struct DeviceOps {
     int NP = 0, precision = 0, n_levels = 0, leaf_side = 0;
     int tab_H = 0, tab_W = 0;             // P2P table half width and row width
-    void* base = nullptr;                 // one allocation
+    void* base = nullptr;                 // one allocation; the operators are its first bytes
     size_t bytes = 0;
     void* tofsT = nullptr;
     void* p2p_table = nullptr;
     std::vector<void*> m2m, l2l, tifo;    // per level k
     std::vector<void*> mono;              // per level k: deflation constants (hi[40], lo[40])
-    std::vector<void*> tc;                // per level k (mixed, NP = 32): tensor-core B tiles,
+    OpsImages have;                       // what is there beside them
+    std::vector<void*> tc;                // TF32 tiles per level k: tensor-core B tiles,
                                           // [40 offsets + 4 L2L classes][hi, lo][32 x 32 fp32]
-    std::vector<void*> tch, tch_scale;    // per level k (mixed): the same operators in fp16 hi, lo, and
+    std::vector<void*> tch, tch_scale;    // fp16 tiles per level k: the same operators in fp16 hi, lo, and
                                           // the float that undoes each one's power-of-two scaling
-    void* sg_base = nullptr;              // binary64-accurate paths, NP = 64: sliced operators
-    std::vector<uint8_t*> sg_tiles;       // per level k (split_tc.h: kSgOps tiles), and
+    std::vector<uint8_t*> sg_tiles;       // sliced operators per level k (split_tc.h: kSgOps tiles), and
     std::vector<int32_t*> sg_e;           // their exponents
-    std::vector<void*> retired;           // earlier, smaller uploads (kept alive)
+    std::vector<void*> retired;           // earlier, smaller uploads, and images added later (kept alive)
 };
 
-const DeviceOps* get_device_ops(ModelOps* mo, int precision, int NP, int n_levels,
+// *want: in, what the plan uses; out, the same without the slices if the device has no
+// memory for them.
+const DeviceOps* get_device_ops(ModelOps* mo, int precision, int NP, int n_levels, OpsImages* want,
                                 cudaStream_t stream, std::string* err);
 
 // ---------------------------------------------------------------- tracing
@@ -474,8 +486,7 @@ constexpr int kDefaultTcMinLevel = 6;
 // Whether level `level` (k levels above the leaves) runs M2L + L2L on the tensor cores:
 // fp32 arithmetic, P <= 32, tiles present, level >= tc_min_level.
 inline bool m2l_uses_tc(const DeviceOps& ops, int k, int level, int tc_min_level, bool fp32) {
-    return fp32 && (ops.NP == 32 || ops.NP == 64) && ops.tc.size() > (size_t)k && ops.tc[k] != nullptr &&
-           level >= tc_min_level;
+    return fp32 && (ops.NP == 32 || ops.NP == 64) && k < ops.n_levels && level >= tc_min_level;
 }
 // M2L + L2L of one level; mixed-path levels >= tc_min_level (P <= 32) run on the
 // tensor cores, which report a timed-out wait in *status.

@@ -1016,7 +1016,7 @@ cudaError_t launch_m2l_tma(const DeviceOps& ops, int k, int level, const float* 
                            int* status, int num_sms, cudaStream_t s, int nvec, int64_t vq, int64_t vQ, int tile,
                            int stages) {
     const int NP = ops.NP;
-    if (NP != 32 && NP != 64) return cudaErrorInvalidValue;
+    if ((NP != 32 && NP != 64) || !ops.tch[k]) return cudaErrorInvalidValue;
     const int lg = level - 1;
     const int np = 1 << lg;
     const bool l2l = u_parent != nullptr;

@@ -30,6 +30,7 @@
 #include <map>
 #include <numeric>
 #include <tuple>
+#include <type_traits>
 
 #include "lfmm_internal.h"
 #include "split_tc.h"
@@ -286,112 +287,113 @@ float tf32_rna(float x) {
 }
 
 // Tensor-core B operand of one operator for K-block h (k in [32h, 32h + 32)): the
-// operator's value(n, k) (n = output p < NP) split into TF32 hi and lo and stacked as one
+// operator's v(n, k) (n = output p < NP) split into TF32 hi and lo and stacked as one
 // K-major matrix of 2 NP rows (hi rows, then lo rows) x 32 K in fp32, laid out as the
 // 128-byte-swizzled shared-memory image (row r at 128 r bytes, 16-byte chunk c of the
 // row at chunk c ^ (r mod 8)).  NP / 32 such blocks per operator, block h at
 // dst + h * 64 NP floats.
-template <typename F>
-void write_tc_tile(float* dst, int NP, int rows, int cols, F value) {
+void write_tc_tile(float* dst, int NP, const float (*v)[64]) {
     for (int h = 0; h < NP / 32; ++h) {
         float* blk = dst + (size_t)h * 64 * NP;
         for (int n = 0; n < NP; ++n)
-            for (int k = 0; k < 32; ++k) {
-                const int kg = 32 * h + k;
-                const float v = (n < rows && kg < cols) ? (float)value(n, kg) : 0.0f;
-                const float hv = tf32_rna(v);
-                const float lv = tf32_rna(v - hv);
-                const size_t sw = ((size_t)(((k >> 2) ^ (n & 7)) << 2)) + (k & 3);  // (NP + n) & 7 == n & 7
-                blk[(size_t)n * 32 + sw] = hv;
-                blk[(size_t)(NP + n) * 32 + sw] = lv;
+            for (int c = 0; c < 8; ++c) {  // ((NP + n) & 7 == n & 7)
+                float* at = blk + (size_t)n * 32 + ((c ^ (n & 7)) << 2);
+                for (int k = 0; k < 4; ++k) {
+                    const float x = v[n][32 * h + 4 * c + k];
+                    const float hv = tf32_rna(x);
+                    at[k] = hv;
+                    at[k + (size_t)NP * 32] = tf32_rna(x - hv);
+                }
             }
     }
 }
 
-// binary16 round to nearest even of a value within the normal range of binary32 (|x| < 2^15
-// here; below 2^-14 on the subnormal grid of spacing 2^-24).
-uint16_t half_rne(float x) {
+uint32_t float_bits(float x) {
     uint32_t u;
     std::memcpy(&u, &x, 4);
-    const uint16_t sign = (uint16_t)((u >> 16) & 0x8000u);
+    return u;
+}
+float bits_float(uint32_t u) {
+    float x;
+    std::memcpy(&x, &u, 4);
+    return x;
+}
+// binary16 round to nearest even of |x| < 2^15; below 2^-14 the grid has a spacing of 2^-24,
+// as binary32 has from 0.5 on, so adding 0.5 rounds to it.
+uint32_t half_rne(float x) {
+    const uint32_t sign = (float_bits(x) >> 16) & 0x8000u;
     const float a = std::fabs(x);
-    if (a < 6.103515625e-05f) return (uint16_t)(sign | (uint16_t)std::nearbyint((double)a * 16777216.0));  // 2^24 a
-    u = (u & 0x7fffffffu) - ((127u - 15u) << 23);
-    u += 0xfffu + ((u >> 13) & 1u);
-    return (uint16_t)(sign | (u >> 13));
+    const uint32_t tiny = float_bits(a + 0.5f) - 0x3f000000u;
+    uint32_t u = float_bits(a) - ((127u - 15u) << 23);
+    u = (u + 0xfffu + ((u >> 13) & 1u)) >> 13;
+    return sign | (a < 6.103515625e-05f ? tiny : u);
 }
-float half_value(uint16_t h) {
-    const int e = (h >> 10) & 31, m = h & 1023;
-    const float v = e ? std::ldexp((float)(1024 + m), e - 25) : std::ldexp((float)m, -24);
-    return h & 0x8000 ? -v : v;
-}
+// the finite binary16 h (its exponent field moved to binary32's, subnormals included)
+float half_value(uint32_t h) { return bits_float((h & 0x7fffu) << 13 | (h & 0x8000u) << 16) * 0x1p112f; }
 
-// The same operators for the fp16 tensor-core M2L: value(n, k) scaled by a power of two so
+// The same operators for the fp16 tensor-core M2L: x(n, k) scaled by a power of two so
 // that the largest magnitude lies in [2^14, 2^15), split into fp16 hi and lo and stacked as
 // one K-major matrix of 2 NP rows (hi rows, then lo rows) of 128 bytes (64 halves; NP = 32
 // uses the first 32), 128-byte swizzled.  Returns the factor that undoes the scaling.
-template <typename F>
-float write_half_tile(uint16_t* dst, int NP, int rows, int cols, F value) {
-    float mx = 0.0f;
-    for (int n = 0; n < rows; ++n)
-        for (int k = 0; k < cols; ++k) mx = std::max(mx, std::fabs((float)value(n, k)));
-    const int sh = mx > 0.0f ? std::min(14 - std::ilogb(mx), 100) : 0;
-    for (int n = 0; n < rows; ++n)
-        for (int k = 0; k < cols; ++k) {
-            const float v = std::ldexp((float)value(n, k), sh);
-            const uint16_t h = half_rne(v), l = half_rne(v - half_value(h));
-            const size_t at = (size_t)n * 64 + (((k >> 3) ^ (n & 7)) << 3) + (k & 7);
-            dst[at] = h;
-            dst[at + (size_t)NP * 64] = l;  // row NP + n: the same swizzle
+float write_half_tile(uint16_t* dst, int NP, const float (*x)[64]) {
+    uint32_t top = 0;  // the largest magnitude's bits
+    for (int n = 0; n < NP; ++n)
+        for (int k = 0; k < NP; ++k) top = std::max(top, float_bits(x[n][k]) & 0x7fffffffu);
+    const int sh = top ? std::min(14 - std::ilogb(bits_float(top)), 100) : 0;
+    const float up = std::ldexp(1.0f, sh);  // (products with it round as ldexp rounds)
+    for (int n = 0; n < NP; ++n) {
+        uint32_t h[64], l[64];  // (words, and a loop of its own, so that it vectorises)
+        for (int k = 0; k < NP; ++k) {
+            const float v = x[n][k] * up;
+            h[k] = half_rne(v);
+            l[k] = half_rne(v - half_value(h[k]));
         }
+        for (int k = 0; k < NP; ++k) {
+            uint16_t* at = dst + (size_t)n * 64 + (((k >> 3) ^ (n & 7)) << 3) + (k & 7);
+            at[0] = (uint16_t)h[k];
+            at[(size_t)NP * 64] = (uint16_t)l[k];  // row NP + n: the same swizzle
+        }
+    }
     return std::ldexp(1.0f, -sh);
 }
 
+// Element offsets of the operators in their image.
+struct ImageOffsets {
+    size_t tofs = 0, tab = 0;
+    std::vector<size_t> m2m, l2l, tifo, mono;  // per level
+};
+
 template <typename T>
-void fill_device_image(const ModelOps& mo, int NP, int n_levels, int H, int W,
-                       std::vector<T>& img, size_t& off_tofs, size_t& off_tab,
-                       std::vector<size_t>& off_m2m, std::vector<size_t>& off_l2l,
-                       std::vector<size_t>& off_tifo, std::vector<size_t>& off_mono,
-                       std::vector<size_t>& off_tc, std::vector<size_t>& off_tch) {
+std::vector<T> operator_image(const ModelOps& mo, int NP, int n_levels, int H, int W, ImageOffsets& off) {
     const int s = mo.leaf_side;
     auto align = [](size_t v) { return (v + 31) & ~(size_t)31; };  // 128/256-byte aligned blocks
     size_t n = 0;
-    off_tofs = n;
+    off.tofs = n;
     n = align(n + (size_t)s * s * NP);
-    off_tab = n;
+    off.tab = n;
     n = align(n + (size_t)(2 * H + 1) * W + 2);
-    off_m2m.assign(n_levels, 0);
-    off_l2l.assign(n_levels, 0);
-    off_tifo.assign(n_levels, 0);
-    off_mono.assign(n_levels, 0);
-    off_tc.assign(n_levels, 0);
-    off_tch.assign(n_levels, 0);
-    const bool tc = sizeof(T) == 4 && (NP == 32 || NP == 64);
+    off.m2m.assign(n_levels, 0);
+    off.l2l.assign(n_levels, 0);
+    off.tifo.assign(n_levels, 0);
+    off.mono.assign(n_levels, 0);
     for (int k = 0; k < n_levels; ++k) {
-        if (tc) {
-            n = (n + 255) & ~(size_t)255;  // 1 KB aligned tiles
-            off_tc[k] = n;
-            n += (size_t)(kNumOffsets + 4) * 2 * NP * NP;  // per operator NP / 32 blocks of 64 NP floats
-            off_tch[k] = n;  // fp16 tiles (2 NP rows of 128 bytes), then their scales
-            n = align(n + (size_t)(kNumOffsets + 4) * (2 * NP * 32 + 1));
-        }
-        off_mono[k] = n;
+        off.mono[k] = n;
         n = align(n + (size_t)2 * kNumOffsets);
         if (k >= 1) {
-            off_m2m[k] = n;
+            off.m2m[k] = n;
             n = align(n + (size_t)4 * NP * NP);
-            off_l2l[k] = n;
+            off.l2l[k] = n;
             n = align(n + (size_t)4 * NP * NP);
         }
-        off_tifo[k] = n;
+        off.tifo[k] = n;
         n = align(n + (size_t)kNumOffsets * NP * NP);
     }
-    img.assign(n, T(0));
+    std::vector<T> img(n, T(0));
     // leaf T_ofs, transposed: tofsT[J][p]
     const LevelOps& leaf = mo.levels[0];
     for (int p = 0; p < leaf.P; ++p)
         for (int J = 0; J < s * s; ++J)
-            img[off_tofs + (size_t)J * NP + p] = (T)mo.tofs[(size_t)p * s * s + J];
+            img[off.tofs + (size_t)J * NP + p] = (T)mo.tofs[(size_t)p * s * s + J];
     // P2P table: entry (dx, dy), |dx|,|dy| <= H, at (dy + H) * W + (dx + H), deflated by
     // phi0 = phi(s, 0) (about the middle of the near-field range); phi0 times the charge of
     // the 3x3 leaf block is added back in the compensated channel.  phi0 as (hi, lo) after
@@ -399,9 +401,9 @@ void fill_device_image(const ModelOps& mo, int NP, int n_levels, int H, int W,
     const double phi0 = phi_host(s, 0);
     for (int dy = -H; dy <= H; ++dy)
         for (int dx = -H; dx <= H; ++dx)
-            img[off_tab + (size_t)(dy + H) * W + (dx + H)] = (T)(phi_host(dx, dy) - phi0);
+            img[off.tab + (size_t)(dy + H) * W + (dx + H)] = (T)(phi_host(dx, dy) - phi0);
     {
-        const size_t e = off_tab + (size_t)(2 * H + 1) * W;
+        const size_t e = off.tab + (size_t)(2 * H + 1) * W;
         const T hi = (T)phi0;
         img[e] = hi;
         img[e + 1] = (T)(phi0 - (double)hi);
@@ -416,8 +418,8 @@ void fill_device_image(const ModelOps& mo, int NP, int n_levels, int H, int W,
                 for (int q = 0; q < ch.P; ++q)
                     for (int p = 0; p < lv.P; ++p) {
                         const double v = lv.S[(size_t)p * cols + c * ch.P + q];
-                        img[off_m2m[k] + (size_t)(c * NP + q) * NP + p] = (T)v;   // [c*NP+q][p]
-                        img[off_l2l[k] + ((size_t)c * NP + p) * NP + q] = (T)v;   // [c][p_par][q_child]
+                        img[off.m2m[k] + (size_t)(c * NP + q) * NP + p] = (T)v;   // [c*NP+q][p]
+                        img[off.l2l[k] + ((size_t)c * NP + p) * NP + q] = (T)v;   // [c][p_par][q_child]
                     }
         }
         // Deflated M2L: T_ifo minus its centre-to-centre value c_o = phi(o * side).  The
@@ -429,43 +431,132 @@ void fill_device_image(const ModelOps& mo, int NP, int n_levels, int H, int W,
             tifo_matrix(lv, o, t);
             const double c = phi_host((int64_t)ot.ox[o] * lv.side, (int64_t)ot.oy[o] * lv.side);
             const T hi = (T)c;
-            img[off_mono[k] + o] = hi;
-            img[off_mono[k] + kNumOffsets + o] = (T)(c - (double)hi);
-            for (int p = 0; p < lv.P; ++p)
-                for (int q = 0; q < lv.P; ++q)
-                    img[off_tifo[k] + ((size_t)o * NP + q) * NP + p] = (T)(t[(size_t)p * lv.P + q] - c);
-            if (tc) {
-                float* base = reinterpret_cast<float*>(img.data() + off_tc[k]) + (size_t)o * 2 * NP * NP;
-                const auto v = [&](int n_, int k_) { return t[(size_t)n_ * lv.P + k_] - c; };
-                write_tc_tile(base, NP, lv.P, lv.P, v);
-                float* half = reinterpret_cast<float*>(img.data() + off_tch[k]);
-                half[(size_t)(kNumOffsets + 4) * 2 * NP * 32 + o] =
-                    write_half_tile(reinterpret_cast<uint16_t*>(half + (size_t)o * 2 * NP * 32), NP, lv.P, lv.P, v);
-            }
-        }
-        // tensor-core L2L tiles for class c: B[n = child p][k = parent q] = S_{k+1}[q][c P_k + p]
-        if (tc && k + 1 < (int)mo.levels.size() && k + 1 < n_levels) {
-            const LevelOps& par = mo.levels[k + 1];
-            for (int c = 0; c < 4; ++c) {
-                float* base = reinterpret_cast<float*>(img.data() + off_tc[k]) + (size_t)(kNumOffsets + c) * 2 * NP * NP;
-                const auto v = [&](int n_, int k_) { return par.S[(size_t)k_ * (4 * lv.P) + c * lv.P + n_]; };
-                write_tc_tile(base, NP, lv.P, par.P, v);
-                float* half = reinterpret_cast<float*>(img.data() + off_tch[k]);
-                half[(size_t)(kNumOffsets + 4) * 2 * NP * 32 + kNumOffsets + c] = write_half_tile(
-                    reinterpret_cast<uint16_t*>(half + (size_t)(kNumOffsets + c) * 2 * NP * 32), NP, lv.P, par.P, v);
-            }
+            img[off.mono[k] + o] = hi;
+            img[off.mono[k] + kNumOffsets + o] = (T)(c - (double)hi);
+            for (int q = 0; q < lv.P; ++q)
+                for (int p = 0; p < lv.P; ++p)
+                    img[off.tifo[k] + ((size_t)o * NP + q) * NP + p] = (T)(t[(size_t)p * lv.P + q] - c);
         }
     }
+    return img;
+}
+
+// Floats of one level's tensor-core tiles: 40 offsets and 4 L2L classes (rows: TF32 hi and lo,
+// NP / 32 blocks of 64 NP floats each; halves: fp16 hi and lo, 2 NP rows of 128 bytes, then the
+// floats that undo the scaling); 1 KB aligned.
+size_t tile_floats(int NP, bool halves) {
+    const size_t n = (size_t)(kNumOffsets + 4) * (halves ? 2 * NP * 32 + 1 : 2 * NP * NP);
+    return (n + 255) & ~(size_t)255;
+}
+size_t tile_bytes(int NP, bool halves, int levels) { return tile_floats(NP, halves) * levels * sizeof(float); }
+size_t sliced_bytes(int n_levels) { return (sg_operator_bytes(n_levels) + 1023) / 1024 * 1024; }
+
+// Tiles of levels have .. want - 1 from the binary32 image, in `mem` (1 KB aligned) or, if null,
+// in an allocation of their own; on the device when the call returns.  L2L tile of class c at
+// the child's level k: B[n = child p][k = parent q] = S_{k+1}[q][c P_k + p].
+cudaError_t add_tiles(DeviceOps& d, bool halves, int want, void* mem, const std::vector<float>& img,
+                      const ImageOffsets& off, cudaStream_t stream) {
+    int& have = halves ? d.have.halves : d.have.rows;
+    const int NP = d.NP, k0 = have;
+    std::vector<float> out(tile_floats(NP, halves) * (want - k0), 0.0f);
+    float v[64][64];
+    for (int k = k0; k < want; ++k) {
+        float* lvl = out.data() + tile_floats(NP, halves) * (k - k0);
+        for (int op = 0; op < kNumOffsets + 4; ++op) {
+            if (op >= kNumOffsets && k + 1 >= d.n_levels) break;
+            const float* from = op < kNumOffsets ? img.data() + off.tifo[k] + (size_t)op * NP * NP
+                                                 : img.data() + off.l2l[k + 1] + (size_t)(op - kNumOffsets) * NP * NP;
+            for (int q = 0; q < NP; ++q)
+                for (int p = 0; p < NP; ++p) v[p][q] = from[(size_t)q * NP + p];
+            if (halves)
+                lvl[(size_t)(kNumOffsets + 4) * 2 * NP * 32 + op] =
+                    write_half_tile(reinterpret_cast<uint16_t*>(lvl + (size_t)op * 2 * NP * 32), NP, v);
+            else
+                write_tc_tile(lvl + (size_t)op * 2 * NP * NP, NP, v);
+        }
+    }
+    void* own = nullptr;
+    cudaError_t e = cudaSuccess;
+    if (!mem) {
+        e = cudaMalloc(&own, out.size() * sizeof(float));
+        if (e != cudaSuccess) return e;
+        mem = own;
+    }
+    e = cudaMemcpyAsync(mem, out.data(), out.size() * sizeof(float), cudaMemcpyHostToDevice, stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+    if (e != cudaSuccess) {
+        if (own) cudaFree(own);
+        return e;
+    }
+    if (own) d.retired.push_back(own);
+    for (int k = k0; k < want; ++k) {
+        float* lvl = (float*)mem + tile_floats(NP, halves) * (k - k0);
+        if (halves) {
+            d.tch[k] = lvl;
+            d.tch_scale[k] = lvl + (size_t)(kNumOffsets + 4) * 2 * NP * 32;
+        } else {
+            d.tc[k] = lvl;
+        }
+    }
+    have = want;
+    return cudaSuccess;
+}
+
+// The sliced operators of every level likewise.
+cudaError_t add_sliced(DeviceOps& d, void* mem, cudaStream_t stream) {
+    void* own = nullptr;
+    cudaError_t e = cudaSuccess;
+    if (!mem) {
+        e = cudaMalloc(&own, sliced_bytes(d.n_levels));
+        if (e != cudaSuccess) return e;
+        mem = own;
+    }
+    e = sg_build_operators(d, mem, stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);  // plans on other streams use them too
+    if (e != cudaSuccess) {
+        if (own) cudaFree(own);
+        return e;
+    }
+    if (own) d.retired.push_back(own);
+    d.have.sliced = true;
+    return cudaSuccess;
 }
 
 }  // namespace
 
-const DeviceOps* get_device_ops(ModelOps* mo, int precision, int NP, int n_levels,
+const DeviceOps* get_device_ops(ModelOps* mo, int precision, int NP, int n_levels, OpsImages* want,
                                 cudaStream_t stream, std::string* err) {
     std::lock_guard<std::mutex> g(mo->mu);
     while ((int)mo->levels.size() < n_levels) build_level(*mo);
     auto& slot = mo->dev[precision == LFMM_MIXED ? 1 : (precision == LFMM_DF ? 2 : 0)][NP == 64 ? 1 : 0];
-    if (slot && slot->n_levels >= n_levels) return slot.get();
+    auto failed = [&](const char* what, cudaError_t e) {
+        cudaGetLastError();
+        if (err) *err = std::string(what) + cudaGetErrorString(e);
+        return nullptr;
+    };
+    if (slot && slot->n_levels >= n_levels) {
+        // brought here by plans that used fewer of the images
+        const bool rows = slot->have.rows < want->rows, halves = slot->have.halves < want->halves;
+        if (rows || halves) {
+            // from the operators on the device (quicker than computing them again)
+            std::vector<float> img(slot->bytes / sizeof(float));
+            ImageOffsets off;
+            for (int k = 0; k < slot->n_levels; ++k) {
+                off.tifo.push_back((float*)slot->tifo[k] - (float*)slot->base);
+                off.l2l.push_back(k >= 1 ? (float*)slot->l2l[k] - (float*)slot->base : 0);
+            }
+            cudaError_t e = cudaMemcpyAsync(img.data(), slot->base, slot->bytes, cudaMemcpyDeviceToHost, stream);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+            if (e == cudaSuccess && rows) e = add_tiles(*slot, false, want->rows, nullptr, img, off, stream);
+            if (e == cudaSuccess && halves) e = add_tiles(*slot, true, want->halves, nullptr, img, off, stream);
+            if (e != cudaSuccess) return failed("operator tiles: ", e);
+        }
+        if (want->sliced && !slot->have.sliced && add_sliced(*slot, nullptr, stream) != cudaSuccess) {
+            cudaGetLastError();
+            want->sliced = false;
+        }
+        return slot.get();
+    }
     const int nl = std::max(n_levels, slot ? slot->n_levels : 0);
     std::unique_ptr<DeviceOps> d(new DeviceOps());
     d->NP = NP;
@@ -474,42 +565,6 @@ const DeviceOps* get_device_ops(ModelOps* mo, int precision, int NP, int n_level
     d->leaf_side = mo->leaf_side;
     d->tab_H = 2 * mo->leaf_side - 1;
     d->tab_W = p2p_table_width(mo->leaf_side);
-    size_t off_tofs, off_tab;
-    std::vector<size_t> om, ol, ot, omono, otc, otch;
-    std::vector<char> bytes;
-    size_t elem;
-    if (precision == LFMM_MIXED) {
-        std::vector<float> img;
-        fill_device_image<float>(*mo, NP, nl, d->tab_H, d->tab_W, img, off_tofs, off_tab, om, ol, ot, omono, otc, otch);
-        elem = sizeof(float);
-        bytes.assign((const char*)img.data(), (const char*)img.data() + img.size() * elem);
-    } else if (precision == LFMM_DF) {
-        std::vector<DF> img;
-        fill_device_image<DF>(*mo, NP, nl, d->tab_H, d->tab_W, img, off_tofs, off_tab, om, ol, ot, omono, otc, otch);
-        elem = sizeof(DF);
-        bytes.assign((const char*)img.data(), (const char*)img.data() + img.size() * elem);
-    } else {
-        std::vector<double> img;
-        fill_device_image<double>(*mo, NP, nl, d->tab_H, d->tab_W, img, off_tofs, off_tab, om, ol, ot, omono, otc, otch);
-        elem = sizeof(double);
-        bytes.assign((const char*)img.data(), (const char*)img.data() + img.size() * elem);
-    }
-    d->bytes = bytes.size();
-    cudaError_t e = cudaMalloc(&d->base, d->bytes);
-    if (e != cudaSuccess) {
-        if (err) *err = std::string("cudaMalloc(operators): ") + cudaGetErrorString(e);
-        return nullptr;
-    }
-    e = cudaMemcpyAsync(d->base, bytes.data(), d->bytes, cudaMemcpyHostToDevice, stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
-    if (e != cudaSuccess) {
-        cudaFree(d->base);
-        if (err) *err = std::string("upload(operators): ") + cudaGetErrorString(e);
-        return nullptr;
-    }
-    char* b = (char*)d->base;
-    d->tofsT = b + off_tofs * elem;
-    d->p2p_table = b + off_tab * elem;
     d->m2m.resize(nl);
     d->l2l.resize(nl);
     d->tifo.resize(nl);
@@ -517,27 +572,45 @@ const DeviceOps* get_device_ops(ModelOps* mo, int precision, int NP, int n_level
     d->tc.assign(nl, nullptr);
     d->tch.assign(nl, nullptr);
     d->tch_scale.assign(nl, nullptr);
-    for (int k = 0; k < nl; ++k) {
-        if (precision == LFMM_MIXED && (NP == 32 || NP == 64)) {
-            d->tc[k] = b + otc[k] * elem;
-            d->tch[k] = b + otch[k] * elem;
-            d->tch_scale[k] = (char*)d->tch[k] + (size_t)(kNumOffsets + 4) * 2 * NP * 128;
+    ImageOffsets off;
+    const char* what = "";
+    auto upload = [&](auto zero) -> cudaError_t {
+        using T = decltype(zero);
+        const std::vector<T> img = operator_image<T>(*mo, NP, nl, d->tab_H, d->tab_W, off);
+        const size_t own = d->bytes = img.size() * sizeof(T);
+        const size_t tiles = (own + 1023) / 1024 * 1024;
+        const size_t slices = tiles + tile_bytes(NP, false, want->rows) + tile_bytes(NP, true, want->halves);
+        what = "cudaMalloc(operators): ";
+        cudaError_t e = cudaErrorMemoryAllocation;
+        if (want->sliced && (e = cudaMalloc(&d->base, slices + sliced_bytes(nl))) != cudaSuccess) {
+            cudaGetLastError();
+            want->sliced = false;  // the plan can do without
         }
-        d->m2m[k] = k >= 1 ? b + om[k] * elem : nullptr;
-        d->l2l[k] = k >= 1 ? b + ol[k] * elem : nullptr;
-        d->tifo[k] = b + ot[k] * elem;
-        d->mono[k] = b + omono[k] * elem;
-    }
-    if (precision != LFMM_MIXED && NP == 64) {
-        e = sg_build_operators(*d, stream);
+        if (e != cudaSuccess) e = cudaMalloc(&d->base, slices);
+        if (e != cudaSuccess) return e;
+        what = "upload(operators): ";
+        char* b = (char*)d->base;
+        e = cudaMemcpyAsync(b, img.data(), own, cudaMemcpyHostToDevice, stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
-        if (e != cudaSuccess) {
-            cudaFree(d->sg_base);
-            cudaFree(d->base);
-            if (err) *err = std::string("sliced operators: ") + cudaGetErrorString(e);
-            return nullptr;
+        d->tofsT = b + off.tofs * sizeof(T);
+        d->p2p_table = b + off.tab * sizeof(T);
+        for (int k = 0; k < nl; ++k) {
+            d->m2m[k] = k >= 1 ? b + off.m2m[k] * sizeof(T) : nullptr;
+            d->l2l[k] = k >= 1 ? b + off.l2l[k] * sizeof(T) : nullptr;
+            d->tifo[k] = b + off.tifo[k] * sizeof(T);
+            d->mono[k] = b + off.mono[k] * sizeof(T);
         }
-    }
+        if constexpr (std::is_same<T, float>::value) {
+            if (e == cudaSuccess && want->rows > 0) e = add_tiles(*d, false, want->rows, b + tiles, img, off, stream);
+            if (e == cudaSuccess && want->halves > 0)
+                e = add_tiles(*d, true, want->halves, b + tiles + tile_bytes(NP, false, want->rows), img, off, stream);
+        }
+        if (e == cudaSuccess && want->sliced) e = add_sliced(*d, b + slices, stream);
+        if (e != cudaSuccess) cudaFree(d->base);
+        return e;
+    };
+    const cudaError_t e = precision == LFMM_MIXED ? upload(0.0f) : precision == LFMM_DF ? upload(DF(0.0)) : upload(0.0);
+    if (e != cudaSuccess) return failed(what, e);
     if (slot) d->retired.push_back(slot.release());  // plans built earlier may still use it
     slot = std::move(d);
     return slot.get();

@@ -984,14 +984,14 @@ int64_t sg_work_bytes(const SgTree& t, int precision, int num_sms) {
     return carve(t, precision == LFMM_DF ? 2 : 3, sg_chunks(t, num_sms), nullptr).bytes;
 }
 
-cudaError_t sg_build_operators(DeviceOps& ops, cudaStream_t s) {
+cudaError_t sg_build_operators(DeviceOps& ops, void* mem, cudaStream_t s) {
     const int nl = ops.n_levels;
     const size_t per = (size_t)kSgOps * kSgTileBytes;
-    cudaError_t e = cudaMalloc(&ops.sg_base, (size_t)nl * (per + kSgOps * sizeof(int32_t)));
-    if (e != cudaSuccess) return clear_and_return(e);
-    uint8_t* tiles = (uint8_t*)ops.sg_base;
+    uint8_t* tiles = (uint8_t*)mem;
     int32_t* exps = (int32_t*)(tiles + nl * per);
     const size_t op = (size_t)64 * 64 * (ops.precision == LFMM_DF ? sizeof(DF) : sizeof(double));
+    ops.sg_tiles.clear();
+    ops.sg_e.clear();
     for (int k = 0; k < nl; ++k) {
         ops.sg_tiles.push_back(tiles + k * per);
         ops.sg_e.push_back(exps + k * kSgOps);
@@ -1005,7 +1005,7 @@ cudaError_t sg_build_operators(DeviceOps& ops, cudaStream_t s) {
             slice_ops_kernel<DF><<<kSgOps, 256, 0, s>>>(l, ops.sg_tiles[k], ops.sg_e[k]);
         else
             slice_ops_kernel<double><<<kSgOps, 256, 0, s>>>(l, ops.sg_tiles[k], ops.sg_e[k]);
-        e = cudaGetLastError();
+        const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

@@ -45,8 +45,12 @@ SgTree forest_sg_tree(const Forest& F);
 int sg_chunks(const SgTree& t, int num_sms);
 // Bytes of the work space of one evaluation.
 int64_t sg_work_bytes(const SgTree& t, int precision, int num_sms);
-// Sliced operators of every level of `ops` (binary64-accurate paths, P_pad 64).
-cudaError_t sg_build_operators(DeviceOps& ops, cudaStream_t s);
+// Sliced operators of every level of `ops` (binary64-accurate paths, P_pad 64), in `mem` (1 KB
+// aligned, sg_operator_bytes of it).
+constexpr size_t sg_operator_bytes(int n_levels) {
+    return (size_t)n_levels * kSgOps * (kSgTileBytes + sizeof(int32_t));
+}
+cudaError_t sg_build_operators(DeviceOps& ops, void* mem, cudaStream_t s);
 // M2M (unless q_all: the expansions of every level are in q already), M2L and L2L: from the
 // leaf expansions and charges in q / Q to the leaf incoming expansions and constants in
 // u / C (rows as in t.lv[k].off; other levels' rows of q and u are scratch).
