@@ -314,6 +314,11 @@ int device_coords(lfmm_plan* p, const int32_t* xy, int64_t n, const int32_t** ou
     return LFMM_OK;
 }
 
+// Work space of the sliced far field (2-4 times the expansions).
+int sliced_workspace(lfmm_plan* p, const SgTree& t, void** work, cudaStream_t s) {
+    return palloc(p, work, (size_t)sg_work_bytes(t, p->opts.precision, p->num_sms), s);
+}
+
 // Operators and workspaces of a pruned tree or forest (tree already in p->forest).
 int forest_workspaces(lfmm_plan* p, cudaStream_t s) {
     int st;
@@ -364,11 +369,6 @@ int forest_workspaces(lfmm_plan* p, cudaStream_t s) {
         if ((st = palloc(p, &c, 32 * sizeof(unsigned long long), s))) return st;
         F.sweep_ctr = (unsigned long long*)c;
     }
-    {  // partial sums of the list M2L levels split along K (few boxes)
-        F.m2l_split = p->opts.m2l_split;
-        const int64_t sb = forest_m2l_split_bytes(F, p->NP, esz, p->num_sms, F.m2l_split);
-        if (sb > 0 && (st = palloc(p, &F.m2l_part, (size_t)sb, s))) return st;
-    }
     if (split_floats > 0) {
         void* b;
         if ((st = palloc(p, &b, (size_t)split_floats * sizeof(float), s))) return st;
@@ -381,17 +381,19 @@ int forest_workspaces(lfmm_plan* p, cudaStream_t s) {
         F.t_leaf = (int32_t*)(F.near_tmp + p->nt);
         LFMM_CUDA_TRY(launch_target_leaves(F, F.t_leaf, s));
     }
-    // sliced far field of the binary64-accurate paths (split_tc.cu)
-    if (images.sliced) {
-        const int64_t need = sg_work_bytes(forest_sg_tree(F), p->opts.precision, p->num_sms);
-        if ((st = palloc(p, &F.sg_work, (size_t)need, s))) return st;
-    }
     if ((st = palloc(p, &p->Qbox, (size_t)boxes * 8, s))) return st;
     if ((st = palloc(p, &p->Cbox, (size_t)boxes * 8, s))) return st;
     void* stbuf;
     if ((st = palloc(p, &stbuf, 16, s))) return st;
     p->status = (int*)stbuf;
     LFMM_CUDA_TRY(cudaMemsetAsync(p->status, 0, 16, s));  // status word + grid-barrier words
+    F.m2l_split = p->opts.m2l_split;
+    // sliced far field of the binary64-accurate paths (split_tc.cu)
+    if (images.sliced && (st = sliced_workspace(p, forest_sg_tree(F), &F.sg_work, s))) return st;
+    if (!F.sg_work) {  // partial sums of the list M2L levels split along K (few boxes)
+        const int64_t sb = forest_m2l_split_bytes(F, p->NP, esz, p->num_sms, F.m2l_split);
+        if (sb > 0 && (st = palloc(p, &F.m2l_part, (size_t)sb, s))) return st;
+    }
     p->tc_min_level = p->opts.tc_min_level == 0 ? kDefaultTcMinLevel : p->opts.tc_min_level;
     p->bytes += F.bytes;
     return LFMM_OK;
@@ -656,10 +658,6 @@ int plan_build(lfmm_plan* p, const int32_t* src_xy, const int32_t* tgt_xy, cudaS
     if ((st = palloc(p, &p->uhat, (size_t)boxes * p->NP * esz, s))) return st;
     if ((st = palloc(p, &p->Qbox, (size_t)boxes * 8, s))) return st;
     if ((st = palloc(p, &p->Cbox, (size_t)boxes * 8, s))) return st;
-    if (images.sliced &&
-        (st = palloc(p, &p->sg_work,
-                     (size_t)sg_work_bytes(sg_uniform_tree(p->L, p->opts.m2l_split), p->opts.precision, p->num_sms), s)))
-        return st;
     if (p->L >= 2) {  // a far field: near and far parts go to these buffers, then one sum
         void* b;
         if ((st = palloc(p, &b, (size_t)2 * p->nt * sizeof(double), s))) return st;
@@ -671,6 +669,7 @@ int plan_build(lfmm_plan* p, const int32_t* src_xy, const int32_t* tgt_xy, cudaS
     p->status = (int*)stbuf;
     LFMM_CUDA_TRY(cudaMemsetAsync(p->status, 0, 16, s));  // status word + grid-barrier words
     p->tc_min_level = p->opts.tc_min_level == 0 ? kDefaultTcMinLevel : p->opts.tc_min_level;
+    if (images.sliced && (st = sliced_workspace(p, sg_uniform_tree(p->L, p->opts.m2l_split), &p->sg_work, s))) return st;
     // the one-vector partial sums of the K-split coarse-level M2L belong to the plan from
     // the start, so that device_bytes counts them before the first evaluation
     if ((st = ensure_m2l_part(p, 1, s))) return st;
@@ -1010,9 +1009,10 @@ int eval_graph(lfmm_plan* p, const double* f, double* const out[3], cudaStream_t
 }
 
 // Room for the partial sums of the K-split fused small-level M2L for nvec vectors
-// (plan-owned, allocated before any evaluation or graph capture needs it).
+// (plan-owned, allocated before any evaluation or graph capture needs it; the sliced far field
+// has sums of its own).
 int ensure_m2l_part(lfmm_plan* p, int nvec, cudaStream_t s) {
-    if (p->forest || p->L < 2 || !p->ops || nvec <= p->m2l_part_nvec) return LFMM_OK;
+    if (p->forest || p->sg_work || p->L < 2 || !p->ops || nvec <= p->m2l_part_nvec) return LFMM_OK;
     const int64_t need =
         p->opts.precision == LFMM_MIXED
             ? m2l_fused_split_bytes<float>(*p->ops, p->L, p->tc_min_level, p->num_sms, nvec, p->opts.m2l_split)
