@@ -81,8 +81,9 @@ typedef struct lfmm_opts {
                               /* and forests: every list level of >= 1024 boxes runs there    */
                               /* unless this is > 30.  Binary64 and float-float at p > 9: the */
                               /* whole far field of pruned trees and forests, and of uniform  */
-                              /* trees whose leaf level is >= this, runs there in exactly     */
-                              /* split operands unless this is > 30                           */
+                              /* trees whose leaf level is >= this, runs there in split       */
+                              /* operands (LFMM_FP64 above) unless this is > 30, or the       */
+                              /* device has no room for the work space at plan creation       */
     int32_t tree;             /* LFMM_TREE_AUTO, LFMM_TREE_UNIFORM or LFMM_TREE_PRUNED         */
     int32_t flags;            /* bitwise OR of LFMM_FLAG_* (0: none)                           */
     /* M2L tiling (0 everywhere: the library's rules; lfmm_autotune picks these).  They    */

@@ -314,9 +314,11 @@ int device_coords(lfmm_plan* p, const int32_t* xy, int64_t n, const int32_t** ou
     return LFMM_OK;
 }
 
-// Work space of the sliced far field (2-4 times the expansions).
+// Work space of the sliced far field (2-4 times the expansions).  *work stays null when the
+// device has no room for it: the other translations then take its place.
 int sliced_workspace(lfmm_plan* p, const SgTree& t, void** work, cudaStream_t s) {
-    return palloc(p, work, (size_t)sg_work_bytes(t, p->opts.precision, p->num_sms), s);
+    const int st = palloc(p, work, (size_t)sg_work_bytes(t, p->opts.precision, p->num_sms), s);
+    return st == LFMM_ENOMEM ? LFMM_OK : st;
 }
 
 // Operators and workspaces of a pruned tree or forest (tree already in p->forest).
@@ -388,7 +390,8 @@ int forest_workspaces(lfmm_plan* p, cudaStream_t s) {
     p->status = (int*)stbuf;
     LFMM_CUDA_TRY(cudaMemsetAsync(p->status, 0, 16, s));  // status word + grid-barrier words
     F.m2l_split = p->opts.m2l_split;
-    // sliced far field of the binary64-accurate paths (split_tc.cu)
+    // sliced far field of the binary64-accurate paths (split_tc.cu), after all that no plan can
+    // do without
     if (images.sliced && (st = sliced_workspace(p, forest_sg_tree(F), &F.sg_work, s))) return st;
     if (!F.sg_work) {  // partial sums of the list M2L levels split along K (few boxes)
         const int64_t sb = forest_m2l_split_bytes(F, p->NP, esz, p->num_sms, F.m2l_split);
@@ -669,6 +672,7 @@ int plan_build(lfmm_plan* p, const int32_t* src_xy, const int32_t* tgt_xy, cudaS
     p->status = (int*)stbuf;
     LFMM_CUDA_TRY(cudaMemsetAsync(p->status, 0, 16, s));  // status word + grid-barrier words
     p->tc_min_level = p->opts.tc_min_level == 0 ? kDefaultTcMinLevel : p->opts.tc_min_level;
+    // (after all that no plan can do without)
     if (images.sliced && (st = sliced_workspace(p, sg_uniform_tree(p->L, p->opts.m2l_split), &p->sg_work, s))) return st;
     // the one-vector partial sums of the K-split coarse-level M2L belong to the plan from
     // the start, so that device_bytes counts them before the first evaluation
