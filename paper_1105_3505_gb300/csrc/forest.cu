@@ -44,7 +44,7 @@ int grid_for(int64_t n, int threads, int cap = 152 * 16) {
 // P2M of compact leaves b0 .. b0 + 3 (those below nb): a quarter warp per leaf, lane h
 // of a quarter owning expansion entries [h PL, h PL + PL), PL = NP / 8; leaf b's sources
 // are [rl_s[j], rl_s[j + 1]), j = the leaf's row-major index.
-template <typename T, int NP>
+template <typename T, int NP, int U = 1>
 __device__ __forceinline__ void p2m_list_quad(int64_t b0, int64_t nb, int lane, const int32_t* __restrict__ leaf_rl,
                                               const int32_t* __restrict__ rl_s, const int32_t* __restrict__ loc,
                                               const int32_t* __restrict__ perm, const double* __restrict__ f,
@@ -101,13 +101,19 @@ __device__ __forceinline__ void p2m_list_quad(int64_t b0, int64_t nb, int lane, 
 #pragma unroll
         for (int u = 0; u < R; ++u) {
             const int cc = min(G, cmax - j0 - u * G);
-            for (int k = 0; k < cc; ++k) {
+            auto one = [&](int k) {
                 // lanes of a quarter with fewer sources multiply row 0 by zero
                 const T fk = shfl(fj[u], (grp << 3) + k);
                 const int Jk = __shfl_sync(kFull, J[u], (grp << 3) + k);
                 const Row r = *reinterpret_cast<const Row*>(tofsT + (size_t)Jk * NP + hl * PL);
 #pragma unroll
                 for (int i = 0; i < PL; ++i) acc[i] = fma(r.v[i], fk, acc[i]);
+            };
+            if constexpr (U > 1) {
+#pragma unroll U
+                for (int k = 0; k < cc; ++k) one(k);
+            } else {
+                for (int k = 0; k < cc; ++k) one(k);
             }
         }
     }
@@ -122,7 +128,10 @@ __device__ __forceinline__ void p2m_list_quad(int64_t b0, int64_t nb, int lane, 
     if (lv && hl == 0) Q[b] = qsum;
 }
 
-template <typename T, int NP>
+// U: operator rows in flight.  Where the leaves fill the chip, one (32 registers; four: clustered_4m
+// 3,660 -> 3,685 us, forest_4096 3,845 -> 3,885); fewer leaves wait for one row after the other
+// (200 sources: 28 -> 20 us a call).
+template <typename T, int NP, int U>
 __global__ void __launch_bounds__(256) p2m_list_kernel(int64_t nb, const int32_t* __restrict__ leaf_rl,
                                                        const int32_t* __restrict__ rl_s,
                                                        const int32_t* __restrict__ loc,
@@ -134,7 +143,7 @@ __global__ void __launch_bounds__(256) p2m_list_kernel(int64_t nb, const int32_t
     const int lane = threadIdx.x & 31;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; 4 * w < nb; w += nw)
-        p2m_list_quad<T, NP>(4 * w, nb, lane, leaf_rl, rl_s, loc, perm, f, f_sorted, tofsT, side, qhat, Q);
+        p2m_list_quad<T, NP, U>(4 * w, nb, lane, leaf_rl, rl_s, loc, perm, f, f_sorted, tofsT, side, qhat, Q);
 }
 
 // P2M of the 8-byte types where the sliced far field follows (leaves of up to 192 sources,
@@ -1305,14 +1314,60 @@ int forest_eval(const Forest& F, const DeviceOps& ops, const double* f, T* f_sor
                                            l0.nb, l0.rl, F.rl_s, F.sloc, F.sperm, f, f_sorted, (const T*)ops.tofsT,
                                            F.side, Qx(0), Qm(0));
             }
-            if (wide) {
-            } else if (NP == 32)
-                (void)launch_dependent(p2m_list_kernel<T, 32>, dim3((int)blocks), dim3(256), 0, s, l0.nb, l0.rl, F.rl_s,
-                                       F.sloc, F.sperm, f, f_sorted, (const T*)ops.tofsT, F.side, Qx(0), Qm(0));
-            else
-                (void)launch_dependent(p2m_list_kernel<T, 64>, dim3((int)blocks), dim3(256), 0, s, l0.nb, l0.rl, F.rl_s,
-                                       F.sloc, F.sperm, f, f_sorted, (const T*)ops.tofsT, F.side, Qx(0), Qm(0));
-            LFMM_CUDA_TRY(cudaGetLastError());
+            if (!wide) {
+                auto go = [&](auto np_tag, auto u_tag) {
+                    (void)launch_dependent(p2m_list_kernel<T, decltype(np_tag)::value, decltype(u_tag)::value>,
+                                           dim3((int)blocks), dim3(256), 0, s, l0.nb, l0.rl, F.rl_s, F.sloc, F.sperm, f,
+                                           f_sorted, (const T*)ops.tofsT, F.side, Qx(0), Qm(0));
+                };
+                using One = std::integral_constant<int, 1>;
+                using Few = std::integral_constant<int, sizeof(T) == 4 ? 4 : 1>;
+                const bool few = blocks <= num_sms;
+                auto by_u = [&](auto np_tag) { few ? go(np_tag, Few()) : go(np_tag, One()); };
+                if (NP == 32) by_u(std::integral_constant<int, 32>());
+                else by_u(std::integral_constant<int, 64>());
+            }
+            pt.add_launches(1);
+        }
+    }
+    // the near field needs the sorted charges and the leaf charges only: it runs beside the
+    // rest of the far field, one of them on the side stream
+    const cudaStream_t s_main = s;
+    cudaStream_t s_near = s;
+    const bool fork = far && side != nullptr && status == nullptr;  // not beside a persistent sweep
+    if (fork) {
+        LFMM_CUDA_TRY(cudaEventRecord(side->fork, s));
+        LFMM_CUDA_TRY(cudaStreamWaitEvent(side->s, side->fork, 0));
+        (side->near ? s_near : s) = side->s;
+    }
+    if (far) {
+        const int st = launch_list_p2p<T>(F, ops, f_sorted, Qm(0), nullptr, nullptr, nullptr, num_sms, s_near, true);
+        if (st) return st;
+    }
+    if constexpr (sizeof(T) == 8) {
+        if (far && sliced) {
+            PhaseTimer pt(LFMM_PHASE_M2L_TC, s);
+            int n = 0;
+            const cudaError_t e = sg_far_field<T>(forest_sg_tree(F), ops, qhat, uhat, Qbox, Cbox, F.sg_work, false,
+                                                  status_word, num_sms, s, &n);
+            if (e != cudaSuccess) return fail(LFMM_ECUDA, std::string("split_gemm_kernel: ") + cudaGetErrorString(e));
+            pt.add_launches(n);
+        }
+    }
+    if (far && !up_done && !sliced) {
+        PhaseTimer pt(LFMM_PHASE_M2M, s);
+        for (int k = 1; k < nk; ++k) {
+            const ForestLevel& lv = F.levels[k];
+            if (lv.nb == 0) continue;
+            if (lv.nb < (int64_t)num_sms * 16) {  // few parents: one block each
+                const int64_t nbk = std::min<int64_t>(lv.nb, (int64_t)num_sms * 16);
+                if (NP == 32)
+                    (void)launch_dependent(m2m_list_block_kernel<T, 32>, dim3((unsigned)nbk), dim3(128), 0, s, lv.nb,
+                                           lv.ch, Qx(k - 1), (const T*)ops.m2m[k], Qm(k - 1), Qx(k), Qm(k));
+                else
+                    (void)launch_dependent(m2m_list_block_kernel<T, 64>, dim3((unsigned)nbk), dim3(256), 0, s, lv.nb,
+                                           lv.ch, Qx(k - 1), (const T*)ops.m2m[k], Qm(k - 1), Qx(k), Qm(k));
+                LFMM_CUDA_TRY(cudaGetLastError());
             pt.add_launches(1);
         }
     }
