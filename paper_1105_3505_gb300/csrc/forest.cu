@@ -798,7 +798,6 @@ struct NearCfg {
     static constexpr int THREADS = sizeof(T) == 8 ? 768 : 192;
     static constexpr int BLOCKS = sizeof(T) == 8 ? 1 : 6;
 };
-
 // A lane's near sum of the 8-byte types.
 //
 // Float-float: four products at a time are summed from zero, their rounding errors gathered in
@@ -853,8 +852,8 @@ struct NearSum<double> {
     __device__ __forceinline__ double total() const { return acc; }
 };
 
-template <typename T>
-__global__ void __launch_bounds__(NearCfg<T>::THREADS, NearCfg<T>::BLOCKS) p2p_list_kernel(
+template <typename T, int BLOCKS>
+__global__ void __launch_bounds__(NearCfg<T>::THREADS, BLOCKS) p2p_list_kernel(
     const int4* __restrict__ strips, const int4* __restrict__ strip_rows, const int32_t* __restrict__ n_strips_d,
     const int32_t* __restrict__ Lp, const uint64_t* __restrict__ rl_key, const int32_t* __restrict__ rl_s,
     const int32_t* __restrict__ rl_t, const int32_t* __restrict__ rl_id, int kb, int side, int SW,
@@ -1213,21 +1212,37 @@ static int launch_list_p2p(const Forest& F, const DeviceOps& ops, const T* f_sor
                         (size_t)3 * (Cfg::MAXSW + 2) * sizeof(V) + (size_t)2 * capt * sizeof(int) +
                         (size_t)(3 * (Cfg::MAXSW + 3) + Cfg::MAXSW + 1) * sizeof(int);
     constexpr int threads = NearCfg<T>::THREADS;
-    const void* fn = (const void*)p2p_list_kernel<T>;
-    cudaError_t e = ensure_dynamic_smem(fn, smem);
-    if (e == cudaSuccess) {
-        const int per_sm = blocks_per_sm(fn, threads, smem);
+    const size_t tab = (size_t)(2 * ops.tab_H + 1) * ops.tab_W * sizeof(T);
+    auto go = [&](auto blocks_tag) -> cudaError_t {
+        constexpr int BLOCKS = decltype(blocks_tag)::value;
+        const void* fn = (const void*)p2p_list_kernel<T, BLOCKS>;
+        const cudaError_t e = ensure_dynamic_smem(fn, smem);
+        if (e != cudaSuccess) return e;
+        const int64_t wave = (int64_t)num_sms * blocks_per_sm(fn, threads, smem);
         // beside the far field: blocks of a few strips, so that the far field's launches (of
         // a higher priority) find free SMs as blocks end; binary32's table is staged faster and
         // its far field takes more of the time (forest_4096 with 2 / 6 / 16 rounds of blocks:
-        // 4,126 / 4,084 / 3,932 us; one stream 4,287 us; clustered_4m 4,020 / 3,880 / 3,867)
-        const int64_t waves = !use_tmp ? 1 : sizeof(T) == 8 ? 6 : 16;
-        const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(F.n_strips, waves * num_sms * per_sm));
-        e = launch_dependent(p2p_list_kernel<T>, dim3((unsigned)grid), dim3(threads), smem, s, F.strips, F.strip_rows,
-                             F.n_strips_d, F.d_L, F.rl_key, F.rl_s, F.rl_t, F.rl_id, F.kb, F.side, F.SW, F.sloc, F.tloc,
-                             F.tperm, f_sorted, (const T*)ops.p2p_table, ops.tab_H, ops.tab_W, (const V*)Qleaf, u, un,
-                             uf, caps, capt, use_tmp ? F.near_tmp : nullptr);
-    }
+        // 4,126 / 4,084 / 3,932 us; one stream 4,287 us; clustered_4m 4,020 / 3,880 / 3,867).
+        // Beyond the first round a block has up to eight leaves, more for a larger table: a
+        // block for every leaf of a sparse tree staged 73 KB for a handful of pairs (20,000
+        // points in a box of 5,656, graph 193 -> 182 us; eight at side 16: 300 small problems
+        // 43 -> 49 us).
+        const int64_t rounds = !use_tmp ? 1 : sizeof(T) == 8 ? 6 : 16;
+        const int64_t per_block = std::max<int64_t>(1, std::min<int64_t>(8, tab / 8192));
+        const int64_t most = std::max(wave, std::min(rounds * wave, F.n_strips / per_block));
+        const int64_t grid = std::max<int64_t>(1, std::min(F.n_strips, most));
+        return launch_dependent(p2p_list_kernel<T, BLOCKS>, dim3((unsigned)grid), dim3(threads), smem, s, F.strips,
+                                F.strip_rows, F.n_strips_d, F.d_L, F.rl_key, F.rl_s, F.rl_t, F.rl_id, F.kb, F.side, F.SW,
+                                F.sloc, F.tloc, F.tperm, f_sorted, (const T*)ops.p2p_table, ops.tab_H, ops.tab_W,
+                                (const V*)Qleaf, u, un, uf, caps, capt, use_tmp ? F.near_tmp : nullptr);
+    };
+    // binary32 without a far field: the blocks that the SM's shared memory holds with registers
+    // for more loads in flight (20,000 problems of 5 to 40 points 306 -> 278 us)
+    cudaError_t e;
+    if constexpr (sizeof(T) == 4)
+        e = use_tmp ? go(std::integral_constant<int, NearCfg<T>::BLOCKS>()) : go(std::integral_constant<int, 4>());
+    else
+        e = go(std::integral_constant<int, NearCfg<T>::BLOCKS>());
     if (e != cudaSuccess) return fail(LFMM_ECUDA, std::string("p2p_list_kernel: ") + cudaGetErrorString(e));
     pt.add_launches(1);
     return LFMM_OK;
@@ -1327,47 +1342,6 @@ int forest_eval(const Forest& F, const DeviceOps& ops, const double* f, T* f_sor
                 if (NP == 32) by_u(std::integral_constant<int, 32>());
                 else by_u(std::integral_constant<int, 64>());
             }
-            pt.add_launches(1);
-        }
-    }
-    // the near field needs the sorted charges and the leaf charges only: it runs beside the
-    // rest of the far field, one of them on the side stream
-    const cudaStream_t s_main = s;
-    cudaStream_t s_near = s;
-    const bool fork = far && side != nullptr && status == nullptr;  // not beside a persistent sweep
-    if (fork) {
-        LFMM_CUDA_TRY(cudaEventRecord(side->fork, s));
-        LFMM_CUDA_TRY(cudaStreamWaitEvent(side->s, side->fork, 0));
-        (side->near ? s_near : s) = side->s;
-    }
-    if (far) {
-        const int st = launch_list_p2p<T>(F, ops, f_sorted, Qm(0), nullptr, nullptr, nullptr, num_sms, s_near, true);
-        if (st) return st;
-    }
-    if constexpr (sizeof(T) == 8) {
-        if (far && sliced) {
-            PhaseTimer pt(LFMM_PHASE_M2L_TC, s);
-            int n = 0;
-            const cudaError_t e = sg_far_field<T>(forest_sg_tree(F), ops, qhat, uhat, Qbox, Cbox, F.sg_work, false,
-                                                  status_word, num_sms, s, &n);
-            if (e != cudaSuccess) return fail(LFMM_ECUDA, std::string("split_gemm_kernel: ") + cudaGetErrorString(e));
-            pt.add_launches(n);
-        }
-    }
-    if (far && !up_done && !sliced) {
-        PhaseTimer pt(LFMM_PHASE_M2M, s);
-        for (int k = 1; k < nk; ++k) {
-            const ForestLevel& lv = F.levels[k];
-            if (lv.nb == 0) continue;
-            if (lv.nb < (int64_t)num_sms * 16) {  // few parents: one block each
-                const int64_t nbk = std::min<int64_t>(lv.nb, (int64_t)num_sms * 16);
-                if (NP == 32)
-                    (void)launch_dependent(m2m_list_block_kernel<T, 32>, dim3((unsigned)nbk), dim3(128), 0, s, lv.nb,
-                                           lv.ch, Qx(k - 1), (const T*)ops.m2m[k], Qm(k - 1), Qx(k), Qm(k));
-                else
-                    (void)launch_dependent(m2m_list_block_kernel<T, 64>, dim3((unsigned)nbk), dim3(256), 0, s, lv.nb,
-                                           lv.ch, Qx(k - 1), (const T*)ops.m2m[k], Qm(k - 1), Qx(k), Qm(k));
-                LFMM_CUDA_TRY(cudaGetLastError());
             pt.add_launches(1);
         }
     }

@@ -45,3 +45,48 @@ def test_sources_per_leaf_mixed(lfmm, p, copies, counts):
         fo.status()
     ref = oracle.lattice_sum(src, f, tgt)
     assert np.abs(u - ref).max() <= 1e-6 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("precision", ["mixed", "df", "fp64"])
+@pytest.mark.parametrize("parts", [False, True])
+def test_problems_of_one_leaf(lfmm, precision, parts):
+    """No far field: the near field alone writes the result, or the parts."""
+    prec, p, tol = {"mixed": (lfmm.LFMM_MIXED, 8, 1e-6), "df": (lfmm.LFMM_DF, 16, 1e-12),
+                    "fp64": (lfmm.LFMM_FP64, 16, 1e-12)}[precision]
+    rng = np.random.default_rng(5)
+    n = [1, 2, 3, 31, 32, 33, 64, 5] * 40
+    m = [64, 1, 33, 32, 31, 5, 2, 64] * 40
+    src = [workloads.distinct_in_box(rng, k, 20, -7, 11) for k in n]
+    tgt = [workloads.distinct_in_box(rng, k, 20, -7, 11) for k in m]
+    f = [rng.standard_normal(k) for k in n]
+    so, to = (np.concatenate([[0], np.cumsum(k)]).astype(np.int64) for k in (n, m))
+    S, T = (np.ascontiguousarray(np.concatenate(a).astype(np.int32)) for a in (src, tgt))
+    with lfmm.Forest(S, so, T, to, opts=lfmm.make_opts(prec, p, 64)) as fo:
+        assert fo.info()["L"] == 0
+        if parts:
+            u, far = fo.eval_parts(np.concatenate(f))
+            assert not far.any()
+        else:
+            u = fo.eval(np.concatenate(f))
+        fo.status()
+    for i in range(len(n)):
+        ref = oracle.lattice_sum(src[i], f[i], tgt[i])
+        assert np.abs(u[to[i]:to[i + 1]] - ref).max() <= tol * np.abs(f[i]).sum()
+
+
+@pytest.mark.parametrize("path", ["mixed", "df"])
+def test_sparse_tree_in_few_blocks(lfmm, path):
+    """Leaves of one or two points in a large box: a block of the near field takes several strips.
+    Eager, recorded and serial evaluations run the same kernels."""
+    prec, p, tol = (lfmm.LFMM_MIXED, 8, 1e-6) if path == "mixed" else (lfmm.LFMM_DF, 16, 1e-10)
+    prob = workloads.uniform_box(9000, 5000, 3300, seed=2)
+    idx = np.arange(0, 5000, 25)
+    ref = oracle.lattice_sum(prob.src, prob.f, prob.tgt[idx])
+    with lfmm.Plan(prob.src, prob.tgt, opts=lfmm.make_opts(prec, p, tree=lfmm.LFMM_TREE_PRUNED)) as pl:
+        assert pl.info()["leaf_side"] == 32 and pl.info()["max_leaf_src"] < 12
+        u = pl.eval(prob.f)
+        for kw in ({"graph": True}, {"serial": True}):
+            pl.set_flags(**kw)
+            assert np.array_equal(pl.eval(prob.f), u)
+        pl.status()
+    assert np.abs(u[idx] - ref).max() <= tol * np.abs(ref).max()
