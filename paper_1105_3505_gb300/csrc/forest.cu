@@ -793,11 +793,22 @@ struct LStripCfg {
 // the number of targets: G = 1 .. 32 lanes take one target and every G-th source of its
 // three rows, and the lanes' sums are added by shuffles; strips of few targets among many
 // sources (clustered points, scattered targets) had kept one warp of six busy.
+// A lane has at least kNearTerms of a target's sources, else the additions across the lanes
+// outweigh its own: 20,000 problems of 60 points, float-float, 1,046 us with as many lanes as
+// there are warps for (32, two terms each), 718 with this line (one thread a target: 782).
+//
+// Binary64: 768 threads of 72 registers leave room on the SM for small launches of the far
+// field (256 threads of 40), the compiler's next step, 80, does not, and 100,003 points then
+// take 348 us a call instead of 305; a bound of 896 threads holds it to 72.  Float-float keeps
+// 80 (400,009 points 495 us; 501 with 72).
 template <typename T>
 struct NearCfg {
     static constexpr int THREADS = sizeof(T) == 8 ? 768 : 192;
+    static constexpr int BOUND = std::is_same<T, double>::value ? 896 : THREADS;
     static constexpr int BLOCKS = sizeof(T) == 8 ? 1 : 6;
 };
+constexpr int kNearTerms = 8;
+
 // A lane's near sum of the 8-byte types.
 //
 // Float-float: four products at a time are summed from zero, their rounding errors gathered in
@@ -853,7 +864,7 @@ struct NearSum<double> {
 };
 
 template <typename T, int BLOCKS>
-__global__ void __launch_bounds__(NearCfg<T>::THREADS, BLOCKS) p2p_list_kernel(
+__global__ void __launch_bounds__(NearCfg<T>::BOUND, BLOCKS) p2p_list_kernel(
     const int4* __restrict__ strips, const int4* __restrict__ strip_rows, const int32_t* __restrict__ n_strips_d,
     const int32_t* __restrict__ Lp, const uint64_t* __restrict__ rl_key, const int32_t* __restrict__ rl_s,
     const int32_t* __restrict__ rl_t, const int32_t* __restrict__ rl_id, int kb, int side, int SW,
@@ -998,9 +1009,11 @@ __global__ void __launch_bounds__(NearCfg<T>::THREADS, BLOCKS) p2p_list_kernel(
         };
         if constexpr (sizeof(T) == 8) {
             const int warps = blockDim.x >> 5;
-            // G = 2^lg lanes per target: at least two units of 32 / G targets per warp
+            // G = 2^lg lanes per target: at least two units of 32 / G targets per warp, and
+            // kNearTerms sources per lane (a target sees three of the strip's columns)
+            const int near = ns_strip * min(3, ncol) / ncol;
             int lg = NearSum<T>::LG_MIN;
-            while (lg < 5 && (nt_strip << lg) < 64 * warps) ++lg;
+            while (lg < 5 && (nt_strip << lg) < 64 * warps && (near >> lg) >= 2 * kNearTerms) ++lg;
             const int G = 1 << lg, sub = lane & (G - 1), per = 32 >> lg;
             const int units = (nt_strip + per - 1) / per;
             for (int unit = warp; unit < units; unit += warps) {

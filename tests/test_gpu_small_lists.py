@@ -1,7 +1,11 @@
-"""P2M of pruned trees and forests on the mixed path (csrc/forest.cu): several operator rows in
-flight where the leaves do not fill the chip, one where they do.
+"""Pruned trees and forests of little work (csrc/forest.cu), where other forms of a kernel run than
+on large ones: P2M with several operator rows in flight where the leaves do not fill the
+chip, the near field with more registers a thread where there is no far field, and its lanes
+per target by the sources that a target has.
 
-Bar: that of the path everywhere in these tests, 1e-6 of the largest value at p = 8 and 16.
+Bars: those of the paths everywhere in these tests (1e-6 of the largest value mixed at p = 8,
+1e-10 float-float and binary64 at p = 16; problems of one leaf have no far field and are held
+to 1e-6 and 1e-12 of sum |f|, the largest |phi| there being below 1).
 """
 import numpy as np
 import pytest
@@ -90,3 +94,25 @@ def test_sparse_tree_in_few_blocks(lfmm, path):
             assert np.array_equal(pl.eval(prob.f), u)
         pl.status()
     assert np.abs(u[idx] - ref).max() <= tol * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("precision", ["df", "fp64"])
+@pytest.mark.parametrize("side", [16, 80])  # one leaf; three by three
+def test_lanes_per_target(lfmm, precision, side):
+    """Every count of sources at which a target gets more lanes, few and many targets."""
+    prec = {"df": lfmm.LFMM_DF, "fp64": lfmm.LFMM_FP64}[precision]
+    rng = np.random.default_rng(side)
+    n = [1, 7, 8, 15, 16, 17, 31, 32, 33, 63, 64, 65, 127, 128, 129, 200] * 2
+    m = [3] * 16 + [150] * 16
+    src = [workloads.distinct_in_box(rng, k, side) for k in n]
+    tgt = [workloads.distinct_in_box(rng, k, side) for k in m]
+    f = [workloads.zero_sum(rng.standard_normal(k)) if k > 1 else np.ones(1) for k in n]
+    so, to = (np.concatenate([[0], np.cumsum(k)]).astype(np.int64) for k in (n, m))
+    S, T = (np.ascontiguousarray(np.concatenate(a).astype(np.int32)) for a in (src, tgt))
+    with lfmm.Forest(S, so, T, to, opts=lfmm.make_opts(prec, 16, 200)) as fo:
+        u = fo.eval(np.concatenate(f))
+        fo.status()
+    for i in range(len(n)):
+        ref = oracle.lattice_sum(src[i], f[i], tgt[i])
+        tol = 1e-12 if side <= 32 else 1e-10
+        assert np.abs(u[to[i]:to[i + 1]] - ref).max() <= tol * np.abs(f[i]).sum()
