@@ -1355,6 +1355,7 @@ int forest_eval(const Forest& F, const DeviceOps& ops, const double* f, T* f_sor
                 if (NP == 32) by_u(std::integral_constant<int, 32>());
                 else by_u(std::integral_constant<int, 64>());
             }
+            LFMM_CUDA_TRY(cudaGetLastError());
             pt.add_launches(1);
         }
     }
