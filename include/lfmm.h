@@ -51,19 +51,26 @@ extern "C" {
 #define LFMM_ECANCELED 8     /* a queued server request was cancelled                   */
 
 /* ---- precision paths ------------------------------------------------------------- */
-/* LFMM_FP64: every step in binary64 (the plain path, relative error <= 1e-10 at p >= 16).
+/* LFMM_FP64: binary64 throughout (the plain path, relative error <= 1e-10 at p >= 16).
  * LFMM_MIXED: near field, expansions and translations in binary32, charges rounded
- *   to binary32, the per-target sum of near and far parts in binary64 (<= 1e-6). */
-#define LFMM_FP64 0   /* every step in binary64 (translations at p > 9: products of       */
-                      /* 53-bit operands split exactly over fp16 tensor-core products)    */
+ *   to binary32, the per-target sum of near and far parts in binary64 (<= 1e-6).
+ * Translations (M2M, M2L, L2L) at p > 9 of the two binary64-accurate paths run on the
+ * tensor cores (tc_min_level below says where): each box's expansion and each operator is
+ * cut into six slices of nine bits under one power of two, so that an entry is kept to
+ * 2^-53 of the largest entry of its expansion or operator (not of itself), and the sliced
+ * products of weight 2^-51 (float-float) or 2^-60 (binary64) of the largest and below are
+ * left out; sums are carried in more than 53 bits.  Measured errors are those of the same
+ * paths with translations in their own arithmetic. */
+#define LFMM_FP64 0   /* every step in binary64; translations as above                    */
 #define LFMM_MIXED 1  /* binary32 near and far field, compensated charge channel,         */
-                      /* tensor-core M2L in three products of 11-bit halves (fp16 on      */
-                      /* uniform levels, TF32 on box lists); binary64 final sum           */
-                      /* (relative error ~1e-7)                                           */
+                      /* tensor-core M2L in three products of 11-bit halves (fp16 under   */
+                      /* one power of two per expansion on uniform levels: 22 bits down   */
+                      /* to 2^-17 of its largest entry, 2^-40 of that below; TF32 on box  */
+                      /* lists: 22 bits of every entry); binary64 final sum (relative     */
+                      /* error ~1e-7)                                                     */
 #define LFMM_DF 2     /* binary64 inputs and outputs, every step in float-float pairs     */
-                      /* (~48 bits) on the FP32 pipes, translations at p > 9 in 53-bit    */
-                      /* split operands on the tensor cores: binary64-level accuracy at a */
-                      /* fraction of the binary64 pipe's cost                             */
+                      /* (~48 bits) on the FP32 pipes, translations as above: binary64-   */
+                      /* level accuracy at a fraction of the binary64 pipe's cost         */
 
 typedef struct lfmm_plan lfmm_plan;
 

@@ -7,8 +7,9 @@
 // K = 27 x 32 source expansions (+ 32 for the parent).  Operands are split into hi + lo
 // parts of 11 bits (round to nearest) and three products hi*hi + hi*lo + lo*hi are formed
 // (the lo*lo term is below 2^-22 relative): on uniform levels in fp16, every row and
-// operator scaled by a power of two (half the operand bytes and half the MMAs of TF32 for
-// the same 22 bits), on box lists in TF32.  The tensor core's fp32 accumulation rounds
+// operator scaled by a power of two (half the operand bytes and half the MMAs of TF32; the
+// same 22 bits down to 2^-17 of the row's largest entry, an absolute 2^-40 of that below), on
+// box lists in TF32.  The tensor core's fp32 accumulation rounds
 // toward zero, and that bias grows linearly with the number of MMAs feeding one
 // accumulator; so every K-step writes fresh TMEM accumulators (hi*hi in one, the small
 // hi*lo + lo*hi terms in another), which are read back after the step and added in

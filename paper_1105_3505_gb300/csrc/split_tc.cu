@@ -7,14 +7,16 @@
 //
 //     x = sum_i a_i 2^(-8 - 9 i),   a_i integer, |a_i| <= 256,   i = 0 .. 5,
 //
-// 53 bits in all, each slice exact in fp16.  A product of two slices is at most 2^16, a sum
+// 53 bits of the row's (operator's) largest entry, each slice exact in fp16; an entry 2^-k of
+// the largest keeps 53 - k.  A product of two slices is at most 2^16, a sum
 // over the 64 coefficients at most 2^22, and the products of equal weight (i + j = g) are
 // added in one fp32 accumulator: up to four of them stay below 2^24, exact whatever the
 // accumulator's rounding; five and more occur only from g = 4 on, 36 bits below the leading
 // weight.  (The splitting follows the error-free matrix products of Ozaki, Ogita, Oishi and
-// Rump, Numer. Algorithms 59 (2012), with power-of-two scaling per row.)  Float-float keeps
-// g <= 5 (21 products, error about 2^-51 of the largest term), binary64 g <= 6 (26
-// products, 2^-60).
+// Rump, Numer. Algorithms 59 (2012), with power-of-two scaling per row.)  Of the 36 products
+// float-float forms those of g <= 5 (21, error about 2^-51 of the largest term), binary64 those
+// of g <= 6 (26, 2^-60).  Rows for the level below that come out under 2^-100 of their reference
+// (sums that cancel to their rounding) are taken for zero.
 //
 // One kernel does the three translations; a work item is 128 target boxes (TMEM lanes) and
 // a chunk of the steps of their sums: 27 interaction offsets (M2L, boxes of one parity
@@ -47,10 +49,11 @@
 // in the downward pass, and small_level_kernel for levels of few boxes (28 and 18 us a
 // level as tensor-core launches) then took eval_df_400k from 968 to 806 us, eval_fp64_100k
 // 636 -> 488, request_178k_1e10 1,456 -> 1,159 and a disk's Krylov iteration 387 -> 188 us.
-// Errors against the exact sum over eight inputs each (geometric means, before -> after):
-// float-float 1.4e-13 -> 1.3e-13, clustered requests 8.8e-14 -> 6.3e-14, a disk's double
-// layer 1.4e-12 -> 9.1e-13, binary64 1.13e-14 -> 1.14e-14 and 3.4e-14 -> 3.4e-14 (these set
-// by the expansions' truncation).
+// Errors against the exact sum, these translations against those on the CUDA cores in the
+// path's own arithmetic, everything else alike (geometric means over twelve inputs each, sizes,
+// orders and leaves over the range in use): kept plans in float-float 8.2e-14 against 8.4e-14,
+// in binary64 1.031e-13 against 1.037e-13 (truncation of the expansions), clustered and
+// uniform requests 4.3e-14 against 4.8e-14, a disk's double layer 1.9e-13 against 3.9e-13.
 #include "split_tc.h"
 
 #include <cuda_fp16.h>
