@@ -51,13 +51,15 @@ struct Job {
 };
 
 // Conservative device footprint of a request before its plan exists (coordinates,
-// buckets, staging, expansions and the tree temporaries), corrected once the plan
-// reports its own size.
+// buckets, staging, expansions and the tree temporaries; float-float plans also sliced rows
+// and sums, about as much as the expansions again), corrected once the plan reports its own
+// size.
 int64_t estimate_bytes(const lfmm_request& r, const lfmm_opts& o) {
     const int64_t n = r.n_src + r.n_tgt;
     const int64_t esz = o.precision == LFMM_MIXED ? 4 : 8;
     const int64_t np = o.p <= 9 ? 32 : 64;
-    return 160 * n + 4 * np * esz * (n / 8 + 1) + ((int64_t)64 << 20);
+    const int64_t per_box = 4 * np * esz + (o.precision == LFMM_MIXED ? 0 : 2200);
+    return 160 * n + per_box * (n / 8 + 1) + ((int64_t)64 << 20);
 }
 
 }  // namespace
